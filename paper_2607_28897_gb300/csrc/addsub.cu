@@ -1,10 +1,11 @@
 // addsub.cu -- batched addition and subtraction (Sec. V-A, Figs. 3 and 4).
 //
-// One CTA per instance.  The CTA's W warps split the instance into W
-// contiguous segments per "super-round"; within its segment a warp reads R
-// rounds of 32 lanes x LPL limbs with coalesced 16-byte loads, straight into
-// registers (step A1: no shared-memory staging is needed because each limb
-// is used by exactly one lane).
+// One CTA per instance (one warp, several to a CTA, for short ones).  The
+// CTA's W warps split the instance into W contiguous segments per
+// "super-round"; within its segment a warp reads R rounds of 32 lanes x LPL
+// limbs with coalesced loads (16 bytes a lane where n is even and the
+// buffers are aligned), straight into registers (step A1: no shared-memory
+// staging is needed because each limb is used by exactly one lane).
 //
 // Carry propagation (step A2) is the exclusive (generate, propagate) scan of
 // Fig. 3 evaluated in three levels:
@@ -17,26 +18,48 @@
 // (Fig. 4, f2).  Subtraction is the same scan with generate = (a < b) and
 // propagate = (a == b), applied as a borrow.
 //
+// The add chain a + b + ... + b (k additions, bigint_add_chain) is the same
+// pass over a_j + k b_j: that sum's high word (at most 255) belongs to limb
+// j + 1, so the low words and the high words one limb up are added with one
+// carry scan, whatever k is.
+//
 // HBM traffic is the algorithmic minimum: 2 limbs read and 1 written per
 // limb position (Table I's 3 x NumInsts x NumBits / 8 bytes).
 #include "common.cuh"
 
 namespace bigint {
 
-template <bool SUB, int LPL, int R>
+// Operations of k_addsub: a + b, a - b, and a + k b (the add chain's k
+// additions at once, k <= 255).
+enum AddSubMode { ADD = 0, SUB = 1, CHAIN = 2 };
+
+// WPI: one warp per instance (n at most one warp's segment), WPI_WARPS
+// instances per CTA and no block barrier.
+constexpr int WPI_WARPS = 8;
+
+template <int MODE, int LPL, int R, bool WPI>
 __global__ void __launch_bounds__(1024)
-    k_addsub(const uint64_t *__restrict__ A, const uint64_t *__restrict__ Bv,
-             uint64_t *__restrict__ Out, uint8_t *__restrict__ carry_out, int n) {
+    k_addsub(const uint64_t *A, const uint64_t *B, uint64_t *Out,
+             uint8_t *__restrict__ carry_out, int64_t count, int n, uint32_t k) {
   constexpr int SEG = 32 * LPL * R;  // limbs per warp per super-round
   __shared__ uint32_t s_g[32], s_p[32];
+  __shared__ uint32_t s_hi;   // CHAIN: high word of the super-round's last limb
+  __shared__ uint32_t s_top;  // CHAIN: high word of limb n - 1
 
-  const int64_t inst = blockIdx.x;
   const uint32_t lane = lane_id();
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
+  const int warp = WPI ? 0 : threadIdx.x >> 5;
+  const int nwarps = WPI ? 1 : blockDim.x >> 5;
+  const int64_t inst =
+      WPI ? (int64_t)blockIdx.x * WPI_WARPS + (threadIdx.x >> 5) : (int64_t)blockIdx.x;
+  if (WPI && inst >= count) return;  // the whole warp: no block barrier below
   const uint64_t *a = A + inst * (int64_t)n;
-  const uint64_t *b = Bv + inst * (int64_t)n;
+  const uint64_t *b = B + inst * (int64_t)n;
   uint64_t *out = Out + inst * (int64_t)n;
+  uint32_t top = 0;  // CHAIN, WPI: high word of limb n - 1
+  if (MODE == CHAIN && !WPI) {
+    if (threadIdx.x == 0) s_hi = 0;
+    __syncthreads();
+  }
 
   uint32_t cin_block = 0;  // carry into the current super-round
   for (int base = 0; base < n; base += SEG * nwarps) {
@@ -59,22 +82,54 @@ __global__ void __launch_bounds__(1024)
         bv[r][0] = j < n ? __ldcs(b + j) : 0;
       }
     }
+    uint32_t hprev = 0;  // CHAIN: high word of the limb below this round's first
+    if (MODE == CHAIN && !WPI) {
+      // the warp's first limb takes the high word of the limb below it: from
+      // the super-round before for warp 0, recomputed from memory otherwise
+      // (this super-round stores nothing before its first barrier)
+      if (lane == 0) {
+        if (warp == 0) hprev = s_hi;
+        else if (wbase <= n) {
+          const uint64_t lo = (uint64_t)k * b[wbase - 1], t = a[wbase - 1] + lo;
+          hprev = (uint32_t)__umul64hi(k, b[wbase - 1]) + (t < lo);
+        }
+      }
+    }
     // ---- A2 level 1: per-limb sums and the lane's (g, p) per round
     uint64_t s[R][LPL];
     uint32_t gbits = 0, pbits = 0;  // per-limb generate/propagate, bit r*LPL+l
     WarpCarry wc[R];
+    uint32_t hlast = 0;
 #pragma unroll
     for (int r = 0; r < R; r++) {
       uint32_t g = 0, p = 1;
+      uint32_t h[LPL];  // CHAIN: high words (at most 255) of the round's limbs
+      if (MODE == CHAIN) {
+#pragma unroll
+        for (int l = 0; l < LPL; l++) {
+          const uint64_t lo = (uint64_t)k * bv[r][l], t = av[r][l] + lo;
+          h[l] = (uint32_t)__umul64hi(k, bv[r][l]) + (t < lo);
+          av[r][l] = t;
+          if (wbase + r * 32 * LPL + (int)lane * LPL + l == n - 1) {
+            if (WPI) top = h[l]; else s_top = h[l];
+          }
+        }
+        const uint32_t below = __shfl_up_sync(FULL, h[LPL - 1], 1);
+        bv[r][0] = lane == 0 ? hprev : below;
+        if constexpr (LPL == 2) bv[r][1] = h[0];
+        hlast = h[LPL - 1];
+        hprev = __shfl_sync(FULL, hlast, 31);
+      }
 #pragma unroll
       for (int l = 0; l < LPL; l++) {
         uint64_t x = av[r][l], y = bv[r][l];
-        uint64_t t = SUB ? x - y : x + y;
-        // positions past the end pass carries through, so the carry out of
-        // the last real limb reaches the end of the warp and of the block
-        const bool in = wbase + r * 32 * LPL + (int)lane * LPL + l < n;
-        uint32_t gl = in && (SUB ? (x < y) : (t < x));
-        uint32_t pl = !in || (SUB ? (t == 0) : (t == ~0ull));
+        uint64_t t = MODE == SUB ? x - y : x + y;
+        // positions past the end pass carries through, so the carry
+        // out of the last limb reaches the end of the warp and of the block
+        const int j = wbase + r * 32 * LPL + (int)lane * LPL + l;
+        const bool in = j < n;
+        uint32_t gl = in && (MODE == SUB ? (x < y) : (t < x));
+        uint32_t pl = !in || (MODE == SUB ? (t == 0) : (t == ~0ull));
         s[r][l] = t;
         gbits |= gl << (r * LPL + l);
         pbits |= pl << (r * LPL + l);
@@ -83,21 +138,27 @@ __global__ void __launch_bounds__(1024)
       }
       wc[r] = warp_gp(g, p);
     }
-    // ---- A2 level 2: fold the rounds into the warp's (g, p)
-    uint32_t wg = 0, wp = 1;
+    uint32_t c = 0, cout_block;
+    if (WPI) {
+      cout_block = 0;  // known after the last round below
+    } else {
+      // ---- A2 level 2: fold the rounds into the warp's (g, p)
+      uint32_t wg = 0, wp = 1;
 #pragma unroll
-    for (int r = 0; r < R; r++) {
-      wg = warp_carry_out(wc[r], 0) | (warp_all_propagate(wc[r]) & wg);
-      wp = wp & warp_all_propagate(wc[r]);
+      for (int r = 0; r < R; r++) {
+        wg = warp_carry_out(wc[r], 0) | (warp_all_propagate(wc[r]) & wg);
+        wp = wp & warp_all_propagate(wc[r]);
+      }
+      if (lane == 0) { s_g[warp] = wg; s_p[warp] = wp; }
+      __syncthreads();
+      // ---- A2 level 3: resolve the warps of the block
+      const uint32_t gw = (int)lane < nwarps ? s_g[lane] : 0;
+      const uint32_t pw = (int)lane < nwarps ? s_p[lane] : 0;
+      const uint64_t cm = warp_carries(warp_gp(gw, pw), cin_block);
+      c = (uint32_t)(cm >> warp) & 1u;
+      cout_block = (uint32_t)(cm >> nwarps) & 1u;
+      if (MODE == CHAIN && warp == nwarps - 1 && lane == 31) s_hi = hlast;
     }
-    if (lane == 0) { s_g[warp] = wg; s_p[warp] = wp; }
-    __syncthreads();
-    // ---- A2 level 3: resolve the warps of the block
-    const uint32_t gw = (int)lane < nwarps ? s_g[lane] : 0;
-    const uint32_t pw = (int)lane < nwarps ? s_p[lane] : 0;
-    const uint64_t cm = warp_carries(warp_gp(gw, pw), cin_block);
-    uint32_t c = (uint32_t)(cm >> warp) & 1u;
-    const uint32_t cout_block = (uint32_t)(cm >> nwarps) & 1u;
     // ---- apply the carries (Fig. 4, f2) and store
 #pragma unroll
     for (int r = 0; r < R; r++) {
@@ -107,7 +168,7 @@ __global__ void __launch_bounds__(1024)
       uint64_t res[LPL];
 #pragma unroll
       for (int l = 0; l < LPL; l++) {
-        res[l] = SUB ? s[r][l] - cl : s[r][l] + cl;
+        res[l] = MODE == SUB ? s[r][l] - cl : s[r][l] + cl;
         const uint32_t gl = (gbits >> (r * LPL + l)) & 1u;
         const uint32_t pl = (pbits >> (r * LPL + l)) & 1u;
         cl = gl | (pl & cl);
@@ -123,41 +184,82 @@ __global__ void __launch_bounds__(1024)
         if (j < n) __stcs(out + j, res[0]);
       }
     }
-    cin_block = cout_block;
-    __syncthreads();  // s_g / s_p are rewritten by the next super-round
+    cin_block = WPI ? c : cout_block;
+    if (!WPI) __syncthreads();  // s_g / s_p are rewritten by the next super-round
   }
-  if (carry_out != nullptr && threadIdx.x == 0) carry_out[inst] = (uint8_t)cin_block;
+  if (carry_out == nullptr) return;
+  if (WPI) {
+    if (MODE == CHAIN) top = __reduce_max_sync(FULL, top);  // one lane holds it
+    if (lane == 0) carry_out[inst] = (uint8_t)(cin_block + top);
+  } else if (threadIdx.x == 0) {
+    carry_out[inst] = (uint8_t)(cin_block + (MODE == CHAIN ? s_top : 0u));
+  }
 }
 
-// Launch shape: R rounds per warp and W warps per CTA, chosen from n so that
-// small instances use few rounds (more CTAs in flight) and large ones use
-// up to 32 warps x 4 rounds (16 KiB of loads in flight per warp).
-template <bool SUB, int LPL>
-static int launch_lpl(const uint64_t *a, const uint64_t *b, uint64_t *out,
-                      uint8_t *carry, int64_t count, int n, cudaStream_t st) {
-  int R = n >= 4096 ? 4 : (n >= 1024 ? 2 : 1);
-  int per_warp = 32 * LPL * R;
-  int W = (n + per_warp - 1) / per_warp;
-  if (W > 32) W = 32;
-  if (W < 1) W = 1;
-  dim3 grid((unsigned)count), block(32 * W);
-  switch (R) {
-    case 4: k_addsub<SUB, LPL, 4><<<grid, block, 0, st>>>(a, b, out, carry, n); break;
-    case 2: k_addsub<SUB, LPL, 2><<<grid, block, 0, st>>>(a, b, out, carry, n); break;
-    default: k_addsub<SUB, LPL, 1><<<grid, block, 0, st>>>(a, b, out, carry, n); break;
+// Launch shape.  Bound: HBM (24 bytes a limb), so what matters is loads in
+// flight on every SM at every moment: one CTA that holds the SM alone reads,
+// waits, then writes.  So a warp always takes R = 4 rounds where the operand
+// has them, and a CTA at most max_warps warps (more limbs: more
+// super-rounds), which leaves an SM several CTAs in different phases.
+// Measured, operand arrays of 2^32 bits: 8192 limbs 5.7 TB/s with 32 warps
+// in one super-round (one CTA per SM) -> 7.0 with 8 warps in four; 1537
+// limbs (8-byte accesses) 5.3 TB/s with two rounds a warp -> 7.1 with four.
+// The chain's extra arithmetic wants more CTAs still: 6.8 against 6.5 TB/s
+// at 8192 limbs with 4 instead of 8 warps.  Operands of at most one warp's
+// segment go one warp per instance: a CTA each starts and ends too often
+// (64 limbs: 3.0 TB/s).  A batch of at most two instances per SM has nothing
+// to overlap with, so there one super-round of up to 32 warps is the fastest.
+static int sm_count() {
+  static int sms = 0;
+  if (sms == 0) {
+    int dev = 0, v = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 0;
+    sms = v;
   }
+  return sms;
+}
+
+template <int MODE, int LPL>
+static int launch_lpl(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
+                      int64_t count, int n, uint32_t k, cudaStream_t st) {
+  constexpr int SEG = 32 * LPL * 4;
+  const int max_warps = count <= 2 * sm_count() ? 32 : (MODE == CHAIN ? 4 : 8);
+  if (n <= SEG) {
+    const unsigned grid = (unsigned)((count + WPI_WARPS - 1) / WPI_WARPS);
+    if (n <= SEG / 4)
+      k_addsub<MODE, LPL, 1, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
+    else if (n <= SEG / 2)
+      k_addsub<MODE, LPL, 2, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
+    else
+      k_addsub<MODE, LPL, 4, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
+    return bigint_launch_status();
+  }
+  const int need = (n + SEG - 1) / SEG;  // warps for one super-round
+  const int rounds = (need + max_warps - 1) / max_warps;
+  const int W = (need + rounds - 1) / rounds;
+  k_addsub<MODE, LPL, 4, false><<<(unsigned)count, 32 * W, 0, st>>>(a, b, out, carry, count, n, k);
   return bigint_launch_status();
+}
+
+template <int MODE>
+static int launch_mode(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
+                       int64_t count, int n, uint32_t k, cudaStream_t st) {
+  const bool vec = (n % 2 == 0) && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)out) % 16 == 0);
+  return vec ? launch_lpl<MODE, 2>(a, b, out, carry, count, n, k, st)
+             : launch_lpl<MODE, 1>(a, b, out, carry, count, n, k, st);
 }
 
 int launch_addsub(bool sub, const uint64_t *a, const uint64_t *b, uint64_t *out,
                   uint8_t *carry, int64_t count, int n, cudaStream_t st) {
-  const bool vec = (n % 2 == 0) && (((uintptr_t)a | (uintptr_t)b | (uintptr_t)out) % 16 == 0);
-  if (sub) {
-    return vec ? launch_lpl<true, 2>(a, b, out, carry, count, n, st)
-               : launch_lpl<true, 1>(a, b, out, carry, count, n, st);
-  }
-  return vec ? launch_lpl<false, 2>(a, b, out, carry, count, n, st)
-             : launch_lpl<false, 1>(a, b, out, carry, count, n, st);
+  return sub ? launch_mode<SUB>(a, b, out, carry, count, n, 0, st)
+             : launch_mode<ADD>(a, b, out, carry, count, n, 0, st);
+}
+
+int launch_add_chain(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
+                     int64_t count, int n, int k, cudaStream_t st) {
+  return launch_mode<CHAIN>(a, b, out, carry, count, n, (uint32_t)k, st);
 }
 
 }  // namespace bigint

@@ -3,93 +3,12 @@
 // on chip (registers) or in a per-CTA scratch region that stays in L2, so
 // global-memory traffic is that of one operation.
 //
-//   add chain:  r = a + b + ... + b  (k additions, k = 6 is Table I's 6-Add),
-//               each a full carry-propagating addition mod B^n; carry_out is
-//               the number of wrap-arounds, floor((a + k b) / B^n).
 //   poly:       r = (a a + b) (b b + b) + a b  mod B^n  (Table II's Poly: four
 //               multiplications and three additions, every value kept to n
 //               limbs as the paper's same-width multiply and add do).
 #include "divcore.cuh"
 
 namespace bigint {
-
-// ---------------------------------------------------------------------------
-// Carry into this thread's segment when every thread holds a segment of
-// consecutive limbs in thread order with (generate, propagate) = (g, p) and
-// the block gets carry cin; *cout = carry out of the last thread.  The scan
-// of Fig. 3 with warp ballots, then across warps (blk_addsub's resolve).
-// ---------------------------------------------------------------------------
-__device__ __forceinline__ uint32_t blk_segment_carry(uint32_t g, uint32_t p, uint32_t cin,
-                                                      uint32_t *sm, uint32_t *cout) {
-  const uint32_t lane = lane_id();
-  const int warp = threadIdx.x >> 5;
-  const int nwarps = blockDim.x >> 5;
-  const WarpCarry wc = warp_gp(g, p);
-  if (lane == 0) {
-    sm[warp] = warp_carry_out(wc, 0);
-    sm[32 + warp] = warp_all_propagate(wc);
-  }
-  __syncthreads();
-  const uint32_t gw = (int)lane < nwarps ? sm[lane] : 0;
-  const uint32_t pw = (int)lane < nwarps ? sm[32 + lane] : 1;
-  const uint64_t cm = warp_carries(warp_gp(gw, pw), cin);
-  const uint32_t cwarp = (uint32_t)(cm >> warp) & 1u;
-  *cout = (uint32_t)(cm >> nwarps) & 1u;
-  const uint64_t lc = warp_carries(wc, cwarp);
-  __syncthreads();  // sm is reused by the next call
-  return (uint32_t)(lc >> lane) & 1u;
-}
-
-// One CTA per instance; thread t holds limbs [t L, t L + L) of the running
-// sum and of b in registers for all k additions.
-template <int L>
-__global__ void __launch_bounds__(1024)
-    k_add_chain(const uint64_t *__restrict__ A, const uint64_t *__restrict__ Bm,
-                uint64_t *__restrict__ Out, uint8_t *carry_out, int n, int k) {
-  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
-  const int64_t inst = blockIdx.x;
-  const uint64_t *a = A + inst * (int64_t)n, *b = Bm + inst * (int64_t)n;
-  uint64_t *o = Out + inst * (int64_t)n;
-  const int base = (int)threadIdx.x * L;
-  int nv = n - base;
-  nv = nv < 0 ? 0 : (nv > L ? L : nv);
-  uint64_t r[L], y[L];
-#pragma unroll
-  for (int j = 0; j < L; j++) {
-    r[j] = j < nv ? a[base + j] : 0ull;
-    y[j] = j < nv ? b[base + j] : 0ull;
-  }
-  uint32_t total = 0;
-  for (int it = 0; it < k; it++) {
-    uint32_t c = 0, all_ones = 1;
-#pragma unroll
-    for (int j = 0; j < L; j++) {
-      if (j < nv) {
-        const uint64_t t = r[j] + y[j];
-        const uint64_t t2 = t + c;
-        c = (uint32_t)(t < r[j]) | (uint32_t)(t2 < t);
-        r[j] = t2;
-        all_ones &= (uint32_t)(t2 == ~0ull);
-      }
-    }
-    // a segment past the end passes carries through
-    const uint32_t g = nv > 0 ? c : 0u, p = nv > 0 ? (c == 0u && all_ones) : 1u;
-    uint32_t cout;
-    uint32_t cin = blk_segment_carry(g, p, 0u, scr, &cout);
-#pragma unroll
-    for (int j = 0; j < L; j++) {
-      if (j < nv && cin) {
-        r[j] += 1;
-        cin = r[j] == 0 ? 1u : 0u;
-      }
-    }
-    total += cout;
-  }
-#pragma unroll
-  for (int j = 0; j < L; j++)
-    if (j < nv) o[base + j] = r[j];
-  if (carry_out && threadIdx.x == 0) carry_out[inst] = (uint8_t)total;
-}
 
 // ---------------------------------------------------------------------------
 // Poly: persistent CTAs; per instance four low-part products (tensor cores
@@ -141,19 +60,6 @@ __global__ void __launch_bounds__(TC ? 2 * NT + 32 : 512, TC ? 256 / NT : 1)
 // ---------------------------------------------------------------------------
 // Host side
 // ---------------------------------------------------------------------------
-int launch_add_chain(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
-                     int64_t count, int n, int k, cudaStream_t st) {
-  if (count == 0) return BIGINT_OK;
-  if (n <= 8 * 1024) {
-    const int T = ((n + 7) / 8 + 31) / 32 * 32;
-    k_add_chain<8><<<(unsigned)count, T, 0, st>>>(a, b, out, carry, n, k);
-  } else {
-    const int T = ((n + 15) / 16 + 31) / 32 * 32;
-    k_add_chain<16><<<(unsigned)count, T, 0, st>>>(a, b, out, carry, n, k);
-  }
-  return bigint_launch_status();
-}
-
 namespace {
 
 template <bool TC, int NT, int G>

@@ -104,3 +104,28 @@ def test_config_sweep_full_size(bi, orc, n):
     # residues: (a - b) + b == a mod p for every instance
     for p in SMALL_PRIMES[:1]:
         assert np.array_equal((residues(to_host(d), p) + residues(sb, p)) % p, residues(sa, p))
+
+
+@pytest.mark.parametrize("n", [64, 65, 128, 130, 255, 256, 257, 258, 1537, 2050, 4097, 8194])
+def test_launch_shapes(bi, orc, n):
+    """Batches of more than two instances per SM: one warp per instance up to
+    a warp's segment (128 limbs for odd n, 256 for even), then CTAs of a few
+    warps in several super-rounds; the stress pairs' carries cross warps and
+    super-rounds, in the first and the last rows of the batch."""
+    import torch
+    from paper_2607_28897_gb300 import inputs
+
+    count = 645
+    a, b = inputs.limbs(300 + n, count, n), inputs.limbs(400 + n, count, n)
+    sa, sb = inputs.stress_pairs(n)
+    a[:8], b[:8], a[-8:], b[-8:] = sa, sb, sa, sb
+    check_add(bi, orc, a, b)
+    check_sub(bi, orc, a, b)
+    for k in (1, 255):
+        da = to_dev(a)
+        carry = torch.zeros(count, dtype=torch.uint8, device="cuda")
+        got = to_host(bi.add_chain(da, to_dev(b), k, out=da, carry=carry))  # in place
+        for i in [*range(9), count // 2, *range(count - 9, count)]:
+            want, c = orc.add_chain(a[i], b[i], k)
+            assert np.array_equal(got[i], want), (i, k)
+            assert int(carry[i]) == c, (i, k)
