@@ -75,7 +75,7 @@ int bigint_sub(const uint64_t *a, const uint64_t *b, uint64_t *out,
 /* ---- multiplication (Sec. V-B, Fig. 5) ----------------------------------
  * out = a * b, the FULL product of na + nb limbs per instance: the
  * schoolbook convolution C_k = sum_{i+j=k} a_i b_j of Sec. V-B, exact.
- * When the shorter operand has 256 limbs or more (and fits one SM's shared
+ * When the shorter operand has 64 limbs or more (and fits one SM's shared
  * memory) the convolution runs on the tensor cores: the operands as signed
  * base-256 digits, the convolution as fp16 matrix products (tcgen05.mma,
  * Toeplitz blocks of one operand times shifted blocks of the other) with
@@ -453,7 +453,7 @@ int bigint_host_sync(void);
  * Selects the kernel variant an operation uses from now on (process-wide,
  * not thread-safe; call it before launching work).  op 0 = multiply:
  *   variant 0 (default): chosen by operand size from GB300 measurements (the
- *   tensor-core product from a shorter operand of 256 limbs, integer
+ *   tensor-core product from a shorter operand of 64 limbs, integer
  *   products below), or the variant bigint_tune recorded for the size class
  *   variant 8: integer product, 29-bit digits, 16-column chunks
  *   variant 9: integer product, 28-bit digits, 8-column chunks

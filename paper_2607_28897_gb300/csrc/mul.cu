@@ -138,18 +138,22 @@ static int launch_kara(const uint64_t *a, const uint64_t *b, uint64_t *out, int6
 }
 
 // Variant table (see bigint_set_variant).  Variant 0 picks by size from
-// measurements on GB300 (full-product sweep, 2^32-bit operand arrays): the
-// tensor-core product (tcmul.cu) once the shorter operand has TC_MIN_LIMBS
-// limbs and fits shared memory; below, the integer product with 28-bit
-// digits and 8-column chunks (variant 9), or 29-bit digits and 16-column
-// chunks (variant 8) past 1535 limbs.  A size class the tuner has measured
+// measurements on GB300: the tensor-core product (tcmul.cu) once the shorter
+// operand has TC_MIN_LIMBS limbs and fits shared memory; below, one warp per
+// product (variant 11) for operands of at most SMALL_LIMBS limbs (65536
+// products of 48 limbs 324 us, 449 us as variant 9), else the integer
+// product with 28-bit digits and 8-column chunks (variant 9), or 29-bit
+// digits and 16-column chunks (variant 8) past 1535 limbs.  A size class the tuner has measured
 // (bigint_tune) takes its recorded variant instead.
 size_t mul_tc_smem(int na, int nb);
 int launch_mul_tc(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t count, int na,
                   int nb, int nout, cudaStream_t st, int force_nt);
 
-// Shorter operand (limbs) from which the default is the tensor-core product.
-constexpr int TC_MIN_LIMBS = 256;
+// Shorter operand (limbs) from which the default is the tensor-core product:
+// 65536 products of 64 limbs 402 us against 504 (one warp each) and 586 us
+// (variant 9), of 128 limbs 579 against 1854 us, 1000 x 64 limbs (16384)
+// 505 against 1033 us; at 48 limbs the warp form is ahead (324 : 376).
+constexpr int TC_MIN_LIMBS = 64;
 
 static int g_mul_variant = 0;
 // Tuned variant per size class (class c: operands of [2^c, 2^(c+1)) limbs),
@@ -186,7 +190,7 @@ int mul_variant_for(int na, int nb, int nout) {
     if (nmin >= TC_MIN_LIMBS && mul_tc_smem(na, nb) > 0)
       v = 12;
     else
-      v = nmax < 1536 ? 9 : 8;
+      v = nmax <= SMALL_LIMBS ? 11 : (nmax < 1536 ? 9 : 8);
   }
   const bool square_full = na == nb && nout == na + nb && na >= 64;
   if (v == 10 && !square_full) v = 8;                // Karatsuba: square full products only

@@ -5,6 +5,7 @@
 // (tccore.cuh: the digit convolution as tcgen05 fp16 MMAs with exact fp32
 // accumulation, Sec. V-B's schoolbook product on the tensor cores).
 #include "tccore.cuh"
+#include "tcone.cuh"
 
 namespace bigint {
 namespace tcm {
@@ -37,6 +38,31 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
   }
   if (c.aborted && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
   tc_release<NT>(c);
+}
+
+// The same for products whose shorter operand has at most ONE_MAX limbs
+// (tcone.cuh): NT tensor-memory columns and 32 W threads per CTA, 512 / NT
+// CTAs per SM.
+template <int NT, int W>
+__global__ void __launch_bounds__(32 * W, 512 / NT)
+    k_mul_one(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
+              uint64_t *__restrict__ Out, int nx, int ny, int nout, int64_t count, int64_t sx,
+              int64_t sy, int64_t so, int lo, int *abort_flag) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ OneShared sh;
+  OneCtx c;
+  one_init<NT>(c, sm, &sh);
+  for (int64_t inst = blockIdx.x; inst < count; inst += gridDim.x) {
+    const int64_t next = inst + gridDim.x;
+    if (threadIdx.x == 0 && next < count) {
+      prefetch_l2(X + next * sx, 8 * (size_t)nx);
+      prefetch_l2(Y + next * sy, 8 * (size_t)ny);
+    }
+    if (!one_product<NT, W>(c, X + inst * sx, nx, Y + inst * sy, ny, Out + inst * so, nout, lo))
+      break;
+  }
+  if (c.aborted && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
+  one_release<NT>(c);
 }
 
 // Split products: unit u is tile u % T of product u / T (tc_product's split
@@ -296,8 +322,8 @@ static int launch_shape(TcShape sh, const TcArgs &A, int64_t count, int nx, int 
 // limbs, low nout limbs, band start lo), following tc_product's tile loop:
 // each MMA of N columns costs the larger of its math (128 x N x 16 fp16
 // multiply-adds at ~6750 flop/cycle per SM) and its operand reads from
-// shared memory (4 KB of A plus 32 N bytes of B at 128 bytes/cycle); the
-// tiles (each a fixed cost: its first Hankel build, last drain and column
+// shared memory (4 KB of A plus 32 N bytes of B at 128 bytes/cycle), and at
+// least 46 (the tightest issue loop); the tiles (each a fixed cost: its first Hankel build, last drain and column
 // sums) count 4000 cycles.  tiles_out: the product's tiles.
 static double tc_model(TcShape sh, int nx, int ny, int nout, int lo, int *tiles_out = nullptr) {
   const ShapeInfo &I = SHAPES[sh];
@@ -321,7 +347,8 @@ static double tc_model(TcShape sh, int nx, int ny, int nout, int lo, int *tiles_
       const int ca = (c0 > S * e ? c0 : S * e) - c0, cb = (c0 + W < S * e + mx ? c0 + W : S * e + mx) - c0;
       const int N = ((cb + 15) & ~15) - (ca & ~15);
       const double math = 4096.0 * N / 6750.0, rd = 32.0 + N / 4.0;
-      cyc += (KB / 16) * (math > rd ? math : rd);
+      const double mma = math > rd ? math : rd;
+      cyc += (KB / 16) * (mma > 46 ? mma : 46);
     }
   }
   if (tiles_out) *tiles_out = tiles;
@@ -384,10 +411,116 @@ static TcShape best_shape(int nx, int ny, int nout, int lo, int kb_mask, int nt,
   return best;
 }
 
-// force: 0 (the 128-digit-block shape by the model, below) or one of the
-// autotuner's candidates -- TC_FORCE_64 / _128 / _256 (128-digit blocks,
-// that tile) and TC_FORCE_N64 / _N32 (narrow blocks).  The shorter operand
-// becomes x.
+// ---- one-drain products (tcone.cuh) -------------------------------------------
+// Warps per CTA.  More of them (8 / 16) shorten a lone product's phases by
+// 15 % but not a batch, where the CTAs sharing the SM overlap anyway
+// (512-limb products 2451 against 2167 us per 65536).
+template <int NT>
+constexpr int one_warps() { return NT == 128 ? 4 : 8; }
+
+// Attributes of k_mul_one<NT>: its largest dynamic shared memory, and the
+// CTAs of a given dynamic shared memory resident on one SM (TMEM allows
+// 512 / NT).
+struct OneAttr {
+  int dyn = 0, smem_sm = 0, overhead = 0;
+  bool ok = false;
+};
+
+template <int NT>
+static const OneAttr &one_attr() {
+  static const OneAttr A = [] {
+    OneAttr a;
+    auto *kern = tcm::k_mul_one<NT, one_warps<NT>()>;
+    int dev = 0, optin = 0, reserved = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&a.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) !=
+            cudaSuccess ||
+        cudaFuncGetAttributes(&fa, kern) != cudaSuccess)
+      return a;
+    a.dyn = optin - (int)fa.sharedSizeBytes;
+    a.overhead = (int)fa.sharedSizeBytes + reserved;
+    a.ok = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, a.dyn) ==
+           cudaSuccess;
+    return a;
+  }();
+  return A;
+}
+
+template <int NT>
+static int one_per_sm(size_t smem) {
+  const OneAttr &a = one_attr<NT>();
+  const int per_sm = a.smem_sm / (int)(smem + a.overhead);
+  return per_sm > 512 / NT ? 512 / NT : (per_sm < 1 ? 1 : per_sm);
+}
+
+// Shared memory of a product (x of nx, y of ny limbs, low nout limbs, band
+// start lo) in the form with NT-column tiles (0: it does not take it), and
+// its modelled time on one SM in tensor-core cycles, comparable with
+// shape_cost: the MMAs (their math, their operands' reads, at least 46
+// cycles each), the shared-memory cycles of a tile's Hankel matrices (16 per
+// block) and transposes (8 per column), and the part of a tile's ~6000
+// cycles of latency and limb work that the CTAs sharing the SM do not hide.
+// Fitted to 25 measured shapes of 8 to 9000 limbs; within 15 % of them.
+template <int NT>
+static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
+  constexpr int R = tcm::ONE_R, S = tcm::ONE_S, W = one_warps<NT>();
+  if ((nx < ny ? nx : ny) > tcm::ONE_MAX || !one_attr<NT>().ok) return 0;
+  const tcm::OneLayout L = tcm::one_layout<W>(nx, ny, 0);
+  int blocks = 0, tiles = 0;
+  double cyc = nx;
+  for (int c0 = lo > 0 ? (lo / R - (S - 1) > 0 ? lo / R - (S - 1) : 0) : 0; R * c0 < nout;
+       c0 += NT) {
+    int Wd = L.cmma + S - 1 - c0 < NT ? L.cmma + S - 1 - c0 : NT;
+    const int need = (nout - R * c0 + R - 1) / R;
+    if (Wd > need) Wd = need;
+    Wd = (Wd + 15) & ~15;
+    int e_lo, e_hi;
+    tcm::one_blocks(L.mx, L.ey, c0, Wd, e_lo, e_hi);
+    const int nb = e_hi >= e_lo ? e_hi - e_lo + 1 : 0;
+    if (nb > blocks) blocks = nb;
+    tiles++;
+    cyc += 16.0 * nb + 8.0 * Wd;
+    for (int e = e_lo; e <= e_hi; e++) {
+      const int ca = (c0 > S * e ? c0 : S * e) - c0;
+      const int cb = (c0 + Wd < S * e + L.mx ? c0 + Wd : S * e + L.mx) - c0;
+      const int N = ((cb + 15) & ~15) - (ca & ~15);
+      const double math = 4096.0 * N / 6750.0, rd = 32.0 + N / 4.0;
+      const double mma = math > rd ? math : rd;
+      cyc += 2 * (mma > 46 ? mma : 46);
+    }
+  }
+  const uint32_t total = tcm::one_layout<W>(nx, ny, blocks).total;
+  if (total > (uint32_t)one_attr<NT>().dyn) return 0;
+  if (cost != nullptr) {
+    const int per_sm = one_per_sm<NT>(total);
+    *cost = cyc + tiles * (per_sm == 1 ? 7400.0 : 6000.0 / per_sm);
+  }
+  return total;
+}
+
+template <int NT>
+static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
+  constexpr int W = one_warps<NT>();
+  const size_t smem = one_plan<NT>(nx, ny, nout, A.lo, nullptr);
+  if (smem == 0) return BIGINT_EINVAL;
+  if (count == 0) return BIGINT_OK;
+  const int sms = sm_count();
+  if (sms == 0) return BIGINT_ECUDA;
+  const int64_t slots = (int64_t)sms * one_per_sm<NT>(smem);
+  const int64_t grid = count < slots ? count : slots;
+  tcm::k_mul_one<NT, W><<<(unsigned)grid, 32 * W, smem, st>>>(
+      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag);
+  return bigint_launch_status();
+}
+
+// force: 0 (the one-drain or 128-digit-block shape by the models above and
+// below) or one of the autotuner's candidates -- TC_FORCE_64 / _128 / _256
+// (128-digit blocks, that tile) and TC_FORCE_N64 / _N32 (narrow blocks).
 int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
                      cudaStream_t st, int force) {
@@ -430,6 +563,29 @@ int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
       const int tn = nx; nx = ny; ny = tn;
       sh = sw;
       keep = swap;
+    }
+  }
+  if (force == 0) {
+    // the one-drain form, either operand as x, where its model is cheaper
+    double best = keep;
+    int nt1 = 0;
+    bool sw = false;
+    for (int k = 0; k < (nx == ny ? 1 : 2); k++) {
+      const int mx = k ? ny : nx, my = k ? nx : ny;
+      double c;
+      if (one_plan<128>(mx, my, nout, lo, &c) && (best < 0 || c < best))
+        best = c, nt1 = 128, sw = k != 0;
+      if (one_plan<256>(mx, my, nout, lo, &c) && (best < 0 || c < best))
+        best = c, nt1 = 256, sw = k != 0;
+    }
+    if (nt1 != 0) {
+      TcArgs B = A;
+      if (sw) {
+        B.x = A.y; B.y = A.x; B.sx = A.sy; B.sy = A.sx;
+      }
+      const int mx = sw ? ny : nx, my = sw ? nx : ny;
+      return nt1 == 128 ? launch_one<128>(B, count, mx, my, nout, st)
+                        : launch_one<256>(B, count, mx, my, nout, st);
     }
   }
   if (keep < 0) return BIGINT_EINVAL;
