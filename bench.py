@@ -214,7 +214,7 @@ def cpu_model() -> str:
 # --------------------------------------------------------------------------
 # committed ncu traffic of the multiply kernel, valid only for its source
 # --------------------------------------------------------------------------
-def kernel_source_hash(files=("tccore.cuh", "tcmul.cu", "mul.cu", "blockops.cuh",
+def kernel_source_hash(files=("tccore.cuh", "tcone.cuh", "tcmul.cu", "mul.cu", "blockops.cuh",
                               "common.cuh")) -> str:
     """Hash of the multiply kernel's code: // comments, blank lines and
     indentation do not count, so a comment edit keeps a profile valid."""
@@ -867,7 +867,7 @@ def batched_block(torch, bi, count, reps, rank=0, world=1, dist=None, dev=None):
     """The batched form: `count` ragged instances (sizes log-uniform over
     2^15..2^19 bits; 40 % mul, 15 % add, 15 % sub, 30 % divmod) in one
     persistent launch with a device-side work queue, in the steps form
-    (large divisions grouped into padded shape classes and divided
+    (large divisions and products grouped step by step, divided
     step-batched, the rest persistent), the faster of the two tuned and
     replayed as a CUDA graph, against one launch per (op, size class).  With
     several ranks the batch is split by estimated cost (ranks.partition) and

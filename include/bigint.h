@@ -249,12 +249,13 @@ typedef struct {
 
 /* Launch forms: one persistent launch with a device-side work queue
  * (cost-sorted, largest first); one launch per (op, size class); or the
- * steps form: the divisions with divisors of 128 limbs or more grouped into
- * classes of nearby shapes (divisors within 1/8, quotients within 1/4 plus
- * 64 limbs, at least 8 members), each class padded to one shape (u and v
- * shifted up by the same number of zero limbs: the quotient is the same,
- * the remainder comes back shifted down) and divided in the step-batched
- * form of bigint_divmod, everything else in one persistent launch.  All
+ * steps form: the divisions with divisors of 128 limbs or more (8 of them at
+ * least) take each step of the step-batched division of bigint_divmod
+ * together, whatever their shapes -- the products of a step in one launch per
+ * product form over all of them, read from the input pool and written to the
+ * output pool in place -- the multiplications with a shorter operand of 64
+ * limbs or more (256 of them at least) run through the same product
+ * launches, and everything else in one persistent launch.  All
  * forms are device work only (a CUDA graph can capture them) and give the
  * same results. */
 #define BIGINT_BATCH_PERSISTENT 0

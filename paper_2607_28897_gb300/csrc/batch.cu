@@ -1,7 +1,7 @@
 // batch.cu -- ragged batches of mixed operations (add, sub, mul, divmod).
 //
 // A batch is a list of operation descriptors (bigint_op, include/bigint.h)
-// over one input pool and one output pool of limbs.  Two ways to run it:
+// over one input pool and one output pool of limbs.  Three ways to run it:
 //
 //   * persistent: ONE launch of grid = SMs x resident CTAs; every CTA takes
 //     the next operation from a device-side work queue (one atomicAdd on a
@@ -9,6 +9,9 @@
 //     the operations sorted by estimated cost, largest first, so the tail of
 //     the launch is made of small operations.  The launch (counter reset +
 //     kernel) contains no host-side step and can be captured in a CUDA graph.
+//   * steps: the large divisions (divisors of 128 limbs and more) and the
+//     products that run on the tensor cores grouped step by step over all
+//     operations (ragged.cu), everything else in one persistent launch.
 //   * per class: one launch per (operation, size class) with size classes
 //     [2^k, 2^(k+1)) limbs, each launch striding over its class -- the
 //     plain form the persistent one is compared against.
@@ -21,6 +24,7 @@
 #include <vector>
 
 #include "divcore.cuh"
+#include "ragged.cuh"
 
 namespace bigint {
 
@@ -79,11 +83,16 @@ template <bool TC>
 __global__ void __launch_bounds__(TC ? tcm::TC_CTA_THREADS : BATCH_MAX_THREADS)
     k_batch(const OpDev *__restrict__ ops, const int32_t *__restrict__ order, int first,
             int count, const uint64_t *in, uint64_t *out, int32_t *status, uint64_t *ws,
-            int64_t ws_per_cta, int *queue, int smem_words) {
+            int64_t ws_per_cta, int *queue, int smem_words, const int *dcount) {
   extern __shared__ __align__(1024) uint32_t smem[];
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   __shared__ int s_idx;
   __shared__ tcm::TcShared tsh;
+  if (dcount != nullptr) {  // a list filled on the device: its length
+    const int n = *(volatile const int *)dcount;
+    if (n < count) count = n;
+    if ((int)blockIdx.x >= count) return;  // before it takes tensor memory
+  }
   uint64_t *my_ws = ws + (int64_t)blockIdx.x * ws_per_cta;
   tcm::TcCtx tcc;
   tcm::TcCtx *tc = nullptr;
@@ -209,54 +218,6 @@ int batch_set_threads(int t) {
 }
 int batch_get_threads() { return g_batch_threads; }
 
-// A class of divisions of nearby shapes run together in the step-batched
-// form: every member u (nu limbs) / v (nv limbs) is padded to u' = u B^s
-// (H limbs) and v' = v B^s (NV limbs), s = NV - nv, so floor(u'/v') =
-// floor(u/v) and u' mod v' = (u mod v) B^s (same quotient, the remainder
-// shifted by s limbs); the quotient has LQ = H - NV + 1 limbs.
-struct DivClass {
-  int H, NV, LQ, first, count;
-};
-
-// One CTA per member of a class: the padded operands.
-__global__ void __launch_bounds__(256)
-    k_cls_gather(const OpDev *__restrict__ ops, const int32_t *__restrict__ order, int first,
-                 const uint64_t *__restrict__ in, uint64_t *Uc, uint64_t *Vc, int H, int NV) {
-  const OpDev o = ops[order[first + blockIdx.x]];
-  const int s = NV - o.nb;
-  const uint64_t *a = in + o.a, *b = in + o.b;
-  uint64_t *u = Uc + (int64_t)blockIdx.x * H, *v = Vc + (int64_t)blockIdx.x * NV;
-  for (int j = threadIdx.x; j < H; j += blockDim.x)
-    u[j] = (j >= s && j - s < o.na) ? a[j - s] : 0ull;
-  for (int j = threadIdx.x; j < NV; j += blockDim.x) v[j] = j >= s ? b[j - s] : 0ull;
-}
-
-// One CTA per member: q (its max(nu - nv + 1, 1) limbs) and r (nv limbs,
-// the padded remainder shifted back by s) into the output pool; status
-// BIGINT_ERANGE where the quotient does not fit its limbs (a divisor with
-// zero top limbs), else the class division's status.
-__global__ void __launch_bounds__(256)
-    k_cls_scatter(const OpDev *__restrict__ ops, const int32_t *__restrict__ order, int first,
-                  const uint64_t *__restrict__ Qc, const uint64_t *__restrict__ Rc,
-                  const int32_t *__restrict__ stc, uint64_t *out, int32_t *status, int LQ, int NV) {
-  const int opi = order[first + blockIdx.x];
-  const OpDev o = ops[opi];
-  const int s = NV - o.nb, nq = o.na - o.nb + 1 > 1 ? o.na - o.nb + 1 : 1;
-  const uint64_t *q = Qc + (int64_t)blockIdx.x * LQ, *r = Rc + (int64_t)blockIdx.x * NV;
-  int high = 0;
-  for (int j = threadIdx.x; j < LQ; j += blockDim.x) {
-    if (j < nq) out[o.o1 + j] = q[j];
-    else if (q[j] != 0) high = 1;
-  }
-  for (int j = threadIdx.x; j < o.nb; j += blockDim.x) out[o.o2 + j] = r[s + j];
-  high = __syncthreads_or(high);
-  if (status != nullptr && threadIdx.x == 0) {
-    int st = stc[blockIdx.x];
-    if (st == BIGINT_OK && high) st = BIGINT_ERANGE;
-    status[opi] = st;
-  }
-}
-
 }  // namespace bigint
 
 // The opaque batch handle of include/bigint.h.
@@ -266,15 +227,14 @@ struct bigint_batch {
   std::vector<int32_t> order_classes;     // grouped by (op, size class)
   std::vector<bigint::Launch> classes;    // one launch per class
   bigint::Launch persistent;
-  // BIGINT_BATCH_STEPS: divisions grouped into shape classes (each run
-  // step-batched on padded operands), the other operations persistent
-  std::vector<int32_t> order_rest;        // order_persistent without the class divisions
-  std::vector<int32_t> order_div;         // the class divisions, class by class
-  std::vector<bigint::DivClass> div_classes;
+  // BIGINT_BATCH_STEPS: large divisions and products grouped (ragged.cu),
+  // the other operations persistent
+  std::vector<int32_t> order_rest;        // order_persistent without the grouped ones
+  bigint::RagPlan rag;
   int64_t ws_limbs_per_cta = 0;
   int max_ctas = 0;
   size_t desc_off = 0, order_p_off = 0, order_c_off = 0, queue_off = 0, scratch_off = 0;
-  size_t order_r_off = 0, order_d_off = 0, cls_off = 0, cls_ws_off = 0, cls_ws_bytes = 0;
+  size_t order_r_off = 0, rag_ops_off = 0, rag_list_off = 0, rag_irr_off = 0, rag_rec_off = 0;
   size_t workspace_bytes = 0;
   int sms = 0, optin = 0;
   int threads_override = 0;  // set by the tuner for this batch
@@ -319,66 +279,41 @@ size_t align256(size_t x) { return (x + 255) / 256 * 256; }
 
 }  // namespace
 
-size_t divmod_workspace(int64_t count, int nu, int nv);
+bool div_steps_on();
+bool mul_tc_on();
 
 namespace {
 
-// Divisions with divisors of at least this many limbs join shape classes.
-constexpr int CLS_MIN_NV = 128;
-// A class keeps divisors within 1/8 and quotient lengths within 1/4 (plus
-// 64 limbs) of its smallest, and has at least CLS_MIN_COUNT members (fewer
-// stay with the persistent launch: a class costs some 50 small launches).
-constexpr int CLS_MIN_COUNT = 8;
+// Divisions with divisors of at least GROUP_MIN_NV limbs run grouped when the
+// batch has GROUP_MIN_DIVS of them (a step of the grouped form is a few
+// launches, however many divisions take it), products with a shorter operand
+// of GROUP_MIN_MUL limbs when it has GROUP_MIN_MULS (more than the persistent
+// launch has CTAs).
+constexpr int GROUP_MIN_NV = 128, GROUP_MIN_DIVS = 8, GROUP_MIN_MUL = 64, GROUP_MIN_MULS = 256;
 
-// Groups the batch's large divisions into classes of nearby shapes and
-// orders the other operations for the persistent launch of the steps form.
-void plan_div_classes(bigint_batch *B) {
-  B->order_div.clear();
-  B->div_classes.clear();
-  std::vector<int32_t> cand;
+// The steps form's plan: the grouped operations, and the order of the rest
+// for the persistent launch.
+int plan_steps(bigint_batch *B) {
+  std::vector<RagOp> divs, muls;
+  std::vector<char> kind(B->ops.size(), 0);
   for (int32_t i = 0; i < (int32_t)B->ops.size(); i++) {
     const bigint_op &o = B->ops[i];
-    if (o.op == BIGINT_OP_DIVMOD && o.nb >= CLS_MIN_NV && o.na >= o.nb) cand.push_back(i);
-  }
-  auto L = [&](int32_t i) { return B->ops[i].na - B->ops[i].nb + 1; };
-  std::stable_sort(cand.begin(), cand.end(),
-                   [&](int32_t x, int32_t y) { return B->ops[x].nb < B->ops[y].nb; });
-  std::vector<char> in_class(B->ops.size(), 0);
-  for (size_t i = 0; i < cand.size();) {
-    const int nv0 = B->ops[cand[i]].nb;
-    size_t j = i;
-    while (j < cand.size() && (int64_t)B->ops[cand[j]].nb * 8 <= (int64_t)nv0 * 9) j++;
-    std::stable_sort(cand.begin() + i, cand.begin() + j,
-                     [&](int32_t x, int32_t y) { return L(x) < L(y); });
-    for (size_t a = i; a < j;) {
-      const int l0 = L(cand[a]);
-      size_t b = a;
-      int nv = 0, lq = 0;
-      while (b < j && (int64_t)L(cand[b]) * 4 <= (int64_t)l0 * 5 + 256) {
-        nv = std::max(nv, (int)B->ops[cand[b]].nb);
-        lq = std::max(lq, L(cand[b]));
-        b++;
-      }
-      if (b - a >= (size_t)CLS_MIN_COUNT) {
-        DivClass c;
-        c.NV = nv;
-        c.LQ = lq;
-        c.H = nv + lq - 1;
-        c.first = (int)B->order_div.size();
-        c.count = (int)(b - a);
-        for (size_t k = a; k < b; k++) {
-          B->order_div.push_back(cand[k]);
-          in_class[cand[k]] = 1;
-        }
-        B->div_classes.push_back(c);
-      }
-      a = b;
+    RagOp r{o.na, o.nb, i, 0, o.a, o.b, o.o1, o.o2, 0};
+    if (o.op == BIGINT_OP_DIVMOD && o.nb >= GROUP_MIN_NV && o.na >= o.nb) {
+      divs.push_back(r);
+      kind[i] = 1;
+    } else if (B->use_tc && o.op == BIGINT_OP_MUL && std::min(o.na, o.nb) >= GROUP_MIN_MUL) {
+      muls.push_back(r);
+      kind[i] = 2;
     }
-    i = j;
   }
+  if (divs.size() < (size_t)GROUP_MIN_DIVS) divs.clear();
+  if (muls.size() < (size_t)GROUP_MIN_MULS) muls.clear();
   B->order_rest.clear();
   for (int32_t i : B->order_persistent)
-    if (!in_class[i]) B->order_rest.push_back(i);
+    if (!(kind[i] == 1 && !divs.empty()) && !(kind[i] == 2 && !muls.empty()))
+      B->order_rest.push_back(i);
+  return rag_plan(std::move(divs), std::move(muls), B->rag);
 }
 
 }  // namespace
@@ -449,37 +384,26 @@ int batch_configure(bigint_batch *B) {
     B->classes.push_back(L);
     i = j;
   }
-  // workspace: descriptors | two orders | queue counter | per-CTA scratch
+  // workspace: descriptors | two orders | queue counter | the steps form's
+  // order and grouped operations, lists, irregular divisions and counters |
+  // per-CTA scratch | the grouped divisions' records.  What batch_upload
+  // copies lies before the scratch, whose size the tuner may change.
   B->desc_off = 0;
   B->order_p_off = align256(n * sizeof(bigint_op));
   B->order_c_off = B->order_p_off + align256(n * 4);
   B->queue_off = B->order_c_off + align256(n * 4);
-  B->scratch_off = B->queue_off + 256;
-  // the steps form: the rest's order, the class divisions' order, then one
-  // set of padded operands / results / statuses and one division workspace,
-  // sized for the largest class (the classes run one after the other)
-  B->order_r_off = B->scratch_off + align256((size_t)B->max_ctas * B->ws_limbs_per_cta * 8);
-  B->order_d_off = B->order_r_off + align256(B->order_rest.size() * 4);
-  B->cls_off = B->order_d_off + align256(B->order_div.size() * 4);
-  size_t cls = 0, cls_ws = 0;
-  for (const DivClass &c : B->div_classes) {
-    const size_t cnt = (size_t)c.count;
-    cls = std::max(cls, align256(8 * cnt * c.H) + align256(8 * cnt * c.NV) +
-                            align256(8 * cnt * c.LQ) + align256(8 * cnt * c.NV) +
-                            align256(4 * cnt));
-    cls_ws = std::max(cls_ws, divmod_workspace(c.count, c.H, c.NV));
-  }
-  B->cls_ws_off = B->cls_off + cls;
-  B->cls_ws_bytes = cls_ws;
-  B->workspace_bytes = B->div_classes.empty() ? B->order_d_off : B->cls_ws_off + cls_ws;
+  B->order_r_off = B->queue_off + 256;
+  B->rag_ops_off = B->order_r_off + align256(B->order_rest.size() * 4);
+  B->rag_list_off = B->rag_ops_off + align256(B->rag.ops.size() * sizeof(RagOp));
+  B->rag_irr_off = B->rag_list_off + align256(B->rag.list.size() * 4);
+  B->scratch_off = B->rag_irr_off + align256((size_t)B->rag.ndiv * 4) + 256;
+  B->rag_rec_off = B->scratch_off + align256((size_t)B->max_ctas * B->ws_limbs_per_cta * 8);
+  B->workspace_bytes = B->rag_rec_off + align256(B->rag.rec_bytes);
   return BIGINT_OK;
 }
 
-int launch_divmod(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r,
-                  int32_t *status, int64_t count, int nu, int nv, void *ws, size_t ws_bytes,
-                  cudaStream_t st);
-
-int batch_create(const bigint_op *ops, int64_t nops, bigint_batch **out) {
+// steps: plan BIGINT_BATCH_STEPS too (without it that mode runs persistent).
+int batch_create(const bigint_op *ops, int64_t nops, bool steps, bigint_batch **out) {
   if (!out || nops < 0 || nops > 0x7fffffff || (nops > 0 && !ops)) return BIGINT_EINVAL;
   for (int64_t i = 0; i < nops; i++) {
     const bigint_op &o = ops[i];
@@ -508,16 +432,21 @@ int batch_create(const bigint_op *ops, int64_t nops, bigint_batch **out) {
   B->order_persistent.resize(nops);
   B->order_classes.resize(nops);
   for (int64_t i = 0; i < nops; i++) B->order_persistent[i] = B->order_classes[i] = (int32_t)i;
+  std::vector<double> cost(nops);
+  std::vector<int32_t> key(nops);
+  for (int64_t i = 0; i < nops; i++) {
+    cost[i] = op_cost(ops[i]);
+    key[i] = ops[i].op * 64 + size_class(ops[i]);
+  }
   std::stable_sort(B->order_persistent.begin(), B->order_persistent.end(),
-                   [&](int32_t x, int32_t y) { return op_cost(ops[x]) > op_cost(ops[y]); });
-  std::stable_sort(B->order_classes.begin(), B->order_classes.end(), [&](int32_t x, int32_t y) {
-    const int kx = ops[x].op * 64 + size_class(ops[x]), ky = ops[y].op * 64 + size_class(ops[y]);
-    return kx < ky;
-  });
+                   [&](int32_t x, int32_t y) { return cost[x] > cost[y]; });
+  std::stable_sort(B->order_classes.begin(), B->order_classes.end(),
+                   [&](int32_t x, int32_t y) { return key[x] < key[y]; });
   for (const bigint_op &o : B->ops)
     if (o.op == BIGINT_OP_DIVMOD) B->ws_limbs_per_cta = std::max(B->ws_limbs_per_cta, ws_limbs(o.na, o.nb, o.na));
-  plan_div_classes(B);
-  const int rc = batch_configure(B);
+  int rc = BIGINT_OK;
+  if (steps) rc = plan_steps(B);
+  if (rc == BIGINT_OK) rc = batch_configure(B);
   if (rc != BIGINT_OK) {
     delete B;
     return rc;
@@ -541,9 +470,12 @@ int batch_upload(bigint_batch *B, void *ws, size_t bytes, cudaStream_t st) {
   if (!B->order_rest.empty())
     BIGINT_CUDA_TRY(cudaMemcpyAsync(w + B->order_r_off, B->order_rest.data(),
                                     B->order_rest.size() * 4, cudaMemcpyHostToDevice, st));
-  if (!B->order_div.empty())
-    BIGINT_CUDA_TRY(cudaMemcpyAsync(w + B->order_d_off, B->order_div.data(),
-                                    B->order_div.size() * 4, cudaMemcpyHostToDevice, st));
+  if (!B->rag.ops.empty()) {
+    BIGINT_CUDA_TRY(cudaMemcpyAsync(w + B->rag_ops_off, B->rag.ops.data(),
+                                    B->rag.ops.size() * sizeof(RagOp), cudaMemcpyHostToDevice, st));
+    BIGINT_CUDA_TRY(cudaMemcpyAsync(w + B->rag_list_off, B->rag.list.data(),
+                                    B->rag.list.size() * 4, cudaMemcpyHostToDevice, st));
+  }
   return BIGINT_OK;
 }
 
@@ -554,6 +486,10 @@ int batch_launch(const bigint_batch *B, const uint64_t *in, uint64_t *out, int32
   char *w = static_cast<char *>(ws);
   const OpDev *ops = reinterpret_cast<const OpDev *>(w + B->desc_off);
   uint64_t *scratch = reinterpret_cast<uint64_t *>(w + B->scratch_off);
+  // a division or multiply variant that keeps those off the grouped form
+  // (bigint_set_variant) runs every operation in the persistent launch
+  if (mode == BIGINT_BATCH_STEPS && (B->rag.ops.empty() || !div_steps_on() || !mul_tc_on()))
+    mode = BIGINT_BATCH_PERSISTENT;
   if (mode == BIGINT_BATCH_PERSISTENT) {
     const Launch &P = B->persistent;
     int *queue = reinterpret_cast<int *>(w + B->queue_off);
@@ -561,11 +497,11 @@ int batch_launch(const bigint_batch *B, const uint64_t *in, uint64_t *out, int32
     auto *kern = P.tc ? k_batch<true> : k_batch<false>;
     kern<<<P.ctas, P.threads, (size_t)P.smem_words * 4, st>>>(
         ops, reinterpret_cast<const int32_t *>(w + B->order_p_off), 0, P.count, in, out, status,
-        scratch, B->ws_limbs_per_cta, queue, P.smem_words);
+        scratch, B->ws_limbs_per_cta, queue, P.smem_words, nullptr);
     return bigint_launch_status();
   }
   if (mode == BIGINT_BATCH_STEPS) {
-    // the operations outside the division classes: one persistent launch
+    // the operations outside the grouped ones: one persistent launch
     const Launch &P = B->persistent;
     const int nrest = (int)B->order_rest.size();
     if (nrest > 0) {
@@ -574,41 +510,31 @@ int batch_launch(const bigint_batch *B, const uint64_t *in, uint64_t *out, int32
       auto *kern = P.tc ? k_batch<true> : k_batch<false>;
       kern<<<std::min(P.ctas, nrest), P.threads, (size_t)P.smem_words * 4, st>>>(
           ops, reinterpret_cast<const int32_t *>(w + B->order_r_off), 0, nrest, in, out, status,
-          scratch, B->ws_limbs_per_cta, queue, P.smem_words);
+          scratch, B->ws_limbs_per_cta, queue, P.smem_words, nullptr);
       const int rc = bigint_launch_status();
       if (rc != BIGINT_OK) return rc;
     }
-    // each class of divisions: padded operands, the step-batched division,
-    // results back into the pool
-    const int32_t *order_d = reinterpret_cast<const int32_t *>(w + B->order_d_off);
-    for (const DivClass &c : B->div_classes) {
-      const size_t cnt = (size_t)c.count;
-      char *p = w + B->cls_off;
-      uint64_t *Uc = reinterpret_cast<uint64_t *>(p); p += align256(8 * cnt * c.H);
-      uint64_t *Vc = reinterpret_cast<uint64_t *>(p); p += align256(8 * cnt * c.NV);
-      uint64_t *Qc = reinterpret_cast<uint64_t *>(p); p += align256(8 * cnt * c.LQ);
-      uint64_t *Rc = reinterpret_cast<uint64_t *>(p); p += align256(8 * cnt * c.NV);
-      int32_t *stc = reinterpret_cast<int32_t *>(p);
-      k_cls_gather<<<(unsigned)c.count, 256, 0, st>>>(ops, order_d, c.first, in, Uc, Vc, c.H,
-                                                        c.NV);
-      int rc = bigint_launch_status();
-      if (rc != BIGINT_OK) return rc;
-      rc = launch_divmod(Uc, Vc, Qc, Rc, stc, c.count, c.H, c.NV, w + B->cls_ws_off,
-                         B->cls_ws_bytes, st);
-      if (rc != BIGINT_OK) return rc;
-      k_cls_scatter<<<(unsigned)c.count, 256, 0, st>>>(ops, order_d, c.first, Qc, Rc, stc, out,
-                                                         status, c.LQ, c.NV);
-      rc = bigint_launch_status();
-      if (rc != BIGINT_OK) return rc;
-    }
-    return BIGINT_OK;
+    RagBuffers R;
+    R.ops = reinterpret_cast<const RagOp *>(w + B->rag_ops_off);
+    R.list = reinterpret_cast<const int32_t *>(w + B->rag_list_off);
+    R.irregular = reinterpret_cast<int32_t *>(w + B->rag_irr_off);
+    R.ctr = reinterpret_cast<int *>(w + B->rag_irr_off + align256((size_t)B->rag.ndiv * 4));
+    R.rec = reinterpret_cast<uint64_t *>(w + B->rag_rec_off);
+    const int rc = rag_launch(B->rag, R, in, out, status, st);
+    if (rc != BIGINT_OK || B->rag.ndiv == 0) return rc;
+    // divisions whose divisor has a zero top limb, one CTA each
+    auto *kern = P.tc ? k_batch<true> : k_batch<false>;
+    kern<<<(unsigned)std::min<int64_t>(P.ctas, B->rag.ndiv), P.threads, (size_t)P.smem_words * 4,
+           st>>>(ops, R.irregular, 0, (int)B->rag.ndiv, in, out, status, scratch,
+                 B->ws_limbs_per_cta, nullptr, P.smem_words, R.ctr);
+    return bigint_launch_status();
   }
   if (mode != BIGINT_BATCH_PER_CLASS) return BIGINT_EINVAL;
   for (const Launch &L : B->classes) {
     auto *kern = L.tc ? k_batch<true> : k_batch<false>;
     kern<<<L.ctas, L.threads, (size_t)L.smem_words * 4, st>>>(
         ops, reinterpret_cast<const int32_t *>(w + B->order_c_off), L.first, L.count, in, out,
-        status, scratch, B->ws_limbs_per_cta, nullptr, L.smem_words);
+        status, scratch, B->ws_limbs_per_cta, nullptr, L.smem_words, nullptr);
     const int rc = bigint_launch_status();
     if (rc != BIGINT_OK) return rc;
   }

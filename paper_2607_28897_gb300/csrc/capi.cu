@@ -30,10 +30,12 @@ int tc_take_timeout();
 int programs_take_timeout();
 int div_take_timeout();
 int batch_take_timeout();
+int rag_take_timeout();
 int tc_set_wait_limit(long long cycles);
 int div_set_wait_limit(long long cycles);
 int programs_set_wait_limit(long long cycles);
 int batch_set_wait_limit(long long cycles);
+int rag_set_wait_limit(long long cycles);
 int launch_add_chain(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
                      int64_t count, int n, int k, cudaStream_t st);
 size_t poly_workspace(int64_t count, int n);
@@ -56,7 +58,7 @@ size_t shinv_workspace(int64_t count, int nv, int h);
 int launch_divmod_inv(const uint64_t *u, const uint64_t *v, const uint64_t *w, uint64_t *q,
                       uint64_t *r, int32_t *status, int64_t count, int nu, int nv, int nw, int h,
                       int64_t v_stride, int64_t w_stride, void *ws, cudaStream_t st);
-int batch_create(const bigint_op *ops, int64_t nops, bigint_batch **out);
+int batch_create(const bigint_op *ops, int64_t nops, bool steps, bigint_batch **out);
 size_t batch_workspace_bytes(const bigint_batch *B);
 int batch_upload(bigint_batch *B, void *ws, size_t bytes, cudaStream_t st);
 int batch_launch(const bigint_batch *B, const uint64_t *in, uint64_t *out, int32_t *status,
@@ -219,7 +221,7 @@ int bigint_shinv(const uint64_t *v, uint64_t *w, int32_t *status, int64_t count,
 }
 
 int bigint_batch_create(const bigint_op *ops_host, int64_t nops, bigint_batch **batch) {
-  return batch_create(ops_host, nops, batch);
+  return batch_create(ops_host, nops, true, batch);
 }
 
 size_t bigint_batch_workspace(const bigint_batch *batch) { return batch_workspace_bytes(batch); }
@@ -301,8 +303,8 @@ int bigint_host_sync(void) { return host_sync(); }
 int bigint_check_timeout(void) {
   // every translation unit that launches tensor-core products keeps its own
   // record: ask them all (each read clears it)
-  const int rc[4] = {tc_take_timeout(), div_take_timeout(), programs_take_timeout(),
-                     batch_take_timeout()};
+  const int rc[5] = {tc_take_timeout(), div_take_timeout(), programs_take_timeout(),
+                     batch_take_timeout(), rag_take_timeout()};
   int out = BIGINT_OK;
   for (int x : rc) {
     if (x == BIGINT_ECUDA) return BIGINT_ECUDA;
@@ -316,8 +318,9 @@ unsigned long long bigint_kernel_launches(void) {
 }
 
 int bigint_set_wait_limit(long long cycles) {
-  const int rc[4] = {tc_set_wait_limit(cycles), div_set_wait_limit(cycles),
-                     programs_set_wait_limit(cycles), batch_set_wait_limit(cycles)};
+  const int rc[5] = {tc_set_wait_limit(cycles), div_set_wait_limit(cycles),
+                     programs_set_wait_limit(cycles), batch_set_wait_limit(cycles),
+                     rag_set_wait_limit(cycles)};
   for (int x : rc)
     if (x != BIGINT_OK) return x;
   return BIGINT_OK;

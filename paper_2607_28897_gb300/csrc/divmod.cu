@@ -172,6 +172,9 @@ int div_set_variant(int v) {
   return BIGINT_OK;
 }
 
+// Whether divisions take the step-batched form where it applies.
+bool div_steps_on() { return g_div_steps != 1; }
+
 // BIGINT_ETIMEOUT if a division kernel's tensor-core product hit a wait
 // limit since the last call (synchronises the device), else BIGINT_OK.
 int div_take_timeout() { return tcm::take_timeout_here(); }

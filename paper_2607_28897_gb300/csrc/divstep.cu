@@ -37,7 +37,7 @@
 // launch, a warp per instance (k_ds_small), instead of four launches each.
 #include <algorithm>
 
-#include "divcore.cuh"
+#include "divstep.cuh"
 
 namespace bigint {
 
@@ -53,7 +53,6 @@ size_t divmod_workspace(int64_t count, int nu, int nv);
 
 namespace dstep {
 
-constexpr int LIN_THREADS = 256;  // CTA of the linear per-instance kernels
 // Shorter operand (limbs) from which a step's product runs on the tensor
 // cores.  The steps' products are rectangular and come in batches of
 // thousands; measured on 2n/n divisions at n = 512 the 132 x 262-limb and
@@ -65,9 +64,8 @@ constexpr int STEP_TC_MIN = 64;
 // leading zero limbs: with h = nu (not prec(u)) w ~ B^h / v still bounds the
 // quotient estimate u w / B^h within a few units of u / v since u < B^h,
 // and the banded u w + B^h < B^(nu + nw) still holds, so such instances
-// (the zero-padded operands of the batched form's division classes, or a
-// short dividend) stay on the step path at the cost of the product work
-// above their precision.
+// stay on the step path at the cost of the product work above their
+// precision.
 __device__ __forceinline__ bool regular(const uint64_t *, int, const uint64_t *v, int nv) {
   return v[nv - 1] != 0;
 }
@@ -91,17 +89,7 @@ __global__ void k_ds_start(const uint64_t *__restrict__ U, const uint64_t *__res
     for (int j = 0; j < l + 2; j++) w[j] = 0;
     return;
   }
-  const int k = nv - 1;
-  uint64_t Vt[6] = {0, 0, 0, 0, 0, 0}, Un[8] = {0, 0, 0, 0, 0, 0, 0, 0}, Qt[8];
-  for (int j = 0; j <= l; j++) Vt[j] = v[k - l + j];
-  int j = 0;
-  while (j <= l && ++Vt[j] == 0) j++;  // V + 1, which may carry into limb l + 1
-  const int nV = j > l ? l + 2 : l + 1;
-  if (j > l) Vt[l + 1] = 1;
-  Un[2 * l] = 1;  // B^(2 l)
-  small_div(Un, 2 * l + 1, Vt, nV, Qt);
-  const int nq = 2 * l + 1 - nV + 1;
-  for (int jj = 0; jj < l + 2; jj++) w[jj] = jj < nq ? Qt[jj] : 0;
+  ds_start_one(v, nv, l, w);
 }
 
 constexpr int WARP_CTA = 256;  // warp-per-instance kernels: 8 instances per CTA
@@ -115,17 +103,14 @@ constexpr int WARP_CTA = 256;  // warp-per-instance kernels: 8 instances per CTA
 // kernels, except that P2 = w |d| is computed whole (so floor(P2 / B^s) is
 // exact, which the step allows).
 // ---------------------------------------------------------------------------
-constexpr int SMALL_STEP_LIMBS = 136, SMALL_STEP_WARPS = 4, SMALL_STEP_MAX = 16;
+constexpr int SMALL_STEP_MAX = 16;
 
-// The steps the fused kernel runs: (l, m, t) of each; N bounds their
-// operands (limbs, a multiple of 8): a warp's shared memory holds two
-// iterates (N each), vt and |d| (N each), P2 (2 N) and the column sums
-// (2 N x 3 words).
+// The steps the fused kernel runs; N bounds their operands (limbs, a
+// multiple of 8).
 struct SmallSteps {
   int n, N;
-  int l[SMALL_STEP_MAX], m[SMALL_STEP_MAX], t[SMALL_STEP_MAX];
+  Step s[SMALL_STEP_MAX];
 };
-__host__ __device__ constexpr int small_step_warp_limbs(int N) { return 2 * N + 2 * N + 2 * N + 6 * N; }
 
 // Steps S of every instance: the iterate from W0 (its first l + 2 limbs),
 // the result (l + m + 2 limbs of the last step) to W0 or W1 as the batched
@@ -143,36 +128,13 @@ __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS)
   uint64_t *z = base + 4 * N, *cs = base + 6 * N;
   const uint64_t *v = V + i * nv;
   const int k = nv - 1;
-  for (int j = lane; j < S.l[0] + 2; j += 32) wb[0][j] = W0[i * sw + j];
+  for (int j = lane; j < S.s[0].l + 2; j += 32) wb[0][j] = W0[i * sw + j];
   int cur = 0;
   for (int st = 0; st < S.n; st++) {
-    const int l = S.l[st], m = S.m[st], t = S.t[st];
-    const int nw = l + 2, nl = t + 2;
-    uint64_t *w = wb[cur], *wn = wb[cur ^ 1];
-    for (int j = lane; j <= t; j += 32) vts[j] = v[k - t + j];
-    __syncwarp();
-    // P = vt w mod B^(t+2); |d| = P (top bit clear: d <= 0) or B^(t+2) - P
-    warp_mul(vts, t + 1, w, nw, d, nl, cs);
-    const bool ng = (d[nl - 1] >> 63) == 0;
-    if (!ng) {
-      warp_addsub<true>(nl, 0u, [&](int j) { return make_ulonglong2(0ull, d[j]); },
-                        [&](int j, uint64_t x) { d[j] = x; });
-      __syncwarp();
-    }
-    // P2 = w |d| (whole); w' = w B^m + floor(P2 / B^s) or w B^m - floor(P2 / B^s) - 1
-    warp_mul(w, nw, d, nl, z, nw + nl, cs);
-    const int s = t + l - m, ny = nw + nl - s;
-    auto load = [&](int j) {
-      const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
-      return make_ulonglong2(x, j < ny ? z[s + j] : 0ull);
-    };
-    auto store = [&](int j, uint64_t x) { wn[j] = x; };
-    if (ng) warp_addsub<true>(l + m + 2, 1u, load, store);
-    else warp_addsub<false>(l + m + 2, 0u, load, store);
-    __syncwarp();
+    ds_small_step(v, k, S.s[st], wb[cur], wb[cur ^ 1], vts, d, z, cs);
     cur ^= 1;
   }
-  const int nlast = S.l[S.n - 1] + S.m[S.n - 1] + 2;
+  const int nlast = S.s[S.n - 1].l + S.s[S.n - 1].m + 2;
   uint64_t *out = (S.n & 1) ? W1 : W0;
   for (int j = lane; j < nlast; j += 32) out[i * sw + j] = wb[cur][j];
 }
@@ -222,16 +184,7 @@ __global__ void __launch_bounds__(LIN_THREADS)
                  int nl, int32_t *neg) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   const int64_t i = blockIdx.x;
-  const uint64_t *p = P + i * sp;
-  uint64_t *d = D + i * sd;
-  const bool ng = (p[nl - 1] >> 63) == 0;
-  auto store = [&](int j, uint64_t x) { d[j] = x; };
-  if (ng) {
-    for (int j = threadIdx.x; j < nl; j += blockDim.x) d[j] = p[j];
-  } else {
-    auto load = [&](int j) { return make_ulonglong2(0ull, p[j]); };
-    blk_addsub<true>(nl, 0u, load, store, scr);
-  }
+  const bool ng = ds_mid_cta(P + i * sp, D + i * sd, nl, scr);
   if (threadIdx.x == 0) neg[i] = ng ? 1 : 0;
 }
 
@@ -241,15 +194,7 @@ __global__ void __launch_bounds__(LIN_THREADS)
                     const int32_t *__restrict__ neg, int m, uint64_t *__restrict__ Wn, int nout) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   const int64_t i = blockIdx.x;
-  const uint64_t *w = W + i * sw, *y = Z + i * sz + s;
-  uint64_t *wn = Wn + i * sw;
-  auto load = [&](int j) {
-    const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
-    return make_ulonglong2(x, j < ny ? y[j] : 0ull);
-  };
-  auto store = [&](int j, uint64_t x) { wn[j] = x; };
-  if (neg[i]) blk_addsub<true>(nout, 1u, load, store, scr);
-  else blk_addsub<false>(nout, 0u, load, store, scr);
+  ds_update_cta(W + i * sw, nw, Z + i * sz + s, ny, neg[i] != 0, m, Wn + i * sw, nout, scr);
 }
 
 // Records up to this many limbs take the warp-per-instance kernels.
@@ -279,36 +224,19 @@ __global__ void __launch_bounds__(LIN_THREADS)
   const int64_t i = blockIdx.x;
   const uint64_t *u = U + i * nu, *v = V + i * nv, *rr = R + i * sp;
   if (!regular(u, nu, v, nv)) return;
-  uint64_t *rh = Rh + i * sd, *qh = Qh + i * sq;
-  {
-    auto load = [&](int j) { return make_ulonglong2(j < nu ? u[j] : 0ull, rr[j]); };
-    auto store = [&](int j, uint64_t x) { rh[j] = x; };
-    blk_addsub<true>(nv + 1, 0u, load, store, scr);
-  }
-  int st = correct(v, nv, rh, qh, nqcap, scr);
-  __syncthreads();
-  const int pq = blk_prec(qh, nqcap, scr);
-  if (pq > nq && st == BIGINT_OK) st = BIGINT_ERANGE;
+  int st = ds_finish_cta(u, nu, v, nv, rr, Rh + i * sd, Qh + i * sq, nqcap, Qo + i * nq, nq,
+                         Ro + i * nv, scr);
   if (*(volatile const int *)aborted) st = BIGINT_ETIMEOUT;
-  uint64_t *q = Qo + i * nq, *r = Ro + i * nv;
-  for (int j = threadIdx.x; j < nq; j += blockDim.x) q[j] = j < nqcap ? qh[j] : 0ull;
-  for (int j = threadIdx.x; j < nv; j += blockDim.x) r[j] = rh[j];
   if (status != nullptr && threadIdx.x == 0) status[i] = st;
 }
 
-// The Newton schedule of a regular instance: (l, m, t) per step.
-struct Step {
-  int l, m, t;
-};
-
+// The Newton schedule of a regular instance.
 int schedule(int k, int h, int l0, Step *steps, int cap) {
   const int L = h - k;
   int l = l0, n = 0;
   while (l < L && n < cap) {
-    const int m = (l - 2 < L - l) ? l - 2 : L - l;
-    const int t = (k < l + m + 2) ? k : l + m + 2;
-    steps[n++] = Step{l, m, t};
-    l += m;
+    steps[n] = newton_next(k, L, l);
+    l += steps[n++].m;
   }
   return n;
 }
@@ -408,10 +336,7 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     const int need = std::max(std::max(S0.l + 2, S0.t + 2), S0.l + S0.m + 2);
     if (need > SMALL_STEP_LIMBS) break;
     SS.N = std::max(SS.N, (need + 7) / 8 * 8);
-    SS.l[SS.n] = S0.l;
-    SS.m[SS.n] = S0.m;
-    SS.t[SS.n] = S0.t;
-    SS.n++;
+    SS.s[SS.n++] = S0;
   }
   if (SS.n > 0) {
     const size_t smem = (size_t)8 * SMALL_STEP_WARPS * small_step_warp_limbs(SS.N);

@@ -178,6 +178,10 @@ int mul_set_variant(int v) {
   return BIGINT_OK;
 }
 
+// Whether the products inside divisions and batches may run on the tensor
+// cores (variants 8-11 keep them on the integer pipes).
+bool mul_tc_on() { return g_mul_variant == 0 || g_mul_variant >= 12; }
+
 // Largest square operand (limbs) whose product fits one CTA's shared memory.
 int mul_max_limbs() { return BIGINT_MUL_MAX_LIMBS; }
 

@@ -1,0 +1,532 @@
+// ragged.cu -- the divisions and products of a ragged batch, grouped.
+//
+// The step-batched division (divstep.cu) for instances of different shapes:
+// all divisions of a wave take each Newton step together.  The known limbs l
+// run through the same sequence 3, 4, 6, 10, ... 130, 258, ... for every
+// division, only a division's last step is shorter, so a step's products
+// differ in size but not in kind: one launch per step, kind and product form
+// (tile), each over the list of the operations that take it, largest first,
+// every CTA reading its operation's sizes and offsets from a table.  The
+// linear parts run one CTA per operation.  Operands are read from the input
+// pool and results written to the output pool in place.  Multiplications of
+// the batch run through the same product launches.
+//
+// Why: grouped by nearby shapes instead (padded classes of at least 8
+// members, each class a chain of ~22 launches of its own), 20000 mixed
+// operations made 199 classes of 30 members on average -- 4474 launches one
+// after the other, each on a fraction of the SMs, 98 ms.  The grouped form
+// takes some 150 launches over thousands of operations each.
+//
+// Bound: the tensor-core products of the last steps; the records of a wave
+// (about 5.5 limbs per divisor limb) are kept to WAVE_BYTES.
+#include "ragged.cuh"
+
+#include <algorithm>
+#include <unordered_map>
+
+#include "divstep.cuh"
+#include "tcone.cuh"
+
+namespace bigint {
+
+// The cheapest form of a product by the models of tcmul.cu, and whether its
+// operands change roles (tcmul.cu).
+int tc_choose(int nx, int ny, int nout, int lo, bool *swap);
+
+namespace {
+
+using namespace dstep;
+
+// Bytes of records of one wave.
+constexpr size_t WAVE_BYTES = (size_t)1 << 30;
+
+// The steps up to this many known limbs run fused in one warp (every operand
+// then has at most SMALL_STEP_LIMBS limbs).
+constexpr int SMALL_L = 66;
+
+struct RagArgs {
+  const RagOp *ops;
+  const int32_t *list;  // products: this launch's list
+  int n;
+  int kind, l, par;
+  const uint64_t *in;
+  uint64_t *out, *rec;
+  int32_t *status;
+  int *abort_flag;
+};
+
+__host__ __device__ inline int rag_L(int nu, int nv) { return nu - nv + 1; }
+
+// Records of an operation: two iterates, low product, |d| (then r^), banded
+// product (its top limbs become q^).
+struct RagRec {
+  uint64_t *w[2], *p, *d, *z;
+};
+__host__ __device__ inline int64_t rag_rec_limbs(int nu, int nv) {
+  const int64_t L = rag_L(nu, nv);
+  return 2 * (L + 4) + 2 * ((int64_t)nv + 2) + (nu + L + 6);
+}
+__device__ __forceinline__ RagRec rag_rec(const RagArgs &A, const RagOp &o) {
+  const int L = rag_L(o.nu, o.nv);
+  RagRec r;
+  r.w[0] = A.rec + o.rec;
+  r.w[1] = r.w[0] + L + 4;
+  r.p = r.w[1] + L + 4;
+  r.d = r.p + o.nv + 2;
+  r.z = r.d + o.nv + 2;
+  return r;
+}
+
+// Steps after the fused ones; the iterate they leave is w[parity of these].
+__host__ __device__ inline int rag_big_steps(int L) {
+  int n = 0;
+  for (int l = 2 * (SMALL_L - 1); l < L; l += l - 2) n++;
+  return n;
+}
+
+struct RagTask {
+  const uint64_t *x, *y;
+  uint64_t *out;
+  int nx, ny, nout, lo;
+};
+// Sizes of the product of a kind (host and device).
+__host__ __device__ inline void rag_sizes(int nu, int nv, int kind, int l, int &nx, int &ny,
+                                          int &nout, int &lo) {
+  const int k = nv - 1, L = rag_L(nu, nv);
+  const Step S = newton_next(k, L, l);
+  switch (kind) {
+    case RAG_P: nx = S.t + 1; ny = l + 2; nout = S.t + 2; lo = 0; break;
+    case RAG_P2: nx = l + 2; ny = S.t + 2; nout = nx + ny; lo = S.t + l - S.m - 2; break;
+    case RAG_UW: nx = nu; ny = L + 2; nout = nx + ny; lo = nu - 2; break;
+    case RAG_QV: nx = L + 2; ny = nv; nout = nv + 1; lo = 0; break;
+    default: nx = nu; ny = nv; nout = nu + nv; lo = 0; break;
+  }
+}
+__device__ __forceinline__ RagTask rag_task(const RagArgs &A, const RagOp &o, bool swap) {
+  RagTask T;
+  rag_sizes(o.nu, o.nv, A.kind, A.l, T.nx, T.ny, T.nout, T.lo);
+  const uint64_t *u = A.in + o.u, *v = A.in + o.v;
+  if (A.kind == RAG_MUL) {
+    T.x = u;
+    T.y = v;
+    T.out = A.out + o.q;
+  } else {
+    const RagRec r = rag_rec(A, o);
+    switch (A.kind) {
+      case RAG_P: T.x = v + (o.nv - T.nx); T.y = r.w[A.par]; T.out = r.p; break;
+      case RAG_P2: T.x = r.w[A.par]; T.y = r.d; T.out = r.z; break;
+      case RAG_UW: T.x = u; T.y = r.w[rag_big_steps(T.ny - 2) & 1]; T.out = r.z; break;
+      default: T.x = r.z + o.nu; T.y = v; T.out = r.p; break;
+    }
+  }
+  if (swap) {
+    const uint64_t *t = T.x; T.x = T.y; T.y = t;
+    const int n = T.nx; T.nx = T.ny; T.ny = n;
+  }
+  return T;
+}
+
+// ---- kernels ---------------------------------------------------------------
+// One thread per division: the Newton start, or (zero top limb of the
+// divisor) its index into the irregular list and a zero iterate, on which
+// the steps stay within their buffers and whose results nobody reads.
+__global__ void k_rag_start(RagArgs A, int32_t *irregular, int *nirr) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= A.n) return;
+  const RagOp o = A.ops[i];
+  const int L = rag_L(o.nu, o.nv), l = L < 3 ? L : 3;
+  uint64_t *w = A.rec + o.rec;
+  const uint64_t *v = A.in + o.v;
+  if (v[o.nv - 1] == 0) {
+    irregular[atomicAdd(nirr, 1)] = o.opi;
+    for (int j = 0; j < l + 2; j++) w[j] = 0;
+    return;
+  }
+  ds_start_one(v, o.nv, l, w);
+}
+
+// One warp per division: the steps from at most SMALL_L known limbs.
+__global__ void __launch_bounds__(32 * SMALL_STEP_WARPS) k_rag_small(RagArgs A) {
+  extern __shared__ __align__(16) uint64_t ssm[];
+  constexpr int N = SMALL_STEP_LIMBS;
+  const int wi = threadIdx.x >> 5, lane = (int)lane_id();
+  const int i = blockIdx.x * SMALL_STEP_WARPS + wi;
+  if (i >= A.n) return;  // the whole warp: no block barrier below
+  const RagOp o = A.ops[i];
+  uint64_t *base = ssm + (size_t)wi * small_step_warp_limbs(N);
+  uint64_t *wb[2] = {base, base + N}, *vts = base + 2 * N, *d = base + 3 * N;
+  uint64_t *z = base + 4 * N, *cs = base + 6 * N;
+  const uint64_t *v = A.in + o.v;
+  uint64_t *w = A.rec + o.rec;
+  const int L = rag_L(o.nu, o.nv);
+  int l = L < 3 ? L : 3, cur = 0;
+  if (l == L) return;  // no steps: the start value stands
+  for (int j = lane; j < l + 2; j += 32) wb[0][j] = w[j];
+  while (l < L && l <= SMALL_L) {
+    const Step S = newton_next(o.nv - 1, L, l);
+    ds_small_step(v, o.nv - 1, S, wb[cur], wb[cur ^ 1], vts, d, z, cs);
+    cur ^= 1;
+    l += S.m;
+  }
+  for (int j = lane; j < l + 2; j += 32) w[j] = wb[cur][j];
+}
+
+// One CTA per division: |d| and its sign (limb nv + 1 of the record's |d|).
+__global__ void __launch_bounds__(LIN_THREADS) k_rag_mid(RagArgs A) {
+  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  const RagOp o = A.ops[blockIdx.x];
+  const RagRec r = rag_rec(A, o);
+  const int nl = newton_next(o.nv - 1, rag_L(o.nu, o.nv), A.l).t + 2;
+  const bool ng = ds_mid_cta(r.p, r.d, nl, scr);
+  if (threadIdx.x == 0) r.p[0] = ng ? 1 : 0;  // the low product is used up
+}
+
+__global__ void __launch_bounds__(LIN_THREADS) k_rag_update(RagArgs A) {
+  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  const RagOp o = A.ops[blockIdx.x];
+  const RagRec r = rag_rec(A, o);
+  const Step S = newton_next(o.nv - 1, rag_L(o.nu, o.nv), A.l);
+  const int nw = S.l + 2, n2 = nw + S.t + 2, s = S.t + S.l - S.m;
+  ds_update_cta(r.w[A.par], nw, r.z + s, n2 - s, r.p[0] != 0, S.m, r.w[A.par ^ 1],
+                S.l + S.m + 2, scr);
+}
+
+__global__ void __launch_bounds__(LIN_THREADS) k_rag_finish(RagArgs A) {
+  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  const RagOp o = A.ops[blockIdx.x];
+  const uint64_t *u = A.in + o.u, *v = A.in + o.v;
+  if (v[o.nv - 1] == 0) return;  // irregular
+  const RagRec r = rag_rec(A, o);
+  const int L = rag_L(o.nu, o.nv), nqh = L + 2;
+  if (threadIdx.x == 0) r.z[o.nu + nqh] = 0;
+  __syncthreads();
+  int st = ds_finish_cta(u, o.nu, v, o.nv, r.p, r.d, r.z + o.nu, nqh + 1, A.out + o.q, L,
+                         A.out + o.r, scr);
+  if (*(volatile int *)A.abort_flag) st = BIGINT_ETIMEOUT;
+  if (A.status != nullptr && threadIdx.x == 0) A.status[o.opi] = st;
+}
+
+// The products of a list: CTA b takes entries b, b + grid, ... (largest
+// first).  A CTA that gives up at a wait limit sets *abort_flag and reports
+// BIGINT_ETIMEOUT for the rest of its multiplications.
+template <class Product>
+__device__ __forceinline__ void rag_products(const RagArgs &A, Product product) {
+  bool ok = true;
+  for (int i = blockIdx.x; i < A.n; i += gridDim.x) {
+    const int32_t e = A.list[i];
+    const RagOp o = A.ops[e & ~RAG_SWAP];
+    if (ok) ok = product(rag_task(A, o, (e & RAG_SWAP) != 0));
+    if (threadIdx.x == 0) {
+      if (!ok) atomicExch(A.abort_flag, 1);
+      if (A.kind == RAG_MUL && A.status != nullptr)
+        A.status[o.opi] = ok ? BIGINT_OK : BIGINT_ETIMEOUT;
+    }
+  }
+}
+
+template <int NT, int G>
+__global__ void __launch_bounds__(2 * NT + 32, 256 / NT) k_rag_tc(RagArgs A) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ tcm::TcShared sh;
+  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  tcm::TcCtx c;
+  tcm::tc_init<NT>(c, sm, &sh, scr);
+  rag_products(A, [&](const RagTask &T) {
+    return tcm::tc_product<NT, G, true>(c, T.x, T.nx, T.y, T.ny, T.out, T.nout, T.lo);
+  });
+  tcm::tc_release<NT>(c);
+}
+
+template <int NT>
+__global__ void __launch_bounds__(32 * tcm::one_warps<NT>(), 512 / NT) k_rag_one(RagArgs A) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ tcm::OneShared sh;
+  tcm::OneCtx c;
+  tcm::one_init<NT>(c, sm, &sh);
+  rag_products(A, [&](const RagTask &T) {
+    return tcm::one_product<NT, tcm::one_warps<NT>()>(c, T.x, T.nx, T.y, T.ny, T.out, T.nout,
+                                                      T.lo);
+  });
+  tcm::one_release<NT>(c);
+}
+
+// ---- host ------------------------------------------------------------------
+struct ShapeAttr {
+  void (*kern)(RagArgs);
+  int threads, cap;    // CTAs per SM the tensor memory allows
+  int dyn, overhead;   // largest dynamic shared memory; static and reserved
+};
+
+// The kernels of the product forms with their attributes on this device
+// (dyn < 0 after an error).
+struct Shapes {
+  ShapeAttr a[RAG_NSHAPES];
+  int sms = 0, smem_sm = 0;
+  bool ok = false;
+};
+const Shapes &shapes() {
+  static const Shapes S = [] {
+    using tcm::one_warps;
+    Shapes s;
+    s.a[RAG_ONE128] = {k_rag_one<128>, 32 * one_warps<128>(), 4, 0, 0};
+    s.a[RAG_ONE256] = {k_rag_one<256>, 32 * one_warps<256>(), 2, 0, 0};
+    s.a[RAG_64] = {k_rag_tc<64, 7>, 2 * 64 + 32, 4, 0, 0};
+    s.a[RAG_128] = {k_rag_tc<128, 8>, 2 * 128 + 32, 2, 0, 0};
+    s.a[RAG_256] = {k_rag_tc<256, 8>, 2 * 256 + 32, 1, 0, 0};
+    s.a[RAG_256_G4] = {k_rag_tc<256, 4>, 2 * 256 + 32, 1, 0, 0};
+    int dev = 0, optin = 0, reserved = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&s.smem_sm, cudaDevAttrMaxSharedMemoryPerMultiprocessor, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&reserved, cudaDevAttrReservedSharedMemoryPerBlock, dev) !=
+            cudaSuccess ||
+        cudaDeviceGetAttribute(&s.sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return s;
+    for (ShapeAttr &x : s.a) {
+      cudaFuncAttributes fa;
+      if (cudaFuncGetAttributes(&fa, x.kern) != cudaSuccess) return s;
+      x.dyn = optin - (int)fa.sharedSizeBytes;
+      x.overhead = (int)fa.sharedSizeBytes + reserved;
+      if (cudaFuncSetAttribute(x.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, x.dyn) !=
+          cudaSuccess)
+        return s;
+    }
+    if (cudaFuncSetAttribute(k_rag_small, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             8 * SMALL_STEP_WARPS * small_step_warp_limbs(SMALL_STEP_LIMBS)) !=
+        cudaSuccess)
+      return s;
+    s.ok = true;
+    return s;
+  }();
+  return S;
+}
+
+uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
+  using namespace tcm;
+  switch (shape) {
+    case RAG_ONE128: return one_bytes<128, one_warps<128>()>(nx, ny, nout, lo);
+    case RAG_ONE256: return one_bytes<256, one_warps<256>()>(nx, ny, nout, lo);
+    case RAG_64: return layout<64, 7>(nx, ny).total;
+    case RAG_128: return layout<128, 8>(nx, ny).total;
+    case RAG_256: return layout<256, 8>(nx, ny).total;
+    default: return layout<256, 4>(nx, ny).total;
+  }
+}
+
+// The form of one product: shape (as an index), swap, shared memory and the
+// CTAs per SM that leaves.  Sizes are rounded up to 1/16 of their highest
+// power of two for the cost models, which a plan then evaluates a few
+// hundred times, and a thread's next plan hardly at all: the choices (a
+// function of the sizes alone) are kept per thread, MEMO_MAX of them at most.
+// The shared memory is that of the actual sizes.
+struct Form {
+  int shape, per_sm;
+  bool swap;
+  uint32_t bytes;
+};
+class Chooser {
+ public:
+  Form get(int nx, int ny, int nout, int lo) {
+    // most operations of a step have the same sizes as the one before
+    if (nx == last_[0] && ny == last_[1] && nout == last_[2] && lo == last_[3]) return last_form_;
+    last_[0] = nx;
+    last_[1] = ny;
+    last_[2] = nout;
+    last_[3] = lo;
+    return last_form_ = choose(nx, ny, nout, lo);
+  }
+
+ private:
+  static constexpr size_t MEMO_MAX = 1 << 15;
+  Form choose(int nx, int ny, int nout, int lo) {
+    static thread_local std::unordered_map<uint64_t, int> memo_;
+    const int qx = up(nx), qy = up(ny);
+    // a banded or low product keeps its kind: the same part of the result
+    const int qo = std::min(qx + qy, nout == nx + ny ? qx + qy : up(nout));
+    const int ql = std::min(lo > 0 ? down(lo) : 0, qo - 1);
+    const uint64_t key = ((uint64_t)qx << 48) ^ ((uint64_t)qy << 32) ^ ((uint64_t)qo << 16) ^ ql;
+    auto it = memo_.find(key);
+    if (it == memo_.end()) {
+      if (memo_.size() >= MEMO_MAX) memo_.clear();
+      bool swap = false;
+      const int sh = tc_choose(qx, qy, qo, ql, &swap);
+      it = memo_.emplace(key, (sh << 1) | (swap ? 1 : 0)).first;
+    }
+    Form f;
+    f.shape = it->second >> 1;
+    f.swap = it->second & 1;
+    if (f.shape == RAG_256_G4) f.shape = RAG_256;
+    int ax = f.swap ? ny : nx, ay = f.swap ? nx : ny;
+    f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
+    if (f.bytes > (uint32_t)shapes().a[f.shape].dyn) {
+      // 256-column tiles, the shorter operand whole in shared memory
+      f.swap = nx > ny;
+      ax = std::min(nx, ny);
+      ay = std::max(nx, ny);
+      f.shape = RAG_256;
+      f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
+      if (f.bytes > (uint32_t)shapes().a[f.shape].dyn) {
+        f.shape = RAG_256_G4;
+        f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
+      }
+    }
+    const ShapeAttr &a = shapes().a[f.shape];
+    f.per_sm = std::max(1, std::min(a.cap, shapes().smem_sm / ((int)f.bytes + a.overhead)));
+    return f;
+  }
+
+  static int step(int n) {
+    int s = 1;
+    while (n >= 32 * s) s *= 2;
+    return s;
+  }
+  static int up(int n) { return (n + step(n) - 1) / step(n) * step(n); }
+  static int down(int n) { return n / step(n) * step(n); }
+  int last_[4] = {-1, -1, -1, -1};
+  Form last_form_{};
+};
+
+// Appends the launches of one kind of product over ops [first, first + n).
+void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, int l, int par) {
+  struct Item {
+    int group;
+    double cost;
+    int32_t entry;
+    uint32_t bytes;
+  };
+  std::vector<Item> items;
+  items.reserve(n);
+  for (int64_t i = 0; i < n; i++) {
+    const RagOp &o = P.ops[first + i];
+    int nx, ny, nout, lo;
+    rag_sizes(o.nu, o.nv, kind, l, nx, ny, nout, lo);
+    const Form f = C.get(nx, ny, nout, lo);
+    items.push_back({f.shape * 8 + f.per_sm, (double)nx * ny,
+                     (int32_t)(first + i) | (f.swap ? RAG_SWAP : 0), f.bytes});
+  }
+  std::stable_sort(items.begin(), items.end(), [](const Item &a, const Item &b) {
+    return a.group != b.group ? a.group > b.group : a.cost > b.cost;
+  });
+  for (size_t i = 0; i < items.size();) {
+    size_t j = i;
+    RagLaunch R{};
+    R.what = RAG_PROD;
+    R.kind = kind;
+    R.l = l;
+    R.par = par;
+    R.shape = items[i].group / 8;
+    R.first = (int64_t)P.list.size();
+    for (; j < items.size() && items[j].group == items[i].group; j++) {
+      P.list.push_back(items[j].entry);
+      R.smem = std::max(R.smem, items[j].bytes);
+    }
+    R.n = (int64_t)(j - i);
+    R.grid = (int)std::min<int64_t>(R.n, (int64_t)shapes().sms * (items[i].group % 8));
+    P.program.push_back(R);
+    i = j;
+  }
+}
+
+}  // namespace
+
+int rag_plan(std::vector<RagOp> divs, std::vector<RagOp> muls, RagPlan &P) {
+  P = RagPlan();
+  if (divs.empty() && muls.empty()) return BIGINT_OK;
+  if (!shapes().ok) return BIGINT_ECUDA;
+  Chooser C;
+  auto linear = [&](int what, int64_t first, int64_t n, int l, int par) {
+    RagLaunch R{};
+    R.what = what;
+    R.l = l;
+    R.par = par;
+    R.first = first;
+    R.n = n;
+    P.program.push_back(R);
+  };
+  // longest quotients first: the divisions still at work in a step are the
+  // first ones of their wave
+  std::stable_sort(divs.begin(), divs.end(), [](const RagOp &a, const RagOp &b) {
+    return rag_L(a.nu, a.nv) > rag_L(b.nu, b.nv);
+  });
+  P.ndiv = (int64_t)divs.size();
+  P.ops = divs;
+  for (int64_t first = 0; first < P.ndiv;) {
+    int64_t n = 0, limbs = 0;
+    while (first + n < P.ndiv) {
+      RagOp &o = P.ops[first + n];
+      const int64_t r = rag_rec_limbs(o.nu, o.nv);
+      if (n > 0 && 8 * (size_t)(limbs + r) > WAVE_BYTES) break;
+      o.rec = limbs;
+      limbs += r;
+      n++;
+    }
+    P.rec_bytes = std::max(P.rec_bytes, 8 * (size_t)limbs);
+    linear(RAG_START, first, n, 0, 0);
+    linear(RAG_SMALL, first, n, 0, 0);
+    int par = 0;
+    for (int l = 2 * (SMALL_L - 1);; l += l - 2, par ^= 1) {
+      int64_t act = 0;
+      while (act < n && rag_L(P.ops[first + act].nu, P.ops[first + act].nv) > l) act++;
+      if (act == 0) break;
+      plan_products(P, C, first, act, RAG_P, l, par);
+      linear(RAG_MID, first, act, l, par);
+      plan_products(P, C, first, act, RAG_P2, l, par);
+      linear(RAG_UPDATE, first, act, l, par);
+    }
+    plan_products(P, C, first, n, RAG_UW, 0, 0);
+    plan_products(P, C, first, n, RAG_QV, 0, 0);
+    linear(RAG_FINISH, first, n, 0, 0);
+    first += n;
+  }
+  if (!muls.empty()) {
+    P.ops.insert(P.ops.end(), muls.begin(), muls.end());
+    plan_products(P, C, P.ndiv, (int64_t)muls.size(), RAG_MUL, 0, 0);
+  }
+  return BIGINT_OK;
+}
+
+int rag_launch(const RagPlan &P, const RagBuffers &B, const uint64_t *in, uint64_t *out,
+               int32_t *status, cudaStream_t st) {
+  BIGINT_CUDA_TRY(cudaMemsetAsync(B.ctr, 0, 2 * sizeof(int), st));
+  for (const RagLaunch &R : P.program) {
+    RagArgs A;
+    A.ops = R.what == RAG_PROD ? B.ops : B.ops + R.first;
+    A.list = R.what == RAG_PROD ? B.list + R.first : nullptr;
+    A.n = (int)R.n;
+    A.kind = R.kind;
+    A.l = R.l;
+    A.par = R.par;
+    A.in = in;
+    A.out = out;
+    A.rec = B.rec;
+    A.status = status;
+    A.abort_flag = B.ctr + 1;
+    const unsigned n = (unsigned)R.n;
+    switch (R.what) {
+      case RAG_START: k_rag_start<<<(n + 127) / 128, 128, 0, st>>>(A, B.irregular, B.ctr); break;
+      case RAG_SMALL:
+        k_rag_small<<<(n + SMALL_STEP_WARPS - 1) / SMALL_STEP_WARPS, 32 * SMALL_STEP_WARPS,
+                      8 * SMALL_STEP_WARPS * small_step_warp_limbs(SMALL_STEP_LIMBS), st>>>(A);
+        break;
+      case RAG_MID: k_rag_mid<<<n, LIN_THREADS, 0, st>>>(A); break;
+      case RAG_UPDATE: k_rag_update<<<n, LIN_THREADS, 0, st>>>(A); break;
+      case RAG_FINISH: k_rag_finish<<<n, LIN_THREADS, 0, st>>>(A); break;
+      default: {
+        const ShapeAttr &a = shapes().a[R.shape];
+        a.kern<<<(unsigned)R.grid, a.threads, R.smem, st>>>(A);
+      }
+    }
+    const int rc = bigint_launch_status();
+    if (rc != BIGINT_OK) return rc;
+  }
+  return BIGINT_OK;
+}
+
+// This unit's record of products that gave up at a wait limit, and its wait
+// limit (see tcm::take_timeout_here).
+int rag_take_timeout() { return tcm::take_timeout_here(); }
+int rag_set_wait_limit(long long cycles) { return tcm::set_wait_limit_here(cycles); }
+
+}  // namespace bigint

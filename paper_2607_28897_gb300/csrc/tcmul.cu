@@ -5,6 +5,7 @@
 // (tccore.cuh: the digit convolution as tcgen05 fp16 MMAs with exact fp32
 // accumulation, Sec. V-B's schoolbook product on the tensor cores).
 #include "tccore.cuh"
+#include "ragged.cuh"
 #include "tcone.cuh"
 
 namespace bigint {
@@ -318,12 +319,23 @@ static int launch_shape(TcShape sh, const TcArgs &A, int64_t count, int nx, int 
   }
 }
 
+// Modelled cycles of an MMA of N columns: the larger of its math (128 x N x
+// 16 fp16 multiply-adds at ~6750 flop/cycle per SM) and its operand reads
+// from shared memory (4 KB of A plus 32 N bytes of B at 128 bytes/cycle),
+// and at least 46 (the tightest issue loop).
+static double mma_cycles(int N) {
+  const double math = 4096.0 * N / 6750.0, rd = 32.0 + N / 4.0;
+  const double c = math > rd ? math : rd;
+  return c > 46 ? c : 46;
+}
+
+// The models look at every st-th of n Toeplitz blocks (their widths change
+// slowly), so that a choice costs a microsecond or two on the host.
+static int sample_step(int n) { return n > 48 ? n / 24 : 1; }
+
 // Modelled tensor-core cycles of one product of a shape (x of nx, y of ny
-// limbs, low nout limbs, band start lo), following tc_product's tile loop:
-// each MMA of N columns costs the larger of its math (128 x N x 16 fp16
-// multiply-adds at ~6750 flop/cycle per SM) and its operand reads from
-// shared memory (4 KB of A plus 32 N bytes of B at 128 bytes/cycle), and at
-// least 46 (the tightest issue loop); the tiles (each a fixed cost: its first Hankel build, last drain and column
+// limbs, low nout limbs, band start lo), following tc_product's tile loop;
+// the tiles (each a fixed cost: its first Hankel build, last drain and column
 // sums) count 4000 cycles.  tiles_out: the product's tiles.
 static double tc_model(TcShape sh, int nx, int ny, int nout, int lo, int *tiles_out = nullptr) {
   const ShapeInfo &I = SHAPES[sh];
@@ -343,12 +355,11 @@ static double tc_model(TcShape sh, int nx, int ny, int nout, int lo, int *tiles_
     tiles++;
     const int e_lo = c0 - mx + 1 > 0 ? (c0 - mx + S) / S : 0;
     const int e_hi = (c0 + W - 1) / S < ey ? (c0 + W - 1) / S : ey;
-    for (int e = e_lo; e <= e_hi; e++) {
+    const int st = sample_step(e_hi - e_lo + 1);
+    for (int e = e_lo; e <= e_hi; e += st) {
       const int ca = (c0 > S * e ? c0 : S * e) - c0, cb = (c0 + W < S * e + mx ? c0 + W : S * e + mx) - c0;
-      const int N = ((cb + 15) & ~15) - (ca & ~15);
-      const double math = 4096.0 * N / 6750.0, rd = 32.0 + N / 4.0;
-      const double mma = math > rd ? math : rd;
-      cyc += (KB / 16) * (mma > 46 ? mma : 46);
+      cyc += (KB / 16) * mma_cycles(((cb + 15) & ~15) - (ca & ~15)) *
+             (e + st <= e_hi + 1 ? st : e_hi + 1 - e);
     }
   }
   if (tiles_out) *tiles_out = tiles;
@@ -412,11 +423,7 @@ static TcShape best_shape(int nx, int ny, int nout, int lo, int kb_mask, int nt,
 }
 
 // ---- one-drain products (tcone.cuh) -------------------------------------------
-// Warps per CTA.  More of them (8 / 16) shorten a lone product's phases by
-// 15 % but not a batch, where the CTAs sharing the SM overlap anyway
-// (512-limb products 2451 against 2167 us per 65536).
-template <int NT>
-constexpr int one_warps() { return NT == 128 ? 4 : 8; }
+using tcm::one_warps;
 
 // Attributes of k_mul_one<NT>: its largest dynamic shared memory, and the
 // CTAs of a given dynamic shared memory resident on one SM (TMEM allows
@@ -468,37 +475,25 @@ static int one_per_sm(size_t smem) {
 // Fitted to 25 measured shapes of 8 to 9000 limbs; within 15 % of them.
 template <int NT>
 static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
-  constexpr int R = tcm::ONE_R, S = tcm::ONE_S, W = one_warps<NT>();
+  constexpr int S = tcm::ONE_S, W = one_warps<NT>();
   if ((nx < ny ? nx : ny) > tcm::ONE_MAX || !one_attr<NT>().ok) return 0;
-  const tcm::OneLayout L = tcm::one_layout<W>(nx, ny, 0);
-  int blocks = 0, tiles = 0;
-  double cyc = nx;
-  for (int c0 = lo > 0 ? (lo / R - (S - 1) > 0 ? lo / R - (S - 1) : 0) : 0; R * c0 < nout;
-       c0 += NT) {
-    int Wd = L.cmma + S - 1 - c0 < NT ? L.cmma + S - 1 - c0 : NT;
-    const int need = (nout - R * c0 + R - 1) / R;
-    if (Wd > need) Wd = need;
-    Wd = (Wd + 15) & ~15;
-    int e_lo, e_hi;
-    tcm::one_blocks(L.mx, L.ey, c0, Wd, e_lo, e_hi);
-    const int nb = e_hi >= e_lo ? e_hi - e_lo + 1 : 0;
-    if (nb > blocks) blocks = nb;
-    tiles++;
-    cyc += 16.0 * nb + 8.0 * Wd;
-    for (int e = e_lo; e <= e_hi; e++) {
-      const int ca = (c0 > S * e ? c0 : S * e) - c0;
-      const int cb = (c0 + Wd < S * e + L.mx ? c0 + Wd : S * e + L.mx) - c0;
-      const int N = ((cb + 15) & ~15) - (ca & ~15);
-      const double math = 4096.0 * N / 6750.0, rd = 32.0 + N / 4.0;
-      const double mma = math > rd ? math : rd;
-      cyc += 2 * (mma > 46 ? mma : 46);
-    }
-  }
-  const uint32_t total = tcm::one_layout<W>(nx, ny, blocks).total;
+  const uint32_t total = tcm::one_bytes<NT, W>(nx, ny, nout, lo);
   if (total > (uint32_t)one_attr<NT>().dyn) return 0;
   if (cost != nullptr) {
-    const int per_sm = one_per_sm<NT>(total);
-    *cost = cyc + tiles * (per_sm == 1 ? 7400.0 : 6000.0 / per_sm);
+    const int mx = tcm::one_layout<W>(nx, ny, 0).mx, per_sm = one_per_sm<NT>(total);
+    double cyc = nx;
+    tcm::one_tiles<NT>(nx, ny, nout, lo, [&](int c0, int Wd, int e_lo, int e_hi) {
+      cyc += 8.0 * Wd + (per_sm == 1 ? 7400.0 : 6000.0 / per_sm);
+      if (e_hi < e_lo) return;
+      cyc += 16.0 * (e_hi - e_lo + 1);
+      const int st = sample_step(e_hi - e_lo + 1);
+      for (int e = e_lo; e <= e_hi; e += st) {
+        const int ca = (c0 > S * e ? c0 : S * e) - c0;
+        const int cb = (c0 + Wd < S * e + mx ? c0 + Wd : S * e + mx) - c0;
+        cyc += 2 * mma_cycles(((cb + 15) & ~15) - (ca & ~15)) * (e + st <= e_hi + 1 ? st : e_hi + 1 - e);
+      }
+    });
+    *cost = cyc;
   }
   return total;
 }
@@ -516,6 +511,44 @@ static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, 
   tcm::k_mul_one<NT, W><<<(unsigned)grid, 32 * W, smem, st>>>(
       A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag);
   return bigint_launch_status();
+}
+
+// Tile columns of the one-drain form, either operand as x (*swap), where its
+// model is cheaper than `than` (< 0: anything); 0 where it is not.
+static int best_one(int nx, int ny, int nout, int lo, double than, bool *swap) {
+  int nt = 0;
+  double c;
+  for (int k = 0; k < (nx == ny ? 1 : 2); k++) {
+    const int mx = k ? ny : nx, my = k ? nx : ny;
+    if (one_plan<128>(mx, my, nout, lo, &c) && (than < 0 || c < than))
+      than = c, nt = 128, *swap = k != 0;
+    if (one_plan<256>(mx, my, nout, lo, &c) && (than < 0 || c < than))
+      than = c, nt = 256, *swap = k != 0;
+  }
+  return nt;
+}
+
+// The same choice for a product of a grouped launch (ragged.cu): a RagShape,
+// with x as the operand of nx limbs unless *swap.
+int tc_choose(int nx, int ny, int nout, int lo, bool *swap) {
+  int sh = RAG_256;
+  double best = -1;
+  *swap = nx > ny;
+  for (int k = 0; k < (nx == ny ? 1 : 2); k++) {
+    const int mx = k ? ny : nx, my = k ? nx : ny;
+    if (mx > 16383) continue;
+    static const struct { TcShape s; int r; } forms[3] = {
+        {TC_64_XC, RAG_64}, {TC_128_XC, RAG_128}, {TC_256, RAG_256}};
+    for (const auto &f : forms) {
+      const double c = shape_cost(f.s, mx, my, nout, lo);
+      if (c >= 0 && (best < 0 || c < best)) best = c, sh = f.r, *swap = k != 0;
+    }
+  }
+  bool sw = false;
+  const int nt = best_one(nx, ny, nout, lo, best, &sw);
+  if (nt == 0) return sh;
+  *swap = sw;
+  return nt == 128 ? RAG_ONE128 : RAG_ONE256;
 }
 
 // force: 0 (the one-drain or 128-digit-block shape by the models above and
@@ -566,18 +599,8 @@ int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
     }
   }
   if (force == 0) {
-    // the one-drain form, either operand as x, where its model is cheaper
-    double best = keep;
-    int nt1 = 0;
     bool sw = false;
-    for (int k = 0; k < (nx == ny ? 1 : 2); k++) {
-      const int mx = k ? ny : nx, my = k ? nx : ny;
-      double c;
-      if (one_plan<128>(mx, my, nout, lo, &c) && (best < 0 || c < best))
-        best = c, nt1 = 128, sw = k != 0;
-      if (one_plan<256>(mx, my, nout, lo, &c) && (best < 0 || c < best))
-        best = c, nt1 = 256, sw = k != 0;
-    }
+    const int nt1 = best_one(nx, ny, nout, lo, keep, &sw);
     if (nt1 != 0) {
       TcArgs B = A;
       if (sw) {

@@ -15,7 +15,7 @@
 #include "common.cuh"
 
 namespace bigint {
-int batch_create(const bigint_op *ops, int64_t nops, bigint_batch **out);
+int batch_create(const bigint_op *ops, int64_t nops, bool steps, bigint_batch **out);
 size_t batch_workspace_bytes(const bigint_batch *B);
 int batch_upload(bigint_batch *B, void *ws, size_t bytes, cudaStream_t st);
 int batch_launch(const bigint_batch *B, const uint64_t *in, uint64_t *out, int32_t *status,
@@ -106,7 +106,7 @@ int run_ops(const std::vector<bigint_op> &ops, const uint64_t *in, uint64_t *out
             int32_t *status, void *ws, size_t bytes, int mode, cudaStream_t st) {
   if (ops.empty()) return BIGINT_OK;
   bigint_batch *B = nullptr;
-  int rc = batch_create(ops.data(), (int64_t)ops.size(), &B);
+  int rc = batch_create(ops.data(), (int64_t)ops.size(), mode == BIGINT_BATCH_STEPS, &B);
   if (rc != BIGINT_OK) return rc;
   if (bytes < batch_workspace_bytes(B)) {
     batch_destroy(B);
@@ -120,10 +120,10 @@ int run_ops(const std::vector<bigint_op> &ops, const uint64_t *in, uint64_t *out
   return rc;
 }
 
-size_t ops_workspace(const std::vector<bigint_op> &ops) {
+size_t ops_workspace(const std::vector<bigint_op> &ops, bool steps) {
   if (ops.empty()) return 0;
   bigint_batch *B = nullptr;
-  if (batch_create(ops.data(), (int64_t)ops.size(), &B) != BIGINT_OK) return 0;
+  if (batch_create(ops.data(), (int64_t)ops.size(), steps, &B) != BIGINT_OK) return 0;
   const size_t b = batch_workspace_bytes(B);
   batch_destroy(B);
   return b;
@@ -163,7 +163,7 @@ size_t bigint_batch_views_workspace(int op, const bigint_batch_cview *a,
     x.flags = (op == BIGINT_OP_ADD || op == BIGINT_OP_SUB) && x.na != x.nb ? BIGINT_ZEXT : 0;
     x.a = x.b = x.o1 = x.o2 = 0;
   }
-  return ops_workspace(ops);
+  return ops_workspace(ops, false);
 }
 
 int bigint_batch_add(const bigint_batch_cview *a, const bigint_batch_cview *b,
@@ -193,7 +193,7 @@ int bigint_batch_divmod(const bigint_batch_cview *u, const bigint_batch_cview *v
 
 size_t bigint_batch_run_workspace(const bigint_op *ops, int64_t nops) {
   if (nops < 0 || (nops > 0 && !ops)) return 0;
-  return ops_workspace(std::vector<bigint_op>(ops, ops + nops));
+  return ops_workspace(std::vector<bigint_op>(ops, ops + nops), true);
 }
 
 int bigint_batch_run(const bigint_op *ops, int64_t nops, const uint64_t *in_pool,

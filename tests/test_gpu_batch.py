@@ -262,3 +262,81 @@ def test_division_classes_with_irregular_members(orc):
         check(ops, to_host(dout), st.cpu().numpy(), exp, exp_st)
         got.append(to_host(dout))
     assert np.array_equal(got[0], got[1])
+
+
+@pytest.mark.parametrize("seed,lo,hi", [(1, 128, 300), (2, 128, 1100), (3, 500, 2600)])
+def test_grouped_divisions_of_mixed_shapes(orc, seed, lo, hi):
+    """Steps form over divisions of unrelated shapes -- quotients of 1 to a
+    few limbs, as long as the divisor and longer, zero and short divisors in
+    between -- and products of unrelated sizes, all grouped by step."""
+    import torch
+
+    import paper_2607_28897_gb300 as bi
+    from paper_2607_28897_gb300 import inputs
+
+    rng = np.random.default_rng(seed)
+    count = 380
+    ops = np.zeros(count, dtype=bi.op_dtype())
+    pos, opos, parts = 0, 0, []
+    for i in range(count):
+        nb = int(rng.integers(lo, hi))
+        if i < 80:
+            kind = bi.OP_DIVMOD
+            na = nb + [0, 1, 2, 3, 5, nb // 3, nb - 1, nb, 2 * nb][i % 9]
+        else:
+            kind = bi.OP_MUL
+            na = int(rng.integers(64, hi))
+        a = inputs.limbs(1000 * seed + i, 1, na, top_nonzero=True)[0]
+        b = inputs.limbs(2000 * seed + i, 1, nb, top_nonzero=True)[0]
+        if i == 7:
+            b[:] = 0
+        elif i in (8, 9):
+            b[-2:] = 0
+        elif i == 10:
+            a[-40:] = 0
+        elif i % 13 == 11:
+            a[:], b[:] = np.uint64(0xFFFFFFFFFFFFFFFF), np.uint64(0x7F807F807F807F80)
+        n1, n2 = (na - nb + 1, nb) if kind == bi.OP_DIVMOD else (na + nb, 0)
+        ops[i] = (kind, na, nb, 0, pos, pos + na, opos, opos + n1 if n2 else 0)
+        parts += [a, b]
+        pos += na + nb
+        opos += n1 + n2
+    pool = np.concatenate(parts)
+    exp, exp_st = oracle_results(orc, ops, pool)
+    dpool = to_dev(pool).view(-1)
+    B = bi.Batch(ops)
+    for _ in range(2):  # the plan replayed
+        dout = torch.zeros(opos, dtype=torch.int64, device="cuda")
+        st = torch.full((count,), 99, dtype=torch.int32, device="cuda")
+        B.launch(dpool, dout, st, mode=bi.BATCH_STEPS)
+        torch.cuda.synchronize()
+        bi.check_timeout()
+        check(ops, to_host(dout), st.cpu().numpy(), exp, exp_st)
+
+
+def test_grouped_divisions_in_waves():
+    """More divisions than one wave's records hold (1 GiB): the second wave
+    reuses them.  Against the uniform division of the same operands."""
+    import torch
+
+    import paper_2607_28897_gb300 as bi
+    from paper_2607_28897_gb300 import inputs
+
+    nu, nv, count = 8192, 4096, 5200
+    u = inputs.limbs_torch(71, count, nu, True, "cuda")
+    v = inputs.limbs_torch(72, count, nv, True, "cuda")
+    q, r, _ = bi.divmod(u, v)
+    ops = np.zeros(count, dtype=bi.op_dtype())
+    i = np.arange(count)
+    nq = nu - nv + 1
+    ops["op"], ops["na"], ops["nb"] = bi.OP_DIVMOD, nu, nv
+    ops["a"], ops["b"] = i * nu, count * nu + i * nv
+    ops["o1"], ops["o2"] = i * nq, count * nq + i * nv
+    pool = torch.cat([u.view(-1), v.view(-1)])
+    out = torch.zeros(count * (nq + nv), dtype=torch.int64, device="cuda")
+    st = torch.full((count,), 99, dtype=torch.int32, device="cuda")
+    bi.Batch(ops).launch(pool, out, st, mode=bi.BATCH_STEPS)
+    assert torch.equal(out[:count * nq].view(count, nq), q)
+    assert torch.equal(out[count * nq:].view(count, nv), r)
+    assert not st.any()
+    bi.check_timeout()
