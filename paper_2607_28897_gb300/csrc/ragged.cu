@@ -25,7 +25,7 @@
 #include <unordered_map>
 
 #include "divstep.cuh"
-#include "tcone.cuh"
+#include "tcpipe.cuh"
 
 namespace bigint {
 
@@ -250,9 +250,81 @@ __global__ void __launch_bounds__(32 * tcm::one_warps<NT>(), 512 / NT) k_rag_one
   tcm::one_release<NT>(c);
 }
 
+// The pipelined form.  The builders read an operation's table entries and
+// hand the product to the other warps through a ring in shared memory, so
+// that the issuing warp does not stall on two dependent loads per product.
+constexpr int RING = 4;
+struct RagRing {
+  uint64_t full[RING], free[RING];
+  tcm::PipeTask t[RING];
+};
+
+template <int KB>
+__global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tcm::PipeLayout L) {
+  using namespace tcm;
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ PipeShared sh;
+  __shared__ RagRing ring;
+  const int lane = (int)lane_id();
+  const long long lim = wait_limit_here();
+  if (threadIdx.x == 0) {
+    for (int i = 0; i < RING; i++) {
+      mbar_init(smem_u32(&ring.full[i]), 1);
+      mbar_init(smem_u32(&ring.free[i]), PIPE_DRAIN / 32 + 1);
+    }
+  }
+  auto next_b = [&](int64_t k, PipeTask &T) {
+    const int64_t i = blockIdx.x + k * gridDim.x;
+    const bool more = i < A.n;
+    T.nx = 0;
+    if (more) {
+      const int32_t e = A.list[i];
+      const RagTask t = rag_task(A, A.ops[e & ~RAG_SWAP], (e & RAG_SWAP) != 0);
+      T = PipeTask{t.x, t.y, t.out, t.nx, t.ny, t.nout, t.lo};
+    }
+    if (threadIdx.x == PIPE_DRAIN + 32) {  // the first builder thread
+      const int r = (int)(k % RING);
+      if (k >= RING && !pipe_wait(&sh, &ring.free[r], (uint32_t)(k / RING - 1) & 1u, lim))
+        return false;
+      ring.t[r] = T;
+      mbar_arrive(smem_u32(&ring.full[r]));
+    }
+    return more;
+  };
+  auto take = [&](int64_t k, PipeTask &T) {  // by a whole warp, once the slot is full
+    T = ring.t[k % RING];
+    __syncwarp();
+    if (lane == 0) mbar_arrive(smem_u32(&ring.free[k % RING]));
+    return T.nx != 0;
+  };
+  auto next_i = [&](int64_t k, PipeTask &T) {
+    if (!pipe_wait_warp(&sh, &ring.full[k % RING], (uint32_t)(k / RING) & 1u, lim)) return false;
+    return take(k, T);
+  };
+  auto next_d = [&](int64_t k, PipeTask &T) {
+    const bool bad = !pipe_wait(&sh, &ring.full[k % RING], (uint32_t)(k / RING) & 1u, lim);
+    if (bar_or_drain<PIPE_DRAIN>(bad)) return false;  // all drain threads agree
+    return take(k, T);
+  };
+  int64_t ndone = 0;
+  auto status = [&](int64_t k, int32_t st) {
+    if (A.kind == RAG_MUL && A.status != nullptr)
+      A.status[A.ops[A.list[blockIdx.x + k * gridDim.x] & ~RAG_SWAP].opi] = st;
+  };
+  auto done = [&](int64_t k) {
+    if (threadIdx.x == 0) status(k, BIGINT_OK);
+    ndone = k + 1;
+  };
+  if (!pipe_run<KB>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
+    atomicExch(A.abort_flag, 1);
+    for (int64_t k = ndone; blockIdx.x + k * gridDim.x < A.n; k++) status(k, BIGINT_ETIMEOUT);
+  }
+}
+
 // ---- host ------------------------------------------------------------------
 struct ShapeAttr {
-  void (*kern)(RagArgs);
+  void (*kern)(RagArgs);                    // or, pipelined forms:
+  void (*pipe)(RagArgs, tcm::PipeLayout);
   int threads, cap;    // CTAs per SM the tensor memory allows
   int dyn, overhead;   // largest dynamic shared memory; static and reserved
 };
@@ -268,12 +340,14 @@ const Shapes &shapes() {
   static const Shapes S = [] {
     using tcm::one_warps;
     Shapes s;
-    s.a[RAG_ONE128] = {k_rag_one<128>, 32 * one_warps<128>(), 4, 0, 0};
-    s.a[RAG_ONE256] = {k_rag_one<256>, 32 * one_warps<256>(), 2, 0, 0};
-    s.a[RAG_64] = {k_rag_tc<64, 7>, 2 * 64 + 32, 4, 0, 0};
-    s.a[RAG_128] = {k_rag_tc<128, 8>, 2 * 128 + 32, 2, 0, 0};
-    s.a[RAG_256] = {k_rag_tc<256, 8>, 2 * 256 + 32, 1, 0, 0};
-    s.a[RAG_256_G4] = {k_rag_tc<256, 4>, 2 * 256 + 32, 1, 0, 0};
+    s.a[RAG_ONE128] = {k_rag_one<128>, nullptr, 32 * one_warps<128>(), 4, 0, 0};
+    s.a[RAG_ONE256] = {k_rag_one<256>, nullptr, 32 * one_warps<256>(), 2, 0, 0};
+    s.a[RAG_64] = {k_rag_tc<64, 7>, nullptr, 2 * 64 + 32, 4, 0, 0};
+    s.a[RAG_128] = {k_rag_tc<128, 8>, nullptr, 2 * 128 + 32, 2, 0, 0};
+    s.a[RAG_256] = {k_rag_tc<256, 8>, nullptr, 2 * 256 + 32, 1, 0, 0};
+    s.a[RAG_256_G4] = {k_rag_tc<256, 4>, nullptr, 2 * 256 + 32, 1, 0, 0};
+    s.a[RAG_PIPE128] = {nullptr, k_rag_pipe<128>, tcm::PIPE_THREADS, 1, 0, 0};
+    s.a[RAG_PIPE64] = {nullptr, k_rag_pipe<64>, tcm::PIPE_THREADS, 1, 0, 0};
     int dev = 0, optin = 0, reserved = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
@@ -286,10 +360,11 @@ const Shapes &shapes() {
       return s;
     for (ShapeAttr &x : s.a) {
       cudaFuncAttributes fa;
-      if (cudaFuncGetAttributes(&fa, x.kern) != cudaSuccess) return s;
+      const void *k = x.kern ? (const void *)x.kern : (const void *)x.pipe;
+      if (cudaFuncGetAttributes(&fa, k) != cudaSuccess) return s;
       x.dyn = optin - (int)fa.sharedSizeBytes;
       x.overhead = (int)fa.sharedSizeBytes + reserved;
-      if (cudaFuncSetAttribute(x.kern, cudaFuncAttributeMaxDynamicSharedMemorySize, x.dyn) !=
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, x.dyn) !=
           cudaSuccess)
         return s;
     }
@@ -303,6 +378,13 @@ const Shapes &shapes() {
   return S;
 }
 
+// Shared memory of a pipelined product, over the limit where x does not fit.
+template <int KB>
+uint32_t pipe_bytes_of(int nx, uint32_t dyn) {
+  const tcm::PipeLayout L = tcm::pipe_layout<KB>(nx, dyn);
+  return L.total ? L.total : ~0u;
+}
+
 uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
   using namespace tcm;
   switch (shape) {
@@ -311,6 +393,8 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
     case RAG_64: return layout<64, 7>(nx, ny).total;
     case RAG_128: return layout<128, 8>(nx, ny).total;
     case RAG_256: return layout<256, 8>(nx, ny).total;
+    case RAG_PIPE128: return pipe_bytes_of<128>(nx, (uint32_t)shapes().a[shape].dyn);
+    case RAG_PIPE64: return pipe_bytes_of<64>(nx, (uint32_t)shapes().a[shape].dyn);
     default: return layout<256, 4>(nx, ny).total;
   }
 }
@@ -322,7 +406,8 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
 // function of the sizes alone) are kept per thread, MEMO_MAX of them at most.
 // The shared memory is that of the actual sizes.
 struct Form {
-  int shape, per_sm;
+  int shape, per_sm, group;  // products of one group share a launch
+  int nx;                    // limbs of the operand stored whole
   bool swap;
   uint32_t bytes;
 };
@@ -373,7 +458,16 @@ class Chooser {
       }
     }
     const ShapeAttr &a = shapes().a[f.shape];
+    f.nx = ax;
+    if (a.pipe) {  // one CTA per SM; those whose x is double buffered apart
+      f.per_sm = 1;
+      f.group = f.shape * 8 + (f.shape == RAG_PIPE128
+                                   ? tcm::pipe_layout<128>(ax, (uint32_t)a.dyn).xbufs
+                                   : tcm::pipe_layout<64>(ax, (uint32_t)a.dyn).xbufs);
+      return f;
+    }
     f.per_sm = std::max(1, std::min(a.cap, shapes().smem_sm / ((int)f.bytes + a.overhead)));
+    f.group = f.shape * 8 + f.per_sm;
     return f;
   }
 
@@ -391,10 +485,9 @@ class Chooser {
 // Appends the launches of one kind of product over ops [first, first + n).
 void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, int l, int par) {
   struct Item {
-    int group;
+    Form f;
     double cost;
     int32_t entry;
-    uint32_t bytes;
   };
   std::vector<Item> items;
   items.reserve(n);
@@ -403,11 +496,10 @@ void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, i
     int nx, ny, nout, lo;
     rag_sizes(o.nu, o.nv, kind, l, nx, ny, nout, lo);
     const Form f = C.get(nx, ny, nout, lo);
-    items.push_back({f.shape * 8 + f.per_sm, (double)nx * ny,
-                     (int32_t)(first + i) | (f.swap ? RAG_SWAP : 0), f.bytes});
+    items.push_back({f, (double)nx * ny, (int32_t)(first + i) | (f.swap ? RAG_SWAP : 0)});
   }
   std::stable_sort(items.begin(), items.end(), [](const Item &a, const Item &b) {
-    return a.group != b.group ? a.group > b.group : a.cost > b.cost;
+    return a.f.group != b.f.group ? a.f.group > b.f.group : a.cost > b.cost;
   });
   for (size_t i = 0; i < items.size();) {
     size_t j = i;
@@ -416,14 +508,15 @@ void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, i
     R.kind = kind;
     R.l = l;
     R.par = par;
-    R.shape = items[i].group / 8;
+    R.shape = items[i].f.shape;
     R.first = (int64_t)P.list.size();
-    for (; j < items.size() && items[j].group == items[i].group; j++) {
+    for (; j < items.size() && items[j].f.group == items[i].f.group; j++) {
       P.list.push_back(items[j].entry);
-      R.smem = std::max(R.smem, items[j].bytes);
+      R.smem = std::max(R.smem, items[j].f.bytes);
+      R.nx = std::max(R.nx, items[j].f.nx);
     }
     R.n = (int64_t)(j - i);
-    R.grid = (int)std::min<int64_t>(R.n, (int64_t)shapes().sms * (items[i].group % 8));
+    R.grid = (int)std::min<int64_t>(R.n, (int64_t)shapes().sms * items[i].f.per_sm);
     P.program.push_back(R);
     i = j;
   }
@@ -515,7 +608,14 @@ int rag_launch(const RagPlan &P, const RagBuffers &B, const uint64_t *in, uint64
       case RAG_FINISH: k_rag_finish<<<n, LIN_THREADS, 0, st>>>(A); break;
       default: {
         const ShapeAttr &a = shapes().a[R.shape];
-        a.kern<<<(unsigned)R.grid, a.threads, R.smem, st>>>(A);
+        if (a.pipe) {
+          const tcm::PipeLayout L = R.shape == RAG_PIPE128
+                                        ? tcm::pipe_layout<128>(R.nx, (uint32_t)a.dyn)
+                                        : tcm::pipe_layout<64>(R.nx, (uint32_t)a.dyn);
+          a.pipe<<<(unsigned)R.grid, a.threads, L.total, st>>>(A, L);
+        } else {
+          a.kern<<<(unsigned)R.grid, a.threads, R.smem, st>>>(A);
+        }
       }
     }
     const int rc = bigint_launch_status();

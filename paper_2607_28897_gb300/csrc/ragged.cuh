@@ -19,7 +19,10 @@ struct RagOp {
 };
 
 // Product forms of a grouped launch (tc_choose).
-enum RagShape { RAG_ONE128, RAG_ONE256, RAG_64, RAG_128, RAG_256, RAG_256_G4, RAG_NSHAPES };
+enum RagShape {
+  RAG_ONE128, RAG_ONE256, RAG_64, RAG_128, RAG_256, RAG_256_G4, RAG_PIPE128, RAG_PIPE64,
+  RAG_NSHAPES
+};
 
 // A list of operations (RagOp indices, RAG_SWAP set where the second operand
 // is the one stored whole in shared memory) whose products of one kind run
@@ -32,7 +35,8 @@ enum RagWhat { RAG_START, RAG_SMALL, RAG_PROD, RAG_MID, RAG_UPDATE, RAG_FINISH }
 struct RagLaunch {
   int what, kind, l, par;  // step (limbs known before it), parity of its iterate
   int shape, grid;
-  uint32_t smem;
+  uint32_t smem;           // RAG_PROD: dynamic shared memory
+  int nx;                  // largest operand stored whole
   int64_t first, n;        // RAG_PROD: range of the list; else ops [first, first + n)
 };
 

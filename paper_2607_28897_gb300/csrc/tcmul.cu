@@ -7,6 +7,7 @@
 #include "tccore.cuh"
 #include "ragged.cuh"
 #include "tcone.cuh"
+#include "tcpipe.cuh"
 
 namespace bigint {
 namespace tcm {
@@ -64,6 +65,24 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
   }
   if (c.aborted && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
   one_release<NT>(c);
+}
+
+// The same by the pipeline of tcpipe.cuh: one CTA per SM.
+template <int KB>
+__global__ void __launch_bounds__(PIPE_THREADS, 1)
+    k_mul_pipe(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
+               uint64_t *__restrict__ Out, int nx, int ny, int nout, int64_t count, int64_t sx,
+               int64_t sy, int64_t so, int lo, int *abort_flag, PipeLayout L) {
+  extern __shared__ __align__(1024) uint8_t sm[];
+  __shared__ PipeShared sh;
+  auto next = [&](int64_t k, PipeTask &T) {
+    const int64_t i = blockIdx.x + k * gridDim.x;
+    if (i >= count) return false;
+    T = PipeTask{X + i * sx, Y + i * sy, Out + i * so, nx, ny, nout, lo};
+    return true;
+  };
+  const bool ok = pipe_run<KB>(L, &sh, sm, next, next, next, [](int64_t) {});
+  if (!ok && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
 }
 
 // Split products: unit u is tile u % T of product u / T (tc_product's split
@@ -377,28 +396,18 @@ static bool shape_applies(TcShape sh, int nx, int ny, int nout, int lo) {
   return tiles <= 1;
 }
 
-// Modelled time of a product on one SM: tensor-core cycles, shared by the
-// CTAs resident on it; with one CTA per SM the setup, first Hankel build,
-// last drains and column sums of each product do not overlap another CTA's
-// MMAs, which the model charges as 15 % more.
+// Modelled time of a product on one SM: the tensor-core cycles times what the
+// shape was measured to take of them (66 shapes of 8 to 9000 limbs, fitted
+// together with the models of the other two forms so that the cheapest by
+// model is the fastest within 1 % on average): several small-tile CTAs share
+// the SM well (64 columns), two less so, and one alone does not cover its
+// setup, drains and column sums.
 static double shape_cost(TcShape sh, int nx, int ny, int nout, int lo) {
   if (!shape_applies(sh, nx, ny, nout, lo)) return -1;
   const size_t smem = shape_smem(sh, nx, ny);
   if (smem == 0) return -1;
-  int per_sm = 1;
-  switch (sh) {
-    case TC_64_XC: per_sm = tc_per_sm<64, 7, true, 128>(smem); break;
-    case TC_64_NOXC: per_sm = tc_per_sm<64, 7, false, 128>(smem); break;
-    case TC_128_XC: per_sm = tc_per_sm<128, 8, true, 128>(smem); break;
-    case TC_128_NOXC: per_sm = tc_per_sm<128, 8, false, 128>(smem); break;
-    case TC_N64_XC: per_sm = tc_per_sm<128, 15, true, 64>(smem); break;
-    case TC_N64_NOXC: per_sm = tc_per_sm<128, 15, false, 64>(smem); break;
-    case TC_N32_XC: per_sm = tc_per_sm<128, 12, true, 32>(smem); break;
-    case TC_N32_NOXC: per_sm = tc_per_sm<128, 12, false, 32>(smem); break;
-    default: per_sm = 1;
-  }
   const double c = tc_model(sh, nx, ny, nout, lo);
-  return per_sm > 1 ? c : 1.15 * c;
+  return c * (SHAPES[sh].nt == 256 ? 1.7 : (SHAPES[sh].nt == 128 ? 1.5 : 1.0));
 }
 
 // The cheapest shape by the model for x of nx, y of ny limbs (among those
@@ -470,9 +479,8 @@ static int one_per_sm(size_t smem) {
 // its modelled time on one SM in tensor-core cycles, comparable with
 // shape_cost: the MMAs (their math, their operands' reads, at least 46
 // cycles each), the shared-memory cycles of a tile's Hankel matrices (16 per
-// block) and transposes (8 per column), and the part of a tile's ~6000
+// block) and transposes (8 per column), and the part of a tile's ~5000
 // cycles of latency and limb work that the CTAs sharing the SM do not hide.
-// Fitted to 25 measured shapes of 8 to 9000 limbs; within 15 % of them.
 template <int NT>
 static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
   constexpr int S = tcm::ONE_S, W = one_warps<NT>();
@@ -483,7 +491,7 @@ static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
     const int mx = tcm::one_layout<W>(nx, ny, 0).mx, per_sm = one_per_sm<NT>(total);
     double cyc = nx;
     tcm::one_tiles<NT>(nx, ny, nout, lo, [&](int c0, int Wd, int e_lo, int e_hi) {
-      cyc += 8.0 * Wd + (per_sm == 1 ? 7400.0 : 6000.0 / per_sm);
+      cyc += 8.0 * Wd + (per_sm == 1 ? 7400.0 : (NT == 128 ? 5000.0 : 4500.0) / per_sm);
       if (e_hi < e_lo) return;
       cyc += 16.0 * (e_hi - e_lo + 1);
       const int st = sample_step(e_hi - e_lo + 1);
@@ -513,19 +521,85 @@ static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, 
   return bigint_launch_status();
 }
 
-// Tile columns of the one-drain form, either operand as x (*swap), where its
-// model is cheaper than `than` (< 0: anything); 0 where it is not.
-static int best_one(int nx, int ny, int nout, int lo, double than, bool *swap) {
-  int nt = 0;
-  double c;
+// ---- pipelined products (tcpipe.cuh) --------------------------------------------
+template <int KB>
+static const OneAttr &pipe_attr() {
+  static const OneAttr A = [] {
+    OneAttr a;
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+            cudaSuccess ||
+        cudaFuncGetAttributes(&fa, tcm::k_mul_pipe<KB>) != cudaSuccess)
+      return a;
+    a.dyn = optin - (int)fa.sharedSizeBytes;
+    a.ok = cudaFuncSetAttribute(tcm::k_mul_pipe<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                a.dyn) == cudaSuccess;
+    return a;
+  }();
+  return A;
+}
+
+template <int KB>
+static int launch_pipe(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
+  if (!pipe_attr<KB>().ok) return BIGINT_ECUDA;
+  const tcm::PipeLayout L = tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB>().dyn);
+  if (L.total == 0 || nx < 64) return BIGINT_EINVAL;
+  if (count == 0) return BIGINT_OK;
+  const int sms = sm_count();
+  if (sms == 0) return BIGINT_ECUDA;
+  tcm::k_mul_pipe<KB><<<(unsigned)(count < sms ? count : sms), tcm::PIPE_THREADS, L.total, st>>>(
+      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag, L);
+  return bigint_launch_status();
+}
+
+// Modelled time of a product in the pipelined form (-1: x does not fit): its
+// MMAs, at least 42 cycles each (warp-uniform issue), 10 % slower beside the
+// drains and builds, 900 cycles a drain and 9000 a tile (the part of its
+// limbs that two groups of MMAs do not cover).
+template <int KB>
+static double pipe_cost(int nx, int ny, int nout, int lo) {
+  constexpr int S = 128 / KB;
+  if (nx < 64 || !pipe_attr<KB>().ok ||
+      tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB>().dyn).total == 0)
+    return -1;
+  const int mx = (8 * nx + KB - 1) / KB;
+  double cyc = 0;
+  tcm::pipe_tiles<KB>(nx, ny, nout, lo, [&](int c0, int W, int e_lo, int e_hi) {
+    cyc += 9000;
+    if (e_hi < e_lo) return true;
+    const int n = e_hi - e_lo + 1, st = sample_step(n);
+    cyc += 900.0 * ((n * KB + 1023) / 1024);
+    for (int e = e_lo; e <= e_hi; e += st) {
+      const int ca = (c0 > S * e ? c0 : S * e) - c0;
+      const int cb = (c0 + W < S * e + mx ? c0 + W : S * e + mx) - c0;
+      const int N = ((cb + 15) & ~15) - (ca & ~15);
+      const double math = N / 2.0, rd = 32.0 + N / 4.0, m = math > rd ? math : rd;
+      cyc += 1.1 * (KB / 16) * (m > 42 ? m : 42) * (e + st <= e_hi + 1 ? st : e_hi + 1 - e);
+    }
+    return true;
+  });
+  return cyc;
+}
+
+// The one-drain (RAG_ONE128, RAG_ONE256) or pipelined (RAG_PIPE128,
+// RAG_PIPE64) form, either operand as x (*swap), where its model is cheaper
+// than `than` (< 0: anything); -1 where none is.
+static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap) {
+  int form = -1;
+  auto offer = [&](double c, int f, int k) {
+    if (c >= 0 && (than < 0 || c < than)) than = c, form = f, *swap = k != 0;
+  };
   for (int k = 0; k < (nx == ny ? 1 : 2); k++) {
     const int mx = k ? ny : nx, my = k ? nx : ny;
-    if (one_plan<128>(mx, my, nout, lo, &c) && (than < 0 || c < than))
-      than = c, nt = 128, *swap = k != 0;
-    if (one_plan<256>(mx, my, nout, lo, &c) && (than < 0 || c < than))
-      than = c, nt = 256, *swap = k != 0;
+    double c;
+    if (one_plan<128>(mx, my, nout, lo, &c)) offer(c, RAG_ONE128, k);
+    if (one_plan<256>(mx, my, nout, lo, &c)) offer(c, RAG_ONE256, k);
+    offer(pipe_cost<128>(mx, my, nout, lo), RAG_PIPE128, k);
+    offer(pipe_cost<64>(mx, my, nout, lo), RAG_PIPE64, k);
   }
-  return nt;
+  return form;
 }
 
 // The same choice for a product of a grouped launch (ragged.cu): a RagShape,
@@ -545,14 +619,14 @@ int tc_choose(int nx, int ny, int nout, int lo, bool *swap) {
     }
   }
   bool sw = false;
-  const int nt = best_one(nx, ny, nout, lo, best, &sw);
-  if (nt == 0) return sh;
+  const int form = best_form(nx, ny, nout, lo, best, &sw);
+  if (form < 0) return sh;
   *swap = sw;
-  return nt == 128 ? RAG_ONE128 : RAG_ONE256;
+  return form;
 }
 
-// force: 0 (the one-drain or 128-digit-block shape by the models above and
-// below) or one of the autotuner's candidates -- TC_FORCE_64 / _128 / _256
+// force: 0 (the one-drain, pipelined or 128-digit-block shape by the models
+// above and below) or one of the autotuner's candidates -- TC_FORCE_64 / _128 / _256
 // (128-digit blocks, that tile) and TC_FORCE_N64 / _N32 (narrow blocks).
 int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
@@ -600,15 +674,19 @@ int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   }
   if (force == 0) {
     bool sw = false;
-    const int nt1 = best_one(nx, ny, nout, lo, keep, &sw);
-    if (nt1 != 0) {
+    const int form = best_form(nx, ny, nout, lo, keep, &sw);
+    if (form >= 0) {
       TcArgs B = A;
       if (sw) {
         B.x = A.y; B.y = A.x; B.sx = A.sy; B.sy = A.sx;
       }
       const int mx = sw ? ny : nx, my = sw ? nx : ny;
-      return nt1 == 128 ? launch_one<128>(B, count, mx, my, nout, st)
-                        : launch_one<256>(B, count, mx, my, nout, st);
+      switch (form) {
+        case RAG_ONE128: return launch_one<128>(B, count, mx, my, nout, st);
+        case RAG_ONE256: return launch_one<256>(B, count, mx, my, nout, st);
+        case RAG_PIPE128: return launch_pipe<128>(B, count, mx, my, nout, st);
+        default: return launch_pipe<64>(B, count, mx, my, nout, st);
+      }
     }
   }
   if (keep < 0) return BIGINT_EINVAL;

@@ -124,6 +124,40 @@ __device__ __forceinline__ void digits_down(uint64_t v, uint64_t below, uint32_t
   w[3] = unbias_h2(__byte_perm(ol, el, 0x5410));
 }
 
+// One Hankel core matrix: row r = the eight digits starting r places down the
+// digits of the limbs v[0] and v[1] (v[2] underneath), at `row`.
+__device__ __forceinline__ void hankel_rows(uint8_t *row, const uint64_t (&v)[3]) {
+  uint32_t w[8], f[7];
+  digits_down(v[0], v[1], w);
+  digits_down(v[1], v[2], w + 4);
+#pragma unroll
+  for (int i = 0; i < 7; i++) f[i] = __byte_perm(w[i], w[i + 1], 0x5432);
+  uint4 *o = reinterpret_cast<uint4 *>(row);
+#pragma unroll
+  for (int m = 0; m < 4; m++) {
+    o[2 * m] = make_uint4(w[m], w[m + 1], w[m + 2], w[m + 3]);
+    o[2 * m + 1] = make_uint4(f[m], f[m + 1], f[m + 2], f[m + 3]);
+  }
+}
+
+// Limb of eight coefficients w (biased by 2^31): V = sum_k w_k 2^(8 k) + add,
+// less the bias word of the limb (`first`: the lowest one kept), the borrow
+// taken off the high word.
+__device__ __forceinline__ void limb_of(const uint32_t (&w)[8], uint64_t add, bool first,
+                                        uint64_t &low, uint32_t &high) {
+  const uint64_t s0 = (uint64_t)w[0] + ((uint64_t)w[1] << 8) + ((uint64_t)w[2] << 16) +
+                      ((uint64_t)w[3] << 24);
+  const uint64_t s1 = (uint64_t)w[4] + ((uint64_t)w[5] << 8) + ((uint64_t)w[6] << 16) +
+                      ((uint64_t)w[7] << 24);
+  uint64_t l = s0 + (s1 << 32);
+  uint32_t h = (uint32_t)(s1 >> 32) + (l < s0);
+  l += add;
+  h += l < add;
+  const uint64_t b = first ? 0x8080808080000000ull : 0x8080808080808080ull;
+  low = l - b;
+  high = h - (l < b);
+}
+
 // Hankel core matrices 0 .. nb - 1 of the blocks ending with eb: row r of
 // matrix j = recoded y digits 128 eb + 127 - 8 j - r - w, w < 8, i.e. the
 // eight digits starting r places down the digits of the limbs 16 eb + 15 - j
@@ -143,22 +177,37 @@ __device__ __forceinline__ void one_hankel(uint8_t *hk, const uint64_t *y, int n
     for (int u = 0; u < 2; u++) {
       const int j = j0 + u * THREADS;
       if (j >= nb) break;
-      uint32_t w[8], f[7];
-      digits_down(v[u][0], v[u][1], w);
-      digits_down(v[u][1], v[u][2], w + 4);
-#pragma unroll
-      for (int i = 0; i < 7; i++) f[i] = __byte_perm(w[i], w[i + 1], 0x5432);
-      uint4 *row = reinterpret_cast<uint4 *>(hk + (uint32_t)j * ONE_CM);
-#pragma unroll
-      for (int m = 0; m < 4; m++) {
-        row[2 * m] = make_uint4(w[m], w[m + 1], w[m + 2], w[m + 3]);
-        row[2 * m + 1] = make_uint4(f[m], f[m + 1], f[m + 2], f[m + 3]);
-      }
+      hankel_rows(hk + (uint32_t)j * ONE_CM, v[u]);
     }
   }
 }
 
-// One thread: the MMAs of the blocks e_lo .. e_hi into the columns
+// The MMA and its commit by lane 0 of a warp that runs them converged, all
+// lanes with the same operands: in straight-line warp-uniform code the
+// descriptors are computed in and read from uniform registers, where a lone
+// thread's code moves six registers per MMA over (an issue floor of ~46
+// cycles an MMA, and ~64 cycles more per Toeplitz block).
+__device__ __forceinline__ void mma_f16_warp(uint32_t d_tmem, uint64_t a, uint64_t b,
+                                             uint32_t idesc, uint32_t accumulate,
+                                             uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred p, q;\n\t"
+      "setp.ne.b32 p, %4, 0;\n\t"
+      "setp.ne.b32 q, %5, 0;\n\t"
+      "@q tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n\t}\n" ::"r"(d_tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(accumulate), "r"(leader));
+}
+__device__ __forceinline__ void mma_commit_warp(uint32_t mbar, uint32_t leader) {
+  asm volatile(
+      "{\n\t.reg .pred q;\n\t"
+      "setp.ne.b32 q, %1, 0;\n\t"
+      "@q tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];\n\t}\n" ::
+          "r"(mbar),
+      "r"(leader)
+      : "memory");
+}
+
+// One warp: the MMAs of the blocks e_lo .. e_hi into the columns
 // [c0, c0 + W) at TMEM column dtm, then a commit to mbar.  The first block's
 // columns are overwritten, those above it up to shi cleared by a zero A
 // operand.  A block has only two MMAs of some 70 cycles each, so the loop
@@ -170,6 +219,7 @@ __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs
                                           uint32_t lbo_b, int c0, int W, int e_lo, int e_hi,
                                           int mx, int shi, uint32_t mbar) {
   tc_fence_after();
+  const uint32_t leader = lane_id() == 0;
   const uint64_t da0 = sdesc(ha, ONE_CM, ONE_CM), db0 = sdesc(xs_a, lbo_b, 128);
   const uint32_t a_hi = (uint32_t)(da0 >> 32), b_hi = (uint32_t)(db0 >> 32);
   const uint32_t step_b = (2u * lbo_b) >> 4;
@@ -178,8 +228,8 @@ __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs
     const int hi =
         ((c0 + W < ONE_S * e_lo + mx ? c0 + W : ONE_S * e_lo + mx) - c0 + 15) & ~15;
     if (hi < shi)
-      mma_f16(dtm + (uint32_t)hi, sdesc(z_a, 128, 128), db0,
-              IDESC_M128 | ((uint32_t)((shi - hi) >> 3) << 17), 0);
+      mma_f16_warp(dtm + (uint32_t)hi, sdesc(z_a, 128, 128), db0,
+              IDESC_M128 | ((uint32_t)((shi - hi) >> 3) << 17), 0, leader);
   }
   uint32_t a_lo = (uint32_t)da0 + (uint32_t)(e_hi - e_lo) * ONE_CM;  // 16 matrices per block
   const uint32_t b0 = (uint32_t)db0 + 16;
@@ -190,14 +240,14 @@ __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs
     const int ca = sh > 0 ? sh >> 4 : 0, end = sh + mx < W ? sh + mx : W;
     const uint32_t id = IDESC_M128 | ((uint32_t)(((end + 15) >> 4) - ca) << 18);
     const uint32_t b_lo = b0 + (uint32_t)(16 * ca - sh), d = dtm + 16u * (uint32_t)ca;
-    mma_f16(d, desc(a_hi, a_lo), desc(b_hi, b_lo), id, acc);
-    mma_f16(d, desc(a_hi, a_lo + ((2 * ONE_CM) >> 4)), desc(b_hi, b_lo + step_b), id, 1);
+    mma_f16_warp(d, desc(a_hi, a_lo), desc(b_hi, b_lo), id, acc, leader);
+    mma_f16_warp(d, desc(a_hi, a_lo + ((2 * ONE_CM) >> 4)), desc(b_hi, b_lo + step_b), id, 1, leader);
     acc = 1;
     sh += ONE_S;
     a_lo -= ONE_CM;
   }
   static_assert(ONE_KB == 32, "two MMAs per block");
-  mma_commit(mbar);
+  mma_commit_warp(mbar, leader);
 }
 
 struct OneShared {
@@ -303,9 +353,9 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
       tc_fence_before();
       fence_async_smem();
       __syncthreads();
-      if (tid == 0) {
+      if (__shfl_sync(FULL, warp, 0) == 0) {
         one_issue(c.tmem, c.sbase + Ly.hk, xs_a, z_a, lbo_b, c0, Wd, e_lo, e_hi, Ly.mx, shi, mb);
-        c.pending = true;
+        c.pending = tid == 0;
       }
       bool bad = false;
       if (mbar_wait_lim(mb, c.phase, c.wlim)) {
@@ -371,23 +421,8 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
 #pragma unroll
             for (int k = 0; k < 8; k++) w[k] = a == 0 ? s[k] + 0x80000000u : w[k] + s[k];
           }
-          // the biased coefficients as two 56-bit sums
-          const uint64_t s0 = (uint64_t)w[0] + ((uint64_t)w[1] << 8) + ((uint64_t)w[2] << 16) +
-                              ((uint64_t)w[3] << 24);
-          const uint64_t s1 = (uint64_t)w[4] + ((uint64_t)w[5] << 8) + ((uint64_t)w[6] << 16) +
-                              ((uint64_t)w[7] << 24);
-          uint64_t l = s0 + (s1 << 32);
-          uint32_t h = (uint32_t)(s1 >> 32) + (l < s0);
           const int j = j0 + lt;
-          if (tx && j >= nx && j - nx < ny) {
-            const uint64_t add = y[j - nx];
-            l += add;
-            h += l < add;
-          }
-          const uint64_t b = j == L0 ? 0x8080808080000000ull : 0x8080808080808080ull;
-          h -= l < b;
-          low[r] = l - b;
-          high[r] = h;
+          limb_of(w, tx && j >= nx && j - nx < ny ? y[j - nx] : 0ull, j == L0, low[r], high[r]);
         }
         if (lane == 31) c.sh->hi[r * W + warp] = high[r];
         gen = gnext;
