@@ -33,7 +33,7 @@
 // squared stays below a unit: the error does not grow from step to step.
 // Then q^ = floor(u w / B^h) (banded from limb h - 2), r^ = u - q^ v modulo
 // B^(nv+1), and the exact correction of divmod.cu settles q and r.  The
-// leading steps whose operands all have at most 136 limbs run in one
+// leading steps whose operands all have at most 72 limbs run in one
 // launch, a warp per instance (k_ds_small), instead of four launches each.
 #include <algorithm>
 
@@ -57,7 +57,7 @@ namespace dstep {
 // cores.  The steps' products are rectangular and come in batches of
 // thousands; measured on 2n/n divisions at n = 512 the 132 x 262-limb and
 // 68 x 134-limb products of the middle steps took 173 and 90 us on the
-// integer pipes for 4096 instances.
+// integer pipes for 4096 instances, 39 and 30 us as one-drain products.
 constexpr int STEP_TC_MIN = 64;
 
 // The step schedule needs k = prec(v) - 1 = nv - 1.  The dividend may have

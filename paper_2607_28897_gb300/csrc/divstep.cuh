@@ -13,10 +13,13 @@ using namespace divc;
 
 constexpr int LIN_THREADS = 256;  // CTA of the linear per-instance kernels
 
-// Fused leading steps: operands of at most SMALL_STEP_LIMBS limbs.  A warp's
+// Fused leading steps: operands of at most SMALL_STEP_LIMBS limbs, i.e. up to
+// 34 known limbs.  (With the step from 66 in the warp too -- 136 limbs -- it
+// took 231 us for 4096 instances; batched on the tensor cores that step is
+// three launches more and 60 us less.)  A warp's
 // shared memory holds, for steps of at most N limbs, two iterates (N each),
 // vt and |d| (N each), P2 (2 N) and the column sums (2 N x 3 words).
-constexpr int SMALL_STEP_LIMBS = 136, SMALL_STEP_WARPS = 4;
+constexpr int SMALL_STEP_LIMBS = 72, SMALL_STEP_WARPS = 4;
 __host__ __device__ constexpr int small_step_warp_limbs(int N) { return 2 * N + 2 * N + 2 * N + 6 * N; }
 
 // One Newton step of an instance: l limbs of the inverse known, m new ones,

@@ -42,7 +42,7 @@ constexpr size_t WAVE_BYTES = (size_t)1 << 30;
 
 // The steps up to this many known limbs run fused in one warp (every operand
 // then has at most SMALL_STEP_LIMBS limbs).
-constexpr int SMALL_L = 66;
+constexpr int SMALL_L = 34;
 
 struct RagArgs {
   const RagOp *ops;
