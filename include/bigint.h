@@ -380,20 +380,20 @@ int bigint_save_tuning(const char *path);
 int bigint_load_tuning(const char *path);
 
 /* ---- fused programs (Sec. VI, Tables I and II) ----------------------------
- * bigint_add_chain: out = a + b + ... + b with k additions (1 <= k <= 255),
- * each a full carry-propagating addition mod B^n (Table I's 6-Add is k = 6);
- * carry_out[i] = floor((a + k b) / B^n) (may be NULL).  One launch, the
- * running sum held in registers: global traffic is that of one addition.
+ * bigint_add_chain: out = a + b + ... + b with k additions (1 <= k <= 255)
+ * mod B^n (Table I's 6-Add is k = 6); carry_out[i] = floor((a + k b) / B^n)
+ * (may be NULL).  One launch and one carry scan, over a_j + k b_j: global
+ * traffic is that of one addition.
  * a, b, out: count x n limbs, device pointers, out may alias a.
  *
  * bigint_poly: out = (a a + b)(b b + b) + a b mod B^n (Table II's Poly: four
  * multiplications, three additions, every value kept to n limbs as the
- * paper's same-width multiply and add).  One persistent launch; products of
- * n >= 256 limbs run on the tensor cores, with the smallest tile that holds
- * a low n x n product's n / 16 columns (up to four CTAs per SM for n <=
- * 1024, two up to 2048, one above); intermediates live in `workspace`
- * (device memory of bigint_poly_workspace(count, n) bytes: 3 n limbs per
- * resident CTA, small enough to stay in L2).  a, b, out: count x n limbs,
+ * paper's same-width multiply and add).  From 64 limbs four launches of
+ * batched tensor-core products, each with an addend taken in as its limbs are
+ * formed, on chunks of the batch; intermediates live in `workspace` (device
+ * memory of bigint_poly_workspace(count, n) bytes: 2 n limbs per instance of
+ * a chunk, about 80 MB at most, so that they stay in L2).  Below 64 limbs one
+ * persistent launch of integer products.  a, b, out: count x n limbs,
  * out disjoint from a and b.  n <= BIGINT_MUL_MAX_LIMBS.
  * Both return BIGINT_EINVAL for bad shapes or pointers, BIGINT_ENOMEM for a
  * short workspace, BIGINT_ECUDA for a launch error.                         */

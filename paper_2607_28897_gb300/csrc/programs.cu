@@ -10,12 +10,21 @@
 
 namespace bigint {
 
+bool mul_add_ok(int n);
+int launch_mul_add(const uint64_t *a, const uint64_t *b, const uint64_t *c, uint64_t *out,
+                   int64_t count, int n, cudaStream_t st);
+
 // ---------------------------------------------------------------------------
-// Poly: persistent CTAs; per instance four low-part products (tensor cores
-// when n >= TC_DIV_MIN, with the tile of NT columns that holds the n / 16
-// columns of a low n x n product, so that small programs run several CTAs
-// per SM; else blk_mul) and three in-place additions through a per-CTA
-// scratch of 3n limbs.
+// Poly: four launches of batched low products with an addend, the additions
+// done as the products' limbs are formed,
+//   T1 = a a + b,  T2 = b b + b,  r = a b,  r = T1 T2 + r,
+// on chunks of the batch whose T1 and T2 stay in L2 (tcone.cuh, tcpipe.cuh:
+// several CTAs per SM or the warp-specialised pipeline; as one persistent
+// kernel a CTA at a time on each product, 16384 Polys of 1024 limbs took 7.9
+// ms).  Sizes those forms do not take run k_poly: persistent CTAs, per
+// instance four low-part products (tensor cores for n beyond what the
+// pipelined form holds, blk_mul below 64 limbs) and three in-place additions
+// through a per-CTA scratch of 3n limbs.
 // ---------------------------------------------------------------------------
 template <bool TC, int NT, int G>
 __global__ void __launch_bounds__(TC ? 2 * NT + 32 : 512, TC ? 256 / NT : 1)
@@ -106,14 +115,23 @@ int sm_count(int *sms) {
   return BIGINT_OK;
 }
 
-// The launch of Poly for n-limb operands: which k_poly, its dynamic shared
-// memory and CTAs per SM.  Tensor cores from TC_DIV_MIN limbs with the
-// smallest tile holding the n / 16 columns of a low n x n product.
+// The launch of Poly for n-limb operands: the form, and for k_poly its
+// dynamic shared memory and CTAs per SM.
 struct PolyPlan {
-  int form;  // 0: integer, 1: NT 64, 2: NT 128, 3: NT 256 G 8, 4: NT 256 G 4
+  int form;  // 0: k_poly, integer, 1: batched products, 3: k_poly NT 256 G 8, 4: NT 256 G 4
   size_t smem;
   int per_sm;
 };
+
+// Instances per chunk of the batched form: whole rounds of the SMs (four CTAs
+// each) whose T1 and T2 take at most POLY_CHUNK_BYTES, well inside the L2.
+constexpr size_t POLY_CHUNK_BYTES = (size_t)80 << 20;
+int64_t poly_chunk(int64_t count, int n, int sms) {
+  const int64_t fit = (int64_t)(POLY_CHUNK_BYTES / (16 * (size_t)n)), round = 4 * (int64_t)sms;
+  int64_t c = fit >= round ? fit / round * round : fit / sms * sms;
+  if (c < sms) c = sms;
+  return c < count ? c : count;
+}
 
 template <bool TC, int NT, int G>
 bool poly_try(int form, size_t smem, PolyPlan &P) {
@@ -126,10 +144,11 @@ bool poly_try(int form, size_t smem, PolyPlan &P) {
 }
 
 bool poly_plan(int n, PolyPlan &P) {
+  if (mul_add_ok(n)) {
+    P = PolyPlan{1, 0, 0};
+    return true;
+  }
   if (n >= divc::TC_DIV_MIN) {
-    const int cols = (n + 15) / 16;
-    if (cols <= 64 && poly_try<true, 64, 7>(1, tcm::layout<64, 7>(n, n).total, P)) return true;
-    if (cols <= 128 && poly_try<true, 128, 8>(2, tcm::layout<128, 8>(n, n).total, P)) return true;
     if (poly_try<true, 256, 8>(3, tcm::layout<256, 8>(n, n).total, P)) return true;
     if (poly_try<true, 256, 4>(4, tcm::layout<256, 4>(n, n).total, P)) return true;
   }
@@ -142,6 +161,34 @@ int64_t poly_grid(const PolyPlan &P, int64_t count) {
   if (sm_count(&sms) != BIGINT_OK) return 0;
   const int64_t slots = (int64_t)sms * P.per_sm;
   return count < slots ? count : slots;
+}
+
+// T1 and T2 of a chunk, or 3n limbs per resident CTA.
+size_t poly_bytes(const PolyPlan &P, int64_t count, int n) {
+  int sms = 0;
+  if (sm_count(&sms) != BIGINT_OK) return 0;
+  if (P.form == 1) return (size_t)poly_chunk(count, n, sms) * 2 * (size_t)n * 8;
+  const int64_t slots = (int64_t)sms * P.per_sm;
+  return (size_t)(count < slots ? count : slots) * 3 * (size_t)n * 8;
+}
+
+int launch_poly_batched(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t count, int n,
+                        void *ws, cudaStream_t st) {
+  int sms = 0;
+  int rc = sm_count(&sms);
+  if (rc != BIGINT_OK) return rc;
+  const int64_t chunk = poly_chunk(count, n, sms);
+  uint64_t *T1 = static_cast<uint64_t *>(ws), *T2 = T1 + chunk * n;
+  for (int64_t i = 0; i < count; i += chunk) {
+    const int64_t c = count - i < chunk ? count - i : chunk;
+    const uint64_t *x = a + i * n, *y = b + i * n;
+    uint64_t *o = out + i * n;
+    if ((rc = launch_mul_add(x, x, y, T1, c, n, st)) != BIGINT_OK) return rc;
+    if ((rc = launch_mul_add(y, y, y, T2, c, n, st)) != BIGINT_OK) return rc;
+    if ((rc = launch_mul_add(x, y, nullptr, o, c, n, st)) != BIGINT_OK) return rc;
+    if ((rc = launch_mul_add(T1, T2, o, o, c, n, st)) != BIGINT_OK) return rc;
+  }
+  return BIGINT_OK;
 }
 
 template <bool TC, int NT, int G>
@@ -162,8 +209,8 @@ int programs_set_wait_limit(long long cycles) { return tcm::set_wait_limit_here(
 size_t poly_workspace(int64_t count, int n) {
   PolyPlan P;
   if (n < 1 || !poly_plan(n, P)) return 0;
-  const int64_t grid = poly_grid(P, count);
-  return (size_t)(grid > 0 ? grid : 1) * 3 * (size_t)n * 8;
+  const size_t bytes = poly_bytes(P, count, n);
+  return bytes ? bytes : 8;
 }
 
 int launch_poly(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t count, int n,
@@ -171,12 +218,12 @@ int launch_poly(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t cou
   if (count == 0) return BIGINT_OK;
   PolyPlan P;
   if (!poly_plan(n, P)) return BIGINT_EINVAL;
+  const size_t need = poly_bytes(P, count, n);
+  if (need == 0) return BIGINT_ECUDA;
+  if (bytes < need) return BIGINT_ENOMEM;
+  if (P.form == 1) return launch_poly_batched(a, b, out, count, n, ws, st);
   const int64_t grid = poly_grid(P, count);
-  if (grid <= 0) return BIGINT_ECUDA;
-  if (bytes < (size_t)grid * 3 * n * 8) return BIGINT_ENOMEM;
   switch (P.form) {
-    case 1: return launch_poly_variant<true, 64, 7>(a, b, out, count, n, ws, grid, P.smem, st);
-    case 2: return launch_poly_variant<true, 128, 8>(a, b, out, count, n, ws, grid, P.smem, st);
     case 3: return launch_poly_variant<true, 256, 8>(a, b, out, count, n, ws, grid, P.smem, st);
     case 4: return launch_poly_variant<true, 256, 4>(a, b, out, count, n, ws, grid, P.smem, st);
     default: return launch_poly_variant<false, 256, 8>(a, b, out, count, n, ws, grid, P.smem, st);

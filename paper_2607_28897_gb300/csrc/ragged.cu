@@ -259,7 +259,7 @@ struct RagRing {
   tcm::PipeTask t[RING];
 };
 
-template <int KB>
+template <int KB, int NT>
 __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tcm::PipeLayout L) {
   using namespace tcm;
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -280,7 +280,13 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
     if (more) {
       const int32_t e = A.list[i];
       const RagTask t = rag_task(A, A.ops[e & ~RAG_SWAP], (e & RAG_SWAP) != 0);
-      T = PipeTask{t.x, t.y, t.out, t.nx, t.ny, t.nout, t.lo};
+      T = PipeTask{t.x, t.y, t.out, t.nx, t.ny, t.nout, t.lo, nullptr};
+    }
+    if (threadIdx.x == PIPE_DRAIN + 64 && i + gridDim.x < A.n) {  // of the second warp
+      const int32_t e = A.list[i + gridDim.x];
+      const RagTask t = rag_task(A, A.ops[e & ~RAG_SWAP], (e & RAG_SWAP) != 0);
+      prefetch_l2(t.x, 8 * (size_t)t.nx);
+      prefetch_l2(t.y, 8 * (size_t)t.ny);
     }
     if (threadIdx.x == PIPE_DRAIN + 32) {  // the first builder thread
       const int r = (int)(k % RING);
@@ -315,7 +321,7 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
     if (threadIdx.x == 0) status(k, BIGINT_OK);
     ndone = k + 1;
   };
-  if (!pipe_run<KB>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
+  if (!pipe_run<KB, NT>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
     atomicExch(A.abort_flag, 1);
     for (int64_t k = ndone; blockIdx.x + k * gridDim.x < A.n; k++) status(k, BIGINT_ETIMEOUT);
   }
@@ -346,8 +352,10 @@ const Shapes &shapes() {
     s.a[RAG_128] = {k_rag_tc<128, 8>, nullptr, 2 * 128 + 32, 2, 0, 0};
     s.a[RAG_256] = {k_rag_tc<256, 8>, nullptr, 2 * 256 + 32, 1, 0, 0};
     s.a[RAG_256_G4] = {k_rag_tc<256, 4>, nullptr, 2 * 256 + 32, 1, 0, 0};
-    s.a[RAG_PIPE128] = {nullptr, k_rag_pipe<128>, tcm::PIPE_THREADS, 1, 0, 0};
-    s.a[RAG_PIPE64] = {nullptr, k_rag_pipe<64>, tcm::PIPE_THREADS, 1, 0, 0};
+    s.a[RAG_PIPE128] = {nullptr, k_rag_pipe<128, 256>, tcm::PIPE_THREADS, 1, 0, 0};
+    s.a[RAG_PIPE64] = {nullptr, k_rag_pipe<64, 256>, tcm::PIPE_THREADS, 1, 0, 0};
+    s.a[RAG_PIPE128N] = {nullptr, k_rag_pipe<128, 128>, tcm::PIPE_THREADS, 1, 0, 0};
+    s.a[RAG_PIPE64N] = {nullptr, k_rag_pipe<64, 128>, tcm::PIPE_THREADS, 1, 0, 0};
     int dev = 0, optin = 0, reserved = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
@@ -378,11 +386,12 @@ const Shapes &shapes() {
   return S;
 }
 
-// Shared memory of a pipelined product, over the limit where x does not fit.
-template <int KB>
-uint32_t pipe_bytes_of(int nx, uint32_t dyn) {
-  const tcm::PipeLayout L = tcm::pipe_layout<KB>(nx, dyn);
-  return L.total ? L.total : ~0u;
+// Shared memory of a pipelined launch for x of at most nx limbs (total = 0:
+// does not fit).
+tcm::PipeLayout pipe_layout_of(int shape, int nx) {
+  const uint32_t dyn = (uint32_t)shapes().a[shape].dyn;
+  return shape == RAG_PIPE128 || shape == RAG_PIPE128N ? tcm::pipe_layout<128>(nx, dyn)
+                                                       : tcm::pipe_layout<64>(nx, dyn);
 }
 
 uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
@@ -393,8 +402,13 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
     case RAG_64: return layout<64, 7>(nx, ny).total;
     case RAG_128: return layout<128, 8>(nx, ny).total;
     case RAG_256: return layout<256, 8>(nx, ny).total;
-    case RAG_PIPE128: return pipe_bytes_of<128>(nx, (uint32_t)shapes().a[shape].dyn);
-    case RAG_PIPE64: return pipe_bytes_of<64>(nx, (uint32_t)shapes().a[shape].dyn);
+    case RAG_PIPE128:
+    case RAG_PIPE64:
+    case RAG_PIPE128N:
+    case RAG_PIPE64N: {
+      const uint32_t t = pipe_layout_of(shape, nx).total;
+      return t ? t : ~0u;
+    }
     default: return layout<256, 4>(nx, ny).total;
   }
 }
@@ -461,9 +475,7 @@ class Chooser {
     f.nx = ax;
     if (a.pipe) {  // one CTA per SM; those whose x is double buffered apart
       f.per_sm = 1;
-      f.group = f.shape * 8 + (f.shape == RAG_PIPE128
-                                   ? tcm::pipe_layout<128>(ax, (uint32_t)a.dyn).xbufs
-                                   : tcm::pipe_layout<64>(ax, (uint32_t)a.dyn).xbufs);
+      f.group = f.shape * 8 + pipe_layout_of(f.shape, ax).xbufs;
       return f;
     }
     f.per_sm = std::max(1, std::min(a.cap, shapes().smem_sm / ((int)f.bytes + a.overhead)));
@@ -609,9 +621,7 @@ int rag_launch(const RagPlan &P, const RagBuffers &B, const uint64_t *in, uint64
       default: {
         const ShapeAttr &a = shapes().a[R.shape];
         if (a.pipe) {
-          const tcm::PipeLayout L = R.shape == RAG_PIPE128
-                                        ? tcm::pipe_layout<128>(R.nx, (uint32_t)a.dyn)
-                                        : tcm::pipe_layout<64>(R.nx, (uint32_t)a.dyn);
+          const tcm::PipeLayout L = pipe_layout_of(R.shape, R.nx);
           a.pipe<<<(unsigned)R.grid, a.threads, L.total, st>>>(A, L);
         } else {
           a.kern<<<(unsigned)R.grid, a.threads, R.smem, st>>>(A);

@@ -21,6 +21,7 @@ struct RagOp {
 // Product forms of a grouped launch (tc_choose).
 enum RagShape {
   RAG_ONE128, RAG_ONE256, RAG_64, RAG_128, RAG_256, RAG_256_G4, RAG_PIPE128, RAG_PIPE64,
+  RAG_PIPE128N, RAG_PIPE64N,  // with 128-column tiles
   RAG_NSHAPES
 };
 

@@ -44,12 +44,13 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
 
 // The same for products whose shorter operand has at most ONE_MAX limbs
 // (tcone.cuh): NT tensor-memory columns and 32 W threads per CTA, 512 / NT
-// CTAs per SM.
-template <int NT, int W>
+// CTAs per SM.  add + i sadd: nout limbs added to product i (null: none).
+template <int NT, int W, bool ADD>
 __global__ void __launch_bounds__(32 * W, 512 / NT)
     k_mul_one(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
-              uint64_t *__restrict__ Out, int nx, int ny, int nout, int64_t count, int64_t sx,
-              int64_t sy, int64_t so, int lo, int *abort_flag) {
+              uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
+              int64_t sy, int64_t so, int lo, int *abort_flag, const uint64_t *add,
+              int64_t sadd) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ OneShared sh;
   OneCtx c;
@@ -60,7 +61,8 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
       prefetch_l2(X + next * sx, 8 * (size_t)nx);
       prefetch_l2(Y + next * sy, 8 * (size_t)ny);
     }
-    if (!one_product<NT, W>(c, X + inst * sx, nx, Y + inst * sy, ny, Out + inst * so, nout, lo))
+    if (!one_product<NT, W, ADD>(c, X + inst * sx, nx, Y + inst * sy, ny, Out + inst * so, nout,
+                                 lo, ADD ? add + inst * sadd : nullptr))
       break;
   }
   if (c.aborted && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
@@ -68,20 +70,31 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
 }
 
 // The same by the pipeline of tcpipe.cuh: one CTA per SM.
-template <int KB>
+template <int KB, int NT>
 __global__ void __launch_bounds__(PIPE_THREADS, 1)
     k_mul_pipe(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
-               uint64_t *__restrict__ Out, int nx, int ny, int nout, int64_t count, int64_t sx,
-               int64_t sy, int64_t so, int lo, int *abort_flag, PipeLayout L) {
+               uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
+               int64_t sy, int64_t so, int lo, int *abort_flag, const uint64_t *add, int64_t sadd,
+               PipeLayout L) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ PipeShared sh;
   auto next = [&](int64_t k, PipeTask &T) {
     const int64_t i = blockIdx.x + k * gridDim.x;
     if (i >= count) return false;
-    T = PipeTask{X + i * sx, Y + i * sy, Out + i * so, nx, ny, nout, lo};
+    T = PipeTask{X + i * sx, Y + i * sy, Out + i * so, nx, ny, nout, lo,
+                 add != nullptr ? add + i * sadd : nullptr};
     return true;
   };
-  const bool ok = pipe_run<KB>(L, &sh, sm, next, next, next, [](int64_t) {});
+  auto next_b = [&](int64_t k, PipeTask &T) {
+    if (!next(k, T)) return false;
+    const int64_t i = blockIdx.x + (k + 1) * gridDim.x;
+    if (threadIdx.x == PIPE_DRAIN + 32 && i < count) {  // the first builder thread
+      prefetch_l2(X + i * sx, 8 * (size_t)nx);
+      prefetch_l2(Y + i * sy, 8 * (size_t)ny);
+    }
+    return true;
+  };
+  const bool ok = pipe_run<KB, NT>(L, &sh, sm, next_b, next, next, [](int64_t) {});
   if (!ok && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
 }
 
@@ -272,6 +285,8 @@ struct TcArgs {
   int64_t sx, sy, so;
   int lo;
   int *abort_flag;
+  const uint64_t *add = nullptr;  // one-drain and pipelined forms: added to the products
+  int64_t sadd = 0;
 };
 
 // CTAs of a shape resident on one SM: TMEM allows 256 / NT, shared memory
@@ -442,11 +457,11 @@ struct OneAttr {
   bool ok = false;
 };
 
-template <int NT>
+template <int NT, bool ADD = false>
 static const OneAttr &one_attr() {
   static const OneAttr A = [] {
     OneAttr a;
-    auto *kern = tcm::k_mul_one<NT, one_warps<NT>()>;
+    auto *kern = tcm::k_mul_one<NT, one_warps<NT>(), ADD>;
     int dev = 0, optin = 0, reserved = 0;
     cudaFuncAttributes fa;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -516,13 +531,15 @@ static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, 
   if (sms == 0) return BIGINT_ECUDA;
   const int64_t slots = (int64_t)sms * one_per_sm<NT>(smem);
   const int64_t grid = count < slots ? count : slots;
-  tcm::k_mul_one<NT, W><<<(unsigned)grid, 32 * W, smem, st>>>(
-      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag);
+  auto *kern = A.add != nullptr ? tcm::k_mul_one<NT, W, true> : tcm::k_mul_one<NT, W, false>;
+  if (A.add != nullptr && !one_attr<NT, true>().ok) return BIGINT_ECUDA;
+  kern<<<(unsigned)grid, 32 * W, smem, st>>>(A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy,
+                                             A.so, A.lo, A.abort_flag, A.add, A.sadd);
   return bigint_launch_status();
 }
 
 // ---- pipelined products (tcpipe.cuh) --------------------------------------------
-template <int KB>
+template <int KB, int NT>
 static const OneAttr &pipe_attr() {
   static const OneAttr A = [] {
     OneAttr a;
@@ -531,43 +548,47 @@ static const OneAttr &pipe_attr() {
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
             cudaSuccess ||
-        cudaFuncGetAttributes(&fa, tcm::k_mul_pipe<KB>) != cudaSuccess)
+        cudaFuncGetAttributes(&fa, tcm::k_mul_pipe<KB, NT>) != cudaSuccess)
       return a;
     a.dyn = optin - (int)fa.sharedSizeBytes;
-    a.ok = cudaFuncSetAttribute(tcm::k_mul_pipe<KB>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    a.ok = cudaFuncSetAttribute(tcm::k_mul_pipe<KB, NT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                 a.dyn) == cudaSuccess;
     return a;
   }();
   return A;
 }
 
-template <int KB>
+template <int KB, int NT>
 static int launch_pipe(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
-  if (!pipe_attr<KB>().ok) return BIGINT_ECUDA;
-  const tcm::PipeLayout L = tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB>().dyn);
+  if (!pipe_attr<KB, NT>().ok) return BIGINT_ECUDA;
+  const tcm::PipeLayout L = tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB, NT>().dyn);
   if (L.total == 0 || nx < 64) return BIGINT_EINVAL;
   if (count == 0) return BIGINT_OK;
   const int sms = sm_count();
   if (sms == 0) return BIGINT_ECUDA;
-  tcm::k_mul_pipe<KB><<<(unsigned)(count < sms ? count : sms), tcm::PIPE_THREADS, L.total, st>>>(
-      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag, L);
+  tcm::k_mul_pipe<KB, NT><<<(unsigned)(count < sms ? count : sms), tcm::PIPE_THREADS, L.total, st>>>(
+      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag, A.add, A.sadd,
+      L);
   return bigint_launch_status();
 }
 
 // Modelled time of a product in the pipelined form (-1: x does not fit): its
 // MMAs, at least 42 cycles each (warp-uniform issue), 10 % slower beside the
-// drains and builds, 900 cycles a drain and 9000 a tile (the part of its
-// limbs that two groups of MMAs do not cover).
-template <int KB>
+// drains and builds, 900 cycles a drain and 9000 (3000 with 128-column tiles)
+// a tile, the part of its limbs that the groups ahead do not cover.  128-
+// column tiles for products of one such tile only.
+template <int KB, int NT>
 static double pipe_cost(int nx, int ny, int nout, int lo) {
   constexpr int S = 128 / KB;
-  if (nx < 64 || !pipe_attr<KB>().ok ||
-      tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB>().dyn).total == 0)
+  if (nx < 64 || !pipe_attr<KB, NT>().ok ||
+      tcm::pipe_layout<KB>(nx, (uint32_t)pipe_attr<KB, NT>().dyn).total == 0)
     return -1;
   const int mx = (8 * nx + KB - 1) / KB;
   double cyc = 0;
-  tcm::pipe_tiles<KB>(nx, ny, nout, lo, [&](int c0, int W, int e_lo, int e_hi) {
-    cyc += 9000;
+  int tiles = 0;
+  tcm::pipe_tiles<KB, NT>(nx, ny, nout, lo, [&](int c0, int W, int e_lo, int e_hi) {
+    tiles++;
+    cyc += NT == 256 ? 9000 : 3000;
     if (e_hi < e_lo) return true;
     const int n = e_hi - e_lo + 1, st = sample_step(n);
     cyc += 900.0 * ((n * KB + 1023) / 1024);
@@ -580,11 +601,10 @@ static double pipe_cost(int nx, int ny, int nout, int lo) {
     }
     return true;
   });
-  return cyc;
+  return NT == 256 || tiles <= 1 ? cyc : -1;
 }
 
-// The one-drain (RAG_ONE128, RAG_ONE256) or pipelined (RAG_PIPE128,
-// RAG_PIPE64) form, either operand as x (*swap), where its model is cheaper
+// The one-drain (RAG_ONE...) or pipelined (RAG_PIPE...) form, either operand as x (*swap), where its model is cheaper
 // than `than` (< 0: anything); -1 where none is.
 static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap) {
   int form = -1;
@@ -596,10 +616,44 @@ static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap) 
     double c;
     if (one_plan<128>(mx, my, nout, lo, &c)) offer(c, RAG_ONE128, k);
     if (one_plan<256>(mx, my, nout, lo, &c)) offer(c, RAG_ONE256, k);
-    offer(pipe_cost<128>(mx, my, nout, lo), RAG_PIPE128, k);
-    offer(pipe_cost<64>(mx, my, nout, lo), RAG_PIPE64, k);
+    offer(pipe_cost<128, 256>(mx, my, nout, lo), RAG_PIPE128, k);
+    offer(pipe_cost<64, 256>(mx, my, nout, lo), RAG_PIPE64, k);
+    offer(pipe_cost<128, 128>(mx, my, nout, lo), RAG_PIPE128N, k);
+    offer(pipe_cost<64, 128>(mx, my, nout, lo), RAG_PIPE64N, k);
   }
   return form;
+}
+
+// Launches a form of best_form (sw: with the operands' roles exchanged).
+static int launch_form(int form, TcArgs A, bool sw, int64_t count, int nx, int ny, int nout,
+                       cudaStream_t st) {
+  if (sw) {
+    const uint64_t *t = A.x; A.x = A.y; A.y = t;
+    const int64_t ts = A.sx; A.sx = A.sy; A.sy = ts;
+    const int tn = nx; nx = ny; ny = tn;
+  }
+  switch (form) {
+    case RAG_ONE128: return launch_one<128>(A, count, nx, ny, nout, st);
+    case RAG_ONE256: return launch_one<256>(A, count, nx, ny, nout, st);
+    case RAG_PIPE128: return launch_pipe<128, 256>(A, count, nx, ny, nout, st);
+    case RAG_PIPE64: return launch_pipe<64, 256>(A, count, nx, ny, nout, st);
+    case RAG_PIPE128N: return launch_pipe<128, 128>(A, count, nx, ny, nout, st);
+    default: return launch_pipe<64, 128>(A, count, nx, ny, nout, st);
+  }
+}
+
+// out = low n limbs of a b + c for a batch of n-limb operands (instance i at
+// a + i sa, ...; c may be null or out), by a form that takes an addend.
+bool mul_add_ok(int n) {
+  bool sw = false;
+  return n >= 64 && best_form(n, n, n, 0, -1, &sw) >= 0;
+}
+int launch_mul_add(const uint64_t *a, const uint64_t *b, const uint64_t *c, uint64_t *out,
+                   int64_t count, int n, cudaStream_t st) {
+  bool sw = false;
+  const int form = best_form(n, n, n, 0, -1, &sw);
+  if (form < 0) return BIGINT_EINVAL;
+  return launch_form(form, TcArgs{a, b, out, n, n, n, 0, nullptr, c, n}, sw, count, n, n, n, st);
 }
 
 // The same choice for a product of a grouped launch (ragged.cu): a RagShape,
@@ -631,6 +685,11 @@ int tc_choose(int nx, int ny, int nout, int lo, bool *swap) {
 int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
                      cudaStream_t st, int force) {
+  if (nout > na + nb) return BIGINT_EINVAL;
+  if (lo == 0) {  // limbs at and above nout do not reach the low nout limbs
+    if (na > nout) na = nout;
+    if (nb > nout) nb = nout;
+  }
   TcArgs A{a, b, out, sa, sb, so, lo, abort_flag};
   int nx = na, ny = nb;
   if (nb < na) {
@@ -675,19 +734,7 @@ int launch_mul_tc_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   if (force == 0) {
     bool sw = false;
     const int form = best_form(nx, ny, nout, lo, keep, &sw);
-    if (form >= 0) {
-      TcArgs B = A;
-      if (sw) {
-        B.x = A.y; B.y = A.x; B.sx = A.sy; B.sy = A.sx;
-      }
-      const int mx = sw ? ny : nx, my = sw ? nx : ny;
-      switch (form) {
-        case RAG_ONE128: return launch_one<128>(B, count, mx, my, nout, st);
-        case RAG_ONE256: return launch_one<256>(B, count, mx, my, nout, st);
-        case RAG_PIPE128: return launch_pipe<128>(B, count, mx, my, nout, st);
-        default: return launch_pipe<64>(B, count, mx, my, nout, st);
-      }
-    }
+    if (form >= 0) return launch_form(form, A, sw, count, nx, ny, nout, st);
   }
   if (keep < 0) return BIGINT_EINVAL;
   return launch_shape(sh, A, count, nx, ny, nout, st);

@@ -303,16 +303,18 @@ __device__ void one_release(OneCtx &c) {
   if (threadIdx.x < 32) tmem_dealloc(c.tmem, NT);
 }
 
-// out[0 .. nout) = low nout limbs of x y by the whole CTA (32 W threads);
+// out[0 .. nout) = low nout limbs of x y (+ add, nout limbs, which may be
+// out itself: each limb is read by the thread that later writes it) by the
+// whole CTA (32 W threads);
 // band mode (lo > 0) as tc_product's: tiles anchored S - 1 columns before
 // limb lo's, limbs below L0 = R floor(lo / R) untouched, out[L0 ..) with
 // 2^32 added at L0.  The shorter operand has at most ONE_MAX limbs; c.sm
 // holds one_layout<W>(nx, ny, blocks of the widest tile).  Returns false
 // (and sets c.aborted) if a wait hit its limit.
-template <int NT, int W>
+template <int NT, int W, bool ADD = false>
 __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx,
                                             const uint64_t *y, int ny, uint64_t *out, int nout,
-                                            int lo) {
+                                            int lo, const uint64_t *add = nullptr) {
   constexpr int THREADS = 32 * W, RUN = 8 * W, NRUN = NT / RUN, S = ONE_S, R = ONE_R;
   constexpr int BUFS = one_bufs<W>();
   static_assert(NRUN * W <= 32, "one warp resolves the carries of a tile");
@@ -423,6 +425,11 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
           }
           const int j = j0 + lt;
           limb_of(w, tx && j >= nx && j - nx < ny ? y[j - nx] : 0ull, j == L0, low[r], high[r]);
+          if constexpr (ADD) {
+            const uint64_t a = add[j];
+            low[r] += a;
+            high[r] += low[r] < a;
+          }
         }
         if (lane == 31) c.sh->hi[r * W + warp] = high[r];
         gen = gnext;

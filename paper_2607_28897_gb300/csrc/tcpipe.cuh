@@ -10,13 +10,16 @@
 //                       stage, straight from registers (tcone.cuh), two or
 //                       three stages ahead;
 //   issuer (1 warp)     the MMAs of a stage once it is full, a group of
-//                       GS stages into one of two 256-column accumulators;
+//                       GS stages into one of 512 / NT accumulators of NT
+//                       columns;
 //   drains (16 warps)   a finished accumulator into int32 column sums in
-//                       registers (64 per thread), and after a tile's last
+//                       registers (NT / 4 per thread), and after a tile's last
 //                       group the column sums into limbs, while the issuer is
-//                       already at work on the next tile or product (the two
-//                       accumulators let it run two groups, ~9K cycles,
-//                       ahead; a tile's limbs take about 5K).
+//                       already at work on the next tile or product: with NT
+//                       = 256 it may run two groups (~9K cycles) ahead, a
+//                       tile's limbs taking ~13K beside them; with NT = 128
+//                       (products of at most 128 columns: low and banded
+//                       ones) four groups, and half the limbs per thread.
 //
 // Every hand-over is an mbarrier: stage full / free, accumulator full / free,
 // x full / free (the "free" ones of operands are tcgen05.commit arrivals).
@@ -40,7 +43,7 @@
 namespace bigint {
 namespace tcm {
 
-constexpr int PIPE_NT = 256, PIPE_HS = 8, PIPE_BUILD = 3, PIPE_DRAIN = 512;
+constexpr int PIPE_HS = 8, PIPE_BUILD = 3, PIPE_DRAIN = 512;
 constexpr int PIPE_THREADS = PIPE_DRAIN + 32 + 32 * PIPE_BUILD;  // 20 warps: 96 registers
 constexpr int PIPE_EX = 264;    // limbs per row of the S = 2 exchange (16 banks from row to row)
 constexpr int PIPE_STAGES = 3;  // at most
@@ -82,7 +85,7 @@ __host__ inline PipeLayout pipe_layout(int nx, uint32_t cap) {
 }
 
 struct PipeShared {
-  uint64_t hfull[PIPE_STAGES], hfree[PIPE_STAGES], afull[2], afree[2], xfull[2], xfree[2], done;
+  uint64_t hfull[PIPE_STAGES], hfree[PIPE_STAGES], afull[4], afree[4], xfull[2], xfree[2], done;
   uint32_t tmem_slot;
   int abort;
   uint32_t hx[4][256];    // high words of each warp's top limb of a column
@@ -90,25 +93,27 @@ struct PipeShared {
 };
 
 // One product: x (the operand stored whole), y, the low nout limbs to out,
-// band start lo (as tc_product's).
+// band start lo (as tc_product's); add: nout limbs added to it (may be out
+// itself), or null.
 struct PipeTask {
   const uint64_t *x, *y;
   uint64_t *out;
   int nx, ny, nout, lo;
+  const uint64_t *add;
 };
 
 // Tiles of a product and their Toeplitz blocks, as every role walks them:
 // f(c0, W, e_lo, e_hi), e_hi < e_lo where no MMA writes the tile; f returns
 // false to stop.
 #pragma nv_exec_check_disable
-template <int KB, class F>
+template <int KB, int NT, class F>
 __host__ __device__ __forceinline__ bool pipe_tiles(int nx, int ny, int nout, int lo, F f) {
   constexpr int S = 128 / KB, R = KB / 8;
   const int mx = (8 * nx + KB - 1) / KB, ey = (8 * ny + KB - 1) / 128;
   const int cols = mx + S * ey + S - 1;
   for (int c0 = lo > 0 ? (lo / R - (S - 1) > 0 ? lo / R - (S - 1) : 0) : 0; R * c0 < nout;
-       c0 += PIPE_NT) {
-    int W = cols - c0 < PIPE_NT ? cols - c0 : PIPE_NT;
+       c0 += NT) {
+    int W = cols - c0 < NT ? cols - c0 : NT;
     const int need = (nout - R * c0 + R - 1) / R;
     if (W > need) W = need;
     W = (W + 15) & ~15;
@@ -177,7 +182,7 @@ __device__ __forceinline__ void pipe_fill(uint8_t *xs, const uint64_t *x, int nx
   }
 }
 
-template <int KB, class Next>
+template <int KB, int NT, class Next>
 __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh, uint8_t *sm,
                                              long long lim, int t, Next next) {
   constexpr int HS = PIPE_HS, NB = pipe_matrices<KB>(), STEP = 32 * PIPE_BUILD;
@@ -198,7 +203,7 @@ __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh
     pipe_fill<KB>(sm + L.xs + xb * L.xbytes, T.x, T.nx, t);
     post(&sh->xfull[xb]);
     items++;
-    const bool ok = pipe_tiles<KB>(T.nx, T.ny, T.nout, T.lo, [&](int, int, int e_lo, int e_hi) {
+    const bool ok = pipe_tiles<KB, NT>(T.nx, T.ny, T.nout, T.lo, [&](int, int, int e_lo, int e_hi) {
       for (int ea = e_lo; ea <= e_hi; ea += HS) {
         const int eb = ea + HS - 1 < e_hi ? ea + HS - 1 : e_hi;
         const int nb = 16 * (eb - ea + 1) + KB / 8 - 1;
@@ -227,10 +232,10 @@ __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh
 }
 
 // ---- issuer ---------------------------------------------------------------------
-template <int KB, class Next>
+template <int KB, int NT, class Next>
 __device__ __forceinline__ void pipe_issuer(const PipeLayout &L, PipeShared *sh, uint32_t sbase,
                                             uint32_t tmem, long long lim, Next next) {
-  constexpr int HS = PIPE_HS, S = 128 / KB, GS = 1024 / (KB * HS);
+  constexpr int HS = PIPE_HS, S = 128 / KB, GS = 1024 / (KB * HS), NACC = 512 / NT;
   uint32_t st = 0, sph = 0, items = 0, grp = 0;
   const uint32_t leader = lane_id() == 0;
   auto desc = [](uint32_t hi, uint32_t lo) { return (uint64_t)hi << 32 | lo; };
@@ -246,13 +251,13 @@ __device__ __forceinline__ void pipe_issuer(const PipeLayout &L, PipeShared *sh,
     const uint32_t lbo = (uint32_t)pipe_ptot<KB>(T.nx) * 16u;
     const uint64_t xd = sdesc(sbase + L.xs + xb * L.xbytes, lbo, 128);
     const uint32_t b_hi = (uint32_t)(xd >> 32), step_b = (2u * lbo) >> 4;
-    const bool ok = pipe_tiles<KB>(T.nx, T.ny, T.nout, T.lo, [&](int c0, int W, int e_lo,
+    const bool ok = pipe_tiles<KB, NT>(T.nx, T.ny, T.nout, T.lo, [&](int c0, int W, int e_lo,
                                                                 int e_hi) {
       for (int eg = e_lo; eg <= e_hi; eg += HS * GS) {
         const int ee = eg + HS * GS - 1 < e_hi ? eg + HS * GS - 1 : e_hi;
-        const uint32_t a = grp & 1u, gn = grp >> 1;
+        const uint32_t a = grp % NACC, gn = grp / NACC;
         if (gn >= 1 && !pipe_wait_warp(sh, &sh->afree[a], (gn - 1) & 1u, lim)) return false;
-        const uint32_t dt = tmem + a * PIPE_NT;
+        const uint32_t dt = tmem + a * NT;
         const int shi = ((c0 + W < S * ee + mx ? c0 + W : S * ee + mx) - c0 + 15) & ~15;
         uint32_t acc = 0;
         for (int ea = eg; ea <= ee; ea += HS) {
@@ -312,15 +317,17 @@ __device__ __forceinline__ void bar_drain() {
 // signed value lo + hi 2^64.  80 shuffles, no barrier: through shared memory
 // the same took 16K cycles beside the MMAs (whose operand reads leave little
 // of its bandwidth), more than the two groups they may run ahead.
-__device__ __forceinline__ void pipe_limbs(int (&acc)[64], uint64_t (&lo)[8], int (&hi)[8]) {
+template <int CW>
+__device__ __forceinline__ void pipe_limbs(int (&acc)[CW], uint64_t (&lo)[CW / 8],
+                                           int (&hi)[CW / 8]) {
   const uint32_t lane = lane_id();
   const bool b0 = lane & 1u, b1 = lane & 2u, b2 = lane & 4u;
   // coefficient 7 - (lane & 7) of a limb; its weight within its half of the
   // limb, and that of the neighbour's coefficient
   const int wo = 1 << (8 * (3 - (lane & 3u))), wg = 1 << (8 * (3 - ((lane ^ 1u) & 3u)));
-  int64_t v[16];
+  int64_t v[CW / 4];
 #pragma unroll
-  for (int m = 0; m < 16; m++) {
+  for (int m = 0; m < CW / 4; m++) {
     int64_t u[2];
 #pragma unroll
     for (int i = 0; i < 2; i++) {
@@ -331,7 +338,7 @@ __device__ __forceinline__ void pipe_limbs(int (&acc)[64], uint64_t (&lo)[8], in
     v[m] = (b1 ? u[1] : u[0]) + __shfl_xor_sync(FULL, b1 ? u[0] : u[1], 2);
   }
 #pragma unroll
-  for (int m = 0; m < 8; m++) {
+  for (int m = 0; m < CW / 8; m++) {
     const int64_t own = b2 ? v[2 * m + 1] : v[2 * m];
     const int64_t got = __shfl_xor_sync(FULL, b2 ? v[2 * m] : v[2 * m + 1], 4);
     const int64_t l = b2 ? own : got, h = b2 ? got : own;
@@ -340,25 +347,50 @@ __device__ __forceinline__ void pipe_limbs(int (&acc)[64], uint64_t (&lo)[8], in
   }
 }
 
-// Byte b of eight words as one 64-bit word.
-__device__ __forceinline__ uint64_t pipe_bytes(const uint32_t (&w)[8], int b) {
+// Byte b of four or eight words, as one.
+template <int N>
+__device__ __forceinline__ uint64_t pipe_bytes(const uint32_t (&w)[N], int b) {
   const uint32_t s = (uint32_t)b | (uint32_t)(4 + b) << 4;  // byte b of both
   const uint32_t a0 = __byte_perm(w[0], w[1], s), a1 = __byte_perm(w[2], w[3], s);
-  const uint32_t a2 = __byte_perm(w[4], w[5], s), a3 = __byte_perm(w[6], w[7], s);
-  return (uint64_t)__byte_perm(a2, a3, 0x5410) << 32 | __byte_perm(a0, a1, 0x5410);
+  const uint64_t low = __byte_perm(a0, a1, 0x5410);
+  if constexpr (N == 4) {
+    return low;
+  } else {
+    const uint32_t a2 = __byte_perm(w[4], w[5], s), a3 = __byte_perm(w[6], w[7], s);
+    return (uint64_t)__byte_perm(a2, a3, 0x5410) << 32 | low;
+  }
 }
 
-template <int KB, class Next, class Done>
+// Adds a warp's 32 lanes and CW columns of an accumulator (the group's
+// columns [lo, hi)) to its column sums.
+template <int CW>
+__device__ __forceinline__ void pipe_drain_acc(uint32_t taddr, int cq, int lo, int hi,
+                                               int (&acc)[CW]) {
+#pragma unroll
+  for (int k = 0; k < CW / 16; k++) {
+    const int col = CW * cq + 16 * k;
+    if (col >= lo && col < hi) {
+      uint32_t r[16];
+      tmem_ld16(taddr + (uint32_t)col, r);
+      tmem_ld_wait();
+#pragma unroll
+      for (int i = 0; i < 16; i++) acc[16 * k + i] += __float2int_rn(__uint_as_float(r[i]));
+    }
+  }
+}
+
+template <int KB, int NT, class Next, class Done>
 __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, uint8_t *sm,
                                            uint32_t tmem, long long lim, Next next, Done done) {
   constexpr int HS = PIPE_HS, S = 128 / KB, R = KB / 8, GS = 1024 / (KB * HS);
+  constexpr int NACC = 512 / NT, CW = NT / 4, CM = CW / 8;  // columns and limbs per lane
   constexpr int QTOP = S == 1 ? 0 : 2;  // warps of the lane quadrants 3 .. QTOP hold the limbs
   // added to a limb's signed high word to make it unsigned, and taken off the
   // next limb: |V_j| < 2^31 sum_k 2^(8 k), so the high word is at least -C
   constexpr uint32_t C = 0x808080u;
   static_assert(S <= 2, "one or two rows per coefficient");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int q = warp & 3, cq = warp >> 2;  // TMEM lane quadrant, 64-column slice
+  const int q = warp & 3, cq = warp >> 2;  // TMEM lane quadrant, CW-column slice
   const uint32_t t_lane = tmem + ((uint32_t)(32 * q) << 16);
   const bool holds = q >= QTOP;
   const int jj = 4 * (3 - q) + 3 - (lane >> 3);  // limb of this lane within a column (holds)
@@ -378,21 +410,21 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
       Xl[tid * PIPE_EX + 256 + gen] = 0ull;
       Xh[tid * PIPE_EX + 256 + gen] = 0;
     }
-    const bool ok = pipe_tiles<KB>(T.nx, T.ny, T.nout, T.lo, [&](int c0, int W, int e_lo,
+    const bool ok = pipe_tiles<KB, NT>(T.nx, T.ny, T.nout, T.lo, [&](int c0, int W, int e_lo,
                                                                 int e_hi) {
-      int acc[64];
+      int acc[CW];
 #pragma unroll
-      for (int i = 0; i < 64; i++) acc[i] = 0;
+      for (int i = 0; i < CW; i++) acc[i] = 0;
       for (int eg = e_lo; eg <= e_hi; eg += HS * GS) {
         const int ee = eg + HS * GS - 1 < e_hi ? eg + HS * GS - 1 : e_hi;
-        const uint32_t a = grp & 1u;
-        const bool bad = !pipe_wait(sh, &sh->afull[a], (grp >> 1) & 1u, lim);
+        const uint32_t a = grp % NACC;
+        const bool bad = !pipe_wait(sh, &sh->afull[a], (grp / NACC) & 1u, lim);
         if (bar_or_drain<PIPE_DRAIN>(bad)) return false;  // all drain threads agree
         grp++;
         tc_fence_after();
         const int slo = (S * eg > c0 ? S * eg - c0 : 0) & ~15;
         const int shi = ((c0 + W < S * ee + mx ? c0 + W : S * ee + mx) - c0 + 15) & ~15;
-        drain(t_lane + a * PIPE_NT, cq, slo, shi, acc);
+        pipe_drain_acc<CW>(t_lane + a * NT, cq, slo, shi, acc);
         tc_fence_before();
         __syncwarp();
         if (lane == 0) mbar_arrive(smem_u32(&sh->afree[a]));
@@ -400,19 +432,19 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
       // ---- column sums -> limbs
       const int j0 = R * c0, nl = R * W < T.nout - j0 ? R * W : T.nout - j0;
       const int skip = L0 > j0 ? L0 - j0 : 0;  // band: limbs below L0 are not kept
-      const int cb = 64 * cq + (lane & 7);     // this lane's columns: cb + 8 m
-      uint64_t low[8];
-      int high[8];
-      pipe_limbs(acc, low, high);
+      const int cb = CW * cq + (lane & 7);     // this lane's columns: cb + 8 m
+      uint64_t low[CM];
+      int high[CM];
+      pipe_limbs<CW>(acc, low, high);
       if (S > 1) {
         // rows 64 .. 127 of column c belong to column c + 1; those of the
         // tile's last column wait for the next tile
         const int row = 4 * (3 - (q | 2)) + 3 - (lane >> 3);
         if (!holds) {
 #pragma unroll
-          for (int m = 0; m < 8; m++) {
+          for (int m = 0; m < CM; m++) {
             const int c = cb + 8 * m;
-            const int at = row * PIPE_EX + (c < 255 ? c + 1 : 256 + (gen ^ 1));
+            const int at = row * PIPE_EX + (c < NT - 1 ? c + 1 : 256 + (gen ^ 1));
             Xl[at] = low[m];
             Xh[at] = high[m];
           }
@@ -420,7 +452,7 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
         bar_drain();
         if (holds) {
 #pragma unroll
-          for (int m = 0; m < 8; m++) {
+          for (int m = 0; m < CM; m++) {
             const int c = cb + 8 * m, at = row * PIPE_EX + (c > 0 ? c : 256 + gen);
             const uint64_t l = Xl[at];
             low[m] += l;
@@ -430,19 +462,28 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
         gen ^= 1;
       }
       // every limb of a whole tile is kept
-      const bool whole = skip == 0 && nl == R * PIPE_NT;
+      const bool whole = skip == 0 && nl == R * NT;
       if (holds) {
         if (tx) {
 #pragma unroll
-          for (int m = 0; m < 8; m++) {
+          for (int m = 0; m < CM; m++) {
             const int j = j0 + R * (cb + 8 * m) + jj - T.nx;
             const uint64_t add = j >= 0 && j < T.ny ? T.y[j] : 0ull;
             low[m] += add;
             high[m] += low[m] < add;
           }
         }
+        if (T.add != nullptr) {
 #pragma unroll
-        for (int m = 0; m < 8; m++) {
+          for (int m = 0; m < CM; m++) {
+            const int lt = R * (cb + 8 * m) + jj;
+            const uint64_t a = lt < nl ? T.add[j0 + lt] : 0ull;
+            low[m] += a;
+            high[m] += low[m] < a;
+          }
+        }
+#pragma unroll
+        for (int m = 0; m < CM; m++) {
           const uint32_t off = j0 + R * (cb + 8 * m) + jj == L0 ? 0u : C;
           high[m] += (int)C - (int)(low[m] < off);
           low[m] -= off;
@@ -451,13 +492,14 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
       }
       bar_drain();
       // ---- low words plus the high words one limb up.  Bit c of the 64-bit
-      // words below stands for column 64 cq + c; a warp's lanes 24-31 hold the
+      // words below stands for column CW cq + c (bits past CW pass carries
+      // on); a warp's lanes 24-31 hold the
       // lowest of its four limbs of a column, quadrant 3 the lowest four.
       uint64_t Gs[4], Ps[4];  // of the limbs in lanes 8 i .. 8 i + 7
       if (holds) {
-        uint32_t G[8], P[8];
+        uint32_t G[CM], P[CM];
 #pragma unroll
-        for (int m = 0; m < 8; m++) {
+        for (int m = 0; m < CM; m++) {
           const int c = cb + 8 * m, lt = R * c + jj;
           uint32_t below = __shfl_down_sync(FULL, (uint32_t)high[m], 8);
           if (lane >= 24)
@@ -476,9 +518,10 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
         const uint64_t g =
             Gs[0] | (Ps[0] & (Gs[1] | (Ps[1] & (Gs[2] | (Ps[2] & Gs[3])))));
         if (lane == 0)
-          sh->gp[cq][q] = make_ulonglong2(g, Ps[0] & Ps[1] & Ps[2] & Ps[3]);
+          sh->gp[cq][q] = make_ulonglong2(
+              g, (Ps[0] & Ps[1] & Ps[2] & Ps[3]) | (CW < 64 ? ~0ull << (CW & 63) : 0ull));
       }
-      const uint32_t hnext = sh->hx[QTOP][255];
+      const uint32_t hnext = sh->hx[QTOP][NT - 1];
       bar_drain();
       uint64_t cin = 0;  // carries into this warp's limbs of its columns
       uint32_t c = cprev;
@@ -511,7 +554,7 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
         cin >>= lane & 7;
         uint64_t *o = T.out + j0 + R * cb + jj;
 #pragma unroll
-        for (int m = 0; m < 8; m++) {
+        for (int m = 0; m < CM; m++) {
           const int lt = R * (cb + 8 * m) + jj;
           if (whole || (lt < nl && lt >= skip)) o[8 * R * m] = low[m] + ((cin >> (8 * m)) & 1u);
         }
@@ -531,7 +574,7 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
 // same sequence; done(k) is called by the drain threads after product k.
 // Returns false if a wait hit its limit (the record for bigint_check_timeout
 // is set).
-template <int KB, class NextB, class NextI, class NextD, class Done>
+template <int KB, int NT, class NextB, class NextI, class NextD, class Done>
 __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, uint8_t *sm,
                                          NextB next_b, NextI next_i, NextD next_d, Done done) {
   constexpr int ISSUER = PIPE_DRAIN / 32;
@@ -542,9 +585,11 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
       mbar_init(smem_u32(&sh->hfull[i]), PIPE_BUILD);
       mbar_init(smem_u32(&sh->hfree[i]), 1);
     }
-    for (int i = 0; i < 2; i++) {
+    for (int i = 0; i < 4; i++) {
       mbar_init(smem_u32(&sh->afull[i]), 1);
       mbar_init(smem_u32(&sh->afree[i]), PIPE_DRAIN / 32);
+    }
+    for (int i = 0; i < 2; i++) {
       mbar_init(smem_u32(&sh->xfull[i]), PIPE_BUILD);
       mbar_init(smem_u32(&sh->xfree[i]), 1);
     }
@@ -553,7 +598,7 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
     sh->abort = 0;
   }
   if (tid < 32) {
-    tmem_alloc(smem_u32(&sh->tmem_slot), 2 * PIPE_NT);
+    tmem_alloc(smem_u32(&sh->tmem_slot), 512);
     tmem_relinquish();
   }
   for (int i = tid; i < ZB * 128 / 16; i += PIPE_THREADS)
@@ -564,14 +609,14 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
   tc_fence_after();
   const uint32_t tmem = sh->tmem_slot;
   if (warp < ISSUER) {
-    pipe_drain<KB>(L, sh, sm, tmem, lim, next_d, done);
+    pipe_drain<KB, NT>(L, sh, sm, tmem, lim, next_d, done);
   } else if (warp == ISSUER) {
-    pipe_issuer<KB>(L, sh, smem_u32(sm), tmem, lim, next_i);
+    pipe_issuer<KB, NT>(L, sh, smem_u32(sm), tmem, lim, next_i);
     // whatever was issued is finished before the tensor memory is freed
     mma_commit_warp(smem_u32(&sh->done), lane_id() == 0);
     mbar_wait(smem_u32(&sh->done), 0, WAIT_LIMIT);
   } else {
-    pipe_builder<KB>(L, sh, sm, lim, tid - 32 * (ISSUER + 1), next_b);
+    pipe_builder<KB, NT>(L, sh, sm, lim, tid - 32 * (ISSUER + 1), next_b);
   }
   __syncwarp();
   tc_fence_before();
@@ -579,7 +624,7 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
   tc_fence_after();
   const bool ok = sh->abort == 0;
   if (!ok && tid == 0) atomicExch(&g_timeout, 1);
-  if (tid < 32) tmem_dealloc(tmem, 2 * PIPE_NT);
+  if (tid < 32) tmem_dealloc(tmem, 512);
   return ok;
 }
 

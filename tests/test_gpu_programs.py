@@ -64,3 +64,23 @@ def test_poly_many_instances(bi, orc):
     out = to_host(bi.poly(to_dev(a), to_dev(b)))
     for i in (0, 1, 151, 152, 153, 607, 608, 609, 1216, 1499):
         assert np.array_equal(out[i], orc.poly(a[i], b[i])), i
+
+
+@pytest.mark.parametrize("n,count", [(63, 700), (64, 1300), (512, 700), (600, 400), (1024, 500),
+                                     (4096, 1300)])
+def test_poly_batched_products(bi, orc, n, count):
+    """Poly as batched products with an addend: several instances per CTA, and
+    at 4096 limbs more than one chunk of the workspace; the instances at the
+    ends of the batch and of its first chunk against the oracle."""
+    from paper_2607_28897_gb300 import inputs
+
+    a, b = inputs.limbs(903 + n, count, n), inputs.limbs(904 + n, count, n)
+    for i, (x, y) in enumerate([(0xFFFFFFFFFFFFFFFF, 0xFFFFFFFFFFFFFFFF),
+                                (0x807F807F807F807F, 0x7F807F807F807F80), (0, 1)]):
+        a[i], b[i] = np.uint64(x), np.uint64(y)
+        a[-1 - i], b[-1 - i] = a[i], b[i]
+    out = to_host(bi.poly(to_dev(a), to_dev(b)))
+    mid = [1215, 1216] if count > 1216 else [count // 2]
+    for i in [0, 1, 2, 3, *mid, count - 4, count - 3, count - 2, count - 1]:
+        assert np.array_equal(out[i], orc.poly(a[i], b[i])), i
+    bi.check_timeout()
