@@ -179,7 +179,7 @@ __global__ void __launch_bounds__(WARP_CTA)
 
 // The same two steps with one CTA per instance, for wide records (a warp
 // takes its limbs 32 at a time, one round after the other).
-__global__ void __launch_bounds__(LIN_THREADS)
+__global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_mid_cta(const uint64_t *__restrict__ P, int64_t sp, uint64_t *__restrict__ D, int64_t sd,
                  int nl, int32_t *neg) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
@@ -188,7 +188,7 @@ __global__ void __launch_bounds__(LIN_THREADS)
   if (threadIdx.x == 0) neg[i] = ng ? 1 : 0;
 }
 
-__global__ void __launch_bounds__(LIN_THREADS)
+__global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_update_cta(const uint64_t *__restrict__ W, int64_t sw, int nw,
                     const uint64_t *__restrict__ Z, int64_t sz, int s, int ny,
                     const int32_t *__restrict__ neg, int m, uint64_t *__restrict__ Wn, int nout) {
@@ -197,35 +197,30 @@ __global__ void __launch_bounds__(LIN_THREADS)
   ds_update_cta(W + i * sw, nw, Z + i * sz + s, ny, neg[i] != 0, m, Wn + i * sw, nout, scr);
 }
 
-// Records up to this many limbs take the warp-per-instance kernels.
+// Records up to this many limbs take the warp-per-instance kernels, except
+// in batches of at most FEW instances (about the SMs).
 constexpr int WARP_LIMBS = 1024;
-
-// One CTA per instance: q^ = Z[h .. h + nqh) into its record (zero above).
-__global__ void __launch_bounds__(LIN_THREADS)
-    k_ds_tail_q(const uint64_t *__restrict__ Z, int64_t sz, int h, int nqh, uint64_t *Qh,
-                int64_t sq, int nqcap) {
-  const int64_t i = blockIdx.x;
-  const uint64_t *z = Z + i * sz + h;
-  uint64_t *qh = Qh + i * sq;
-  for (int j = threadIdx.x; j < nqcap; j += blockDim.x) qh[j] = j < nqh ? z[j] : 0ull;
-}
+constexpr int64_t FEW = 128;
 
 // One CTA per regular instance: r^ = (u - R) mod B^(nv+1) with R the low
-// nv + 1 limbs of q^ v, the exact correction of q^ and r^ (divmod.cu), and
-// the results.  Irregular instances are left to the one-CTA-per-division
+// nv + 1 limbs of q^ v, the exact correction of q^ (in place: the top limbs
+// of the banded product) and r^ (divmod.cu), and the results.  Irregular instances are left to the one-CTA-per-division
 // kernel.  A tensor-core product of this division that gave up at a wait
 // limit (*aborted) voids the results: BIGINT_ETIMEOUT.
-__global__ void __launch_bounds__(LIN_THREADS)
+__global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_finish(const uint64_t *__restrict__ U, int nu, const uint64_t *__restrict__ V, int nv,
                 const uint64_t *__restrict__ R, int64_t sp, uint64_t *Rh, int64_t sd, uint64_t *Qh,
-                int64_t sq, int nqcap, uint64_t *Qo, int nq, uint64_t *Ro, int32_t *status,
+                int64_t sq, int nqh, uint64_t *Qo, int nq, uint64_t *Ro, int32_t *status,
                 const int *aborted) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   const int64_t i = blockIdx.x;
   const uint64_t *u = U + i * nu, *v = V + i * nv, *rr = R + i * sp;
   if (!regular(u, nu, v, nv)) return;
-  int st = ds_finish_cta(u, nu, v, nv, rr, Rh + i * sd, Qh + i * sq, nqcap, Qo + i * nq, nq,
-                         Ro + i * nv, scr);
+  uint64_t *qh = Qh + i * sq;
+  if (threadIdx.x == 0) qh[nqh] = 0;  // room for a carry of the correction
+  __syncthreads();
+  int st = ds_finish_cta(u, nu, v, nv, rr, Rh + i * sd, qh, nqh + 1, Qo + i * nq, nq, Ro + i * nv,
+                         scr);
   if (*(volatile const int *)aborted) st = BIGINT_ETIMEOUT;
   if (status != nullptr && threadIdx.x == 0) status[i] = st;
 }
@@ -243,8 +238,8 @@ int schedule(int k, int h, int l0, Step *steps, int cap) {
 
 // Per-instance record widths (limbs) and the workspace layout.
 struct Layout {
-  int64_t sw, sp, sd, sz, sq;  // iterate, low product, |d| / r^, banded product, q^
-  size_t w0, w1, p, d, z, qh, neg, total;
+  int64_t sw, sp, sd, sz;  // iterate, low product, |d| / r^, banded product (then q^)
+  size_t w0, w1, p, d, z, neg, total;
 };
 
 size_t align256(size_t x) { return (x + 255) / 256 * 256; }
@@ -255,8 +250,7 @@ Layout layout(int64_t count, int nu, int nv) {
   Y.sw = L + 4;
   Y.sp = nv + 2;
   Y.sd = nv + 2;
-  Y.sz = nu + L + 4;
-  Y.sq = L + 4;
+  Y.sz = nu + L + 6;
   size_t o = 0;
   auto take = [&](size_t bytes) {
     const size_t at = o;
@@ -268,7 +262,6 @@ Layout layout(int64_t count, int nu, int nv) {
   Y.p = take(8 * count * Y.sp);
   Y.d = take(8 * count * Y.sd);
   Y.z = take(8 * count * Y.sz);
-  Y.qh = take(8 * count * Y.sq);
   Y.neg = take(4 * count);
   Y.total = o;
   return Y;
@@ -308,7 +301,6 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   uint64_t *P = reinterpret_cast<uint64_t *>(base + Y.p);
   uint64_t *D = reinterpret_cast<uint64_t *>(base + Y.d);
   uint64_t *Z = reinterpret_cast<uint64_t *>(base + Y.z);
-  uint64_t *Qh = reinterpret_cast<uint64_t *>(base + Y.qh);
   int32_t *neg = reinterpret_cast<int32_t *>(base + Y.neg);
   int32_t *list = static_cast<int32_t *>(list_and_counters);
   // [0] irregular instances listed, [1] a tensor-core product gave up
@@ -325,6 +317,8 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   int rc = bigint_launch_status();
   if (rc != BIGINT_OK) return rc;
   int cur = 0;
+  const bool few = count <= FEW;
+  const int lin = few ? LIN_THREADS_FEW : LIN_THREADS;
   const unsigned gw = (unsigned)((count + WARP_CTA / 32 - 1) / (WARP_CTA / 32));
   // the leading steps whose operands are all small, fused into one launch
   SmallSteps SS;
@@ -359,35 +353,33 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     rc = launch_mul_ex(v + (k - S.t), nv, W[cur], Y.sw, P, Y.sp, count, S.t + 1, nw, nl, 0,
                        ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
     if (rc != BIGINT_OK) return rc;
-    if (nl <= WARP_LIMBS)
+    if (nl <= WARP_LIMBS && !few)
       k_ds_mid<<<gw, WARP_CTA, 0, st>>>(P, Y.sp, D, Y.sd, nl, neg, count);
     else
-      k_ds_mid_cta<<<(unsigned)count, LIN_THREADS, 0, st>>>(P, Y.sp, D, Y.sd, nl, neg);
+      k_ds_mid_cta<<<(unsigned)count, lin, 0, st>>>(P, Y.sp, D, Y.sd, nl, neg);
     if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
     // P2 = w |d|, its limbs from s on
     const int s = S.t + S.l - S.m, n2 = nw + nl;
     rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
     if (rc != BIGINT_OK) return rc;
-    if (S.l + S.m + 2 <= WARP_LIMBS)
+    if (S.l + S.m + 2 <= WARP_LIMBS && !few)
       k_ds_update<<<gw, WARP_CTA, 0, st>>>(W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s, neg, S.m,
                                            W[cur ^ 1], S.l + S.m + 2, count);
     else
-      k_ds_update_cta<<<(unsigned)count, LIN_THREADS, 0, st>>>(
+      k_ds_update_cta<<<(unsigned)count, lin, 0, st>>>(
           W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s, neg, S.m, W[cur ^ 1], S.l + S.m + 2);
     if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
     cur ^= 1;
   }
   // q^ = floor(u w / B^h), w of L + 2 limbs
-  const int nw = L + 2, nz = nu + nw, nqh = nz - h, nqcap = nqh + 1;
+  const int nw = L + 2, nz = nu + nw, nqh = nz - h;
   rc = launch_mul_ex(u, nu, W[cur], Y.sw, Z, Y.sz, count, nu, nw, nz, h - 2, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
   if (rc != BIGINT_OK) return rc;
-  k_ds_tail_q<<<(unsigned)count, LIN_THREADS, 0, st>>>(Z, Y.sz, h, nqh, Qh, Y.sq, nqcap);
-  if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
   // R = q^ v mod B^(nv+1)
-  rc = launch_mul_ex(Qh, Y.sq, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
+  rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
   if (rc != BIGINT_OK) return rc;
-  k_ds_finish<<<(unsigned)count, LIN_THREADS, 0, st>>>(u, nu, v, nv, P, Y.sp, D, Y.sd, Qh, Y.sq,
-                                                       nqcap, q, nq, r, status, ctr + 1);
+  k_ds_finish<<<(unsigned)count, lin, 0, st>>>(u, nu, v, nv, P, Y.sp, D, Y.sd, Z + h, Y.sz, nqh, q,
+                                               nq, r, status, ctr + 1);
   if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
   // the irregular instances, one CTA per division (the workspace is free
   // again: everything above is stream-ordered before this launch)

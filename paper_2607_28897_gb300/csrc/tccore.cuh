@@ -902,7 +902,7 @@ __device__ __forceinline__ bool tc_product(TcCtx &c, const uint64_t *x, int nx, 
 // the coefficient 128 (c0 + c) + t is added to colsum[c * 128 + t] with an
 // atomic add (exact and order-independent: a coefficient's full sum is below
 // 2^31 in magnitude, so every partial sum is too).  The CTAs of one product
-// thus share its tiles' Toeplitz blocks, and tc_colsum_limbs turns the sums
+// thus share its tiles' Toeplitz blocks, and k_tc_sk_finish turns the sums
 // into limbs.  Returns false (and sets c.aborted) if a wait hit its limit.
 template <int NT, int G>
 __device__ bool tc_partial(TcCtx &c, const uint64_t *x, int nx, const uint64_t *y, int ny,
@@ -989,33 +989,6 @@ __device__ bool tc_partial(TcCtx &c, const uint64_t *x, int nx, const uint64_t *
   }
   __syncthreads();  // the shared memory (x, Hankel buffers) is reused by the next unit
   return true;
-}
-
-// out[L0 .. nout) of the product whose column sums (coefficients 128 c + t
-// for the columns c from cfirst = L0 / 16 on) are in colsum[(c - cfirst) *
-// 128 + t], by the whole CTA: limb j is V_j = sum_k (coef(8 j + k) + 2^31)
-// 2^(8 k), i.e. its low word plus the high word of V_(j-1) (plus `margin` at
-// L0), less the bias sum of the column sums (0x8080808080000000 at L0,
-// 0x8080808080808080 above); one carry scan then one borrow scan
-// (blk_add_then_sub), as at the end of each of tc_product's tiles.
-__device__ inline void tc_colsum_limbs(const int *colsum, int L0, int nout, uint64_t margin,
-                                uint64_t *out, uint32_t *scr) {
-  auto V = [&](int j) {
-    const int *cs = colsum + (size_t)(j - L0) * 8;  // 16 limbs per 128-position column
-    unsigned __int128 v = 0;
-#pragma unroll
-    for (int k = 0; k < 8; k++) v += (unsigned __int128)((uint32_t)cs[k] ^ 0x80000000u) << (8 * k);
-    return v;
-  };
-  auto load = [&](int jj) {
-    const int j = L0 + jj;
-    const uint64_t hi = jj == 0 ? margin : (uint64_t)(V(j - 1) >> 64);
-    return make_ulonglong2((uint64_t)V(j), hi);
-  };
-  auto bias = [&](int jj) { return jj == 0 ? 0x8080808080000000ull : 0x8080808080808080ull; };
-  auto store = [&](int jj, uint64_t v) { out[L0 + jj] = v; };
-  uint32_t cc = 0, bb = 0;
-  blk_add_then_sub(nout - L0, &cc, &bb, load, bias, store, scr);
 }
 
 // ---- host side, per translation unit ---------------------------------------

@@ -159,12 +159,73 @@ __global__ void __launch_bounds__(2 * NT + 32, 1)
   tc_release<NT>(c);
 }
 
-// One CTA per product: its limbs [L0, nout) from its column sums.
-__global__ void __launch_bounds__(512)
+// One CTA per product: its limbs [L0, nout) from its column sums (limb j from
+// the coefficients 8 j .. 8 j + 7, biased, with `margin` in place of what limb
+// L0 - 1 would carry; one carry scan, as in tcone.cuh).  A lone CTA is bound
+// by its latency, so it has 1024 threads with four limbs each in flight.
+constexpr int SKF_THREADS = 1024, SKF_R = 4;
+
+__global__ void __launch_bounds__(SKF_THREADS)
     k_tc_sk_finish(const int *colsum, int64_t cs_stride, uint64_t *Out, int64_t so, int L0,
                    int nout, uint64_t margin) {
-  __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
-  tc_colsum_limbs(colsum + blockIdx.x * cs_stride, L0, nout, margin, Out + blockIdx.x * so, scr);
+  constexpr int W = SKF_THREADS / 32;
+  __shared__ uint32_t s_hi[SKF_R * W], s_g[SKF_R * W], s_p[SKF_R * W];
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int *cs = colsum + blockIdx.x * cs_stride;
+  uint64_t *out = Out + blockIdx.x * so + L0;
+  const int n = nout - L0;
+  uint32_t hprev = 0, cprev = 0;
+  for (int base = 0; base < n; base += SKF_R * SKF_THREADS) {
+    uint64_t low[SKF_R];
+    uint32_t high[SKF_R];
+#pragma unroll
+    for (int r = 0; r < SKF_R; r++) {
+      const int j = base + r * SKF_THREADS + tid;
+      low[r] = 0;
+      high[r] = 0;
+      if (j < n) {
+        // (the workspace of bigint_mul_split is 8-byte aligned)
+        const int2 *p = reinterpret_cast<const int2 *>(cs + (size_t)j * 8);
+        const int2 u0 = p[0], u1 = p[1], u2 = p[2], u3 = p[3];
+        constexpr uint32_t B = 0x80000000u;
+        const uint32_t w[8] = {u0.x + B, u0.y + B, u1.x + B, u1.y + B,
+                               u2.x + B, u2.y + B, u3.x + B, u3.y + B};
+        limb_of(w, 0ull, j == 0, low[r], high[r]);
+      }
+      if (lane == 31) s_hi[r * W + warp] = high[r];
+    }
+    __syncthreads();
+    WarpCarry wc[SKF_R];
+#pragma unroll
+    for (int r = 0; r < SKF_R; r++) {
+      const int j = base + r * SKF_THREADS + tid;
+      uint32_t below = __shfl_up_sync(FULL, high[r], 1);
+      if (lane == 0) below = r * W + warp > 0 ? s_hi[r * W + warp - 1] : hprev;
+      uint32_t g = 0, p = 1;
+      if (j < n) {
+        const uint64_t add = j == 0 ? margin : (uint64_t)below;
+        low[r] += add;
+        g = low[r] < add;
+        p = low[r] == ~0ull;
+      }
+      wc[r] = warp_gp(g, p);
+      if (lane == 0) {
+        s_g[r * W + warp] = warp_carry_out(wc[r], 0);
+        s_p[r * W + warp] = warp_all_propagate(wc[r]);
+      }
+    }
+    hprev = s_hi[SKF_R * W - 1];
+    __syncthreads();
+#pragma unroll
+    for (int r = 0; r < SKF_R; r++) {
+      const int j = base + r * SKF_THREADS + tid;
+      const uint64_t cm = warp_carries(warp_gp(s_g[r * W + lane], s_p[r * W + lane]), cprev);
+      const uint64_t lc = warp_carries(wc[r], (uint32_t)(cm >> warp) & 1u);
+      if (j < n) out[j] = low[r] + ((lc >> lane) & 1u);
+      cprev = (uint32_t)(cm >> 32);
+    }
+    __syncthreads();  // the shared arrays are rewritten
+  }
 }
 
 // One CTA per product: tile t (limbs [t L, t L + L), L = tile_limbs) was
@@ -884,7 +945,7 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   int rc = bigint_launch_status();
   if (rc != BIGINT_OK) return rc;
   const int L0 = 16 * P.cfirst;
-  tcm::k_tc_sk_finish<<<(unsigned)count, 512, 0, st>>>(static_cast<const int *>(colsum), stride,
+  tcm::k_tc_sk_finish<<<(unsigned)count, tcm::SKF_THREADS, 0, st>>>(static_cast<const int *>(colsum), stride,
                                                        out, so, L0, nout,
                                                        lo > 0 ? (1ull << 32) : 0ull);
   return bigint_launch_status();
