@@ -81,6 +81,8 @@ __global__ void k_ds_start(const uint64_t *__restrict__ U, const uint64_t *__res
                            int nv, int l, uint64_t *W, int64_t sw, int64_t count,
                            int32_t *irregular, int *nirr) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  pdl_trigger();
+  pdl_wait();
   if (i >= count) return;
   const uint64_t *u = U + i * nu, *v = V + i * nv;
   uint64_t *w = W + i * sw;
@@ -121,6 +123,8 @@ __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS)
   extern __shared__ __align__(16) uint64_t ssm[];
   const int wi = threadIdx.x >> 5, lane = (int)lane_id();
   const int64_t i = (int64_t)blockIdx.x * SMALL_STEP_WARPS + wi;
+  pdl_trigger();
+  pdl_wait();
   if (i >= count) return;  // the whole warp: no block barrier below
   const int N = S.N;
   uint64_t *base = ssm + (size_t)wi * small_step_warp_limbs(N);
@@ -145,6 +149,8 @@ __global__ void __launch_bounds__(WARP_CTA)
     k_ds_mid(const uint64_t *__restrict__ P, int64_t sp, uint64_t *__restrict__ D, int64_t sd,
              int nl, int32_t *neg, int64_t count) {
   const int64_t i = (int64_t)blockIdx.x * (WARP_CTA / 32) + (threadIdx.x >> 5);
+  pdl_trigger();
+  pdl_wait();
   if (i >= count) return;
   const uint64_t *p = P + i * sp;
   uint64_t *d = D + i * sd;
@@ -165,6 +171,8 @@ __global__ void __launch_bounds__(WARP_CTA)
                 int64_t sz, int s, int ny, const int32_t *__restrict__ neg, int m,
                 uint64_t *__restrict__ Wn, int nout, int64_t count) {
   const int64_t i = (int64_t)blockIdx.x * (WARP_CTA / 32) + (threadIdx.x >> 5);
+  pdl_trigger();
+  pdl_wait();
   if (i >= count) return;
   const uint64_t *w = W + i * sw, *y = Z + i * sz + s;
   uint64_t *wn = Wn + i * sw;
@@ -183,6 +191,8 @@ __global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_mid_cta(const uint64_t *__restrict__ P, int64_t sp, uint64_t *__restrict__ D, int64_t sd,
                  int nl, int32_t *neg) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = blockIdx.x;
   const bool ng = ds_mid_cta(P + i * sp, D + i * sd, nl, scr);
   if (threadIdx.x == 0) neg[i] = ng ? 1 : 0;
@@ -193,6 +203,8 @@ __global__ void __launch_bounds__(LIN_THREADS_FEW)
                     const uint64_t *__restrict__ Z, int64_t sz, int s, int ny,
                     const int32_t *__restrict__ neg, int m, uint64_t *__restrict__ Wn, int nout) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = blockIdx.x;
   ds_update_cta(W + i * sw, nw, Z + i * sz + s, ny, neg[i] != 0, m, Wn + i * sw, nout, scr);
 }
@@ -213,6 +225,8 @@ __global__ void __launch_bounds__(LIN_THREADS_FEW)
                 int64_t sq, int nqh, uint64_t *Qo, int nq, uint64_t *Ro, int32_t *status,
                 const int *aborted) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
+  pdl_trigger();
+  pdl_wait();
   const int64_t i = blockIdx.x;
   const uint64_t *u = U + i * nu, *v = V + i * nv, *rr = R + i * sp;
   if (!regular(u, nu, v, nv)) return;
@@ -312,13 +326,13 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   Step steps[64];
   const int ns = schedule(k, h, l0, steps, 64);
   BIGINT_CUDA_TRY(cudaMemsetAsync(ctr, 0, 8, st));
-  k_ds_start<<<(unsigned)((count + 127) / 128), 128, 0, st>>>(u, v, nu, nv, l0, W[0], Y.sw, count,
-                                                              list, ctr);
-  int rc = bigint_launch_status();
-  if (rc != BIGINT_OK) return rc;
-  int cur = 0;
+  if (sk != nullptr) BIGINT_CUDA_TRY(cudaMemsetAsync(sk, 0, sk_bytes, st));
   const bool few = count <= FEW;
   const int lin = few ? LIN_THREADS_FEW : LIN_THREADS;
+  int rc = chain_launch(few, k_ds_start, (unsigned)((count + 127) / 128), 128, 0, st, u, v, nu, nv,
+                        l0, W[0], Y.sw, count, list, ctr);
+  if (rc != BIGINT_OK) return rc;
+  int cur = 0;
   const unsigned gw = (unsigned)((count + WARP_CTA / 32 - 1) / (WARP_CTA / 32));
   // the leading steps whose operands are all small, fused into one launch
   SmallSteps SS;
@@ -341,9 +355,10 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
           8 * SMALL_STEP_WARPS * small_step_warp_limbs(SMALL_STEP_LIMBS)));
       attr = true;
     }
-    k_ds_small<<<(unsigned)((count + SMALL_STEP_WARPS - 1) / SMALL_STEP_WARPS),
-                 32 * SMALL_STEP_WARPS, smem, st>>>(v, nv, W[0], W[1], Y.sw, count, SS);
-    if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
+    rc = chain_launch(few, k_ds_small,
+                      (unsigned)((count + SMALL_STEP_WARPS - 1) / SMALL_STEP_WARPS),
+                      32 * SMALL_STEP_WARPS, smem, st, v, nv, W[0], W[1], Y.sw, count, SS);
+    if (rc != BIGINT_OK) return rc;
     cur = SS.n & 1;
   }
   for (int i = SS.n; i < ns; i++) {
@@ -354,21 +369,21 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
                        ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
     if (rc != BIGINT_OK) return rc;
     if (nl <= WARP_LIMBS && !few)
-      k_ds_mid<<<gw, WARP_CTA, 0, st>>>(P, Y.sp, D, Y.sd, nl, neg, count);
+      rc = chain_launch(few, k_ds_mid, gw, WARP_CTA, 0, st, P, Y.sp, D, Y.sd, nl, neg, count);
     else
-      k_ds_mid_cta<<<(unsigned)count, lin, 0, st>>>(P, Y.sp, D, Y.sd, nl, neg);
-    if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
+      rc = chain_launch(few, k_ds_mid_cta, (unsigned)count, lin, 0, st, P, Y.sp, D, Y.sd, nl, neg);
+    if (rc != BIGINT_OK) return rc;
     // P2 = w |d|, its limbs from s on
     const int s = S.t + S.l - S.m, n2 = nw + nl;
     rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
     if (rc != BIGINT_OK) return rc;
     if (S.l + S.m + 2 <= WARP_LIMBS && !few)
-      k_ds_update<<<gw, WARP_CTA, 0, st>>>(W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s, neg, S.m,
-                                           W[cur ^ 1], S.l + S.m + 2, count);
+      rc = chain_launch(few, k_ds_update, gw, WARP_CTA, 0, st, W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s,
+                        neg, S.m, W[cur ^ 1], S.l + S.m + 2, count);
     else
-      k_ds_update_cta<<<(unsigned)count, lin, 0, st>>>(
-          W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s, neg, S.m, W[cur ^ 1], S.l + S.m + 2);
-    if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
+      rc = chain_launch(few, k_ds_update_cta, (unsigned)count, lin, 0, st, W[cur], Y.sw, nw, Z, Y.sz,
+                        s, n2 - s, neg, S.m, W[cur ^ 1], S.l + S.m + 2);
+    if (rc != BIGINT_OK) return rc;
     cur ^= 1;
   }
   // q^ = floor(u w / B^h), w of L + 2 limbs
@@ -378,9 +393,9 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   // R = q^ v mod B^(nv+1)
   rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
   if (rc != BIGINT_OK) return rc;
-  k_ds_finish<<<(unsigned)count, lin, 0, st>>>(u, nu, v, nv, P, Y.sp, D, Y.sd, Z + h, Y.sz, nqh, q,
-                                               nq, r, status, ctr + 1);
-  if ((rc = bigint_launch_status()) != BIGINT_OK) return rc;
+  rc = chain_launch(few, k_ds_finish, (unsigned)count, lin, 0, st, u, nu, v, nv, P, Y.sp, D, Y.sd,
+                    Z + h, Y.sz, nqh, q, nq, r, status, ctr + 1);
+  if (rc != BIGINT_OK) return rc;
   // the irregular instances, one CTA per division (the workspace is free
   // again: everything above is stream-ordered before this launch)
   return launch_divmod_cta(u, v, q, r, status, count, nu, nv, ws, list, ctr, st);

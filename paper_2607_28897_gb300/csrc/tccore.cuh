@@ -402,6 +402,36 @@ __device__ __forceinline__ void fill_x(uint8_t *xs, const uint64_t *x, int nx, i
   }
 }
 
+// The same for the blocks p0 <= p < p1 of 128 digits only, with x's carry
+// digit.
+__device__ __forceinline__ void fill_x_window(uint8_t *xs, const uint64_t *x, int nx, int ptot,
+                                              int p0, int p1) {
+  constexpr int U = 8;
+  const int total = 16 * (p1 - p0), step = (int)blockDim.x;
+  for (int i0 = threadIdx.x; i0 < total; i0 += U * step) {
+    uint64_t v[U], below[U];
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int i = i0 + u * step, L = 16 * p0 + i;
+      v[u] = (L >= 0 && L < nx && i < total) ? x[L] : 0ull;
+      below[u] = (L >= 1 && L - 1 < nx && i < total) ? x[L - 1] : 0ull;
+    }
+#pragma unroll
+    for (int u = 0; u < U; u++) {
+      const int i = i0 + u * step;
+      if (i < total) {
+        const int pp = p0 + 16 + (i >> 4), h = i & 15;
+        const Digits16 d = recode16(v[u], below[u]);
+        const uint32_t el = (uint32_t)d.ev, eh = (uint32_t)(d.ev >> 32);
+        const uint32_t ol = (uint32_t)d.od, oh = (uint32_t)(d.od >> 32);
+        *reinterpret_cast<uint4 *>(xs + (size_t)(pp + h * ptot) * 16) = make_uint4(
+            unbias_h2(__byte_perm(el, ol, 0x5410)), unbias_h2(__byte_perm(el, ol, 0x7632)),
+            unbias_h2(__byte_perm(eh, oh, 0x5410)), unbias_h2(__byte_perm(eh, oh, 0x7632)));
+      }
+    }
+  }
+}
+
 // Hankel core matrices of the group whose last block is eb: matrix j, row r,
 // element w = recoded y digit at 128 eb + 127 - 8 j - r - w.  Row s = 8 j + r
 // is the run D[s .. s + 8) of the reversed digit sequence D[i] = digit at
@@ -462,7 +492,8 @@ __device__ __forceinline__ void hank_build(uint8_t *hb, uint8_t *st, HankLimbs v
 // of the tile that meet x are computed, widened to multiples of 16; the
 // group's first MMA overwrites the accumulator if it spans the group's
 // columns (group_span), otherwise a clearing MMA with a zero A operand over
-// those columns comes first.
+// those columns comes first (its B operand is x from clear_off bytes on,
+// which must hold finite values).
 // Tile columns [lo, hi) (multiples of 16) that the MMAs of blocks ea..eb
 // write: block e meets columns [max(c0, S e), min(c0 + W, S e + mx)), both
 // ends growing with e.
@@ -477,7 +508,7 @@ __device__ __forceinline__ void group_span(int c0, int W, int ea, int eb, int mx
 template <int KB = 128>
 __device__ __forceinline__ void issue_group(uint32_t dtm, uint32_t ha, uint32_t xs_a,
                                             uint32_t z_a, uint32_t lbo_b, int c0, int W, int ea,
-                                            int eb, int mx, uint32_t mbar) {
+                                            int eb, int mx, uint32_t mbar, uint32_t clear_off = 0) {
   constexpr int S = 128 / KB;
   tc_fence_after();
   int slo, shi;
@@ -496,7 +527,7 @@ __device__ __forceinline__ void issue_group(uint32_t dtm, uint32_t ha, uint32_t 
       if (lo == slo && hi == shi) {
         accf = 0;
       } else {
-        mma_f16(dtm + (uint32_t)slo, sdesc(z_a, 128, 128), sdesc(xs_a, lbo_b, 128),
+        mma_f16(dtm + (uint32_t)slo, sdesc(z_a, 128, 128), sdesc(xs_a + clear_off, lbo_b, 128),
                 IDESC_M128 | ((uint32_t)((shi - slo) >> 3) << 17), 0);
       }
     }
@@ -930,8 +961,13 @@ __device__ bool tc_partial(TcCtx &c, const uint64_t *x, int nx, const uint64_t *
 
   for (int i = tid; i < ZB * 128 / 16; i += THREADS)
     reinterpret_cast<uint4 *>(sm + Ly.z)[i] = make_uint4(0u, 0u, 0u, 0u);
-  fill_x<true>(sm + Ly.xs, x, nx, Ly.ptot);
   auto last_block = [&](int gi) { return e_lo + gi * G + G - 1 < e_hi ? e_lo + gi * G + G - 1 : e_hi; };
+  // only the x blocks that the unit's Toeplitz blocks meet in the tile (with
+  // the 16-column rounding of the MMAs), eight limbs' loads in flight
+  const int pb0 = c0 - last_block(g1 - 1) - 15 > -16 ? c0 - last_block(g1 - 1) - 15 : -16;
+  const int pb1 = c0 + W - (e_lo + g0 * G) + 16 < Ly.mx + 16 ? c0 + W - (e_lo + g0 * G) + 16 : Ly.mx + 16;
+  fill_x_window(sm + Ly.xs, x, nx, Ly.ptot, pb0, pb1);
+  const uint32_t clear_off = (uint32_t)(pb0 + 16) * 16u;
   if (worker) hank_build<G, DRAIN>(sm + Ly.h0, sm + Ly.st, hank_load<G>(y, ny, last_block(g0), tid), tid);
   fence_async_smem();
   __syncthreads();
@@ -941,7 +977,7 @@ __device__ bool tc_partial(TcCtx &c, const uint64_t *x, int nx, const uint64_t *
     const int ea = e_lo + gi * G, eb = last_block(gi);
     if (issuer)
       issue_group(c.tmem + (uint32_t)(b * NT), b ? sbase + Ly.h1 : sbase + Ly.h0, xs_a, z_a,
-                  lbo_b, c0, W, ea, eb, Ly.mx, mb[b]);
+                  lbo_b, c0, W, ea, eb, Ly.mx, mb[b], clear_off);
     c.pending |= 1u << b;
     const bool more = k + 1 < ng && worker;
     HankLimbs hv{0ull, 0ull};

@@ -28,6 +28,8 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   TcCtx c;
   tc_init<NT>(c, sm, &sh, scr);
+  pdl_trigger();  // not before this CTA has its tensor memory
+  pdl_wait();
   for (int64_t inst = blockIdx.x; inst < count; inst += gridDim.x) {
     const int64_t next = inst + gridDim.x;
     if (threadIdx.x == 0 && next < count) {
@@ -55,6 +57,8 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
   __shared__ OneShared sh;
   OneCtx c;
   one_init<NT>(c, sm, &sh);
+  pdl_trigger();  // not before this CTA has its tensor memory
+  pdl_wait();
   for (int64_t inst = blockIdx.x; inst < count; inst += gridDim.x) {
     const int64_t next = inst + gridDim.x;
     if (threadIdx.x == 0 && next < count) {
@@ -144,6 +148,8 @@ __global__ void __launch_bounds__(2 * NT + 32, 1)
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   TcCtx c;
   tc_init<NT>(c, sm, &sh, scr);
+  pdl_trigger();  // not before this CTA has its tensor memory
+  pdl_wait();
   const int upi = P.first[P.T];
   for (int64_t u = blockIdx.x; u < count * upi; u += gridDim.x) {
     const int64_t inst = u / upi;
@@ -161,17 +167,20 @@ __global__ void __launch_bounds__(2 * NT + 32, 1)
 
 // One CTA per product: its limbs [L0, nout) from its column sums (limb j from
 // the coefficients 8 j .. 8 j + 7, biased, with `margin` in place of what limb
-// L0 - 1 would carry; one carry scan, as in tcone.cuh).  A lone CTA is bound
+// L0 - 1 would carry; one carry scan, as in tcone.cuh), then `zero` of the
+// sums cleared.  A lone CTA is bound
 // by its latency, so it has 1024 threads with four limbs each in flight.
 constexpr int SKF_THREADS = 1024, SKF_R = 4;
 
 __global__ void __launch_bounds__(SKF_THREADS)
-    k_tc_sk_finish(const int *colsum, int64_t cs_stride, uint64_t *Out, int64_t so, int L0,
-                   int nout, uint64_t margin) {
+    k_tc_sk_finish(int *colsum, int64_t cs_stride, uint64_t *Out, int64_t so, int L0,
+                   int nout, uint64_t margin, int zero) {
   constexpr int W = SKF_THREADS / 32;
   __shared__ uint32_t s_hi[SKF_R * W], s_g[SKF_R * W], s_p[SKF_R * W];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-  const int *cs = colsum + blockIdx.x * cs_stride;
+  pdl_trigger();
+  pdl_wait();
+  int *cs = colsum + blockIdx.x * cs_stride;
   uint64_t *out = Out + blockIdx.x * so + L0;
   const int n = nout - L0;
   uint32_t hprev = 0, cprev = 0;
@@ -226,6 +235,10 @@ __global__ void __launch_bounds__(SKF_THREADS)
     }
     __syncthreads();  // the shared arrays are rewritten
   }
+  // the sums back to zero for the chain's next product (zero ints, a multiple
+  // of 4; everything was read before the last barrier)
+  for (int i = 4 * tid; i < zero; i += 4 * SKF_THREADS)
+    *reinterpret_cast<int4 *>(cs + i) = make_int4(0, 0, 0, 0);
 }
 
 // One CTA per product: tile t (limbs [t L, t L + L), L = tile_limbs) was
@@ -391,9 +404,8 @@ static int launch_tc(const TcArgs &A, int64_t count, int nx, int ny, int nout, c
   if (sms == 0) return BIGINT_ECUDA;
   const int64_t slots = (int64_t)sms * tc_per_sm<NT, G, XC, KB>(smem);
   const int64_t grid = count < slots ? count : slots;
-  tcm::k_mul_tc<NT, G, XC, KB><<<(unsigned)grid, 2 * NT + 32, smem, st>>>(
-      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag);
-  return bigint_launch_status();
+  return chain_launch(grid <= sms, tcm::k_mul_tc<NT, G, XC, KB>, (unsigned)grid, 2 * NT + 32, smem, st, A.x,
+                      A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag);
 }
 
 static int launch_shape(TcShape sh, const TcArgs &A, int64_t count, int nx, int ny, int nout,
@@ -594,9 +606,8 @@ static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, 
   const int64_t grid = count < slots ? count : slots;
   auto *kern = A.add != nullptr ? tcm::k_mul_one<NT, W, true> : tcm::k_mul_one<NT, W, false>;
   if (A.add != nullptr && !one_attr<NT, true>().ok) return BIGINT_ECUDA;
-  kern<<<(unsigned)grid, 32 * W, smem, st>>>(A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy,
-                                             A.so, A.lo, A.abort_flag, A.add, A.sadd);
-  return bigint_launch_status();
+  return chain_launch(grid <= sms, kern, (unsigned)grid, 32 * W, smem, st, A.x, A.y, A.out, nx, ny, nout, count,
+                      A.sx, A.sy, A.so, A.lo, A.abort_flag, A.add, A.sadd);
 }
 
 // ---- pipelined products (tcpipe.cuh) --------------------------------------------
@@ -627,10 +638,9 @@ static int launch_pipe(const TcArgs &A, int64_t count, int nx, int ny, int nout,
   if (count == 0) return BIGINT_OK;
   const int sms = sm_count();
   if (sms == 0) return BIGINT_ECUDA;
-  tcm::k_mul_pipe<KB, NT><<<(unsigned)(count < sms ? count : sms), tcm::PIPE_THREADS, L.total, st>>>(
-      A.x, A.y, A.out, nx, ny, nout, count, A.sx, A.sy, A.so, A.lo, A.abort_flag, A.add, A.sadd,
-      L);
-  return bigint_launch_status();
+  return chain_launch(true, tcm::k_mul_pipe<KB, NT>, (unsigned)(count < sms ? count : sms),
+                      tcm::PIPE_THREADS, L.total, st, A.x, A.y, A.out, nx, ny, nout, count, A.sx,
+                      A.sy, A.so, A.lo, A.abort_flag, A.add, A.sadd, L);
 }
 
 // Modelled time of a product in the pipelined form (-1: x does not fit): its
@@ -882,10 +892,12 @@ size_t mul_sk_bytes_per_product(int na, int nb, int nout, int lo) {
 }
 
 // True if the split-K form would run more units than the ordinary launch
-// has CTAs busy: few products (count x tiles well below the SMs).
+// has CTAs busy: few products (count x tiles well below the SMs).  Not for
+// products the one-drain form takes: one of 512 limbs is 12 us there on one
+// CTA, 18 us as units, sums and finish.
 bool mul_sk_worth(int64_t count, int na, int nb, int nout, int lo) {
   const int nx = na < nb ? na : nb, ny = na < nb ? nb : na;
-  if (nx < 256 || mul_sk_bytes_per_product(na, nb, nout, lo) == 0) return false;
+  if (nx <= tcm::ONE_MAX || mul_sk_bytes_per_product(na, nb, nout, lo) == 0) return false;
   tcm::SkPlan P;
   int groups[tcm::SK_MAX_TILES];
   if (!sk_tiles(nx, ny, nout, lo, 8, P, groups)) return false;
@@ -896,11 +908,11 @@ bool mul_sk_worth(int64_t count, int na, int nb, int nout, int lo) {
 // The low nout limbs (from limb lo: band mode, as tc_product) of a batch of
 // products, each cut into units of (tile, groups) spread over the SMs; the
 // units add their column sums into `colsum` (count x
-// mul_sk_bytes_per_product bytes, zeroed here), then one CTA per product
-// forms the limbs.  Results are those of tc_product (bit-identical).
+// mul_sk_bytes_per_product bytes, zeroed here, or with `zeroed` found and left
+// all zero: 16-byte aligned then), then one CTA per product forms the limbs.  Results are those of tc_product (bit-identical).
 int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, void *colsum,
-                     size_t colsum_bytes, int *abort_flag, cudaStream_t st) {
+                     size_t colsum_bytes, int *abort_flag, cudaStream_t st, bool zeroed) {
   const uint64_t *x = a, *y = b;
   int64_t sx = sa, sy = sb;
   int nx = na, ny = nb;
@@ -933,22 +945,17 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   P.first[0] = 0;
   for (int t = 0; t < P.T; t++) P.first[t + 1] = P.first[t] + (int)((groups[t] + gpc - 1) / gpc);
   const int64_t units = count * P.first[P.T];
-  BIGINT_CUDA_TRY(cudaMemsetAsync(colsum, 0, per * (size_t)count, st));
+  if (!zeroed) BIGINT_CUDA_TRY(cudaMemsetAsync(colsum, 0, per * (size_t)count, st));
   const int64_t stride = (int64_t)(per / sizeof(int));
   const unsigned grid = (unsigned)(units < sms ? units : sms);
-  if (G == 8)
-    tcm::k_mul_tc_sk<256, 8><<<grid, 2 * 256 + 32, smem, st>>>(
-        x, y, nx, ny, sx, sy, count, P, static_cast<int *>(colsum), stride, abort_flag);
-  else
-    tcm::k_mul_tc_sk<256, 4><<<grid, 2 * 256 + 32, smem, st>>>(
-        x, y, nx, ny, sx, sy, count, P, static_cast<int *>(colsum), stride, abort_flag);
-  int rc = bigint_launch_status();
+  int rc = chain_launch(true, G == 8 ? tcm::k_mul_tc_sk<256, 8> : tcm::k_mul_tc_sk<256, 4>, grid,
+                        2 * 256 + 32, smem, st, x, y, nx, ny, sx, sy, count, P,
+                        static_cast<int *>(colsum), stride, abort_flag);
   if (rc != BIGINT_OK) return rc;
   const int L0 = 16 * P.cfirst;
-  tcm::k_tc_sk_finish<<<(unsigned)count, tcm::SKF_THREADS, 0, st>>>(static_cast<const int *>(colsum), stride,
-                                                       out, so, L0, nout,
-                                                       lo > 0 ? (1ull << 32) : 0ull);
-  return bigint_launch_status();
+  return chain_launch(true, tcm::k_tc_sk_finish, (unsigned)count, tcm::SKF_THREADS, 0, st,
+                      static_cast<int *>(colsum), stride, out, so, L0, nout,
+                      lo > 0 ? (1ull << 32) : 0ull, zeroed ? (int)stride : 0);
 }
 
 // ---- split products ----------------------------------------------------------
@@ -1040,7 +1047,7 @@ int launch_mul_split(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_
   // a few products: each cut into (tile, groups) units over the SMs
   if (count <= SPLIT_SK_MAX_COUNT && mul_sk_worth(count, na, nb, na + nb, 0))
     return launch_mul_tc_sk(a, na, b, nb, out, na + nb, count, na, nb, na + nb, 0, ws, bytes,
-                            nullptr, st);
+                            nullptr, st, false);
   const uint64_t *x = a, *y = b;
   int nx = na, ny = nb;
   if (nb < na) { x = b; y = a; nx = nb; ny = na; }

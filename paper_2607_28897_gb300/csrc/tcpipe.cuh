@@ -608,6 +608,8 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
   __syncthreads();
   tc_fence_after();
   const uint32_t tmem = sh->tmem_slot;
+  pdl_trigger();  // not before this CTA has its tensor memory
+  pdl_wait();
   if (warp < ISSUER) {
     pipe_drain<KB, NT>(L, sh, sm, tmem, lim, next_d, done);
   } else if (warp == ISSUER) {
