@@ -95,6 +95,16 @@ namespace bigint {
 // Counts the kernel launches the library enqueues (bigint_kernel_launches).
 void count_launch();
 
+// Column sums of a chain of split-K products: two buffers of `bytes`, all
+// zero at the start; a product takes buf[cur], and its finish clears what the
+// product before left in the other (`used` bytes of each instance's `used`).
+struct SkBuffers {
+  void *buf[2] = {nullptr, nullptr};
+  size_t bytes = 0;
+  int cur = 0;
+  size_t used = 0;  // bytes the last product dirtied in buf[cur ^ 1]
+};
+
 // Shapes the tensor-core product can be forced to (the autotuner's
 // candidates; 0 = chosen by the cost model): 128-digit x blocks with the
 // 64-, 128- or 256-column tile, or narrow x blocks of 64 or 32 digits.
@@ -116,8 +126,9 @@ namespace bigint {
 // put at most one CTA on an SM: with several, those that start early crowd on
 // the SMs that empty first and queue there for tensor memory (4096 divisions
 // of 1024 by 512 limbs 810 -> 874 us), while a chain of small launches gains
-// (one division of 16384 by 8192 limbs 470 -> 359 us).
-template <class... P, class... A>
+// (one division of 16384 by 8192 limbs 470 -> 359 us).  CLUSTER: CTAs per
+// thread-block cluster (grid a multiple of it).
+template <int CLUSTER = 1, class... P, class... A>
 inline int chain_launch(bool overlap, void (*kern)(P...), unsigned grid, unsigned threads,
                         size_t smem, cudaStream_t st, A... args) {
   cudaLaunchConfig_t c = {};
@@ -125,11 +136,19 @@ inline int chain_launch(bool overlap, void (*kern)(P...), unsigned grid, unsigne
   c.blockDim = dim3(threads);
   c.dynamicSmemBytes = smem;
   c.stream = st;
-  cudaLaunchAttribute at;
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  c.attrs = &at;
-  c.numAttrs = overlap ? 1 : 0;
+  cudaLaunchAttribute at[2];
+  c.attrs = at;
+  if (CLUSTER > 1) {
+    at[c.numAttrs].id = cudaLaunchAttributeClusterDimension;
+    at[c.numAttrs].val.clusterDim.x = CLUSTER;
+    at[c.numAttrs].val.clusterDim.y = at[c.numAttrs].val.clusterDim.z = 1;
+    c.numAttrs++;
+  }
+  if (overlap) {
+    at[c.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at[c.numAttrs].val.programmaticStreamSerializationAllowed = 1;
+    c.numAttrs++;
+  }
   if (cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...) != cudaSuccess) return BIGINT_ECUDA;
   return bigint_launch_status();
 }

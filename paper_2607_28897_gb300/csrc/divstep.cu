@@ -45,7 +45,7 @@ using namespace divc;
 
 int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                   int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
-                  cudaStream_t st, int tc_min, void *sk_ws, size_t sk_bytes);
+                  cudaStream_t st, int tc_min, SkBuffers *sk);
 int launch_divmod_cta(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r,
                       int32_t *status, int64_t count, int nu, int nv, void *ws,
                       const int32_t *list, const int *nlist, cudaStream_t st);
@@ -301,7 +301,7 @@ bool divmod_steps_default(int nu, int nv) { return nv >= DIV_STEP_MIN && nu >= n
 // ws: ws_bytes for the step records (the one-CTA-per-division kernel's
 // per-instance regions, reused); list_and_counters: 4 count bytes rounded to
 // 256, then two ints, OUTSIDE those regions (that kernel reads the list
-// while it writes its regions); sk: sk_bytes for the column sums of the
+// while it writes its regions); sk: sk_bytes for two sets of column sums of the
 // split-K products of a small batch (null: none).
 int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r,
                         int32_t *status, int64_t count, int nu, int nv, void *ws, size_t ws_bytes,
@@ -326,7 +326,14 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   Step steps[64];
   const int ns = schedule(k, h, l0, steps, 64);
   BIGINT_CUDA_TRY(cudaMemsetAsync(ctr, 0, 8, st));
-  if (sk != nullptr) BIGINT_CUDA_TRY(cudaMemsetAsync(sk, 0, sk_bytes, st));
+  SkBuffers skb, *skp = nullptr;
+  if (sk != nullptr) {
+    BIGINT_CUDA_TRY(cudaMemsetAsync(sk, 0, sk_bytes, st));
+    skb.bytes = sk_bytes / 2;
+    skb.buf[0] = sk;
+    skb.buf[1] = static_cast<char *>(sk) + skb.bytes;
+    skp = &skb;
+  }
   const bool few = count <= FEW;
   const int lin = few ? LIN_THREADS_FEW : LIN_THREADS;
   int rc = chain_launch(few, k_ds_start, (unsigned)((count + 127) / 128), 128, 0, st, u, v, nu, nv,
@@ -366,7 +373,7 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     const int nw = S.l + 2, nl = S.t + 2;
     // P = vt w mod B^(t+2)
     rc = launch_mul_ex(v + (k - S.t), nv, W[cur], Y.sw, P, Y.sp, count, S.t + 1, nw, nl, 0,
-                       ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
+                       ctr + 1, st, STEP_TC_MIN, skp);
     if (rc != BIGINT_OK) return rc;
     if (nl <= WARP_LIMBS && !few)
       rc = chain_launch(few, k_ds_mid, gw, WARP_CTA, 0, st, P, Y.sp, D, Y.sd, nl, neg, count);
@@ -375,7 +382,7 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     if (rc != BIGINT_OK) return rc;
     // P2 = w |d|, its limbs from s on
     const int s = S.t + S.l - S.m, n2 = nw + nl;
-    rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
+    rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st, STEP_TC_MIN, skp);
     if (rc != BIGINT_OK) return rc;
     if (S.l + S.m + 2 <= WARP_LIMBS && !few)
       rc = chain_launch(few, k_ds_update, gw, WARP_CTA, 0, st, W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s,
@@ -388,10 +395,10 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   }
   // q^ = floor(u w / B^h), w of L + 2 limbs
   const int nw = L + 2, nz = nu + nw, nqh = nz - h;
-  rc = launch_mul_ex(u, nu, W[cur], Y.sw, Z, Y.sz, count, nu, nw, nz, h - 2, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
+  rc = launch_mul_ex(u, nu, W[cur], Y.sw, Z, Y.sz, count, nu, nw, nz, h - 2, ctr + 1, st, STEP_TC_MIN, skp);
   if (rc != BIGINT_OK) return rc;
   // R = q^ v mod B^(nv+1)
-  rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, sk, sk_bytes);
+  rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, skp);
   if (rc != BIGINT_OK) return rc;
   rc = chain_launch(few, k_ds_finish, (unsigned)count, lin, 0, st, u, nu, v, nv, P, Y.sp, D, Y.sd,
                     Z + h, Y.sz, nqh, q, nq, r, status, ctr + 1);
@@ -434,7 +441,7 @@ size_t divmod_sk_bytes(int64_t count, int nu, int nv) {
   const int nw = L + 2;
   take(nu, nw, nu + nw, h - 2);
   take(nw, nv, nv + 1, 0);
-  return (size_t)count * per;
+  return 2 * (size_t)count * per;  // two buffers in turn
 }
 
 }  // namespace bigint

@@ -21,7 +21,7 @@ namespace bigint {
 
 int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                   int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
-                  cudaStream_t st, int tc_min, void *sk_ws, size_t sk_bytes);
+                  cudaStream_t st, int tc_min, SkBuffers *sk);
 int launch_mul(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t count, int na,
                int nb, int nout, cudaStream_t st);
 
@@ -122,7 +122,7 @@ int run(const uint64_t *x, int64_t sx, const uint64_t *y, int64_t sy, uint64_t *
         int64_t count, int n, int levels, char *ws, cudaStream_t st) {
   if (levels <= 0)
     return launch_mul_ex(x, sx, y, sy, out, so, count, n, n, 2 * n, 0, nullptr, st, TC_LEAF_MIN,
-                         nullptr, 0);
+                         nullptr);
   const int k = n / 2;
   uint64_t *DA = reinterpret_cast<uint64_t *>(ws);
   char *p = ws + align256(8 * (size_t)count * k);

@@ -228,26 +228,25 @@ size_t mul_sk_bytes_per_product(int na, int nb, int nout, int lo);
 bool mul_sk_worth(int64_t count, int na, int nb, int nout, int lo);
 int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, void *colsum,
-                     size_t colsum_bytes, int *abort_flag, cudaStream_t st, bool zeroed);
+                     size_t colsum_bytes, SkBuffers *chain, int *abort_flag, cudaStream_t st);
 
 // The products inside divisions and programs: variant 0 or 12 runs the
 // tensor-core product with its shape by the cost model (split-K for a few
-// products, with sk_ws, sk_bytes of zeros that it leaves zero), variants
-// 13-17 force its shape as for launch_mul, and variants 8-10 keep them on the
-// integer pipes.
+// products of a chain with column-sum buffers `sk`), variants 13-17 force its
+// shape as for launch_mul, and variants 8-10 keep them on the integer pipes.
 int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                   int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
-                  cudaStream_t st, int tc_min, void *sk_ws, size_t sk_bytes) {
+                  cudaStream_t st, int tc_min, SkBuffers *sk) {
   if (count == 0) return BIGINT_OK;
   const int nmin = na < nb ? na : nb;
   const int v = g_mul_variant;
   if (v == 0 || (v >= 12 && v <= 17)) {
     if (nmin >= tc_min && mul_tc_smem(na, nb) > 0) {
       // few products: cut each into units over the SMs (split-K)
-      if (v <= 12 && sk_ws != nullptr && mul_sk_worth(count, na, nb, nout, lo) &&
-          sk_bytes >= (size_t)count * mul_sk_bytes_per_product(na, nb, nout, lo))
-        return launch_mul_tc_sk(a, sa, b, sb, out, so, count, na, nb, nout, lo, sk_ws, sk_bytes,
-                                abort_flag, st, true);
+      if (v <= 12 && sk != nullptr && mul_sk_worth(count, na, nb, nout, lo) &&
+          sk->bytes >= (size_t)count * mul_sk_bytes_per_product(na, nb, nout, lo))
+        return launch_mul_tc_sk(a, sa, b, sb, out, so, count, na, nb, nout, lo, sk->buf[sk->cur],
+                                sk->bytes, sk, abort_flag, st);
       static const int force[6] = {0, TC_FORCE_64, TC_FORCE_128, TC_FORCE_256, TC_FORCE_N64,
                                    TC_FORCE_N32};
       return launch_mul_tc_ex(a, sa, b, sb, out, so, count, na, nb, nout, lo, abort_flag, st,

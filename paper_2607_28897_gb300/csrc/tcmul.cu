@@ -5,6 +5,8 @@
 // (tccore.cuh: the digit convolution as tcgen05 fp16 MMAs with exact fp32
 // accumulation, Sec. V-B's schoolbook product on the tensor cores).
 #include "tccore.cuh"
+#include <cooperative_groups.h>
+
 #include "ragged.cuh"
 #include "tcone.cuh"
 #include "tcpipe.cuh"
@@ -165,31 +167,47 @@ __global__ void __launch_bounds__(2 * NT + 32, 1)
   tc_release<NT>(c);
 }
 
-// One CTA per product: its limbs [L0, nout) from its column sums (limb j from
-// the coefficients 8 j .. 8 j + 7, biased, with `margin` in place of what limb
-// L0 - 1 would carry; one carry scan, as in tcone.cuh), then `zero` of the
-// sums cleared.  A lone CTA is bound
-// by its latency, so it has 1024 threads with four limbs each in flight.
-constexpr int SKF_THREADS = 1024, SKF_R = 4;
+// A cluster of SKF_CLUSTER CTAs per product: its limbs [L0, nout) from its
+// column sums (limb j from the coefficients 8 j .. 8 j + 7, biased, with
+// `margin` in place of what limb L0 - 1 would carry; one carry scan, as in
+// tcone.cuh), SKF_SPAN limbs per CTA and round; the CTAs exchange the high
+// word of their last limb and their (generate, propagate) through distributed
+// shared memory.  Bound by latency: 16384 limbs on one CTA, 512 threads and
+// two scans took 27 us, 1024 threads and one scan 13.  CTAs past the products'
+// clear `zero` ints of zbuf (the column sums of the product before).
+constexpr int SKF_THREADS = 1024, SKF_R = 4, SKF_CLUSTER = 4, SKF_SPAN = SKF_R * SKF_THREADS;
 
 __global__ void __launch_bounds__(SKF_THREADS)
-    k_tc_sk_finish(int *colsum, int64_t cs_stride, uint64_t *Out, int64_t so, int L0,
-                   int nout, uint64_t margin, int zero) {
+    k_tc_sk_finish(const int *colsum, int64_t cs_stride, uint64_t *Out, int64_t so, int L0,
+                   int nout, uint64_t margin, int64_t count, int *zbuf, int64_t zero) {
   constexpr int W = SKF_THREADS / 32;
   __shared__ uint32_t s_hi[SKF_R * W], s_g[SKF_R * W], s_p[SKF_R * W];
+  __shared__ uint32_t c_hi[SKF_CLUSTER], c_g[SKF_CLUSTER], c_p[SKF_CLUSTER];
+  namespace cg = cooperative_groups;
+  cg::cluster_group cl = cg::this_cluster();
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   pdl_trigger();
   pdl_wait();
-  int *cs = colsum + blockIdx.x * cs_stride;
-  uint64_t *out = Out + blockIdx.x * so + L0;
+  const int64_t inst = blockIdx.x / SKF_CLUSTER;
+  if (inst >= count) {  // the whole cluster
+    const int64_t nz = gridDim.x - count * SKF_CLUSTER, z = blockIdx.x - count * SKF_CLUSTER;
+    for (int64_t i = 4 * (z * SKF_THREADS + tid); i < zero; i += 4 * nz * SKF_THREADS)
+      *reinterpret_cast<int4 *>(zbuf + i) = make_int4(0, 0, 0, 0);
+    return;
+  }
+  const int rank = (int)(blockIdx.x % SKF_CLUSTER);
+  const int *cs = colsum + inst * cs_stride;
+  uint64_t *out = Out + inst * so + L0;
   const int n = nout - L0;
-  uint32_t hprev = 0, cprev = 0;
-  for (int base = 0; base < n; base += SKF_R * SKF_THREADS) {
+  uint32_t hprev = 0, cprev = 0;  // into the cluster's round
+  cl.sync();                      // every CTA of the cluster runs: its shared memory is there
+  for (int base = 0; base < n; base += SKF_CLUSTER * SKF_SPAN) {
+    const int b = base + rank * SKF_SPAN;
     uint64_t low[SKF_R];
     uint32_t high[SKF_R];
 #pragma unroll
     for (int r = 0; r < SKF_R; r++) {
-      const int j = base + r * SKF_THREADS + tid;
+      const int j = b + r * SKF_THREADS + tid;
       low[r] = 0;
       high[r] = 0;
       if (j < n) {
@@ -203,13 +221,16 @@ __global__ void __launch_bounds__(SKF_THREADS)
       }
       if (lane == 31) s_hi[r * W + warp] = high[r];
     }
-    __syncthreads();
+    if (tid == SKF_THREADS - 1)
+      for (int i = 0; i < SKF_CLUSTER; i++) *cl.map_shared_rank(&c_hi[rank], i) = high[SKF_R - 1];
+    cl.sync();
+    const uint32_t hin = rank > 0 ? c_hi[rank - 1] : hprev;
     WarpCarry wc[SKF_R];
 #pragma unroll
     for (int r = 0; r < SKF_R; r++) {
-      const int j = base + r * SKF_THREADS + tid;
+      const int j = b + r * SKF_THREADS + tid;
       uint32_t below = __shfl_up_sync(FULL, high[r], 1);
-      if (lane == 0) below = r * W + warp > 0 ? s_hi[r * W + warp - 1] : hprev;
+      if (lane == 0) below = r * W + warp > 0 ? s_hi[r * W + warp - 1] : hin;
       uint32_t g = 0, p = 1;
       if (j < n) {
         const uint64_t add = j == 0 ? margin : (uint64_t)below;
@@ -223,22 +244,40 @@ __global__ void __launch_bounds__(SKF_THREADS)
         s_p[r * W + warp] = warp_all_propagate(wc[r]);
       }
     }
-    hprev = s_hi[SKF_R * W - 1];
+    hprev = c_hi[SKF_CLUSTER - 1];
     __syncthreads();
+    WarpCarry bc[SKF_R];  // the CTA's warps, round by round
+    uint32_t bg = 0, bp = 1;
 #pragma unroll
     for (int r = 0; r < SKF_R; r++) {
-      const int j = base + r * SKF_THREADS + tid;
-      const uint64_t cm = warp_carries(warp_gp(s_g[r * W + lane], s_p[r * W + lane]), cprev);
-      const uint64_t lc = warp_carries(wc[r], (uint32_t)(cm >> warp) & 1u);
-      if (j < n) out[j] = low[r] + ((lc >> lane) & 1u);
-      cprev = (uint32_t)(cm >> 32);
+      bc[r] = warp_gp(s_g[r * W + lane], s_p[r * W + lane]);
+      bg = warp_carry_out(bc[r], 0) | (warp_all_propagate(bc[r]) & bg);
+      bp &= warp_all_propagate(bc[r]);
     }
-    __syncthreads();  // the shared arrays are rewritten
+    if (tid < SKF_CLUSTER) {
+      *cl.map_shared_rank(&c_g[rank], tid) = bg;
+      *cl.map_shared_rank(&c_p[rank], tid) = bp;
+    }
+    cl.sync();
+    uint32_t c = cprev;  // carry into this CTA's span, then through the cluster
+#pragma unroll
+    for (int i = 0; i < SKF_CLUSTER; i++) {
+      if (i == rank) {
+        uint32_t cc = c;
+#pragma unroll
+        for (int r = 0; r < SKF_R; r++) {
+          const int j = b + r * SKF_THREADS + tid;
+          const uint64_t cm = warp_carries(bc[r], cc);
+          const uint64_t lc = warp_carries(wc[r], (uint32_t)(cm >> warp) & 1u);
+          if (j < n) out[j] = low[r] + ((lc >> lane) & 1u);
+          cc = (uint32_t)(cm >> 32);
+        }
+      }
+      c = c_g[i] | (c_p[i] & c);
+    }
+    cprev = c;
+    cl.sync();  // the exchange words are rewritten, or the CTA leaves
   }
-  // the sums back to zero for the chain's next product (zero ints, a multiple
-  // of 4; everything was read before the last barrier)
-  for (int i = 4 * tid; i < zero; i += 4 * SKF_THREADS)
-    *reinterpret_cast<int4 *>(cs + i) = make_int4(0, 0, 0, 0);
 }
 
 // One CTA per product: tile t (limbs [t L, t L + L), L = tile_limbs) was
@@ -908,11 +947,12 @@ bool mul_sk_worth(int64_t count, int na, int nb, int nout, int lo) {
 // The low nout limbs (from limb lo: band mode, as tc_product) of a batch of
 // products, each cut into units of (tile, groups) spread over the SMs; the
 // units add their column sums into `colsum` (count x
-// mul_sk_bytes_per_product bytes, zeroed here, or with `zeroed` found and left
-// all zero: 16-byte aligned then), then one CTA per product forms the limbs.  Results are those of tc_product (bit-identical).
+// mul_sk_bytes_per_product bytes), zeroed here or, in a chain of products,
+// by the finish of the product before, then a cluster per product forms the
+// limbs.  Results are those of tc_product (bit-identical).
 int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, void *colsum,
-                     size_t colsum_bytes, int *abort_flag, cudaStream_t st, bool zeroed) {
+                     size_t colsum_bytes, SkBuffers *chain, int *abort_flag, cudaStream_t st) {
   const uint64_t *x = a, *y = b;
   int64_t sx = sa, sy = sb;
   int nx = na, ny = nb;
@@ -945,7 +985,16 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   P.first[0] = 0;
   for (int t = 0; t < P.T; t++) P.first[t + 1] = P.first[t] + (int)((groups[t] + gpc - 1) / gpc);
   const int64_t units = count * P.first[P.T];
-  if (!zeroed) BIGINT_CUDA_TRY(cudaMemsetAsync(colsum, 0, per * (size_t)count, st));
+  int *zbuf = nullptr;
+  int64_t zero = 0;
+  if (chain != nullptr) {
+    zbuf = static_cast<int *>(chain->buf[chain->cur ^ 1]);
+    zero = (int64_t)(chain->used / sizeof(int));
+    chain->used = per * (size_t)count;
+    chain->cur ^= 1;
+  } else {
+    BIGINT_CUDA_TRY(cudaMemsetAsync(colsum, 0, per * (size_t)count, st));
+  }
   const int64_t stride = (int64_t)(per / sizeof(int));
   const unsigned grid = (unsigned)(units < sms ? units : sms);
   int rc = chain_launch(true, G == 8 ? tcm::k_mul_tc_sk<256, 8> : tcm::k_mul_tc_sk<256, 4>, grid,
@@ -953,9 +1002,14 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
                         static_cast<int *>(colsum), stride, abort_flag);
   if (rc != BIGINT_OK) return rc;
   const int L0 = 16 * P.cfirst;
-  return chain_launch(true, tcm::k_tc_sk_finish, (unsigned)count, tcm::SKF_THREADS, 0, st,
-                      static_cast<int *>(colsum), stride, out, so, L0, nout,
-                      lo > 0 ? (1ull << 32) : 0ull, zeroed ? (int)stride : 0);
+  // clearing CTAs: 16 KB each
+  int64_t clear = (zero + 4095) / 4096;
+  if (clear > 64) clear = 64;
+  clear = (clear + tcm::SKF_CLUSTER - 1) / tcm::SKF_CLUSTER * tcm::SKF_CLUSTER;
+  return chain_launch<tcm::SKF_CLUSTER>(
+      true, tcm::k_tc_sk_finish, (unsigned)(count * tcm::SKF_CLUSTER + clear), tcm::SKF_THREADS, 0,
+      st, static_cast<const int *>(colsum), stride, out, so, L0, nout,
+      lo > 0 ? (1ull << 32) : 0ull, count, zbuf, zero);
 }
 
 // ---- split products ----------------------------------------------------------
@@ -1047,7 +1101,7 @@ int launch_mul_split(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_
   // a few products: each cut into (tile, groups) units over the SMs
   if (count <= SPLIT_SK_MAX_COUNT && mul_sk_worth(count, na, nb, na + nb, 0))
     return launch_mul_tc_sk(a, na, b, nb, out, na + nb, count, na, nb, na + nb, 0, ws, bytes,
-                            nullptr, st, false);
+                            nullptr, nullptr, st);
   const uint64_t *x = a, *y = b;
   int nx = na, ny = nb;
   if (nb < na) { x = b; y = a; nx = nb; ny = na; }
