@@ -624,7 +624,10 @@ int rag_launch(const RagPlan &P, const RagBuffers &B, const uint64_t *in, uint64
           const tcm::PipeLayout L = pipe_layout_of(R.shape, R.nx);
           a.pipe<<<(unsigned)R.grid, a.threads, L.total, st>>>(A, L);
         } else {
-          a.kern<<<(unsigned)R.grid, a.threads, R.smem, st>>>(A);
+          // no more CTAs on an SM than its tensor memory serves (one too many
+          // would queue for it through all of another's products)
+          const uint32_t least = (uint32_t)(shapes().smem_sm / (a.cap + 1) - a.overhead + 1);
+          a.kern<<<(unsigned)R.grid, a.threads, std::max(R.smem, least), st>>>(A);
         }
       }
     }

@@ -601,6 +601,17 @@ static int one_per_sm(size_t smem) {
   return per_sm > 512 / NT ? 512 / NT : (per_sm < 1 ? 1 : per_sm);
 }
 
+// At least so much shared memory that no SM takes more CTAs than its tensor
+// memory serves: one too many queues for it through all of another CTA's
+// products (65536 products of 64 limbs 390 us, 440 to 590 with five CTAs on
+// some SMs).
+template <int NT>
+static size_t one_smem_floor(size_t smem) {
+  const OneAttr &a = one_attr<NT>();
+  const size_t least = (size_t)(a.smem_sm / (512 / NT + 1) - a.overhead + 1);
+  return smem > least ? smem : least;
+}
+
 // Shared memory of a product (x of nx, y of ny limbs, low nout limbs, band
 // start lo) in the form with NT-column tiles (0: it does not take it), and
 // its modelled time on one SM in tensor-core cycles, comparable with
@@ -636,13 +647,14 @@ static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
 template <int NT>
 static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
   constexpr int W = one_warps<NT>();
-  const size_t smem = one_plan<NT>(nx, ny, nout, A.lo, nullptr);
+  size_t smem = one_plan<NT>(nx, ny, nout, A.lo, nullptr);
   if (smem == 0) return BIGINT_EINVAL;
   if (count == 0) return BIGINT_OK;
   const int sms = sm_count();
   if (sms == 0) return BIGINT_ECUDA;
   const int64_t slots = (int64_t)sms * one_per_sm<NT>(smem);
   const int64_t grid = count < slots ? count : slots;
+  smem = one_smem_floor<NT>(smem);
   auto *kern = A.add != nullptr ? tcm::k_mul_one<NT, W, true> : tcm::k_mul_one<NT, W, false>;
   if (A.add != nullptr && !one_attr<NT, true>().ok) return BIGINT_ECUDA;
   return chain_launch(grid <= sms, kern, (unsigned)grid, 32 * W, smem, st, A.x, A.y, A.out, nx, ny, nout, count,
