@@ -696,7 +696,7 @@ static int launch_pipe(const TcArgs &A, int64_t count, int nx, int ny, int nout,
 
 // Modelled time of a product in the pipelined form (-1: x does not fit): its
 // MMAs, at least 42 cycles each (warp-uniform issue), 10 % slower beside the
-// drains and builds, 900 cycles a drain and 9000 (3000 with 128-column tiles)
+// drains and builds, 900 cycles a drain and 9000 (5000 with 128-column tiles)
 // a tile, the part of its limbs that the groups ahead do not cover.  128-
 // column tiles for products of one such tile only.
 template <int KB, int NT>
@@ -710,7 +710,7 @@ static double pipe_cost(int nx, int ny, int nout, int lo) {
   int tiles = 0;
   tcm::pipe_tiles<KB, NT>(nx, ny, nout, lo, [&](int c0, int W, int e_lo, int e_hi) {
     tiles++;
-    cyc += NT == 256 ? 9000 : 3000;
+    cyc += NT == 256 ? 9000 : 5000;
     if (e_hi < e_lo) return true;
     const int n = e_hi - e_lo + 1, st = sample_step(n);
     cyc += 900.0 * ((n * KB + 1023) / 1024);
@@ -726,9 +726,15 @@ static double pipe_cost(int nx, int ny, int nout, int lo) {
   return NT == 256 || tiles <= 1 ? cyc : -1;
 }
 
+// The pipeline with 32-digit blocks, for uniform batches only: a grouped
+// launch per form more costs a step of a ragged batch more than it saves
+// (20000 mixed operations 17.4 -> 17.8 ms).
+constexpr int FORM_PIPE32 = RAG_NSHAPES;
+
 // The one-drain (RAG_ONE...) or pipelined (RAG_PIPE...) form, either operand as x (*swap), where its model is cheaper
 // than `than` (< 0: anything); -1 where none is.
-static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap) {
+static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap,
+                     bool grouped = false) {
   int form = -1;
   auto offer = [&](double c, int f, int k) {
     if (c >= 0 && (than < 0 || c < than)) than = c, form = f, *swap = k != 0;
@@ -742,6 +748,7 @@ static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap) 
     offer(pipe_cost<64, 256>(mx, my, nout, lo), RAG_PIPE64, k);
     offer(pipe_cost<128, 128>(mx, my, nout, lo), RAG_PIPE128N, k);
     offer(pipe_cost<64, 128>(mx, my, nout, lo), RAG_PIPE64N, k);
+    if (!grouped) offer(pipe_cost<32, 256>(mx, my, nout, lo), FORM_PIPE32, k);
   }
   return form;
 }
@@ -760,7 +767,8 @@ static int launch_form(int form, TcArgs A, bool sw, int64_t count, int nx, int n
     case RAG_PIPE128: return launch_pipe<128, 256>(A, count, nx, ny, nout, st);
     case RAG_PIPE64: return launch_pipe<64, 256>(A, count, nx, ny, nout, st);
     case RAG_PIPE128N: return launch_pipe<128, 128>(A, count, nx, ny, nout, st);
-    default: return launch_pipe<64, 128>(A, count, nx, ny, nout, st);
+    case RAG_PIPE64N: return launch_pipe<64, 128>(A, count, nx, ny, nout, st);
+    default: return launch_pipe<32, 256>(A, count, nx, ny, nout, st);
   }
 }
 
@@ -795,7 +803,7 @@ int tc_choose(int nx, int ny, int nout, int lo, bool *swap) {
     }
   }
   bool sw = false;
-  const int form = best_form(nx, ny, nout, lo, best, &sw);
+  const int form = best_form(nx, ny, nout, lo, best, &sw, true);
   if (form < 0) return sh;
   *swap = sw;
   return form;

@@ -31,8 +31,9 @@
 // and the ~20K cycles between products were not covered: 122K cycles for a
 // 2048-limb product whose MMAs take 74K.
 //
-// KB digits per x block: 128 (S = 1 row per coefficient) or 64 (S = 2, MMAs
-// twice as wide: operands below 2048 limbs).  KB * HS * GS = 1024 digit
+// KB digits per x block: 128 (S = 1 row per coefficient), 64 (S = 2, MMAs
+// twice as wide: operands below 2048 limbs) or 32 (S = 4, again twice: low and
+// banded products of a few hundred columns).  KB * HS * GS = 1024 digit
 // products per accumulated sum: exact (tccore.cuh).  x goes without its carry
 // digit; where its top bit is set, limb j of the result takes limb j - nx of
 // y more as its coefficients are summed.  Limbs, bias and the single carry
@@ -45,7 +46,7 @@ namespace tcm {
 
 constexpr int PIPE_HS = 8, PIPE_BUILD = 3, PIPE_DRAIN = 512;
 constexpr int PIPE_THREADS = PIPE_DRAIN + 32 + 32 * PIPE_BUILD;  // 20 warps: 96 registers
-constexpr int PIPE_EX = 264;    // limbs per row of the S = 2 exchange (16 banks from row to row)
+constexpr int PIPE_EX = 264;    // limbs per row of the S > 1 exchange (16 banks from row to row)
 constexpr int PIPE_STAGES = 3;  // at most
 
 template <int KB>
@@ -56,6 +57,10 @@ struct PipeLayout {
   uint32_t xs, xbytes, z, hk, hbytes, ex, total;
   int xbufs, stages;
 };
+
+// Rows of the exchange (limbs of a column times the row parts it collects).
+template <int KB>
+__host__ __device__ constexpr int pipe_ex_rows() { return KB == 128 ? 0 : (KB == 64 ? 8 : 12); }
 
 template <int KB>
 __host__ __device__ inline int pipe_ptot(int nx) {
@@ -69,7 +74,7 @@ __host__ inline PipeLayout pipe_layout(int nx, uint32_t cap) {
   constexpr int R = KB / 8;
   L.xbytes = ((uint32_t)pipe_ptot<KB>(nx) * 16u * R + 127) / 128 * 128;
   L.hbytes = (uint32_t)pipe_matrices<KB>() * ONE_CM;
-  const uint32_t fixed = ZB * 128 + (KB == 64 ? 8 * PIPE_EX * 12 : 0);
+  const uint32_t fixed = ZB * 128 + pipe_ex_rows<KB>() * PIPE_EX * 12;
   for (L.xbufs = 2; L.xbufs >= 1; L.xbufs--)
     for (L.stages = PIPE_STAGES; L.stages >= 2; L.stages--) {
       const uint32_t t = fixed + L.xbufs * L.xbytes + L.stages * L.hbytes;
@@ -156,7 +161,7 @@ __device__ __forceinline__ bool pipe_wait_warp(PipeShared *sh, uint64_t *bar, ui
 // x into the B layout (fill_x without the carry digit), by the builders.
 template <int KB>
 __device__ __forceinline__ void pipe_fill(uint8_t *xs, const uint64_t *x, int nx, int t) {
-  constexpr int U = 4, R = KB / 8, LR = KB == 128 ? 4 : 3, STEP = 32 * PIPE_BUILD;
+  constexpr int U = 4, R = KB / 8, LR = KB == 128 ? 4 : (KB == 64 ? 3 : 2), STEP = 32 * PIPE_BUILD;
   const int ptot = pipe_ptot<KB>(nx), total = R * ptot;
   for (int i0 = t; i0 < total; i0 += U * STEP) {
     uint64_t v[U], below[U];
@@ -384,19 +389,23 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
                                            uint32_t tmem, long long lim, Next next, Done done) {
   constexpr int HS = PIPE_HS, S = 128 / KB, R = KB / 8, GS = 1024 / (KB * HS);
   constexpr int NACC = 512 / NT, CW = NT / 4, CM = CW / 8;  // columns and limbs per lane
-  constexpr int QTOP = S == 1 ? 0 : 2;  // warps of the lane quadrants 3 .. QTOP hold the limbs
+  constexpr int QTOP = S == 1 ? 0 : (S == 2 ? 2 : 3);  // lane quadrants 3 .. QTOP hold the limbs
   // added to a limb's signed high word to make it unsigned, and taken off the
   // next limb: |V_j| < 2^31 sum_k 2^(8 k), so the high word is at least -C
   constexpr uint32_t C = 0x808080u;
-  static_assert(S <= 2, "one or two rows per coefficient");
+  static_assert(S <= 4, "one, two or four rows per coefficient");
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int q = warp & 3, cq = warp >> 2;  // TMEM lane quadrant, CW-column slice
   const uint32_t t_lane = tmem + ((uint32_t)(32 * q) << 16);
   const bool holds = q >= QTOP;
   const int jj = 4 * (3 - q) + 3 - (lane >> 3);  // limb of this lane within a column (holds)
-  // S = 2: the upper rows' limbs, at the column they belong to
+  // S > 1: rows 128 / S and up are parts of limbs of later columns, exchanged
+  // at the column they belong to: quadrant q's go `ahead` columns on, to the
+  // holder with the same limbs, in exchange row xrow (limb, and part for S = 4)
   uint64_t *Xl = reinterpret_cast<uint64_t *>(sm + L.ex);
-  int *Xh = reinterpret_cast<int *>(sm + L.ex + 8 * 8 * PIPE_EX);
+  int *Xh = reinterpret_cast<int *>(sm + L.ex + 8 * pipe_ex_rows<KB>() * PIPE_EX);
+  const int ahead = S == 2 ? 1 : 3 - q;
+  const int xrow = 3 - (lane >> 3) + 4 * (S == 2 ? 3 - (q | 2) : 2 - q);
   uint32_t grp = 0;
   int gen = 0;
   PipeTask T;
@@ -406,9 +415,10 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
     const bool tx = (T.x[T.nx - 1] >> 63) != 0;
     uint32_t hprev = 0, cprev = 0;  // high word and carry into the tile
     const uint64_t margin = T.lo > 0 ? 1ull << 32 : 0ull;
-    if (S > 1 && tid < 8) {  // nothing before the first column
-      Xl[tid * PIPE_EX + 256 + gen] = 0ull;
-      Xh[tid * PIPE_EX + 256 + gen] = 0;
+    if (S > 1 && tid < 4 * pipe_ex_rows<KB>()) {  // nothing before the first column
+      const int at = (tid >> 2) * PIPE_EX + 256 + 4 * gen + (tid & 3);
+      Xl[at] = 0ull;
+      Xh[at] = 0;
     }
     const bool ok = pipe_tiles<KB, NT>(T.nx, T.ny, T.nout, T.lo, [&](int c0, int W, int e_lo,
                                                                 int e_hi) {
@@ -437,14 +447,12 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
       int high[CM];
       pipe_limbs<CW>(acc, low, high);
       if (S > 1) {
-        // rows 64 .. 127 of column c belong to column c + 1; those of the
-        // tile's last column wait for the next tile
-        const int row = 4 * (3 - (q | 2)) + 3 - (lane >> 3);
+        // parts beyond the tile's last column wait for the next tile
         if (!holds) {
 #pragma unroll
           for (int m = 0; m < CM; m++) {
-            const int c = cb + 8 * m;
-            const int at = row * PIPE_EX + (c < NT - 1 ? c + 1 : 256 + (gen ^ 1));
+            const int c = cb + 8 * m + ahead;
+            const int at = xrow * PIPE_EX + (c < NT ? c : 256 + 4 * (gen ^ 1) + c - NT);
             Xl[at] = low[m];
             Xh[at] = high[m];
           }
@@ -453,10 +461,15 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
         if (holds) {
 #pragma unroll
           for (int m = 0; m < CM; m++) {
-            const int c = cb + 8 * m, at = row * PIPE_EX + (c > 0 ? c : 256 + gen);
-            const uint64_t l = Xl[at];
-            low[m] += l;
-            high[m] += Xh[at] + (int)(low[m] < l);
+#pragma unroll
+            for (int a = 1; a < S; a++) {
+              const int c = cb + 8 * m;
+              const int row = S == 2 ? xrow : 3 - (lane >> 3) + 4 * (a - 1);
+              const int at = row * PIPE_EX + (c >= a ? c : 256 + 4 * gen + c);
+              const uint64_t l = Xl[at];
+              low[m] += l;
+              high[m] += Xh[at] + (int)(low[m] < l);
+            }
           }
         }
         gen ^= 1;
