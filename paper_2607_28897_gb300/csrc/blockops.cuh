@@ -247,59 +247,101 @@ __device__ __forceinline__ void warp_addsub(int n, uint32_t cin, Load load, Stor
   }
 }
 
-// out[0..nout) = low nout limbs of x y (x, y, out in shared memory, cs
-// room for nout columns of 3 words), by one warp: each lane forms whole
-// columns of the schoolbook product (column j = sum_i x_i y_(j-i), 128-bit
-// limb products summed into lo + hi B + top B^2, two partial sums in
-// flight), then the columns' words are added as three shifted numbers --
-// lo, hi one limb up, top two limbs up -- with the warp carry scan.
-__device__ __forceinline__ void warp_mul(const uint64_t *x, int nx, const uint64_t *y, int ny,
-                                         uint64_t *out, int nout, uint64_t *cs) {
-  const int lane = (int)lane_id();
-  for (int j = lane; j < nout; j += 32) {
-    uint64_t lo0 = 0, hi0 = 0, top0 = 0, lo1 = 0, hi1 = 0, top1 = 0;
-    const int i0 = j - ny + 1 > 0 ? j - ny + 1 : 0, i1 = j < nx - 1 ? j : nx - 1;
-    int i = i0;
-    for (; i + 1 <= i1; i += 2) {
-      const uint64_t p0 = x[i], q0 = y[j - i], p1 = x[i + 1], q1 = y[j - i - 1];
-      const uint64_t l0 = p0 * q0, h0 = __umul64hi(p0, q0);
-      const uint64_t l1 = p1 * q1, h1 = __umul64hi(p1, q1);
-      lo0 += l0;
-      const uint64_t u0 = h0 + (lo0 < l0);  // h <= 2^64 - 2: no overflow
-      hi0 += u0;
-      top0 += hi0 < u0;
-      lo1 += l1;
-      const uint64_t u1 = h1 + (lo1 < l1);
-      hi1 += u1;
-      top1 += hi1 < u1;
-    }
-    if (i <= i1) {
-      const uint64_t p = x[i], q = y[j - i];
-      const uint64_t l = p * q, h = __umul64hi(p, q);
-      lo0 += l;
-      const uint64_t u = h + (lo0 < l);
-      hi0 += u;
-      top0 += hi0 < u;
-    }
-    lo0 += lo1;
-    const uint64_t u = hi1 + (lo0 < lo1);
-    const uint64_t carry_u = u < hi1;  // hi1 + 1 overflowed
-    hi0 += u;
-    top0 += top1 + carry_u + (hi0 < u);
-    cs[3 * j] = lo0;
-    cs[3 * j + 1] = hi0;
-    cs[3 * j + 2] = top0;
+// Sum of 64 x 64-bit products, one of the limb columns of a product: the
+// 32-bit partial products of even weight in e, the two of odd weight in a
+// and b, each with its own carry word, so that a product is four 32-bit
+// multiply-adds with 64-bit results and three carry additions in three
+// independent chains (in 64-bit arithmetic, the low and high words
+// formed and compared apart, it was some 30 instructions).
+struct ColSum {
+  uint32_t e[5] = {0, 0, 0, 0, 0}, a[3] = {0, 0, 0}, b[3] = {0, 0, 0};
+  __device__ __forceinline__ void mac(uint64_t x, uint64_t y) {
+    const uint32_t x0 = (uint32_t)x, x1 = (uint32_t)(x >> 32);
+    const uint32_t y0 = (uint32_t)y, y1 = (uint32_t)(y >> 32);
+    asm("mad.lo.cc.u32 %0, %5, %7, %0;\n\t"
+        "madc.hi.cc.u32 %1, %5, %7, %1;\n\t"
+        "madc.lo.cc.u32 %2, %6, %8, %2;\n\t"
+        "madc.hi.cc.u32 %3, %6, %8, %3;\n\t"
+        "addc.u32 %4, %4, 0;\n\t"
+        : "+r"(e[0]), "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4])
+        : "r"(x0), "r"(x1), "r"(y0), "r"(y1));
+    odd(a, x0, y1);
+    odd(b, x1, y0);
   }
-  __syncwarp();
-  // lo + hi B (each column's hi one limb up), into the lo words
-  warp_addsub<false>(nout, 0u,
-                     [&](int j) { return make_ulonglong2(cs[3 * j], j >= 1 ? cs[3 * j - 2] : 0ull); },
-                     [&](int j, uint64_t v) { cs[3 * j] = v; });
-  __syncwarp();
-  // + top B^2
-  warp_addsub<false>(nout, 0u,
-                     [&](int j) { return make_ulonglong2(cs[3 * j], j >= 2 ? cs[3 * j - 4] : 0ull); },
-                     [&](int j, uint64_t v) { out[j] = v; });
+  // The sum: low and high 64 bits and what lies above them.
+  __device__ __forceinline__ void get(uint64_t &lo, uint64_t &hi, uint32_t &top) {
+    asm("add.cc.u32 %0, %0, %3;\n\t"
+        "addc.cc.u32 %1, %1, %4;\n\t"
+        "addc.u32 %2, %2, %5;\n\t"
+        : "+r"(a[0]), "+r"(a[1]), "+r"(a[2])
+        : "r"(b[0]), "r"(b[1]), "r"(b[2]));
+    asm("add.cc.u32 %0, %0, %4;\n\t"
+        "addc.cc.u32 %1, %1, %5;\n\t"
+        "addc.cc.u32 %2, %2, %6;\n\t"
+        "addc.u32 %3, %3, 0;\n\t"
+        : "+r"(e[1]), "+r"(e[2]), "+r"(e[3]), "+r"(e[4])
+        : "r"(a[0]), "r"(a[1]), "r"(a[2]));
+    lo = (uint64_t)e[1] << 32 | e[0];
+    hi = (uint64_t)e[3] << 32 | e[2];
+    top = e[4];
+  }
+
+ private:
+  static __device__ __forceinline__ void odd(uint32_t (&v)[3], uint32_t x, uint32_t y) {
+    asm("mad.lo.cc.u32 %0, %3, %4, %0;\n\t"
+        "madc.hi.cc.u32 %1, %3, %4, %1;\n\t"
+        "addc.u32 %2, %2, 0;\n\t"
+        : "+r"(v[0]), "+r"(v[1]), "+r"(v[2])
+        : "r"(x), "r"(y));
+  }
+};
+
+// out[lo..nout) = limbs of x y (x, y, out in shared memory; fewer than 2^31
+// products a column), by one warp: each lane forms whole columns of the
+// schoolbook product (column j = sum_i x_i y_(j-i)), 32 of them a round, then
+// limb j is the low word of column j plus the high word of column j - 1 plus
+// the top of column j - 2, which one carry scan a round settles.  lo > 0:
+// the columns below lo - 1 are left out, which is less than 2^31 units of
+// limb lo, and 2^32 are added there, so that the limbs above it are exact or
+// one unit high.
+__device__ __forceinline__ void warp_mul(const uint64_t *x, int nx, const uint64_t *y, int ny,
+                                         uint64_t *out, int nout, int lo = 0) {
+  const int lane = (int)lane_id();
+  uint64_t hi_r = 0;                     // on lane 0 (top: 0 and 1): of the round before
+  uint32_t top_r = 0, c_r = 0, cin = 0;
+  for (int base = lo > 0 ? lo - 1 : 0; base < nout; base += 32) {
+    const int j = base + lane;
+    ColSum s;
+    if (j < nout) {
+      const int i0 = j - ny + 1 > 0 ? j - ny + 1 : 0, i1 = j < nx - 1 ? j : nx - 1;
+      const uint64_t *xp = x + i0, *yp = y + (j - i0);
+      const int n = i1 - i0 + 1;
+#pragma unroll 4
+      for (int i = 0; i < n; i++) s.mac(xp[i], yp[-i]);
+    }
+    __syncwarp();
+    uint64_t low, high;
+    uint32_t top;
+    s.get(low, high, top);
+    const uint64_t hs = __shfl_sync(FULL, high, (lane + 31) & 31);
+    const uint32_t ts = __shfl_sync(FULL, top, (lane + 30) & 31);
+    const uint64_t hb = lane == 0 ? hi_r : hs;
+    uint64_t tb = lane < 2 ? top_r : ts;
+    hi_r = hs;
+    top_r = ts;
+    if (lo > 0 && j == lo) tb += 1ull << 32;
+    low += hb;
+    uint32_t c = low < hb;
+    low += tb;
+    c += low < tb;
+    const uint32_t cs = __shfl_sync(FULL, c, (lane + 31) & 31);
+    const uint32_t cb = lane == 0 ? c_r : cs;
+    c_r = cs;
+    low += cb;  // at most 2: a limb that overflows is not all ones after it
+    const uint64_t cm = warp_carries(warp_gp(low < cb, low == ~0ull), cin);
+    if (j >= lo && j < nout) out[j] = low + ((cm >> lane) & 1u);
+    cin = (uint32_t)(cm >> 32) & 1u;
+  }
   __syncwarp();
 }
 

@@ -100,10 +100,9 @@ constexpr int WARP_CTA = 256;  // warp-per-instance kernels: 8 instances per CTA
 // The early Newton steps, while every operand of a step has at most
 // SMALL_STEP_LIMBS limbs, in one launch with one warp per instance: each
 // such step is four small launches otherwise (P, |d|, P2, update), whose
-// fixed costs are most of their time.  Per step the warp keeps w, vt, P /
-// |d| and P2 in shared memory and runs the same arithmetic as the batched
-// kernels, except that P2 = w |d| is computed whole (so floor(P2 / B^s) is
-// exact, which the step allows).
+// fixed costs are most of their time.  The warp keeps w, the divisor's top
+// limbs, P / |d| and P2 in shared memory and runs the same arithmetic as the
+// batched kernels (warp_mul's band makes floor(P2 / B^s) exact or one high).
 // ---------------------------------------------------------------------------
 constexpr int SMALL_STEP_MAX = 16;
 
@@ -128,14 +127,15 @@ __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS)
   if (i >= count) return;  // the whole warp: no block barrier below
   const int N = S.N;
   uint64_t *base = ssm + (size_t)wi * small_step_warp_limbs(N);
-  uint64_t *wb[2] = {base, base + N}, *vts = base + 2 * N, *d = base + 3 * N;
-  uint64_t *z = base + 4 * N, *cs = base + 6 * N;
-  const uint64_t *v = V + i * nv;
-  const int k = nv - 1;
+  uint64_t *wb[2] = {base, base + N}, *vt = base + 2 * N, *d = base + 3 * N, *z = base + 4 * N;
+  const int t = S.s[S.n - 1].t;  // the largest
+  const uint64_t *v = V + i * nv + (nv - 1 - t);
+  for (int j = lane; j <= t; j += 32) vt[j] = v[j];
   for (int j = lane; j < S.s[0].l + 2; j += 32) wb[0][j] = W0[i * sw + j];
+  __syncwarp();
   int cur = 0;
   for (int st = 0; st < S.n; st++) {
-    ds_small_step(v, k, S.s[st], wb[cur], wb[cur ^ 1], vts, d, z, cs);
+    ds_small_step(vt + (t - S.s[st].t), S.s[st], wb[cur], wb[cur ^ 1], d, z);
     cur ^= 1;
   }
   const int nlast = S.s[S.n - 1].l + S.s[S.n - 1].m + 2;
@@ -349,7 +349,7 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     const Step &S0 = steps[SS.n];
     // every operand and result of the step within N limbs (w' too)
     const int need = std::max(std::max(S0.l + 2, S0.t + 2), S0.l + S0.m + 2);
-    if (need > SMALL_STEP_LIMBS) break;
+    if (need > (few ? SMALL_STEP_LIMBS_FEW : SMALL_STEP_LIMBS)) break;
     SS.N = std::max(SS.N, (need + 7) / 8 * 8);
     SS.s[SS.n++] = S0;
   }

@@ -18,13 +18,13 @@ using namespace divc;
 constexpr int LIN_THREADS = 256, LIN_THREADS_FEW = 1024;
 
 // Fused leading steps: operands of at most SMALL_STEP_LIMBS limbs, i.e. up to
-// 34 known limbs.  (With the step from 66 in the warp too -- 136 limbs -- it
-// took 231 us for 4096 instances; batched on the tensor cores that step is
-// three launches more and 60 us less.)  A warp's
+// 66 known limbs, in a batch of few instances SMALL_STEP_LIMBS_FEW, i.e. 34
+// (a lone warp's serial products then cost more than the four launches of
+// the step).  A warp's
 // shared memory holds, for steps of at most N limbs, two iterates (N each),
-// vt and |d| (N each), P2 (2 N) and the column sums (2 N x 3 words).
-constexpr int SMALL_STEP_LIMBS = 72, SMALL_STEP_WARPS = 4;
-__host__ __device__ constexpr int small_step_warp_limbs(int N) { return 2 * N + 2 * N + 2 * N + 6 * N; }
+// the divisor's top limbs and |d| (N each) and P2 (2 N).
+constexpr int SMALL_STEP_LIMBS = 136, SMALL_STEP_LIMBS_FEW = 72, SMALL_STEP_WARPS = 4;
+__host__ __device__ constexpr int small_step_warp_limbs(int N) { return 6 * N; }
 
 // One Newton step of an instance: l limbs of the inverse known, m new ones,
 // the divisor truncated to its top t + 1 limbs.
@@ -56,25 +56,22 @@ __device__ void ds_start_one(const uint64_t *v, int nv, int l, uint64_t *w) {
 }
 
 // One warp: the step S on the iterate w (l + 2 limbs) into wn (l + m + 2),
-// everything in shared memory (vts, d: N limbs, z: 2 N, cs: 6 N); v in
-// global memory.
-__device__ __forceinline__ void ds_small_step(const uint64_t *v, int k, Step S, const uint64_t *w,
-                                              uint64_t *wn, uint64_t *vts, uint64_t *d,
-                                              uint64_t *z, uint64_t *cs) {
-  const int lane = (int)lane_id(), l = S.l, m = S.m, t = S.t, nw = l + 2, nl = t + 2;
-  for (int j = lane; j <= t; j += 32) vts[j] = v[k - t + j];
-  __syncwarp();
+// everything in shared memory (vt: the divisor's top t + 1 limbs, d: N limbs,
+// z: 2 N).
+__device__ __forceinline__ void ds_small_step(const uint64_t *vt, Step S, const uint64_t *w,
+                                              uint64_t *wn, uint64_t *d, uint64_t *z) {
+  const int l = S.l, m = S.m, t = S.t, nw = l + 2, nl = t + 2;
   // P = vt w mod B^(t+2); |d| = P (top bit clear: d <= 0) or B^(t+2) - P
-  warp_mul(vts, t + 1, w, nw, d, nl, cs);
+  warp_mul(vt, t + 1, w, nw, d, nl);
   const bool ng = (d[nl - 1] >> 63) == 0;
   if (!ng) {
     warp_addsub<true>(nl, 0u, [&](int j) { return make_ulonglong2(0ull, d[j]); },
                       [&](int j, uint64_t x) { d[j] = x; });
     __syncwarp();
   }
-  // P2 = w |d| (whole); w' = w B^m + floor(P2 / B^s) or w B^m - floor(P2 / B^s) - 1
-  warp_mul(w, nw, d, nl, z, nw + nl, cs);
+  // P2 = w |d| (band); w' = w B^m + floor(P2 / B^s) or w B^m - floor(P2 / B^s) - 1
   const int s = t + l - m, ny = nw + nl - s;
+  warp_mul(w, nw, d, nl, z, nw + nl, s - 2);
   auto load = [&](int j) {
     const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
     return make_ulonglong2(x, j < ny ? z[s + j] : 0ull);

@@ -33,7 +33,7 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS)
                 uint64_t *__restrict__ Out, int na, int nb, int nout, int64_t count, int64_t sa,
                 int64_t sb, int64_t so) {
   __shared__ uint64_t xs[SMALL_WARPS][SMALL_LIMBS], ys[SMALL_WARPS][SMALL_LIMBS];
-  __shared__ uint64_t os[SMALL_WARPS][2 * SMALL_LIMBS], cs[SMALL_WARPS][6 * SMALL_LIMBS];
+  __shared__ uint64_t os[SMALL_WARPS][2 * SMALL_LIMBS];
   const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int64_t inst = (int64_t)blockIdx.x * SMALL_WARPS + w;
   if (inst >= count) return;  // the whole warp: no block barrier below
@@ -41,7 +41,7 @@ __global__ void __launch_bounds__(32 * SMALL_WARPS)
   for (int i = lane; i < na; i += 32) xs[w][i] = a[i];
   for (int i = lane; i < nb; i += 32) ys[w][i] = b[i];
   __syncwarp();
-  warp_mul(xs[w], na, ys[w], nb, os[w], nout, cs[w]);
+  warp_mul(xs[w], na, ys[w], nb, os[w], nout);
   uint64_t *o = Out + inst * so;
   for (int j = lane; j < nout; j += 32) o[j] = os[w][j];
 }
@@ -191,7 +191,7 @@ int mul_variant_for(int na, int nb, int nout) {
   if (v == 0) v = g_mul_tuned[mul_size_class(na, nb)];
   if (v == 0) {
     const int nmax = na > nb ? na : nb, nmin = na < nb ? na : nb;
-    if (nmin >= TC_MIN_LIMBS && mul_tc_smem(na, nb) > 0)
+    if (nmin >= TC_MIN_LIMBS && nmax > SMALL_LIMBS && mul_tc_smem(na, nb) > 0)
       v = 12;
     else
       v = nmax <= SMALL_LIMBS ? 11 : (nmax < 1536 ? 9 : 8);

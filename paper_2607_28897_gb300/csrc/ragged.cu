@@ -42,7 +42,7 @@ constexpr size_t WAVE_BYTES = (size_t)1 << 30;
 
 // The steps up to this many known limbs run fused in one warp (every operand
 // then has at most SMALL_STEP_LIMBS limbs).
-constexpr int SMALL_L = 34;
+constexpr int SMALL_L = 66;
 
 struct RagArgs {
   const RagOp *ops;
@@ -154,17 +154,23 @@ __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS) k_rag_small(RagArgs A) 
   if (i >= A.n) return;  // the whole warp: no block barrier below
   const RagOp o = A.ops[i];
   uint64_t *base = ssm + (size_t)wi * small_step_warp_limbs(N);
-  uint64_t *wb[2] = {base, base + N}, *vts = base + 2 * N, *d = base + 3 * N;
-  uint64_t *z = base + 4 * N, *cs = base + 6 * N;
-  const uint64_t *v = A.in + o.v;
+  uint64_t *wb[2] = {base, base + N}, *vt = base + 2 * N, *d = base + 3 * N, *z = base + 4 * N;
   uint64_t *w = A.rec + o.rec;
   const int L = rag_L(o.nu, o.nv);
-  int l = L < 3 ? L : 3, cur = 0;
+  int l = L < 3 ? L : 3, cur = 0, t = 0;
   if (l == L) return;  // no steps: the start value stands
+  for (int ll = l; ll < L && ll <= SMALL_L;) {  // t of the last step: the largest
+    const Step S = newton_next(o.nv - 1, L, ll);
+    t = S.t;
+    ll += S.m;
+  }
+  const uint64_t *v = A.in + o.v + (o.nv - 1 - t);
+  for (int j = lane; j <= t; j += 32) vt[j] = v[j];
   for (int j = lane; j < l + 2; j += 32) wb[0][j] = w[j];
+  __syncwarp();
   while (l < L && l <= SMALL_L) {
     const Step S = newton_next(o.nv - 1, L, l);
-    ds_small_step(v, o.nv - 1, S, wb[cur], wb[cur ^ 1], vts, d, z, cs);
+    ds_small_step(vt + (t - S.t), S, wb[cur], wb[cur ^ 1], d, z);
     cur ^= 1;
     l += S.m;
   }
