@@ -153,12 +153,13 @@ int bigint_mul_kara(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t
  * workspace: device scratch of at least bigint_divmod_workspace(count, nu,
  * nv) bytes, 256-byte aligned, owned by the caller, contents clobbered.
  * 1 <= nu, nv <= BIGINT_MAX_LIMBS.
- * Schedule: with divisors of 128 limbs or more (and nu >= nv) every Newton
- * step runs for all instances at once -- each product one batched launch
- * of the multiply kernels, each linear step one small launch -- and only
- * instances whose divisor has a zero top limb are divided one CTA each at
- * the end; smaller divisions run one CTA per division (the paper's
- * intragroup form).  Results are the same either way.                     */
+ * Schedule: with divisors of 8 limbs or more (and nu >= nv) every Newton
+ * step runs for all instances at once -- the leading ones in one launch, then
+ * each product one batched launch of the multiply kernels, each linear step
+ * one small launch -- and only instances whose divisor has a zero top limb
+ * are divided one CTA each at the end.  Smaller divisions, and small batches
+ * with quotients of at most four limbs, run one CTA per division (the
+ * paper's intragroup form).  Results are the same either way.             */
 int bigint_divmod(const uint64_t *u, const uint64_t *v, uint64_t *q,
                   uint64_t *r, int32_t *status, int64_t count, int32_t nu,
                   int32_t nv, void *workspace, size_t workspace_bytes,
@@ -476,15 +477,16 @@ int bigint_host_sync(void);
  *   divisions (where a forced shape cannot take a product, the model's
  *   choice runs); variants 8-10 keep those on the integer pipes.
  * op 1 = division (divmod, shinv, divmod_inv):
- *   variant 0 (default): bigint_divmod on divisors of 128 limbs or more in
- *   the step-batched form (see bigint_divmod), everything else as variant 1
+ *   variant 0 (default): bigint_divmod on divisors of 8 limbs or more in
+ *   the step-batched form except small batches with short quotients (see
+ *   bigint_divmod), everything else as variant 1
  *   variant 1: one CTA per division; operands of 1536 limbs and more run in
  *   a kernel that holds its SM's tensor memory and computes products whose
  *   shorter operand has at least 256 limbs on the tensor cores (as variant
  *   12 of the multiply); smaller divisions use the integer products
  *   variant 2: one CTA per division, integer products (blk_mul) only
- *   variant 3: as 0, with the step-batched form for divisors of 8 limbs
- *   and more
+ *   variant 3: as 0, with the step-batched form for every divisor of 8
+ *   limbs and more
  * op 2 = ragged batches (bigint_batch_*, for batches created afterwards):
  *   variant 0 (default) or 1: a batch with multiplications or divisions
  *   whose products have a shorter operand of 256 limbs or more runs them in

@@ -160,9 +160,9 @@ __global__ void __launch_bounds__(div_max_threads<Q, TC>())
 // Division kernels for H >= DIV_SMALL_LIMBS run their large products on the
 // tensor cores unless switched off (bigint_set_variant(1, ...)).
 static int g_div_tc = 1;
-// Uniform divisions: the step-batched form (divstep.cu) for divisors of
-// DIV_STEP_MIN limbs and more (0), never (1, 2: one CTA per division), or
-// for every divisor of 8 limbs and more (3).
+// Uniform divisions: the step-batched form (divstep.cu) where it is the
+// faster one (0, divmod_steps_default), never (1, 2: one CTA per division),
+// or for every divisor of 8 limbs and more (3).
 static int g_div_steps = 0;
 
 int div_set_variant(int v) {
@@ -264,14 +264,18 @@ static int launch_div_variant(const uint64_t *u, const uint64_t *v, uint64_t *q,
   const int hcap = mode == 1 ? h : nu;
   const int64_t stride = ws_limbs(nu, nv, hcap);
   int64_t grid = count;
-  if (x.list != nullptr) {  // a listed subset: a few CTAs per SM loop over it
+  if (x.list != nullptr) {  // a listed subset: as many CTAs as fit loop over it
     static int sms = 0;
     if (sms == 0) {
       int dev = 0;
       BIGINT_CUDA_TRY(cudaGetDevice(&dev));
       BIGINT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
     }
-    const int64_t slots = (int64_t)sms * (TC ? 1 : 2);
+    int per = 1;
+    if (!TC && grid > sms)
+      BIGINT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(
+          &per, k_divmod<RB, Q, F, TC>, T, (size_t)smem_words * 4));
+    const int64_t slots = (int64_t)sms * (per > 1 ? per : 1);
     if (grid > slots) grid = slots;
   }
   k_divmod<RB, Q, F, TC><<<(unsigned)grid, T, (size_t)smem_words * 4, st>>>(
@@ -295,7 +299,7 @@ static int launch_div_common(const uint64_t *u, const uint64_t *v, uint64_t *q, 
 }
 
 bool divmod_steps_ok(int64_t count, int nu, int nv, size_t ws_bytes);
-bool divmod_steps_default(int nu, int nv);
+bool divmod_steps_default(int64_t count, int nu, int nv);
 int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r,
                         int32_t *status, int64_t count, int nu, int nv, void *ws, size_t ws_bytes,
                         void *list_and_counters, void *sk, size_t sk_bytes, cudaStream_t st);
@@ -317,7 +321,8 @@ int launch_divmod(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r
                   int32_t *status, int64_t count, int nu, int nv, void *ws, size_t ws_bytes,
                   cudaStream_t st) {
   const size_t regions = cta_regions_bytes(count, nu, nv);
-  const bool steps = g_div_steps == 2 ? true : (g_div_steps == 0 && divmod_steps_default(nu, nv));
+  const bool steps =
+      g_div_steps == 2 ? true : (g_div_steps == 0 && divmod_steps_default(count, nu, nv));
   if (steps && ws_bytes >= divmod_workspace(count, nu, nv) &&
       divmod_steps_ok(count, nu, nv, regions)) {
     const size_t skb = divmod_sk_bytes(count, nu, nv);

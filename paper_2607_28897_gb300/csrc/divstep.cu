@@ -283,17 +283,26 @@ Layout layout(int64_t count, int nu, int nv) {
 
 }  // namespace dstep
 
-// Smallest divisor (limbs) for which a uniform batch takes the step-batched
-// form by default; smaller divisions stay in one CTA each.
-constexpr int DIV_STEP_MIN = 128;
-
 // True if divmod_steps can run this shape (with enough workspace).
 bool divmod_steps_ok(int64_t count, int nu, int nv, size_t ws_bytes) {
   if (count < 1 || nv < 8 || nu < nv) return false;
   return dstep::layout(count, nu, nv).total <= ws_bytes;
 }
 
-bool divmod_steps_default(int nu, int nv) { return nv >= DIV_STEP_MIN && nu >= nv; }
+// Whether a uniform batch takes the step-batched form by default: all but
+// few divisions with short quotients.  Up to four quotient limbs take one
+// Newton step at most, and a CTA's two short products then end before the
+// step form's eight launches (1 to 200 divisions of 67 by 64 limbs 32 us
+// against 40, of 515 by 512 limbs 38 against 46), unless the batch fills the SMs
+// (4096 of 66 by 64 limbs 94 against 58 us) or the divisor is long (one
+// division of 4099 by 4096 limbs 110 against 65 us).  With longer quotients
+// the step form is ahead from 8-limb divisors on: 16 by 8 limbs 47 : 37 us
+// for up to 200 divisions and 1187 : 164 us for 20000, 192 by 96 limbs
+// 142 : 66 us for 200 and 5093 : 714 us for 20000.
+bool divmod_steps_default(int64_t count, int nu, int nv) {
+  if (nv < 8 || nu < nv) return false;
+  return !(nu - nv + 1 <= 4 && nv <= 1024 && count <= 1024 && count * nv <= (1 << 18));
+}
 
 // q = floor(u / v), r = u - q v for a uniform batch, step by step across the
 // batch (see the top of this file); irregular instances by the

@@ -101,6 +101,29 @@ def test_step_form_adversarial_and_irregular(bi, orc):
         assert np.array_equal(r, orr), variant
 
 
+@pytest.mark.parametrize("nu,nv,count", [
+    (8, 7, 40), (8, 8, 40), (11, 8, 40), (12, 8, 40), (16, 8, 2500), (50, 9, 700), (64, 64, 1024),
+    (67, 64, 1025), (68, 64, 24), (90, 33, 400), (192, 96, 300), (400, 127, 40), (127, 127, 1300),
+    (1027, 1024, 3), (1028, 1025, 3)])
+def test_default_form_small_divisors(bi, orc, nu, nv, count):
+    """Both sides of the rule between the forms (variant 0): short quotients,
+    small divisors, batches of few and of many; some divisors with zero top
+    limbs and one zero divisor."""
+    from paper_2607_28897_gb300 import inputs
+
+    u = inputs.limbs(nu * 13 + nv + count, count, nu, top_nonzero=True)
+    v = inputs.limbs(nu * 17 + nv + count, count, nv, top_nonzero=True)
+    v[1::2, -1] = (v[1::2, -1] % np.uint64(1 << 32)) | np.uint64(1)
+    v[::5, :] = np.uint64(0xFFFFFFFFFFFFFFFF)
+    v[2::7, nv - nv // 4 - 1:] = 0
+    v[2] = 0
+    u[3::6] = np.uint64(0xFFFFFFFFFFFFFFFF)
+    q, r, st = run(bi, u, v, 0)
+    oq, orr, est = expect(bi, orc, u, v)
+    assert np.array_equal(st, est)
+    assert np.array_equal(q, oq) and np.array_equal(r, orr)
+
+
 @pytest.mark.parametrize("n,count", [(512, 96), (2048, 20), (8192, 3)])
 def test_default_form_equals_one_cta_form(bi, n, count):
     """The default (step-batched at these sizes) and the one-CTA-per-division
