@@ -28,9 +28,15 @@ constexpr int TC_DIV_MIN = 256;
 // One-thread long division for the Newton start value (tiny operands:
 // u <= 7 limbs, v <= 5 limbs).  Knuth's Algorithm D with 64-bit digits and
 // 128-bit intermediates.  q[0 .. nu-nv] receives floor(u / v); v[nv-1] != 0.
+// A quotient digit is a 128 by 64-bit division by the same top digit each
+// time: after one such division for its reciprocal, two multiplications
+// (Moeller and Granlund, "Improved division by invariant integers", 2011).
 // ---------------------------------------------------------------------------
-__device__ void small_div(const uint64_t *u, int nu, const uint64_t *v, int nv, uint64_t *q) {
+// small_div_body with constant sizes stays in registers.
+__device__ __forceinline__ void small_div_body(const uint64_t *u, int nu, const uint64_t *v,
+                                               int nv, uint64_t *q) {
   typedef unsigned __int128 u128;
+#pragma unroll
   for (int j = 0; j <= nu - nv; j++) q[j] = 0;
   if (nu < nv) return;
   if (nv == 1) {
@@ -44,24 +50,45 @@ __device__ void small_div(const uint64_t *u, int nu, const uint64_t *v, int nv, 
   }
   uint64_t vn[5], un[8];
   const int s = __clzll(v[nv - 1]);
+#pragma unroll
   for (int i = nv - 1; i > 0; i--) vn[i] = (v[i] << s) | (s ? v[i - 1] >> (64 - s) : 0);
   vn[0] = v[0] << s;
   un[nu] = s ? u[nu - 1] >> (64 - s) : 0;
+#pragma unroll
   for (int i = nu - 1; i > 0; i--) un[i] = (u[i] << s) | (s ? u[i - 1] >> (64 - s) : 0);
   un[0] = u[0] << s;
-  const u128 B = (u128)1 << 64;
+  const uint64_t vt = vn[nv - 1];  // bit 63 set
+  const uint64_t rec = (uint64_t)((((u128)~vt << 64) | ~0ull) / vt);  // floor((B^2 - 1) / vt) - B
+#pragma unroll
   for (int j = nu - nv; j >= 0; j--) {
-    const u128 num = ((u128)un[j + nv] << 64) | un[j + nv - 1];
-    u128 qh = num / vn[nv - 1];
-    u128 rh = num % vn[nv - 1];
-    while (qh >= B || qh * vn[nv - 2] > ((rh << 64) | un[j + nv - 2])) {
+    const uint64_t n1 = un[j + nv], n0 = un[j + nv - 1];  // n1 <= vt
+    uint64_t qh;
+    u128 rh;
+    if (n1 >= vt) {
+      qh = ~0ull;
+      rh = (u128)n0 + vt;
+    } else {
+      const u128 e = (u128)rec * n1 + (((u128)n1 << 64) | n0);
+      qh = (uint64_t)(e >> 64) + 1;
+      uint64_t r0 = n0 - qh * vt;
+      if (r0 > (uint64_t)e) {
+        qh--;
+        r0 += vt;
+      }
+      if (r0 >= vt) {
+        qh++;
+        r0 -= vt;
+      }
+      rh = r0;
+    }
+    while ((rh >> 64) == 0 && (u128)qh * vn[nv - 2] > ((rh << 64) | un[j + nv - 2])) {
       qh--;
-      rh += vn[nv - 1];
-      if (rh >= B) break;
+      rh += vt;
     }
     u128 borrow = 0, carry = 0;
+#pragma unroll
     for (int i = 0; i < nv; i++) {
-      const u128 p = qh * vn[i] + carry;
+      const u128 p = (u128)qh * vn[i] + carry;
       carry = p >> 64;
       const u128 t = (u128)un[i + j] - (uint64_t)p - borrow;
       un[i + j] = (uint64_t)t;
@@ -72,6 +99,7 @@ __device__ void small_div(const uint64_t *u, int nu, const uint64_t *v, int nv, 
     if (t >> 64) {  // estimate one too large: add back
       qh--;
       u128 c = 0;
+#pragma unroll
       for (int i = 0; i < nv; i++) {
         const u128 s2 = (u128)un[i + j] + vn[i] + c;
         un[i + j] = (uint64_t)s2;
@@ -81,6 +109,28 @@ __device__ void small_div(const uint64_t *u, int nu, const uint64_t *v, int nv, 
     }
     q[j] = (uint64_t)qh;
   }
+}
+__device__ void small_div(const uint64_t *u, int nu, const uint64_t *v, int nv, uint64_t *q) {
+  small_div_body(u, nu, v, nv, q);
+}
+
+// The Newton start of three limbs: floor(B^6 / (t + 1)), t the divisor's top
+// four limbs (the top one nonzero), into w[0 .. 5).  False (w untouched) if
+// t + 1 = B^4.
+__device__ __forceinline__ bool start_div(const uint64_t *t, uint64_t *w) {
+  uint64_t vt[4], un[7] = {0, 0, 0, 0, 0, 0, 1}, q[4];
+  uint64_t c = 1;
+#pragma unroll
+  for (int j = 0; j < 4; j++) {
+    vt[j] = t[j] + c;
+    c = vt[j] < c;
+  }
+  if (c) return false;
+  small_div_body(un, 7, vt, 4, q);
+#pragma unroll
+  for (int j = 0; j < 4; j++) w[j] = q[j];
+  w[4] = 0;
+  return true;
 }
 
 // Per-instance workspace, in limbs.
@@ -245,7 +295,9 @@ __device__ void mul_any(const uint64_t *x, int nx, const uint64_t *y, int ny, ui
 // + 1 (k >= l) or V = v B^(l-k) (k < l).  Thread 0 computes, all wait.
 // ---------------------------------------------------------------------------
 __device__ void newton_start(const uint64_t *v, int k, int l, uint64_t *w, int cap_w) {
-  if (threadIdx.x == 0) {
+  if (threadIdx.x == 0 && l == 3 && k >= l && cap_w >= 5 && start_div(v + k - 3, w)) {
+    for (int i = 5; i < cap_w; i++) w[i] = 0;
+  } else if (threadIdx.x == 0) {
     uint64_t V[6] = {0, 0, 0, 0, 0, 0}, U[8] = {0, 0, 0, 0, 0, 0, 0, 0}, Qt[8];
     int nV;
     if (k >= l) {

@@ -43,6 +43,7 @@ __host__ __device__ inline Step newton_next(int k, int L, int l) {
 // + 1, into w[0 .. l + 2) (the divisor's top limb is nonzero).
 __device__ void ds_start_one(const uint64_t *v, int nv, int l, uint64_t *w) {
   const int k = nv - 1;
+  if (l == 3 && start_div(v + k - 3, w)) return;
   uint64_t Vt[6] = {0, 0, 0, 0, 0, 0}, Un[8] = {0, 0, 0, 0, 0, 0, 0, 0}, Qt[8];
   for (int j = 0; j <= l; j++) Vt[j] = v[k - l + j];
   int j = 0;
