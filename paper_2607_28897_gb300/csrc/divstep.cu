@@ -22,13 +22,15 @@
 //
 // Per step, with the iterate w ~ B^(k+l) / v kept to l + 2 limbs,
 // m = min(l - 2, L - l), t = min(k, l + m + 2), vt = top t + 1 limbs of v:
-//   P  = vt w mod B^(t+2)                    (low product, exact)
-//   d  = B^(t+l) - vt w: |d| = P if P < B^(t+2)/2 (d <= 0), else B^(t+2) - P
+//   P  = vt w mod B^(t+2)                    (banded from limb c - 2)
+//   d  = B^(t+l) - vt w: |d| = P if P < B^(t+2)/2 (d <= 0), else B^(t+2) - P,
+//        from limb c = t - m - 2 on (within a unit there, step_cut)
 //   P2 = w |d|, banded from limb s - 2, s = t + l - m
 //   w' = w B^m + floor(P2 / B^s)             (d >= 0)
 //   w' = w B^m - floor(P2 / B^s) - 1         (d <  0; the ceiling of Fig. 6
 //                                             rounded up by at most one)
-// The band makes floor(P2 / B^s) exact or one unit high; so each step lands
+// The band makes floor(P2 / B^s) exact or one unit high, and the unit of limb
+// c by which |d| may be off moves it by less than 2 / B^2; so each step lands
 // within a few units of B^(k+l+m) / v, and since m <= l - 2 the Newton error
 // squared stays below a unit: the error does not grow from step to step.
 // Then q^ = floor(u w / B^h) (banded from limb h - 2), r^ = u - q^ v modulo
@@ -379,19 +381,20 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   }
   for (int i = SS.n; i < ns; i++) {
     const Step S = steps[i];
-    const int nw = S.l + 2, nl = S.t + 2;
-    // P = vt w mod B^(t+2)
-    rc = launch_mul_ex(v + (k - S.t), nv, W[cur], Y.sw, P, Y.sp, count, S.t + 1, nw, nl, 0,
-                       ctr + 1, st, STEP_TC_MIN, skp);
+    const int nw = S.l + 2, c = step_cut(S), nl = S.t + 2 - c;
+    // P = vt w mod B^(t+2) from the cut on
+    rc = launch_mul_ex(v + (k - S.t), nv, W[cur], Y.sw, P, Y.sp, count, S.t + 1, nw, S.t + 2,
+                       c > 0 ? c - 2 : 0, ctr + 1, st, STEP_TC_MIN, skp);
     if (rc != BIGINT_OK) return rc;
     if (nl <= WARP_LIMBS && !few)
-      rc = chain_launch(few, k_ds_mid, gw, WARP_CTA, 0, st, P, Y.sp, D, Y.sd, nl, neg, count);
+      rc = chain_launch(few, k_ds_mid, gw, WARP_CTA, 0, st, P + c, Y.sp, D, Y.sd, nl, neg, count);
     else
-      rc = chain_launch(few, k_ds_mid_cta, (unsigned)count, lin, 0, st, P, Y.sp, D, Y.sd, nl, neg);
+      rc = chain_launch(few, k_ds_mid_cta, (unsigned)count, lin, 0, st, P + c, Y.sp, D, Y.sd, nl, neg);
     if (rc != BIGINT_OK) return rc;
     // P2 = w |d|, its limbs from s on
-    const int s = S.t + S.l - S.m, n2 = nw + nl;
-    rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st, STEP_TC_MIN, skp);
+    const int s = S.t + S.l - S.m - c, n2 = nw + nl;
+    rc = launch_mul_ex(W[cur], Y.sw, D, Y.sd, Z, Y.sz, count, nw, nl, n2, s - 2, ctr + 1, st,
+                       STEP_TC_MIN, skp);
     if (rc != BIGINT_OK) return rc;
     if (S.l + S.m + 2 <= WARP_LIMBS && !few)
       rc = chain_launch(few, k_ds_update, gw, WARP_CTA, 0, st, W[cur], Y.sw, nw, Z, Y.sz, s, n2 - s,
@@ -443,9 +446,9 @@ size_t divmod_sk_bytes(int64_t count, int nu, int nv) {
   };
   for (int i = 0; i < ns; i++) {
     const dstep::Step S = steps[i];
-    const int nw = S.l + 2, nl = S.t + 2;
-    take(S.t + 1, nw, nl, 0);
-    take(nw, nl, nw + nl, S.t + S.l - S.m - 2);
+    const int nw = S.l + 2, c = dstep::step_cut(S), nl = S.t + 2 - c;
+    take(S.t + 1, nw, S.t + 2, c > 0 ? c - 2 : 0);
+    take(nw, nl, nw + nl, S.t + S.l - S.m - c - 2);
   }
   const int nw = L + 2;
   take(nu, nw, nu + nw, h - 2);

@@ -39,6 +39,15 @@ __host__ __device__ inline Step newton_next(int k, int L, int l) {
   return s;
 }
 
+// The step's residue d = B^(t+l) - vt w is only needed from limb t - m - 2 on:
+// what lies below, times w / B^s, is less than 2 / B^2 of a unit of the new
+// iterate.  So vt w is a banded product from two limbs below this cut, and |d|
+// starts at it.  0: no cut.
+__host__ __device__ inline int step_cut(Step S) {
+  const int c = S.t - S.m - 2;
+  return c > 2 ? c : 0;
+}
+
 // One thread: the Newton start w = floor(B^(2 l) / V), V = floor(v / B^(k-l))
 // + 1, into w[0 .. l + 2) (the divisor's top limb is nonzero).
 __device__ void ds_start_one(const uint64_t *v, int nv, int l, uint64_t *w) {
@@ -61,9 +70,11 @@ __device__ void ds_start_one(const uint64_t *v, int nv, int l, uint64_t *w) {
 // z: 2 N).
 __device__ __forceinline__ void ds_small_step(const uint64_t *vt, Step S, const uint64_t *w,
                                               uint64_t *wn, uint64_t *d, uint64_t *z) {
-  const int l = S.l, m = S.m, t = S.t, nw = l + 2, nl = t + 2;
-  // P = vt w mod B^(t+2); |d| = P (top bit clear: d <= 0) or B^(t+2) - P
-  warp_mul(vt, t + 1, w, nw, d, nl);
+  const int l = S.l, m = S.m, t = S.t, nw = l + 2, c = step_cut(S), nl = t + 2 - c;
+  // P = vt w mod B^(t+2) from the cut on; |d| = P (top bit clear: d <= 0) or
+  // B^(t+2) - P
+  warp_mul(vt, t + 1, w, nw, d, t + 2, c > 0 ? c - 1 : 0);
+  d += c;
   const bool ng = (d[nl - 1] >> 63) == 0;
   if (!ng) {
     warp_addsub<true>(nl, 0u, [&](int j) { return make_ulonglong2(0ull, d[j]); },
@@ -71,8 +82,8 @@ __device__ __forceinline__ void ds_small_step(const uint64_t *vt, Step S, const 
     __syncwarp();
   }
   // P2 = w |d| (band); w' = w B^m + floor(P2 / B^s) or w B^m - floor(P2 / B^s) - 1
-  const int s = t + l - m, ny = nw + nl - s;
-  warp_mul(w, nw, d, nl, z, nw + nl, s - 2);
+  const int s = t + l - m - c, ny = nw + nl - s;
+  warp_mul(w, nw, d, nl, z, nw + nl, s - 1);
   auto load = [&](int j) {
     const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
     return make_ulonglong2(x, j < ny ? z[s + j] : 0ull);

@@ -94,9 +94,10 @@ __host__ __device__ inline void rag_sizes(int nu, int nv, int kind, int l, int &
                                           int &nout, int &lo) {
   const int k = nv - 1, L = rag_L(nu, nv);
   const Step S = newton_next(k, L, l);
+  const int c = step_cut(S);
   switch (kind) {
-    case RAG_P: nx = S.t + 1; ny = l + 2; nout = S.t + 2; lo = 0; break;
-    case RAG_P2: nx = l + 2; ny = S.t + 2; nout = nx + ny; lo = S.t + l - S.m - 2; break;
+    case RAG_P: nx = S.t + 1; ny = l + 2; nout = S.t + 2; lo = c > 0 ? c - 2 : 0; break;
+    case RAG_P2: nx = l + 2; ny = S.t + 2 - c; nout = nx + ny; lo = S.t + l - S.m - c - 2; break;
     case RAG_UW: nx = nu; ny = L + 2; nout = nx + ny; lo = nu - 2; break;
     case RAG_QV: nx = L + 2; ny = nv; nout = nv + 1; lo = 0; break;
     default: nx = nu; ny = nv; nout = nu + nv; lo = 0; break;
@@ -182,8 +183,9 @@ __global__ void __launch_bounds__(LIN_THREADS) k_rag_mid(RagArgs A) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   const RagOp o = A.ops[blockIdx.x];
   const RagRec r = rag_rec(A, o);
-  const int nl = newton_next(o.nv - 1, rag_L(o.nu, o.nv), A.l).t + 2;
-  const bool ng = ds_mid_cta(r.p, r.d, nl, scr);
+  const Step S = newton_next(o.nv - 1, rag_L(o.nu, o.nv), A.l);
+  const int c = step_cut(S);
+  const bool ng = ds_mid_cta(r.p + c, r.d, S.t + 2 - c, scr);
   if (threadIdx.x == 0) r.p[0] = ng ? 1 : 0;  // the low product is used up
 }
 
@@ -192,7 +194,7 @@ __global__ void __launch_bounds__(LIN_THREADS) k_rag_update(RagArgs A) {
   const RagOp o = A.ops[blockIdx.x];
   const RagRec r = rag_rec(A, o);
   const Step S = newton_next(o.nv - 1, rag_L(o.nu, o.nv), A.l);
-  const int nw = S.l + 2, n2 = nw + S.t + 2, s = S.t + S.l - S.m;
+  const int nw = S.l + 2, c = step_cut(S), n2 = nw + S.t + 2 - c, s = S.t + S.l - S.m - c;
   ds_update_cta(r.w[A.par], nw, r.z + s, n2 - s, r.p[0] != 0, S.m, r.w[A.par ^ 1],
                 S.l + S.m + 2, scr);
 }
