@@ -209,17 +209,33 @@ __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh
     post(&sh->xfull[xb]);
     items++;
     const bool ok = pipe_tiles<KB, NT>(T.nx, T.ny, T.nout, T.lo, [&](int, int, int e_lo, int e_hi) {
-      for (int ea = e_lo; ea <= e_hi; ea += HS) {
+      // AHEAD: the next stage's limbs are loaded while this one's rows are
+      // written (32-digit blocks, whose stages are short: 16384 low products of
+      // 1024 limbs 2 % faster; with the longer ones it only cost registers)
+      constexpr bool AHEAD = KB == 32;
+      uint64_t ahead[2][3];
+      auto load = [&](int ea) {
         const int eb = ea + HS - 1 < e_hi ? ea + HS - 1 : e_hi;
         const int nb = 16 * (eb - ea + 1) + KB / 8 - 1;
-        uint64_t v[2][3];
 #pragma unroll
         for (int u = 0; u < 2; u++) {
           const int Lm = 16 * eb + 15 - (t + u * STEP);
 #pragma unroll
           for (int i = 0; i < 3; i++)
-            v[u][i] = t + u * STEP < nb && Lm >= i && Lm - i < T.ny ? T.y[Lm - i] : 0ull;
+            ahead[u][i] = t + u * STEP < nb && Lm >= i && Lm - i < T.ny ? T.y[Lm - i] : 0ull;
         }
+      };
+      if (AHEAD && e_lo <= e_hi) load(e_lo);
+      for (int ea = e_lo; ea <= e_hi; ea += HS) {
+        const int eb = ea + HS - 1 < e_hi ? ea + HS - 1 : e_hi;
+        const int nb = 16 * (eb - ea + 1) + KB / 8 - 1;
+        if (!AHEAD) load(ea);
+        uint64_t v[2][3];
+#pragma unroll
+        for (int u = 0; u < 2; u++)
+#pragma unroll
+          for (int i = 0; i < 3; i++) v[u][i] = ahead[u][i];
+        if (AHEAD && ea + HS <= e_hi) load(ea + HS);
         if ((used >> st & 1u) && !pipe_wait(sh, &sh->hfree[st], sph >> st & 1u, lim)) return false;
         if (used >> st & 1u) sph ^= 1u << st;
         used |= 1u << st;
