@@ -214,14 +214,20 @@ __global__ void __launch_bounds__(LIN_THREADS) k_rag_finish(RagArgs A) {
   if (A.status != nullptr && threadIdx.x == 0) A.status[o.opi] = st;
 }
 
-// The products of a list: CTA b takes entries b, b + grid, ... (largest
-// first).  A CTA that gives up at a wait limit sets *abort_flag and reports
+// Entry k of this CTA: a list (largest first) is dealt to the CTAs in rounds,
+// every second one backwards, so that no CTA gets the larger one each time
+// (20000 mixed operations 16.67 -> 15.96 ms).
+__device__ __forceinline__ int64_t rag_entry(int64_t k) {
+  return k * gridDim.x + (k & 1 ? gridDim.x - 1 - blockIdx.x : blockIdx.x);
+}
+
+// The products of a list.  A CTA that gives up at a wait limit sets *abort_flag and reports
 // BIGINT_ETIMEOUT for the rest of its multiplications.
 template <class Product>
 __device__ __forceinline__ void rag_products(const RagArgs &A, Product product) {
   bool ok = true;
-  for (int i = blockIdx.x; i < A.n; i += gridDim.x) {
-    const int32_t e = A.list[i];
+  for (int64_t k = 0; rag_entry(k) < A.n; k++) {
+    const int32_t e = A.list[rag_entry(k)];
     const RagOp o = A.ops[e & ~RAG_SWAP];
     if (ok) ok = product(rag_task(A, o, (e & RAG_SWAP) != 0));
     if (threadIdx.x == 0) {
@@ -282,7 +288,7 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
     }
   }
   auto next_b = [&](int64_t k, PipeTask &T) {
-    const int64_t i = blockIdx.x + k * gridDim.x;
+    const int64_t i = rag_entry(k), in = rag_entry(k + 1);
     const bool more = i < A.n;
     T.nx = 0;
     if (more) {
@@ -290,8 +296,8 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
       const RagTask t = rag_task(A, A.ops[e & ~RAG_SWAP], (e & RAG_SWAP) != 0);
       T = PipeTask{t.x, t.y, t.out, t.nx, t.ny, t.nout, t.lo, nullptr};
     }
-    if (threadIdx.x == PIPE_DRAIN + 64 && i + gridDim.x < A.n) {  // of the second warp
-      const int32_t e = A.list[i + gridDim.x];
+    if (threadIdx.x == PIPE_DRAIN + 64 && in < A.n) {  // of the second warp
+      const int32_t e = A.list[in];
       const RagTask t = rag_task(A, A.ops[e & ~RAG_SWAP], (e & RAG_SWAP) != 0);
       prefetch_l2(t.x, 8 * (size_t)t.nx);
       prefetch_l2(t.y, 8 * (size_t)t.ny);
@@ -323,7 +329,7 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
   int64_t ndone = 0;
   auto status = [&](int64_t k, int32_t st) {
     if (A.kind == RAG_MUL && A.status != nullptr)
-      A.status[A.ops[A.list[blockIdx.x + k * gridDim.x] & ~RAG_SWAP].opi] = st;
+      A.status[A.ops[A.list[rag_entry(k)] & ~RAG_SWAP].opi] = st;
   };
   auto done = [&](int64_t k) {
     if (threadIdx.x == 0) status(k, BIGINT_OK);
@@ -331,7 +337,7 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
   };
   if (!pipe_run<KB, NT>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
     atomicExch(A.abort_flag, 1);
-    for (int64_t k = ndone; blockIdx.x + k * gridDim.x < A.n; k++) status(k, BIGINT_ETIMEOUT);
+    for (int64_t k = ndone; rag_entry(k) < A.n; k++) status(k, BIGINT_ETIMEOUT);
   }
 }
 
