@@ -255,7 +255,7 @@ typedef struct {
  * together, whatever their shapes -- the products of a step in one launch per
  * product form over all of them, read from the input pool and written to the
  * output pool in place -- the multiplications with a shorter operand of 64
- * limbs or more (256 of them at least) run through the same product
+ * limbs or more (32 of them at least) run through the same product
  * launches, and everything else in one persistent launch.  All
  * forms are device work only (a CUDA graph can capture them) and give the
  * same results. */

@@ -238,6 +238,15 @@ __device__ __forceinline__ void rag_products(const RagArgs &A, Product product) 
   }
 }
 
+// Product launches of one set (one kind and step, one form each; also the
+// batch's multiplications) depend on what came before the set but not on one
+// another, and each may fill only some of the SMs.  So all but the first are
+// launched as dependents (chain_launch) of the one before, which lets them
+// start once all its CTAs have: every CTA triggers when it has its tensor
+// memory, and CTA 0 waits for the launch before at its end, so that the last
+// one's completion is the set's.  The first starts after everything before.
+// Launches one after the other took 15.9 ms for 20000 mixed operations and
+// 4.5 for 1500.
 template <int NT, int G>
 __global__ void __launch_bounds__(2 * NT + 32, 256 / NT) k_rag_tc(RagArgs A) {
   extern __shared__ __align__(1024) uint8_t sm[];
@@ -245,10 +254,12 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT) k_rag_tc(RagArgs A) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   tcm::TcCtx c;
   tcm::tc_init<NT>(c, sm, &sh, scr);
+  pdl_trigger();
   rag_products(A, [&](const RagTask &T) {
     return tcm::tc_product<NT, G, true>(c, T.x, T.nx, T.y, T.ny, T.out, T.nout, T.lo);
   });
   tcm::tc_release<NT>(c);
+  if (blockIdx.x == 0) pdl_wait();
 }
 
 template <int NT>
@@ -257,11 +268,13 @@ __global__ void __launch_bounds__(32 * tcm::one_warps<NT>(), 512 / NT) k_rag_one
   __shared__ tcm::OneShared sh;
   tcm::OneCtx c;
   tcm::one_init<NT>(c, sm, &sh);
+  pdl_trigger();
   rag_products(A, [&](const RagTask &T) {
     return tcm::one_product<NT, tcm::one_warps<NT>()>(c, T.x, T.nx, T.y, T.ny, T.out, T.nout,
                                                       T.lo);
   });
   tcm::one_release<NT>(c);
+  if (blockIdx.x == 0) pdl_wait();
 }
 
 // The pipelined form.  The builders read an operation's table entries and
@@ -335,10 +348,11 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
     if (threadIdx.x == 0) status(k, BIGINT_OK);
     ndone = k + 1;
   };
-  if (!pipe_run<KB, NT>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
+  if (!pipe_run<KB, NT, false>(L, &sh, sm, next_b, next_i, next_d, done) && threadIdx.x == 0) {
     atomicExch(A.abort_flag, 1);
     for (int64_t k = ndone; rag_entry(k) < A.n; k++) status(k, BIGINT_ETIMEOUT);
   }
+  if (blockIdx.x == 0) pdl_wait();
 }
 
 // ---- host ------------------------------------------------------------------
@@ -509,7 +523,9 @@ class Chooser {
 };
 
 // Appends the launches of one kind of product over ops [first, first + n).
-void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, int l, int par) {
+// joined: they belong to the set of launches appended last.
+void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, int l, int par,
+                   bool joined = false) {
   struct Item {
     Form f;
     double cost;
@@ -531,6 +547,7 @@ void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, i
     size_t j = i;
     RagLaunch R{};
     R.what = RAG_PROD;
+    R.sibling = joined || i > 0;
     R.kind = kind;
     R.l = l;
     R.par = par;
@@ -571,6 +588,7 @@ int rag_plan(std::vector<RagOp> divs, std::vector<RagOp> muls, RagPlan &P) {
   });
   P.ndiv = (int64_t)divs.size();
   P.ops = divs;
+  P.ops.insert(P.ops.end(), muls.begin(), muls.end());
   for (int64_t first = 0; first < P.ndiv;) {
     int64_t n = 0, limbs = 0;
     while (first + n < P.ndiv) {
@@ -595,14 +613,12 @@ int rag_plan(std::vector<RagOp> divs, std::vector<RagOp> muls, RagPlan &P) {
       linear(RAG_UPDATE, first, act, l, par);
     }
     plan_products(P, C, first, n, RAG_UW, 0, 0);
+    if (first == 0) plan_products(P, C, P.ndiv, (int64_t)muls.size(), RAG_MUL, 0, 0, true);
     plan_products(P, C, first, n, RAG_QV, 0, 0);
     linear(RAG_FINISH, first, n, 0, 0);
     first += n;
   }
-  if (!muls.empty()) {
-    P.ops.insert(P.ops.end(), muls.begin(), muls.end());
-    plan_products(P, C, P.ndiv, (int64_t)muls.size(), RAG_MUL, 0, 0);
-  }
+  if (P.ndiv == 0) plan_products(P, C, 0, (int64_t)muls.size(), RAG_MUL, 0, 0);
   return BIGINT_OK;
 }
 
@@ -634,15 +650,19 @@ int rag_launch(const RagPlan &P, const RagBuffers &B, const uint64_t *in, uint64
       case RAG_FINISH: k_rag_finish<<<n, LIN_THREADS, 0, st>>>(A); break;
       default: {
         const ShapeAttr &a = shapes().a[R.shape];
+        int rc;
         if (a.pipe) {
           const tcm::PipeLayout L = pipe_layout_of(R.shape, R.nx);
-          a.pipe<<<(unsigned)R.grid, a.threads, L.total, st>>>(A, L);
+          rc = chain_launch(R.sibling, a.pipe, (unsigned)R.grid, a.threads, L.total, st, A, L);
         } else {
           // no more CTAs on an SM than its tensor memory serves (one too many
           // would queue for it through all of another's products)
           const uint32_t least = (uint32_t)(shapes().smem_sm / (a.cap + 1) - a.overhead + 1);
-          a.kern<<<(unsigned)R.grid, a.threads, std::max(R.smem, least), st>>>(A);
+          rc = chain_launch(R.sibling, a.kern, (unsigned)R.grid, a.threads,
+                            std::max(R.smem, least), st, A);
         }
+        if (rc != BIGINT_OK) return rc;
+        continue;
       }
     }
     const int rc = bigint_launch_status();

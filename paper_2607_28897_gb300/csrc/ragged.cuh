@@ -35,6 +35,7 @@ enum RagKind { RAG_P, RAG_P2, RAG_UW, RAG_QV, RAG_MUL };
 enum RagWhat { RAG_START, RAG_SMALL, RAG_PROD, RAG_MID, RAG_UPDATE, RAG_FINISH };
 struct RagLaunch {
   int what, kind, l, par;  // step (limbs known before it), parity of its iterate
+  bool sibling;            // RAG_PROD: independent of the launch before it
   int shape, grid;
   uint32_t smem;           // RAG_PROD: dynamic shared memory
   int nx;                  // largest operand stored whole

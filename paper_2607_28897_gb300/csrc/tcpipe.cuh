@@ -602,8 +602,8 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
 // builders, the issuing warp and the drain threads, which must all see the
 // same sequence; done(k) is called by the drain threads after product k.
 // Returns false if a wait hit its limit (the record for bigint_check_timeout
-// is set).
-template <int KB, int NT, class NextB, class NextI, class NextD, class Done>
+// is set).  WAIT: the products depend on the launch before (pdl_wait).
+template <int KB, int NT, bool WAIT = true, class NextB, class NextI, class NextD, class Done>
 __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, uint8_t *sm,
                                          NextB next_b, NextI next_i, NextD next_d, Done done) {
   constexpr int ISSUER = PIPE_DRAIN / 32;
@@ -638,7 +638,7 @@ __device__ __forceinline__ bool pipe_run(const PipeLayout &L, PipeShared *sh, ui
   tc_fence_after();
   const uint32_t tmem = sh->tmem_slot;
   pdl_trigger();  // not before this CTA has its tensor memory
-  pdl_wait();
+  if constexpr (WAIT) pdl_wait();
   if (warp < ISSUER) {
     pipe_drain<KB, NT>(L, sh, sm, tmem, lim, next_d, done);
   } else if (warp == ISSUER) {

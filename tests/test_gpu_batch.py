@@ -340,3 +340,49 @@ def test_grouped_divisions_in_waves():
     assert torch.equal(out[count * nq:].view(count, nv), r)
     assert not st.any()
     bi.check_timeout()
+
+
+@pytest.mark.parametrize("nmul,ndiv", [(32, 0), (40, 9), (170, 60)])
+def test_grouped_sets_overlap(nmul, ndiv):
+    """Product launches of one set run side by side (few products of very
+    different sizes, more forms than fill the SMs), captured in a graph and
+    replayed on fresh results, against the persistent form."""
+    import torch
+
+    import paper_2607_28897_gb300 as bi
+    from paper_2607_28897_gb300 import inputs
+
+    sizes = [64, 70, 4096, 130, 511, 700, 90, 1500, 2100, 300]
+    ops = np.zeros(nmul + ndiv, dtype=bi.op_dtype())
+    pos = opos = 0
+    for i in range(nmul + ndiv):
+        n = sizes[i % len(sizes)] + i // 10
+        if i < nmul:
+            kind, na, nb, n1, n2 = bi.OP_MUL, n, sizes[(3 * i + 1) % len(sizes)], 0, 0
+            n1 = na + nb
+        else:
+            kind, nb = bi.OP_DIVMOD, max(n, 128)
+            na = nb + [nb, 5, nb // 2][i % 3]
+            n1, n2 = na - nb + 1, nb
+        ops[i] = (kind, na, nb, 0, pos, pos + na, opos, opos + n1 if n2 else 0)
+        pos += na + nb
+        opos += n1 + n2
+    pool = inputs.limbs_torch(5, 1, pos, True, "cuda").view(-1)
+    B = bi.Batch(ops)
+    want = torch.zeros(opos, dtype=torch.int64, device="cuda")
+    wst = torch.full((len(ops),), 99, dtype=torch.int32, device="cuda")
+    B.launch(pool, want, wst, mode=bi.BATCH_PERSISTENT)
+    got, st = torch.zeros_like(want), torch.full_like(wst, 99)
+    B.launch(pool, got, st, mode=bi.BATCH_STEPS)
+    torch.cuda.synchronize()
+    assert torch.equal(got, want) and torch.equal(st, wst)
+    g = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(g):
+        B.launch(pool, got, st, mode=bi.BATCH_STEPS)
+    for _ in range(3):
+        got.zero_()
+        st.fill_(99)
+        g.replay()
+        torch.cuda.synchronize()
+        assert torch.equal(got, want) and torch.equal(st, wst)
+    bi.check_timeout()
