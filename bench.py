@@ -214,8 +214,8 @@ def cpu_model() -> str:
 # --------------------------------------------------------------------------
 # committed ncu traffic of the multiply kernel, valid only for its source
 # --------------------------------------------------------------------------
-def kernel_source_hash(files=("tccore.cuh", "tcone.cuh", "tcmul.cu", "mul.cu", "blockops.cuh",
-                              "common.cuh")) -> str:
+def kernel_source_hash(files=("tccore.cuh", "tcone.cuh", "tcpipe.cuh", "tcmul.cu", "mul.cu",
+                              "blockops.cuh", "common.cuh")) -> str:
     """Hash of the multiply kernel's code: // comments, blank lines and
     indentation do not count, so a comment edit keeps a profile valid."""
     h = hashlib.sha256()
@@ -537,7 +537,7 @@ def main():
     all_ms = sum(school_ms(n) for n in sizes)
     tr = committed_traffic()
     vk = bi.mul_variant_for(nk, nk)
-    kernel = (f"{'k_mul_tc<256, 8, 1, 128>' if vk == 12 else 'k_mul_kara' if vk in (10, 11) else 'k_mul'}"
+    kernel = (f"{'k_mul_pipe<128, 256>' if vk == 12 else 'k_mul_kara' if vk in (10, 11) else 'k_mul'}"
               f" (variant {vk}), {nk}-limb operands, batch {sweep_batch(nk)}: the launch shape "
               f"of the step's tensor-core products (the {nk}-limb sweep product and the leaves "
               f"of the Karatsuba products)")

@@ -76,7 +76,7 @@ int bigint_sub(const uint64_t *a, const uint64_t *b, uint64_t *out,
  * out = a * b, the FULL product of na + nb limbs per instance: the
  * schoolbook convolution C_k = sum_{i+j=k} a_i b_j of Sec. V-B, exact.
  * When the shorter operand has 64 limbs or more (and fits one SM's shared
- * memory) the convolution runs on the tensor cores: the operands as signed
+ * memory), the longer one more than 64, the convolution runs on the tensor cores: the operands as signed
  * base-256 digits, the convolution as fp16 matrix products (tcgen05.mma,
  * Toeplitz blocks of one operand times shifted blocks of the other) with
  * exact fp32 accumulation in tensor memory, the column sums turned into
@@ -104,8 +104,8 @@ int bigint_mul_lo(const uint64_t *a, const uint64_t *b, uint64_t *out,
  * more: each product's output tiles (4096 limbs each) are cut further into
  * units of consecutive groups of Toeplitz blocks, about one unit per SM;
  * every unit adds its tile's partial column sums into a buffer in the
- * workspace with integer atomic adds (exact, in any order), and one CTA per
- * product turns the sums into limbs.  Larger batches: each product's output
+ * workspace with integer atomic adds (exact, in any order), and a cluster of
+ * four CTAs per product turns the sums into limbs.  Larger batches: each product's output
  * tiles on different CTAs, linked by a second small kernel (the carries
  * between tiles and the column-sum bias are settled there).  Any other
  * product runs as bigint_mul.  Results are bit-identical to bigint_mul.
@@ -455,15 +455,14 @@ int bigint_host_sync(void);
  * Selects the kernel variant an operation uses from now on (process-wide,
  * not thread-safe; call it before launching work).  op 0 = multiply:
  *   variant 0 (default): chosen by operand size from GB300 measurements (the
- *   tensor-core product from a shorter operand of 64 limbs, integer
- *   products below), or the variant bigint_tune recorded for the size class
+ *   tensor-core product from a shorter operand of 64 limbs and a longer one
+ *   of more, integer products below), or the variant bigint_tune recorded for the size class
  *   variant 8: integer product, 29-bit digits, 16-column chunks
  *   variant 9: integer product, 28-bit digits, 8-column chunks
  *   variant 10: one level of Karatsuba (square full products of at least 64
  *   limbs; otherwise variant 8) over variant 8's half products
- *   variant 11: one warp per instance, 128-bit column sums (operands of at
- *   most 64 limbs; otherwise variant 9) -- what the products inside
- *   step-batched divisions use for operands of at most 64 limbs
+ *   variant 11: one warp per instance, whole limb columns per lane (operands
+ *   of at most 64 limbs; otherwise variant 9) -- the default for them
  *   variant 12: the tensor-core product -- the digit convolution of the
  *   schoolbook product (Sec. V-B) as fp16 matrix products (tcgen05.mma)
  *   over signed base-256 digits with exact fp32 accumulation -- with its

@@ -42,7 +42,8 @@ __host__ __device__ inline Step newton_next(int k, int L, int l) {
 // The step's residue d = B^(t+l) - vt w is only needed from limb t - m - 2 on:
 // what lies below, times w / B^s, is less than 2 / B^2 of a unit of the new
 // iterate.  So vt w is a banded product from two limbs below this cut, and |d|
-// starts at it.  0: no cut.
+// starts at it: l x 2l and l x l limbs become two products of about l x l
+// (4096 divisions of 1024 by 512 limbs 721 -> 675 us).  0: no cut.
 __host__ __device__ inline int step_cut(Step S) {
   const int c = S.t - S.m - 2;
   return c > 2 ? c : 0;

@@ -139,10 +139,10 @@ static int launch_kara(const uint64_t *a, const uint64_t *b, uint64_t *out, int6
 
 // Variant table (see bigint_set_variant).  Variant 0 picks by size from
 // measurements on GB300: the tensor-core product (tcmul.cu) once the shorter
-// operand has TC_MIN_LIMBS limbs and fits shared memory; below, one warp per
-// product (variant 11) for operands of at most SMALL_LIMBS limbs (65536
-// products of 48 limbs 324 us, 449 us as variant 9), else the integer
-// product with 28-bit digits and 8-column chunks (variant 9), or 29-bit
+// operand has TC_MIN_LIMBS limbs, the longer one more than SMALL_LIMBS, and it
+// fits shared memory; one warp per product (variant 11) for operands of at
+// most SMALL_LIMBS limbs (65536 products of 48 limbs 174 us, 450 us as
+// variant 9), else the integer product with 28-bit digits and 8-column chunks (variant 9), or 29-bit
 // digits and 16-column chunks (variant 8) past 1535 limbs.  A size class the tuner has measured
 // (bigint_tune) takes its recorded variant instead.
 size_t mul_tc_smem(int na, int nb);
@@ -150,9 +150,9 @@ int launch_mul_tc(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t c
                   int nb, int nout, cudaStream_t st, int force_nt);
 
 // Shorter operand (limbs) from which the default is the tensor-core product:
-// 65536 products of 64 limbs 402 us against 504 (one warp each) and 586 us
-// (variant 9), of 128 limbs 579 against 1854 us, 1000 x 64 limbs (16384)
-// 505 against 1033 us; at 48 limbs the warp form is ahead (324 : 376).
+// 65536 products of 128 limbs 579 us against 1854 (variant 9), 16384 of 1000
+// x 64 limbs 505 against 1033 us.  Products of 64 x 64 limbs and less are ahead
+// with a warp each (65536 of 64 limbs 273 us, 393 as a one-drain product).
 constexpr int TC_MIN_LIMBS = 64;
 
 static int g_mul_variant = 0;

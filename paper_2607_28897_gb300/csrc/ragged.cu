@@ -15,10 +15,14 @@
 // members, each class a chain of ~22 launches of its own), 20000 mixed
 // operations made 199 classes of 30 members on average -- 4474 launches one
 // after the other, each on a fraction of the SMs, 98 ms.  The grouped form
-// takes some 150 launches over thousands of operations each.
+// takes some 70 launches over thousands of operations each, and the product
+// launches of a step run side by side (below): 14.35 ms.
 //
-// Bound: the tensor-core products of the last steps; the records of a wave
-// (about 5.5 limbs per divisor limb) are kept to WAVE_BYTES.
+// Bound: the tensor-core products, whose floor is 10.5 ms at the cuBLAS rate;
+// they run at about 0.85 of it, the linear parts take 0.9 ms and the
+// persistent launch of the rest 0.3 ms.  In a batch of few operations each set of
+// launches lasts as long as its largest product on one CTA.  The records of a
+// wave (about 5.5 limbs per divisor limb) are kept to WAVE_BYTES.
 #include "ragged.cuh"
 
 #include <algorithm>

@@ -1,9 +1,20 @@
 // tcmul.cu -- batched full (and low-part) products on the tensor cores.
 //
-// Persistent CTAs, one per SM (NT = 256), two (NT = 128) or three (NT = 64),
-// loop over the instances of a uniform batch, each product computed by tc_product
-// (tccore.cuh: the digit convolution as tcgen05 fp16 MMAs with exact fp32
-// accumulation, Sec. V-B's schoolbook product on the tensor cores).
+// Persistent CTAs loop over the instances of a uniform batch, each product the
+// digit convolution of tccore.cuh (tcgen05 fp16 MMAs with exact fp32
+// accumulation, Sec. V-B's schoolbook product on the tensor cores) in the form
+// the cost models below pick:
+//   k_mul_one   one drain, two or four CTAs per SM (tcone.cuh): a shorter
+//               operand of at most 512 limbs
+//   k_mul_pipe  builder, issuing and drain warps, one CTA per SM
+//               (tcpipe.cuh): most larger ones
+//   k_mul_tc    all warps doing all of it in turn, one, two or three CTAs per
+//               SM (tc_product): the largest operands, and the forced shapes
+//   k_mul_tc_sk, k_mul_tc_split  a few products, each over several CTAs
+//
+// Measured, 0.x of 1900 TFLOP/s: 512 limbs 0.55 (131072 products 4182 us,
+// 6770 as tc_product), 1701 x 1103 limbs 0.73 (16384: 2815, 3860), 2048 limbs
+// as Karatsuba leaves 0.87.
 #include "tccore.cuh"
 #include <cooperative_groups.h>
 

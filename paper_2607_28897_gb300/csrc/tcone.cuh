@@ -32,7 +32,12 @@
 //    so one carry scan of the low words plus the high words one limb up
 //    finishes the tile; the words stay in registers until then.
 //
-// Product of 512 x 512 limbs, 131072 of them: see launch_mul_tc_ex's rule.
+// Bound: shared memory (the MMAs' operands, the transposes, the Hankel
+// stores: 7K of 9.5K cycles a product at 512 limbs, tensor pipe 0.55 of the
+// cuBLAS rate) and, below 200 limbs, latency: 16 warps an SM, all that the
+// tensor memory admits, issue half the time.  131072 products of 512 limbs
+// 4182 us (6770 as tc_product), 65536 of 160 limbs 662 us (2281 on the
+// integer pipes), 72 of 512 limbs 10.6 us (24.6).
 #pragma once
 #include "tccore.cuh"
 
