@@ -19,7 +19,7 @@
 // launches of a step run side by side (below): 14.35 ms.
 //
 // Bound: the tensor-core products, whose floor is 10.5 ms at the cuBLAS rate;
-// they run at about 0.85 of it, the linear parts take 0.9 ms and the
+// they run at about 0.8 of it, the linear parts take 0.9 ms and the
 // persistent launch of the rest 0.3 ms.  In a batch of few operations each set of
 // launches lasts as long as its largest product on one CTA.  The records of a
 // wave (about 5.5 limbs per divisor limb) are kept to WAVE_BYTES.

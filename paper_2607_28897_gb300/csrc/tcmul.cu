@@ -8,8 +8,9 @@
 //               operand of at most 512 limbs
 //   k_mul_pipe  builder, issuing and drain warps, one CTA per SM
 //               (tcpipe.cuh): most larger ones
-//   k_mul_tc    all warps doing all of it in turn, one, two or three CTAs per
-//               SM (tc_product): the largest operands, and the forced shapes
+//   k_mul_tc    all warps doing all of it in turn, one, two or four CTAs per
+//               SM (tc_product): operands beyond the pipeline's shared memory,
+//               some narrow products, and the forced shapes
 //   k_mul_tc_sk, k_mul_tc_split  a few products, each over several CTAs
 //
 // Measured, 0.x of 1900 TFLOP/s: 512 limbs 0.55 (131072 products 4182 us,
