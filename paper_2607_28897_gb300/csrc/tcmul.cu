@@ -5,7 +5,8 @@
 // accumulation, Sec. V-B's schoolbook product on the tensor cores) in the form
 // the cost models below pick:
 //   k_mul_one   one drain, two or four CTAs per SM (tcone.cuh): a shorter
-//               operand of at most 512 limbs
+//               operand of at most 512 limbs, with two accumulators of up to
+//               about 640
 //   k_mul_pipe  builder, issuing and drain warps, one CTA per SM
 //               (tcpipe.cuh): most larger ones
 //   k_mul_tc    all warps doing all of it in turn, one, two or four CTAs per
@@ -59,10 +60,10 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
 }
 
 // The same for products whose shorter operand has at most ONE_MAX limbs
-// (tcone.cuh): NT tensor-memory columns and 32 W threads per CTA, 512 / NT
-// CTAs per SM.  add + i sadd: nout limbs added to product i (null: none).
-template <int NT, int W, bool ADD>
-__global__ void __launch_bounds__(32 * W, 512 / NT)
+// (ONE_MAX2 with ACC = 2 accumulators; tcone.cuh): NT ACC tensor-memory columns
+// and 32 W threads per CTA, 512 / (NT ACC) CTAs per SM.  add + i sadd: nout limbs added to product i (null: none).
+template <int NT, int W, bool ADD, int ACC>
+__global__ void __launch_bounds__(32 * W, 512 / (NT * ACC))
     k_mul_one(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
               uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
               int64_t sy, int64_t so, int lo, int *abort_flag, const uint64_t *add,
@@ -70,7 +71,7 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ OneShared sh;
   OneCtx c;
-  one_init<NT>(c, sm, &sh);
+  one_init<NT * ACC>(c, sm, &sh);
   pdl_trigger();  // not before this CTA has its tensor memory
   pdl_wait();
   for (int64_t inst = blockIdx.x; inst < count; inst += gridDim.x) {
@@ -79,12 +80,12 @@ __global__ void __launch_bounds__(32 * W, 512 / NT)
       prefetch_l2(X + next * sx, 8 * (size_t)nx);
       prefetch_l2(Y + next * sy, 8 * (size_t)ny);
     }
-    if (!one_product<NT, W, ADD>(c, X + inst * sx, nx, Y + inst * sy, ny, Out + inst * so, nout,
+    if (!one_product<NT, W, ADD, ACC>(c, X + inst * sx, nx, Y + inst * sy, ny, Out + inst * so, nout,
                                  lo, ADD ? add + inst * sadd : nullptr))
       break;
   }
   if (c.aborted && abort_flag != nullptr && threadIdx.x == 0) atomicExch(abort_flag, 1);
-  one_release<NT>(c);
+  one_release<NT * ACC>(c);
 }
 
 // The same by the pipeline of tcpipe.cuh: one CTA per SM.
@@ -581,11 +582,11 @@ struct OneAttr {
   bool ok = false;
 };
 
-template <int NT, bool ADD = false>
+template <int NT, int ACC, bool ADD = false>
 static const OneAttr &one_attr() {
   static const OneAttr A = [] {
     OneAttr a;
-    auto *kern = tcm::k_mul_one<NT, one_warps<NT>(), ADD>;
+    auto *kern = tcm::k_mul_one<NT, one_warps<NT, ACC>(), ADD, ACC>;
     int dev = 0, optin = 0, reserved = 0;
     cudaFuncAttributes fa;
     if (cudaGetDevice(&dev) != cudaSuccess ||
@@ -606,21 +607,21 @@ static const OneAttr &one_attr() {
   return A;
 }
 
-template <int NT>
+template <int NT, int ACC>
 static int one_per_sm(size_t smem) {
-  const OneAttr &a = one_attr<NT>();
-  const int per_sm = a.smem_sm / (int)(smem + a.overhead);
-  return per_sm > 512 / NT ? 512 / NT : (per_sm < 1 ? 1 : per_sm);
+  const OneAttr &a = one_attr<NT, ACC>();
+  const int per_sm = a.smem_sm / (int)(smem + a.overhead), cap = 512 / (NT * ACC);
+  return per_sm > cap ? cap : (per_sm < 1 ? 1 : per_sm);
 }
 
 // At least so much shared memory that no SM takes more CTAs than its tensor
 // memory serves: one too many queues for it through all of another CTA's
 // products (65536 products of 64 limbs 390 us, 440 to 590 with five CTAs on
 // some SMs).
-template <int NT>
+template <int NT, int ACC>
 static size_t one_smem_floor(size_t smem) {
-  const OneAttr &a = one_attr<NT>();
-  const size_t least = (size_t)(a.smem_sm / (512 / NT + 1) - a.overhead + 1);
+  const OneAttr &a = one_attr<NT, ACC>();
+  const size_t least = (size_t)(a.smem_sm / (512 / (NT * ACC) + 1) - a.overhead + 1);
   return smem > least ? smem : least;
 }
 
@@ -631,14 +632,16 @@ static size_t one_smem_floor(size_t smem) {
 // cycles each), the shared-memory cycles of a tile's Hankel matrices (16 per
 // block) and transposes (8 per column), and the part of a tile's ~5000
 // cycles of latency and limb work that the CTAs sharing the SM do not hide.
-template <int NT>
+template <int NT, int ACC = 1>
 static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
-  constexpr int S = tcm::ONE_S, W = one_warps<NT>();
-  if ((nx < ny ? nx : ny) > tcm::ONE_MAX || !one_attr<NT>().ok) return 0;
+  constexpr int S = tcm::ONE_S, W = one_warps<NT, ACC>();
+  const int ns = nx < ny ? nx : ny;
+  if (ns > (ACC == 2 ? tcm::ONE_MAX2 : tcm::ONE_MAX) || (ACC == 2 && ns <= tcm::ONE_MAX)) return 0;
+  if (!one_attr<NT, ACC>().ok) return 0;
   const uint32_t total = tcm::one_bytes<NT, W>(nx, ny, nout, lo);
-  if (total > (uint32_t)one_attr<NT>().dyn) return 0;
+  if (total > (uint32_t)one_attr<NT, ACC>().dyn) return 0;
   if (cost != nullptr) {
-    const int mx = tcm::one_layout<W>(nx, ny, 0).mx, per_sm = one_per_sm<NT>(total);
+    const int mx = tcm::one_layout<W>(nx, ny, 0).mx, per_sm = one_per_sm<NT, ACC>(total);
     double cyc = nx;
     tcm::one_tiles<NT>(nx, ny, nout, lo, [&](int c0, int Wd, int e_lo, int e_hi) {
       cyc += 8.0 * Wd + (per_sm == 1 ? 7400.0 : (NT == 128 ? 5000.0 : 4500.0) / per_sm);
@@ -656,19 +659,20 @@ static size_t one_plan(int nx, int ny, int nout, int lo, double *cost) {
   return total;
 }
 
-template <int NT>
+template <int NT, int ACC = 1>
 static int launch_one(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
-  constexpr int W = one_warps<NT>();
-  size_t smem = one_plan<NT>(nx, ny, nout, A.lo, nullptr);
+  constexpr int W = one_warps<NT, ACC>();
+  size_t smem = one_plan<NT, ACC>(nx, ny, nout, A.lo, nullptr);
   if (smem == 0) return BIGINT_EINVAL;
   if (count == 0) return BIGINT_OK;
   const int sms = sm_count();
   if (sms == 0) return BIGINT_ECUDA;
-  const int64_t slots = (int64_t)sms * one_per_sm<NT>(smem);
+  const int64_t slots = (int64_t)sms * one_per_sm<NT, ACC>(smem);
   const int64_t grid = count < slots ? count : slots;
-  smem = one_smem_floor<NT>(smem);
-  auto *kern = A.add != nullptr ? tcm::k_mul_one<NT, W, true> : tcm::k_mul_one<NT, W, false>;
-  if (A.add != nullptr && !one_attr<NT, true>().ok) return BIGINT_ECUDA;
+  smem = one_smem_floor<NT, ACC>(smem);
+  auto *kern =
+      A.add != nullptr ? tcm::k_mul_one<NT, W, true, ACC> : tcm::k_mul_one<NT, W, false, ACC>;
+  if (A.add != nullptr && !one_attr<NT, ACC, true>().ok) return BIGINT_ECUDA;
   return chain_launch(grid <= sms, kern, (unsigned)grid, 32 * W, smem, st, A.x, A.y, A.out, nx, ny, nout, count,
                       A.sx, A.sy, A.so, A.lo, A.abort_flag, A.add, A.sadd);
 }
@@ -742,6 +746,8 @@ static double pipe_cost(int nx, int ny, int nout, int lo) {
 // launch per form more costs a step of a ragged batch more than it saves
 // (20000 mixed operations 17.4 -> 17.8 ms).
 constexpr int FORM_PIPE32 = RAG_NSHAPES;
+// The one-drain form with two accumulators, likewise.
+constexpr int FORM_ONE2 = RAG_NSHAPES + 1;
 
 // The one-drain (RAG_ONE...) or pipelined (RAG_PIPE...) form, either operand as x (*swap), where its model is cheaper
 // than `than` (< 0: anything); -1 where none is.
@@ -760,7 +766,9 @@ static int best_form(int nx, int ny, int nout, int lo, double than, bool *swap,
     offer(pipe_cost<64, 256>(mx, my, nout, lo), RAG_PIPE64, k);
     offer(pipe_cost<128, 128>(mx, my, nout, lo), RAG_PIPE128N, k);
     offer(pipe_cost<64, 128>(mx, my, nout, lo), RAG_PIPE64N, k);
-    if (!grouped) offer(pipe_cost<32, 256>(mx, my, nout, lo), FORM_PIPE32, k);
+    if (grouped) continue;
+    offer(pipe_cost<32, 256>(mx, my, nout, lo), FORM_PIPE32, k);
+    if (one_plan<128, 2>(mx, my, nout, lo, &c)) offer(c, FORM_ONE2, k);
   }
   return form;
 }
@@ -776,6 +784,7 @@ static int launch_form(int form, TcArgs A, bool sw, int64_t count, int nx, int n
   switch (form) {
     case RAG_ONE128: return launch_one<128>(A, count, nx, ny, nout, st);
     case RAG_ONE256: return launch_one<256>(A, count, nx, ny, nout, st);
+    case FORM_ONE2: return launch_one<128, 2>(A, count, nx, ny, nout, st);
     case RAG_PIPE128: return launch_pipe<128, 256>(A, count, nx, ny, nout, st);
     case RAG_PIPE64: return launch_pipe<64, 256>(A, count, nx, ny, nout, st);
     case RAG_PIPE128N: return launch_pipe<128, 128>(A, count, nx, ny, nout, st);

@@ -18,8 +18,16 @@
 //    the 1024 products has magnitude 2^14; then it is a multiple of 128 below
 //    2^25, exact as well.  (If one of them is not 128 * 128 it is at most
 //    128 * 127 = 2^14 - 128, which makes room for the carry digit's 128.)
-//  * So a CTA needs NT tensor-memory columns and no registers for column
-//    sums, and 512 / NT CTAs share an SM: while one forms limbs, the others'
+//  * Shorter operands of up to ONE_MAX2 limbs take two accumulators (ACC = 2):
+//    even Toeplitz blocks add into one, odd ones into the other.  A column meets
+//    at most ceil(n / 16) consecutive blocks, so each sums the products of at most
+//    32 of them, within the same bound, and a column sum is the sum of two
+//    drains at the end.  With 128-column tiles that is two CTAs per SM, as
+//    long as the Hankel matrices of a tile's blocks (up to about 640 limbs) leave
+//    room for two.  4096 products of 515 limbs by the top of 1024: 141 us, 192
+//    in the pipeline; 6080 of 520 limbs 351, 399.
+//  * So a CTA needs NT ACC tensor-memory columns and no registers for column
+//    sums, and 512 / (NT ACC) CTAs share an SM: while one forms limbs, the others'
 //    MMAs run.  The Hankel core matrices of all of y's blocks lie in shared
 //    memory at once; the column sums are transposed through the same memory.
 //  * Core matrices of A are 144 bytes apart instead of 128: a thread writes
@@ -46,6 +54,7 @@ namespace tcm {
 
 constexpr int ONE_KB = 32, ONE_S = 128 / ONE_KB, ONE_R = ONE_KB / 8;
 constexpr int ONE_MAX = 1024 / ONE_KB * 16;  // limbs of the shorter operand
+constexpr int ONE_MAX2 = 2 * ONE_MAX - 16;   // with two accumulators
 constexpr int ONE_CM = 144;                  // bytes from core matrix to core matrix of A
 constexpr int ONE_CS = 132;                  // words per transposed column
 
@@ -87,8 +96,8 @@ __host__ __device__ inline void one_blocks(int mx, int ey, int c0, int W, int &e
 // Warps per CTA.  More of them (8 / 16) shorten a lone product's phases by
 // 15 % but not a batch, where the CTAs sharing the SM overlap anyway
 // (512-limb products 2451 against 2167 us per 65536).
-template <int NT>
-__host__ __device__ constexpr int one_warps() { return NT == 128 ? 4 : 8; }
+template <int NT, int ACC = 1>
+__host__ __device__ constexpr int one_warps() { return NT * ACC == 128 ? 4 : 8; }
 
 // The tiles of NT columns of a product (low nout limbs, band start lo):
 // f(c0, W, e_lo, e_hi) for each.
@@ -215,11 +224,12 @@ __device__ __forceinline__ void mma_commit_warp(uint32_t mbar, uint32_t leader) 
 // One warp: the MMAs of the blocks e_lo .. e_hi into the columns
 // [c0, c0 + W) at TMEM column dtm, then a commit to mbar.  The first block's
 // columns are overwritten, those above it up to shi cleared by a zero A
-// operand.  A block has only two MMAs of some 70 cycles each, so the loop
+// operand (ACC = 2: all W columns of both accumulators, NT apart).  A block has only two MMAs of some 70 cycles each, so the loop
 // keeps a block's bookkeeping to a few independent integer operations
 // (descriptor start addresses and the column count are low-word fields) and
 // is unrolled so that they run ahead of the MMAs (otherwise ~105 cycles per
 // MMA whatever its width).
+template <int NT, int ACC>
 __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs_a, uint32_t z_a,
                                           uint32_t lbo_b, int c0, int W, int e_lo, int e_hi,
                                           int mx, int shi, uint32_t mbar) {
@@ -229,7 +239,12 @@ __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs
   const uint32_t a_hi = (uint32_t)(da0 >> 32), b_hi = (uint32_t)(db0 >> 32);
   const uint32_t step_b = (2u * lbo_b) >> 4;
   auto desc = [](uint32_t hi, uint32_t lo) { return (uint64_t)hi << 32 | lo; };
-  {
+  if (ACC == 2) {  // every column of both accumulators
+#pragma unroll
+    for (int a = 0; a < 2; a++)
+      mma_f16_warp(dtm + a * NT, sdesc(z_a, 128, 128), db0,
+                   IDESC_M128 | ((uint32_t)(W >> 3) << 17), 0, leader);
+  } else {
     const int hi =
         ((c0 + W < ONE_S * e_lo + mx ? c0 + W : ONE_S * e_lo + mx) - c0 + 15) & ~15;
     if (hi < shi)
@@ -239,12 +254,13 @@ __device__ __forceinline__ void one_issue(uint32_t dtm, uint32_t ha, uint32_t xs
   uint32_t a_lo = (uint32_t)da0 + (uint32_t)(e_hi - e_lo) * ONE_CM;  // 16 matrices per block
   const uint32_t b0 = (uint32_t)db0 + 16;
   int sh = ONE_S * e_lo - c0;  // column of the block's x block 0
-  uint32_t acc = 0;
+  uint32_t acc = ACC == 2;
 #pragma unroll 4
   for (int e = e_lo; e <= e_hi; e++) {
     const int ca = sh > 0 ? sh >> 4 : 0, end = sh + mx < W ? sh + mx : W;
     const uint32_t id = IDESC_M128 | ((uint32_t)(((end + 15) >> 4) - ca) << 18);
-    const uint32_t b_lo = b0 + (uint32_t)(16 * ca - sh), d = dtm + 16u * (uint32_t)ca;
+    const uint32_t b_lo = b0 + (uint32_t)(16 * ca - sh);
+    const uint32_t d = dtm + 16u * (uint32_t)ca + (ACC == 2 && (e & 1) ? NT : 0);
     mma_f16_warp(d, desc(a_hi, a_lo), desc(b_hi, b_lo), id, acc, leader);
     mma_f16_warp(d, desc(a_hi, a_lo + ((2 * ONE_CM) >> 4)), desc(b_hi, b_lo + step_b), id, 1, leader);
     acc = 1;
@@ -313,10 +329,11 @@ __device__ void one_release(OneCtx &c) {
 // whole CTA (32 W threads);
 // band mode (lo > 0) as tc_product's: tiles anchored S - 1 columns before
 // limb lo's, limbs below L0 = R floor(lo / R) untouched, out[L0 ..) with
-// 2^32 added at L0.  The shorter operand has at most ONE_MAX limbs; c.sm
+// 2^32 added at L0.  The shorter operand has at most ONE_MAX limbs (ONE_MAX2
+// with two accumulators); c.sm
 // holds one_layout<W>(nx, ny, blocks of the widest tile).  Returns false
 // (and sets c.aborted) if a wait hit its limit.
-template <int NT, int W, bool ADD = false>
+template <int NT, int W, bool ADD = false, int ACC = 1>
 __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx,
                                             const uint64_t *y, int ny, uint64_t *out, int nout,
                                             int lo, const uint64_t *add = nullptr) {
@@ -351,9 +368,10 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
     int e_lo, e_hi;
     one_blocks(Ly.mx, Ly.ey, c0, Wd, e_lo, e_hi);
     // columns of the tile the MMAs write
-    const int slo = ((c0 > S * e_lo ? c0 : S * e_lo) - c0) & ~15;
+    const int slo = ACC == 2 ? 0 : ((c0 > S * e_lo ? c0 : S * e_lo) - c0) & ~15;
     const int shi = e_hi >= e_lo
-                        ? ((c0 + Wd < S * e_hi + Ly.mx ? c0 + Wd : S * e_hi + Ly.mx) - c0 + 15) & ~15
+                        ? ACC == 2 ? Wd
+                        : ((c0 + Wd < S * e_hi + Ly.mx ? c0 + Wd : S * e_hi + Ly.mx) - c0 + 15) & ~15
                         : 0;
     if (shi > 0) {
       one_hankel<THREADS>(hk, y, ny, e_hi, 16 * (e_hi - e_lo + 1) + R - 1);
@@ -361,7 +379,7 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
       fence_async_smem();
       __syncthreads();
       if (__shfl_sync(FULL, warp, 0) == 0) {
-        one_issue(c.tmem, c.sbase + Ly.hk, xs_a, z_a, lbo_b, c0, Wd, e_lo, e_hi, Ly.mx, shi, mb);
+        one_issue<NT, ACC>(c.tmem, c.sbase + Ly.hk, xs_a, z_a, lbo_b, c0, Wd, e_lo, e_hi, Ly.mx, shi, mb);
         c.pending = tid == 0;
       }
       bool bad = false;
@@ -401,6 +419,13 @@ __device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx
 #pragma unroll
             for (int i = 0; i < 16; i++)
               v[i] = (uint32_t)__float2int_rn(__uint_as_float(v[i]));
+            if constexpr (ACC == 2) {
+              uint32_t o[16];
+              tmem_ld16(c.tmem + ((uint32_t)(32 * q) << 16) + (uint32_t)(NT + col0), o);
+              tmem_ld_wait();
+#pragma unroll
+              for (int i = 0; i < 16; i++) v[i] += (uint32_t)__float2int_rn(__uint_as_float(o[i]));
+            }
           } else {
 #pragma unroll
             for (int i = 0; i < 16; i++) v[i] = 0u;

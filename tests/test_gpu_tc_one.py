@@ -76,3 +76,32 @@ def test_banded_in_division(bi, orc, nu, nv):
     assert np.array_equal(to_host(q), oq) and np.array_equal(to_host(r), orr)
     assert np.array_equal(st.cpu().numpy(), ost)
     bi.check_timeout()
+
+
+@pytest.mark.parametrize("na,nb", [
+    (513, 513), (520, 513), (515, 1024), (1024, 527), (528, 528), (544, 640), (600, 600),
+    (513, 1500)])
+def test_two_accumulators(bi, orc, na, nb):
+    """Shorter operands just above one accumulator's bound, where even and odd
+    blocks are summed apart: full and low products, more of them than CTAs."""
+    count = 330
+    a, b = operands(na, nb, count)
+    a[-20:], b[-20:] = a[:20], b[:20]
+    want = orc.batch_mul(a, b)
+    assert np.array_equal(to_host(bi.mul(to_dev(a), to_dev(b))), want)
+    for m in (min(na, nb), na + nb - 3):
+        got = to_host(bi.mul_lo(to_dev(a), to_dev(b), m))
+        assert np.array_equal(got, want[:, :m]), m
+    bi.check_timeout()
+
+
+@pytest.mark.parametrize("nu,nv", [(1024, 512), (1040, 520), (1200, 640), (1100, 512)])
+def test_two_accumulators_banded(bi, orc, nu, nv):
+    """The banded products of divisions with quotients of 513 to 700 limbs."""
+    a, b = operands(nu, nv, 200)
+    b[b[:, -1] == 0, -1] = 1
+    q, r, st = bi.divmod(to_dev(a), to_dev(b))
+    oq, orr, _ = orc.batch_divmod(a, b)
+    assert not to_host(st).any()
+    assert np.array_equal(to_host(q), oq) and np.array_equal(to_host(r), orr)
+    bi.check_timeout()
