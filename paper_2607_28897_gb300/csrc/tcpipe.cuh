@@ -35,7 +35,7 @@
 // bandwidth at 144 columns, at the clock the chip's power leaves (2048-limb
 // products 1650 TFLOP/s, 94K cycles a product, 84K of them MMAs); for products
 // of a single narrow tile the drain warps' serial work (515 limbs by the top
-// 530: tensor pipe 20 % busy, issue slots 50 %).  16384 products of 1701 x
+// 530, now a one-drain product: tensor pipe 20 % busy, issue slots 50 %).  16384 products of 1701 x
 // 1103 limbs 3860 -> 2815 us, 8192 of 8192 limbs by Karatsuba 30.9 -> 25.4 ms.
 //
 // KB digits per x block: 128 (S = 1 row per coefficient), 64 (S = 2, MMAs
