@@ -41,7 +41,7 @@
 //
 // Measured: 4096 divisions of 1024 by 512 limbs 626 us, of which the products
 // take 475 (their tensor-core floor is 145 us: low and banded triangles of
-// small products, bound by the builds, drains and limb scans of tcone.cuh); one division of 16384 by 8192 limbs 286 us, a chain of 44
+// small products, bound by the builds, drains and limb scans of tcone.cuh); one division of 16384 by 8192 limbs 286 us, a chain of 40
 // dependent launches of 4 to 27 us.
 #include <algorithm>
 
@@ -366,7 +366,7 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
     const Step &S0 = steps[SS.n];
     // every operand and result of the step within N limbs (w' too)
     const int need = std::max(std::max(S0.l + 2, S0.t + 2), S0.l + S0.m + 2);
-    if (need > (few ? SMALL_STEP_LIMBS_FEW : SMALL_STEP_LIMBS)) break;
+    if (need > SMALL_STEP_LIMBS) break;
     SS.N = std::max(SS.N, (need + 7) / 8 * 8);
     SS.s[SS.n++] = S0;
   }

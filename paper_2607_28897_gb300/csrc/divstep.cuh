@@ -18,12 +18,12 @@ using namespace divc;
 constexpr int LIN_THREADS = 256, LIN_THREADS_FEW = 1024;
 
 // Fused leading steps: operands of at most SMALL_STEP_LIMBS limbs, i.e. up to
-// 66 known limbs, in a batch of few instances SMALL_STEP_LIMBS_FEW, i.e. 34
-// (a lone warp's serial products then cost more than the four launches of
-// the step).  A warp's
+// 66 known limbs.  (Up to 34 only, the step from 66 as four launches: 3000
+// divisions of 1024 by 512 limbs 522 us against 487, 40 of 200 by 100 limbs 66
+// against 49, one of 16384 by 8192 limbs 294 against 290.)  A warp's
 // shared memory holds, for steps of at most N limbs, two iterates (N each),
 // the divisor's top limbs and |d| (N each) and P2 (2 N).
-constexpr int SMALL_STEP_LIMBS = 136, SMALL_STEP_LIMBS_FEW = 72, SMALL_STEP_WARPS = 4;
+constexpr int SMALL_STEP_LIMBS = 136, SMALL_STEP_WARPS = 4;
 __host__ __device__ constexpr int small_step_warp_limbs(int N) { return 6 * N; }
 
 // One Newton step of an instance: l limbs of the inverse known, m new ones,
