@@ -39,10 +39,11 @@
 // leading steps whose operands all have at most SMALL_STEP_LIMBS limbs run in
 // one launch, a warp per instance (k_ds_small), instead of four launches each.
 //
-// Measured: 4096 divisions of 1024 by 512 limbs 626 us, of which the products
+// Measured: 4096 divisions of 1024 by 512 limbs 628 us, of which the products
 // take 475 (their tensor-core floor is 145 us: low and banded triangles of
-// small products, bound by the builds, drains and limb scans of tcone.cuh); one division of 16384 by 8192 limbs 286 us, a chain of 40
-// dependent launches of 4 to 27 us.
+// small products, bound by the builds, drains and limb scans of tcone.cuh); one
+// division of 16384 by 8192 limbs 282 us, a chain of 40 dependent launches of
+// 4 to 27 us.
 #include <algorithm>
 
 #include "divstep.cuh"
