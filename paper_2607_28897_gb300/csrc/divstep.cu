@@ -55,6 +55,7 @@ using namespace divc;
 int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, uint64_t *out,
                   int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
                   cudaStream_t st, int tc_min, SkBuffers *sk);
+bool mul_ex_ok(int na, int nb, int tc_min);
 int launch_divmod_cta(const uint64_t *u, const uint64_t *v, uint64_t *q, uint64_t *r,
                       int32_t *status, int64_t count, int nu, int nv, void *ws,
                       const int32_t *list, const int *nlist, cudaStream_t st);
@@ -259,6 +260,18 @@ int schedule(int k, int h, int l0, Step *steps, int cap) {
   return n;
 }
 
+// Limbs that a fused step takes per operand or result (w' too).
+int small_step_need(const Step &S) {
+  return std::max(std::max(S.l + 2, S.t + 2), S.l + S.m + 2);
+}
+
+// How many of the leading steps run fused in one launch.
+int small_steps(const Step *steps, int ns) {
+  int n = 0;
+  while (n < ns && n < SMALL_STEP_MAX && small_step_need(steps[n]) <= SMALL_STEP_LIMBS) n++;
+  return n;
+}
+
 // Per-instance record widths (limbs) and the workspace layout.
 struct Layout {
   int64_t sw, sp, sd, sz;  // iterate, low product, |d| / r^, banded product (then q^)
@@ -290,12 +303,34 @@ Layout layout(int64_t count, int nu, int nv) {
   return Y;
 }
 
+// The products of a division outside the fused steps, f(na, nb, nout, lo) for
+// each: every step's two, then those of the tail.  f returns false to stop.
+template <class F>
+bool products(int nu, int nv, F f) {
+  const int k = nv - 1, h = nu, L = h - k, l0 = L < 3 ? L : 3, nw = L + 2;
+  Step steps[64];
+  const int ns = schedule(k, h, l0, steps, 64);
+  for (int i = small_steps(steps, ns); i < ns; i++) {
+    const Step S = steps[i];
+    const int c = step_cut(S), nl = S.t + 2 - c;
+    if (!f(S.t + 1, S.l + 2, S.t + 2, c > 0 ? c - 2 : 0)) return false;
+    if (!f(S.l + 2, nl, S.l + 2 + nl, S.t + S.l - S.m - c - 2)) return false;
+  }
+  return f(nu, nw, nu + nw, h - 2) && f(nw, nv, nv + 1, 0);
+}
+
 }  // namespace dstep
 
-// True if divmod_steps can run this shape (with enough workspace).
+// True if divmod_steps can run this shape (with enough workspace): u w has a
+// shorter operand of nu - nv + 3 limbs, and where that fits no product form
+// (quotients of some 11000 limbs and more) the division is left to the
+// one-CTA-per-division kernel, which slices its products.
 bool divmod_steps_ok(int64_t count, int nu, int nv, size_t ws_bytes) {
   if (count < 1 || nv < 8 || nu < nv) return false;
-  return dstep::layout(count, nu, nv).total <= ws_bytes;
+  if (dstep::layout(count, nu, nv).total > ws_bytes) return false;
+  return dstep::products(nu, nv, [](int na, int nb, int, int) {
+    return mul_ex_ok(na, nb, dstep::STEP_TC_MIN);
+  });
 }
 
 // Whether a uniform batch takes the step-batched form by default: all but
@@ -361,15 +396,11 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   const unsigned gw = (unsigned)((count + WARP_CTA / 32 - 1) / (WARP_CTA / 32));
   // the leading steps whose operands are all small, fused into one launch
   SmallSteps SS;
-  SS.n = 0;
+  SS.n = small_steps(steps, ns);
   SS.N = 8;
-  while (SS.n < ns && SS.n < SMALL_STEP_MAX) {
-    const Step &S0 = steps[SS.n];
-    // every operand and result of the step within N limbs (w' too)
-    const int need = std::max(std::max(S0.l + 2, S0.t + 2), S0.l + S0.m + 2);
-    if (need > SMALL_STEP_LIMBS) break;
-    SS.N = std::max(SS.N, (need + 7) / 8 * 8);
-    SS.s[SS.n++] = S0;
+  for (int i = 0; i < SS.n; i++) {
+    SS.N = std::max(SS.N, (small_step_need(steps[i]) + 7) / 8 * 8);
+    SS.s[i] = steps[i];
   }
   if (SS.n > 0) {
     const size_t smem = (size_t)8 * SMALL_STEP_WARPS * small_step_warp_limbs(SS.N);
@@ -443,23 +474,11 @@ constexpr int64_t DIV_SK_MAX_COUNT = 16;
 // the step schedule and of the tail.
 size_t divmod_sk_bytes(int64_t count, int nu, int nv) {
   if (count < 1 || count > DIV_SK_MAX_COUNT || nu < nv) return 0;
-  const int k = nv - 1, h = nu, L = h - k, l0 = L < 3 ? L : 3;
-  dstep::Step steps[64];
-  const int ns = dstep::schedule(k, h, l0, steps, 64);
   size_t per = 0;
-  auto take = [&](int na, int nb, int nout, int lo) {
-    const size_t b = mul_sk_bytes_per_product(na, nb, nout, lo);
-    if (b > per) per = b;
-  };
-  for (int i = 0; i < ns; i++) {
-    const dstep::Step S = steps[i];
-    const int nw = S.l + 2, c = dstep::step_cut(S), nl = S.t + 2 - c;
-    take(S.t + 1, nw, S.t + 2, c > 0 ? c - 2 : 0);
-    take(nw, nl, nw + nl, S.t + S.l - S.m - c - 2);
-  }
-  const int nw = L + 2;
-  take(nu, nw, nu + nw, h - 2);
-  take(nw, nv, nv + 1, 0);
+  dstep::products(nu, nv, [&](int na, int nb, int nout, int lo) {
+    per = std::max(per, mul_sk_bytes_per_product(na, nb, nout, lo));
+    return true;
+  });
   return 2 * (size_t)count * per;  // two buffers in turn
 }
 

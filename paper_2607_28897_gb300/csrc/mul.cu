@@ -91,23 +91,36 @@ static int smem_optin() {
   return g_smem_optin;
 }
 
+// Largest dynamic shared memory of k_mul<RB, Q, F>: the opt-in limit minus its
+// static shared memory (< 0: a CUDA error).
+template <int RB, int Q, int F>
+static int variant_dyn_max() {
+  static int dyn_max = -1;
+  if (dyn_max < 0) {
+    const int optin = smem_optin();
+    cudaFuncAttributes fa;
+    if (optin == 0 || cudaFuncGetAttributes(&fa, k_mul<RB, Q, F>) != cudaSuccess) return -1;
+    const int d = optin - (int)fa.sharedSizeBytes;
+    if (cudaFuncSetAttribute(k_mul<RB, Q, F>, cudaFuncAttributeMaxDynamicSharedMemorySize, d) !=
+        cudaSuccess)
+      return -1;
+    dyn_max = d;
+  }
+  return dyn_max;
+}
+
+template <int RB, int Q>
+static size_t variant_smem(int na, int nb) {
+  return sizeof(uint32_t) * (size_t)blk_mul_smem_words<RB, Q>(na, nb);
+}
+
 template <int RB, int Q, int F>
 static int launch_variant(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t count,
                           int na, int nb, int nout, cudaStream_t st, int64_t sa = -1,
                           int64_t sb = -1, int64_t so = -1) {
-  const size_t smem = sizeof(uint32_t) * (size_t)blk_mul_smem_words<RB, Q>(na, nb);
-  const int optin = smem_optin();
-  if (optin == 0) return BIGINT_ECUDA;
-  if (smem > (size_t)optin) return BIGINT_EINVAL;
-  static int dyn_max = -1;  // opt-in limit minus the kernel's static shared memory
-  if (dyn_max < 0) {
-    cudaFuncAttributes fa;
-    BIGINT_CUDA_TRY(cudaFuncGetAttributes(&fa, k_mul<RB, Q, F>));
-    BIGINT_CUDA_TRY(cudaFuncSetAttribute(k_mul<RB, Q, F>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         optin - (int)fa.sharedSizeBytes));
-    dyn_max = optin - (int)fa.sharedSizeBytes;
-  }
+  const size_t smem = variant_smem<RB, Q>(na, nb);
+  const int dyn_max = variant_dyn_max<RB, Q, F>();
+  if (dyn_max < 0) return BIGINT_ECUDA;
   if (smem > (size_t)dyn_max) return BIGINT_EINVAL;
   const int T = pick_threads(blk_mul_units<RB, Q>(na, nb), Q >= 16 ? 640 : 1024);
   k_mul<RB, Q, F><<<(unsigned)count, T, smem, st>>>(
@@ -230,6 +243,25 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
                      int64_t so, int64_t count, int na, int nb, int nout, int lo, void *colsum,
                      size_t colsum_bytes, SkBuffers *chain, int *abort_flag, cudaStream_t st);
 
+// The kernel family of a product inside a division or program (launch_mul_ex).
+enum MulRoute { ROUTE_TC, ROUTE_SMALL, ROUTE_28, ROUTE_29 };
+static MulRoute mul_ex_route(int na, int nb, int tc_min) {
+  const int nmin = na < nb ? na : nb, nmax = na > nb ? na : nb;
+  if (mul_tc_on() && nmin >= tc_min && mul_tc_smem(na, nb) > 0) return ROUTE_TC;
+  return nmax <= SMALL_LIMBS ? ROUTE_SMALL : (nmax < 1536 ? ROUTE_28 : ROUTE_29);
+}
+
+// Whether launch_mul_ex has a form for products of these sizes: the integer
+// kernels hold both operands in shared memory, and the tensor-core forms at
+// least the shorter one (up to 11215 limbs).
+bool mul_ex_ok(int na, int nb, int tc_min) {
+  switch (mul_ex_route(na, nb, tc_min)) {
+    case ROUTE_28: return (int64_t)variant_smem<28, 8>(na, nb) <= variant_dyn_max<28, 8, 128>();
+    case ROUTE_29: return (int64_t)variant_smem<29, 16>(na, nb) <= variant_dyn_max<29, 16, 32>();
+    default: return true;
+  }
+}
+
 // The products inside divisions and programs: variant 0 or 12 runs the
 // tensor-core product with its shape by the cost model (split-K for a few
 // products of a chain with column-sum buffers `sk`), variants 13-17 force its
@@ -238,10 +270,9 @@ int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, 
                   int64_t so, int64_t count, int na, int nb, int nout, int lo, int *abort_flag,
                   cudaStream_t st, int tc_min, SkBuffers *sk) {
   if (count == 0) return BIGINT_OK;
-  const int nmin = na < nb ? na : nb;
   const int v = g_mul_variant;
-  if (v == 0 || (v >= 12 && v <= 17)) {
-    if (nmin >= tc_min && mul_tc_smem(na, nb) > 0) {
+  switch (mul_ex_route(na, nb, tc_min)) {
+    case ROUTE_TC: {
       // few products: cut each into units over the SMs (split-K)
       if (v <= 12 && sk != nullptr && mul_sk_worth(count, na, nb, nout, lo) &&
           sk->bytes >= (size_t)count * mul_sk_bytes_per_product(na, nb, nout, lo))
@@ -252,11 +283,11 @@ int launch_mul_ex(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t sb, 
       return launch_mul_tc_ex(a, sa, b, sb, out, so, count, na, nb, nout, lo, abort_flag, st,
                               v <= 12 ? 0 : force[v - 12]);
     }
+    case ROUTE_SMALL: return launch_mul_small(a, sa, b, sb, out, so, count, na, nb, nout, st);
+    case ROUTE_28:
+      return launch_variant<28, 8, 128>(a, b, out, count, na, nb, nout, st, sa, sb, so);
+    default: return launch_variant<29, 16, 32>(a, b, out, count, na, nb, nout, st, sa, sb, so);
   }
-  const int nmax = na > nb ? na : nb;
-  if (nmax <= SMALL_LIMBS) return launch_mul_small(a, sa, b, sb, out, so, count, na, nb, nout, st);
-  if (nmax < 1536) return launch_variant<28, 8, 128>(a, b, out, count, na, nb, nout, st, sa, sb, so);
-  return launch_variant<29, 16, 32>(a, b, out, count, na, nb, nout, st, sa, sb, so);
 }
 
 }  // namespace bigint

@@ -148,3 +148,27 @@ def test_single_division_2_20_bits(bi, orc):
     q, r, st = run(bi, u, v, 0)
     oq, orr, est = expect(bi, orc, u, v)
     assert np.array_equal(st, est) and np.array_equal(q, oq) and np.array_equal(r, orr)
+
+
+@pytest.mark.parametrize("nu,nv,mul", [(12000, 8, 0), (16384, 8, 0), (12000, 64, 0),
+                                       (16384, 64, 0), (12000, 127, 0), (16384, 127, 0),
+                                       (12000, 1000, 0), (16384, 1000, 0), (16384, 4096, 0),
+                                       (11224, 12, 0), (11225, 12, 0), (11700, 12, 0),
+                                       (16384, 8192, 8)])
+def test_long_quotients(bi, orc, nu, nv, mul):
+    """Quotients whose product u w fits no batched product form (with the
+    integer products, 8, a shorter one), and lengths around the last that the
+    tensor-core and the integer products take: the default form divides them
+    all."""
+    from paper_2607_28897_gb300 import inputs
+
+    u = inputs.limbs(nu + nv, 2, nu, top_nonzero=True)
+    v = inputs.limbs(nu - nv, 2, nv, top_nonzero=True)
+    bi.set_variant(0, mul)
+    try:
+        q, r, st = run(bi, u, v, 0)
+    finally:
+        bi.set_variant(0, 0)
+    oq, orr, est = expect(bi, orc, u, v)
+    assert np.array_equal(st, est)
+    assert np.array_equal(q, oq) and np.array_equal(r, orr)
