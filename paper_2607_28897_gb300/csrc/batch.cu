@@ -289,7 +289,8 @@ namespace {
 // launches, however many divisions take it), products with a shorter operand
 // of GROUP_MIN_MUL limbs when it has GROUP_MIN_MULS (a batch of 40 such
 // products, 28 divisions and 32 additions 1.54 ms, 2.14 ms with the products
-// in the persistent launch).
+// in the persistent launch).  Operations too long for the grouped products'
+// shared memory (rag_takes) stay in the persistent launch, which slices them.
 constexpr int GROUP_MIN_NV = 128, GROUP_MIN_DIVS = 8, GROUP_MIN_MUL = 64, GROUP_MIN_MULS = 32;
 
 // The steps form's plan: the grouped operations, and the order of the rest
@@ -300,10 +301,12 @@ int plan_steps(bigint_batch *B) {
   for (int32_t i = 0; i < (int32_t)B->ops.size(); i++) {
     const bigint_op &o = B->ops[i];
     RagOp r{o.na, o.nb, i, 0, o.a, o.b, o.o1, o.o2, 0};
-    if (o.op == BIGINT_OP_DIVMOD && o.nb >= GROUP_MIN_NV && o.na >= o.nb) {
+    if (o.op == BIGINT_OP_DIVMOD && o.nb >= GROUP_MIN_NV && o.na >= o.nb &&
+        rag_takes(o.na, o.nb, false)) {
       divs.push_back(r);
       kind[i] = 1;
-    } else if (B->use_tc && o.op == BIGINT_OP_MUL && std::min(o.na, o.nb) >= GROUP_MIN_MUL) {
+    } else if (B->use_tc && o.op == BIGINT_OP_MUL && std::min(o.na, o.nb) >= GROUP_MIN_MUL &&
+               rag_takes(o.na, o.nb, true)) {
       muls.push_back(r);
       kind[i] = 2;
     }

@@ -383,7 +383,6 @@ const Shapes &shapes() {
     s.a[RAG_64] = {k_rag_tc<64, 7>, nullptr, 2 * 64 + 32, 4, 0, 0};
     s.a[RAG_128] = {k_rag_tc<128, 8>, nullptr, 2 * 128 + 32, 2, 0, 0};
     s.a[RAG_256] = {k_rag_tc<256, 8>, nullptr, 2 * 256 + 32, 1, 0, 0};
-    s.a[RAG_256_G4] = {k_rag_tc<256, 4>, nullptr, 2 * 256 + 32, 1, 0, 0};
     s.a[RAG_PIPE128] = {nullptr, k_rag_pipe<128, 256>, tcm::PIPE_THREADS, 1, 0, 0};
     s.a[RAG_PIPE64] = {nullptr, k_rag_pipe<64, 256>, tcm::PIPE_THREADS, 1, 0, 0};
     s.a[RAG_PIPE128N] = {nullptr, k_rag_pipe<128, 128>, tcm::PIPE_THREADS, 1, 0, 0};
@@ -433,7 +432,6 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
     case RAG_ONE256: return one_bytes<256, one_warps<256>()>(nx, ny, nout, lo);
     case RAG_64: return layout<64, 7>(nx, ny).total;
     case RAG_128: return layout<128, 8>(nx, ny).total;
-    case RAG_256: return layout<256, 8>(nx, ny).total;
     case RAG_PIPE128:
     case RAG_PIPE64:
     case RAG_PIPE128N:
@@ -441,7 +439,7 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
       const uint32_t t = pipe_layout_of(shape, nx).total;
       return t ? t : ~0u;
     }
-    default: return layout<256, 4>(nx, ny).total;
+    default: return layout<256, 8>(nx, ny).total;
   }
 }
 
@@ -450,7 +448,10 @@ uint32_t shape_bytes(int shape, int nx, int ny, int nout, int lo) {
 // power of two for the cost models, which a plan then evaluates a few
 // hundred times, and a thread's next plan hardly at all: the choices (a
 // function of the sizes alone) are kept per thread, MEMO_MAX of them at most.
-// The shared memory is that of the actual sizes.
+// The shared memory is that of the actual sizes; a product that the chosen form
+// does not hold takes the 256-column tile with its shorter operand whole in
+// shared memory, and one that this does not hold either has no form
+// (rag_takes).
 struct Form {
   int shape, per_sm, group;  // products of one group share a launch
   int nx;                    // limbs of the operand stored whole
@@ -488,20 +489,14 @@ class Chooser {
     Form f;
     f.shape = it->second >> 1;
     f.swap = it->second & 1;
-    if (f.shape == RAG_256_G4) f.shape = RAG_256;
     int ax = f.swap ? ny : nx, ay = f.swap ? nx : ny;
     f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
     if (f.bytes > (uint32_t)shapes().a[f.shape].dyn) {
-      // 256-column tiles, the shorter operand whole in shared memory
       f.swap = nx > ny;
       ax = std::min(nx, ny);
       ay = std::max(nx, ny);
       f.shape = RAG_256;
       f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
-      if (f.bytes > (uint32_t)shapes().a[f.shape].dyn) {
-        f.shape = RAG_256_G4;
-        f.bytes = shape_bytes(f.shape, ax, ay, nout, lo);
-      }
     }
     const ShapeAttr &a = shapes().a[f.shape];
     f.nx = ax;
@@ -570,6 +565,14 @@ void plan_products(RagPlan &P, Chooser &C, int64_t first, int64_t n, int kind, i
 }
 
 }  // namespace
+
+bool rag_takes(int nu, int nv, bool mul) {
+  if (!shapes().ok) return true;  // rag_plan reports the error
+  // no product of a division has longer operands than u w, w of L + 2 limbs
+  const int nx = mul ? nu : rag_L(nu, nv) + 2, ny = mul ? nv : nu + 1;
+  return shape_bytes(RAG_256, std::min(nx, ny), std::max(nx, ny), nx + ny, 0) <=
+         (uint32_t)shapes().a[RAG_256].dyn;
+}
 
 int rag_plan(std::vector<RagOp> divs, std::vector<RagOp> muls, RagPlan &P) {
   P = RagPlan();

@@ -20,7 +20,7 @@ struct RagOp {
 
 // Product forms of a grouped launch (tc_choose).
 enum RagShape {
-  RAG_ONE128, RAG_ONE256, RAG_64, RAG_128, RAG_256, RAG_256_G4, RAG_PIPE128, RAG_PIPE64,
+  RAG_ONE128, RAG_ONE256, RAG_64, RAG_128, RAG_256, RAG_PIPE128, RAG_PIPE64,
   RAG_PIPE128N, RAG_PIPE64N,  // with 128-column tiles
   RAG_NSHAPES
 };
@@ -50,8 +50,13 @@ struct RagPlan {
   size_t rec_bytes = 0;         // largest wave's records
 };
 
-// Plans the given operations (divisions with nv >= 8 and nu >= nv, products);
-// BIGINT_OK or BIGINT_ECUDA.
+// Whether every product of a division of nu by nv limbs (mul: the product
+// itself) has a form: an operand of each has to lie in shared memory whole,
+// which a quotient of some 11000 limbs and more is too long for.
+bool rag_takes(int nu, int nv, bool mul);
+
+// Plans the given operations (divisions with nv >= 8 and nu >= nv, products,
+// all of which rag_takes); BIGINT_OK or BIGINT_ECUDA.
 int rag_plan(std::vector<RagOp> divs, std::vector<RagOp> muls, RagPlan &P);
 
 // Device buffers of a launch: plan copies, records, the irregular divisions'

@@ -386,3 +386,33 @@ def test_grouped_sets_overlap(nmul, ndiv):
         torch.cuda.synchronize()
         assert torch.equal(got, want) and torch.equal(st, wst)
     bi.check_timeout()
+
+
+def test_steps_form_with_a_long_quotient(orc):
+    """Divisions whose products are too long for the grouped form's shared
+    memory run in the persistent launch beside the grouped ones, and the calls
+    after the batch are not disturbed."""
+    import torch
+
+    import paper_2607_28897_gb300 as bi
+    from paper_2607_28897_gb300 import inputs
+
+    sizes = [(16384, 4096), (16384, 128), (11400, 180)] + [(1000 + 300 * i, 400 + 100 * i)
+                                                           for i in range(7)]
+    ops = np.zeros(len(sizes), dtype=bi.op_dtype())
+    nin = nout = 0
+    for i, (na, nb) in enumerate(sizes):
+        nq = na - nb + 1
+        ops[i] = (4, na, nb, 0, nin, nin + na, nout, nout + nq)
+        nin, nout = nin + na + nb, nout + nq + nb
+    pool = inputs.ragged_pool(21, ops, nin)
+    exp, exp_st = oracle_results(orc, ops, pool)
+    batch = bi.Batch(ops)
+    out = torch.zeros(nout, dtype=torch.int64, device="cuda")
+    st = torch.full((len(ops),), -99, dtype=torch.int32, device="cuda")
+    batch.launch(to_dev(pool), out, st, mode=bi.BATCH_STEPS)
+    check(ops, to_host(out), st.cpu().numpy(), exp, exp_st)
+    a, b = inputs.config_small(seed=1, n=64, count=6)
+    s, c = bi.add(to_dev(a), to_dev(b))
+    so, co = orc.batch_add(a, b)
+    assert np.array_equal(to_host(s), so) and np.array_equal(c.cpu().numpy(), co)
