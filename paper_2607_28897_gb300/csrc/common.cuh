@@ -85,10 +85,17 @@ __device__ __forceinline__ void pdl_wait() {
 }  // namespace bigint
 
 // Host-side helpers --------------------------------------------------------
-#define BIGINT_CUDA_TRY(expr)                   \
-  do {                                          \
-    cudaError_t e__ = (expr);                   \
-    if (e__ != cudaSuccess) return BIGINT_ECUDA; \
+// BIGINT_ECUDA for a CUDA call that failed; takes the error off the calling
+// thread, whose later calls would report it as theirs.
+static inline int bigint_cuda_error() {
+  cudaGetLastError();
+  return BIGINT_ECUDA;
+}
+
+#define BIGINT_CUDA_TRY(expr)                          \
+  do {                                                 \
+    cudaError_t e__ = (expr);                          \
+    if (e__ != cudaSuccess) return bigint_cuda_error(); \
   } while (0)
 
 namespace bigint {
@@ -113,10 +120,10 @@ constexpr int TC_FORCE_N64 = 1064, TC_FORCE_N32 = 1032;
 }  // namespace bigint
 
 // Called right after every kernel launch of the library: counts it and
-// reports a launch error.
+// reports a launch error, which it takes off the thread.
 static inline int bigint_launch_status() {
   bigint::count_launch();
-  return cudaPeekAtLastError() == cudaSuccess ? BIGINT_OK : BIGINT_ECUDA;
+  return cudaGetLastError() == cudaSuccess ? BIGINT_OK : BIGINT_ECUDA;
 }
 
 namespace bigint {
@@ -149,7 +156,8 @@ inline int chain_launch(bool overlap, void (*kern)(P...), unsigned grid, unsigne
     at[c.numAttrs].val.programmaticStreamSerializationAllowed = 1;
     c.numAttrs++;
   }
-  if (cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...) != cudaSuccess) return BIGINT_ECUDA;
+  if (cudaLaunchKernelEx(&c, kern, static_cast<P>(args)...) != cudaSuccess)
+    return bigint_cuda_error();
   return bigint_launch_status();
 }
 }  // namespace bigint
