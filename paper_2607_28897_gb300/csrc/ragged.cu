@@ -319,12 +319,14 @@ __global__ void __launch_bounds__(tcm::PIPE_THREADS, 1) k_rag_pipe(RagArgs A, tc
       prefetch_l2(t.x, 8 * (size_t)t.nx);
       prefetch_l2(t.y, 8 * (size_t)t.ny);
     }
-    if (threadIdx.x == PIPE_DRAIN + 32) {  // the first builder thread
+    if (threadIdx.x / 32 == PIPE_DRAIN / 32 + 1) {  // the first builder warp, as one
       const int r = (int)(k % RING);
-      if (k >= RING && !pipe_wait(&sh, &ring.free[r], (uint32_t)(k / RING - 1) & 1u, lim))
+      if (k >= RING && !pipe_wait_warp(&sh, &ring.free[r], (uint32_t)(k / RING - 1) & 1u, lim))
         return false;
-      ring.t[r] = T;
-      mbar_arrive(smem_u32(&ring.full[r]));
+      if (lane == 0) {
+        ring.t[r] = T;
+        mbar_arrive(smem_u32(&ring.full[r]));
+      }
     }
     return more;
   };

@@ -165,6 +165,8 @@ __device__ __forceinline__ bool pipe_wait_warp(PipeShared *sh, uint64_t *bar, ui
 }
 
 // ---- builders -----------------------------------------------------------------
+// Their waits are decided by whole warps (pipe_wait_warp): a lane that gave up
+// alone would leave the others of its warp at the next __syncwarp for ever.
 // x into the B layout (fill_x without the carry digit), by the builders.
 template <int KB>
 __device__ __forceinline__ void pipe_fill(uint8_t *xs, const uint64_t *x, int nx, int t) {
@@ -211,7 +213,7 @@ __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh
   PipeTask T;
   for (int64_t k = 0; next(k, T); k++) {
     const uint32_t xb = L.xbufs == 2 ? items & 1u : 0u, n = L.xbufs == 2 ? items >> 1 : items;
-    if (n >= 1 && !pipe_wait(sh, &sh->xfree[xb], (n - 1) & 1u, lim)) return;
+    if (n >= 1 && !pipe_wait_warp(sh, &sh->xfree[xb], (n - 1) & 1u, lim)) return;
     pipe_fill<KB>(sm + L.xs + xb * L.xbytes, T.x, T.nx, t);
     post(&sh->xfull[xb]);
     items++;
@@ -243,7 +245,8 @@ __device__ __forceinline__ void pipe_builder(const PipeLayout &L, PipeShared *sh
 #pragma unroll
           for (int i = 0; i < 3; i++) v[u][i] = ahead[u][i];
         if (AHEAD && ea + HS <= e_hi) load(ea + HS);
-        if ((used >> st & 1u) && !pipe_wait(sh, &sh->hfree[st], sph >> st & 1u, lim)) return false;
+        if ((used >> st & 1u) && !pipe_wait_warp(sh, &sh->hfree[st], sph >> st & 1u, lim))
+          return false;
         if (used >> st & 1u) sph ^= 1u << st;
         used |= 1u << st;
         uint8_t *hk = sm + L.hk + st * L.hbytes;
@@ -605,9 +608,9 @@ __device__ __forceinline__ bool pipe_drain(const PipeLayout &L, PipeShared *sh, 
 
 // ---- the CTA ----------------------------------------------------------------------
 // Runs the products 0, 1, ... on PIPE_THREADS threads with 512 TMEM columns:
-// next_b(k, T), next_i and next_d give product k (false: no more) to the
-// builders, the issuing warp and the drain threads, which must all see the
-// same sequence; done(k) is called by the drain threads after product k.
+// next_b(k, T), next_i and next_d give product k (false: no more, the same
+// answer for all lanes of a warp) to the builders, the issuing warp and the drain
+// threads, which must all see the same sequence; done(k) is called by the drain threads after product k.
 // Returns false if a wait hit its limit (the record for bigint_check_timeout
 // is set).  WAIT: the products depend on the launch before (pdl_wait).
 template <int KB, int NT, bool WAIT = true, class NextB, class NextI, class NextD, class Done>

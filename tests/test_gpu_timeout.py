@@ -51,3 +51,62 @@ def test_wait_limit_timeout_then_recovery(orc):
     assert np.array_equal(to_host(q), oq) and np.array_equal(to_host(r), orr)
     assert not st.cpu().numpy().any()
     bi.check_timeout()
+
+
+def test_pipeline_and_batch_give_up_then_recover(orc):
+    """The same for the pipelined products (several per CTA, full ones and
+    Poly's low ones with an addend) and the grouped products and divisions of
+    a ragged batch."""
+    import torch
+
+    import paper_2607_28897_gb300 as bi
+    from paper_2607_28897_gb300 import inputs
+
+    n = 400  # more products than SMs
+    a, b = (inputs.limbs(s, n, 2048, top_nonzero=True) for s in (31, 32))
+    pa, pb = (inputs.limbs(s, n, 1024, top_nonzero=True) for s in (33, 34))
+    ops, nin, nout = inputs.ragged_ops(35, 400, min_limbs=300, max_limbs=2000)
+    pool = inputs.ragged_pool(36, ops, nin)
+    da, db, dpa, dpb, dpool = (to_dev(x) for x in (a, b, pa, pb, pool))
+    batch = bi.Batch(ops)
+    out = torch.zeros(nout, dtype=torch.int64, device="cuda")
+    st = torch.zeros(len(ops), dtype=torch.int32, device="cuda")
+
+    def gave_up():
+        with pytest.raises(bi.BigIntError) as e:
+            bi.check_timeout()
+        assert e.value.code == bi.ETIMEOUT
+
+    bi.check_timeout()
+    bi.set_wait_limit(-2000)
+    try:
+        bi.mul(da, db)
+        gave_up()
+        bi.poly(dpa, dpb)
+        gave_up()
+        batch.launch(dpool, out, st, mode=bi.BATCH_STEPS)
+        gave_up()
+        got = st.cpu().numpy()
+        assert (got[ops["op"] >= 3] == bi.ETIMEOUT).all(), got
+    finally:
+        bi.set_wait_limit(0)
+    bi.check_timeout()
+    assert np.array_equal(to_host(bi.mul(da, db))[::40], orc.batch_mul(a[::40], b[::40]))
+    got = to_host(bi.poly(dpa, dpb))
+    for i in (0, 151, 152, n - 1):
+        x, y = (int.from_bytes(v[i].tobytes(), "little") for v in (pa, pb))
+        want = ((x * x + y) * (y * y + y) + x * y) % (1 << (64 * 1024))
+        assert int.from_bytes(got[i].tobytes(), "little") == want, i
+    batch.launch(dpool, out, st, mode=bi.BATCH_STEPS)
+    got, status = to_host(out), st.cpu().numpy()
+    for i in np.nonzero(ops["op"] >= 3)[0][::9]:
+        o = ops[i]
+        x, y = (int.from_bytes(pool[o[k]:o[k] + o[m]].tobytes(), "little")
+                for k, m in (("a", "na"), ("b", "nb")))
+        want = [(x * y, o["o1"], o["na"] + o["nb"])]
+        if o["op"] == 4:
+            want = [(x // y, o["o1"], o["na"] - o["nb"] + 1), (x % y, o["o2"], o["nb"])]
+        assert status[i] == 0
+        for value, at, size in want:
+            assert int.from_bytes(got[at:at + size].tobytes(), "little") == value, i
+    bi.check_timeout()
