@@ -801,7 +801,8 @@ __device__ __forceinline__ bool tc_product(TcCtx &c, const uint64_t *x, int nx, 
         }
         if (!bad) {
           const int lb = (NG - 1) & 1;
-          if (!mbar_wait_lim(mb[lb], (c.phase >> lb) & 1u, c.wlim)) {
+          // a warp drains (tcgen05.ld, by whole warps) or gives up as one
+          if (!__all_sync(FULL, mbar_wait_lim(mb[lb], (c.phase >> lb) & 1u, c.wlim))) {
             bad = true;
           } else {
             c.phase ^= 1u << lb;
