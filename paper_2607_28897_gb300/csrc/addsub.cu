@@ -196,19 +196,42 @@ __global__ void __launch_bounds__(1024)
   }
 }
 
-// Launch shape.  Bound: HBM (24 bytes a limb), so what matters is loads in
+// Launch shape: rounds per warp, and warps per CTA or (0) one warp per instance.
+//
+// A large batch is bound by HBM (24 bytes a limb), so what matters is loads in
 // flight on every SM at every moment: one CTA that holds the SM alone reads,
-// waits, then writes.  So a warp always takes R = 4 rounds where the operand
-// has them, and a CTA at most max_warps warps (more limbs: more
-// super-rounds), which leaves an SM several CTAs in different phases.
-// Measured, operand arrays of 2^32 bits: 8192 limbs 5.7 TB/s with 32 warps
-// in one super-round (one CTA per SM) -> 7.0 with 8 warps in four; 1537
-// limbs (8-byte accesses) 5.3 TB/s with two rounds a warp -> 7.1 with four.
-// The chain's extra arithmetic wants more CTAs still: 6.8 against 6.5 TB/s
-// at 8192 limbs with 4 instead of 8 warps.  Operands of at most one warp's
-// segment go one warp per instance: a CTA each starts and ends too often
-// (64 limbs: 3.0 TB/s).  A batch of at most two instances per SM has nothing
-// to overlap with, so there one super-round of up to 32 warps is the fastest.
+// waits, then writes (operand arrays of 2^32 bits, 8192 limbs: 5.7 TB/s with 32
+// warps of four rounds, 7.0 with 8).  A small one lasts as long as its last CTA,
+// which wants less work per warp and more warps.  128 limbs a warp and up to 16
+// warps serve both; where they do not:
+//  * Batches of MANY instances per SM and MANY_LIMBS limbs take 8 warps of four
+//    rounds for more than 4096 limbs (600 of 8192 limbs 16.9 us, 17.7 as 16 warps
+//    of two) and for odd sizes (8-byte accesses: 2^26 limbs of 1025 234 us, 236
+//    as 9 warps).
+//  * Up to 1024 limbs, batches of at most HALF_LIMBS limbs per SM take 64 limbs a
+//    warp (64 of 512 limbs 1.75 -> 1.66 us; 600 of 1024 limbs 2.90 -> 3.14, so
+//    not there).
+//  * At most one instance per SM (odd sizes: two) gets 32 warps (16 of 4096 limbs
+//    2.9 us, 3.2 with 16), of four rounds above 4096 limbs (6000 limbs 3.6 us, 3.7
+//    with two), and one of two 24 if that makes one super-round.
+// Against 8 warps of four rounds (32 up to two instances per SM) at every size:
+// 64 additions of 512 limbs 1.97 -> 1.68 us, 400 of 1024 limbs 2.79 -> 2.63, 600
+// of 1536 limbs 3.70 -> 3.31, 304 of 8192 limbs 8.54 -> 7.29, 400 of 8193 limbs
+// 15.4 -> 12.0, 2^26 limbs of 300 242 -> 224.
+//
+// The chain keeps 4 warps of four rounds (32 up to two instances per SM): its
+// extra arithmetic wants more CTAs (8192 limbs: 6.8 against 6.5 TB/s with 8).
+//
+// Short operands go one warp per instance in larger batches, because a CTA each
+// starts and ends too often (64 limbs, HBM-bound: 3.0 TB/s); a few instances are
+// faster with several warps each (128 limbs x 152 1.77 -> 1.66 us, 256 limbs x 64
+// 2.05 -> 1.56, x 400 2.08 -> 1.98).
+struct Shape {
+  int R, W;
+};
+constexpr int MANY = 3;
+constexpr int64_t MANY_LIMBS = 3 << 20, HALF_LIMBS = 2048;
+
 static int sm_count() {
   static int sms = 0;
   if (sms == 0) {
@@ -222,25 +245,49 @@ static int sm_count() {
 }
 
 template <int MODE, int LPL>
+static Shape shape_of(int64_t count, int n) {
+  constexpr int ROUND = 32 * LPL;  // limbs of a warp's round
+  const int sms = sm_count();
+  const bool chain = MODE == CHAIN;
+  if (n <= ROUND || (n <= 4 * ROUND && (chain || count > 2 * LPL * sms)))
+    return Shape{n <= ROUND ? 1 : (n <= 2 * ROUND ? 2 : 4), 0};
+  const bool many = count > MANY * sms && count * n > MANY_LIMBS && (LPL == 1 || n > 4096);
+  const bool half = n <= 1024 && count * n <= HALF_LIMBS * sms;
+  const bool four = chain || many || (n > 4096 && count <= sms);
+  const int R = four ? 4 : (half ? 64 : 128) / ROUND;
+  const int need = (n + R * ROUND - 1) / (R * ROUND);  // warps for one super-round
+  int max_warps;
+  if (chain)
+    max_warps = count <= 2 * sms ? 32 : 4;
+  else if (LPL == 1)
+    max_warps = count <= 2 * sms ? 32 : (many ? 8 : 16);
+  else
+    max_warps = count <= sms ? 32 : (count <= 2 * sms && need <= 24 ? 24 : (many ? 8 : 16));
+  const int rounds = (need + max_warps - 1) / max_warps;
+  return Shape{R, (need + rounds - 1) / rounds};
+}
+
+template <int MODE, int LPL, int R>
+static int launch_shape(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
+                        int64_t count, int n, uint32_t k, int W, cudaStream_t st) {
+  if (W == 0)
+    k_addsub<MODE, LPL, R, true><<<(unsigned)((count + WPI_WARPS - 1) / WPI_WARPS), 32 * WPI_WARPS,
+                                   0, st>>>(a, b, out, carry, count, n, k);
+  else if constexpr (MODE != CHAIN || R == 4)
+    k_addsub<MODE, LPL, R, false><<<(unsigned)count, 32 * W, 0, st>>>(a, b, out, carry, count, n,
+                                                                      k);
+  return bigint_launch_status();
+}
+
+template <int MODE, int LPL>
 static int launch_lpl(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
                       int64_t count, int n, uint32_t k, cudaStream_t st) {
-  constexpr int SEG = 32 * LPL * 4;
-  const int max_warps = count <= 2 * sm_count() ? 32 : (MODE == CHAIN ? 4 : 8);
-  if (n <= SEG) {
-    const unsigned grid = (unsigned)((count + WPI_WARPS - 1) / WPI_WARPS);
-    if (n <= SEG / 4)
-      k_addsub<MODE, LPL, 1, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
-    else if (n <= SEG / 2)
-      k_addsub<MODE, LPL, 2, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
-    else
-      k_addsub<MODE, LPL, 4, true><<<grid, 32 * WPI_WARPS, 0, st>>>(a, b, out, carry, count, n, k);
-    return bigint_launch_status();
+  const Shape S = shape_of<MODE, LPL>(count, n);
+  switch (S.R) {
+    case 1: return launch_shape<MODE, LPL, 1>(a, b, out, carry, count, n, k, S.W, st);
+    case 2: return launch_shape<MODE, LPL, 2>(a, b, out, carry, count, n, k, S.W, st);
+    default: return launch_shape<MODE, LPL, 4>(a, b, out, carry, count, n, k, S.W, st);
   }
-  const int need = (n + SEG - 1) / SEG;  // warps for one super-round
-  const int rounds = (need + max_warps - 1) / max_warps;
-  const int W = (need + rounds - 1) / rounds;
-  k_addsub<MODE, LPL, 4, false><<<(unsigned)count, 32 * W, 0, st>>>(a, b, out, carry, count, n, k);
-  return bigint_launch_status();
 }
 
 template <int MODE>

@@ -129,3 +129,18 @@ def test_launch_shapes(bi, orc, n):
             want, c = orc.add_chain(a[i], b[i], k)
             assert np.array_equal(got[i], want), (i, k)
             assert int(carry[i]) == c, (i, k)
+
+
+@pytest.mark.parametrize("n", [63, 64, 65, 128, 129, 256, 257, 512, 1024, 1025, 1026, 4097, 8194,
+                               16384])
+@pytest.mark.parametrize("count", [16, 310])
+def test_launch_shapes_of_few_instances(bi, orc, n, count):
+    """Batches that do not fill the GPU: one, two or four rounds a warp, up to
+    16 or 32 warps, one super-round or several."""
+    from paper_2607_28897_gb300 import inputs
+
+    a, b = inputs.limbs(500 + n, count, n), inputs.limbs(600 + n, count, n)
+    sa, sb = inputs.stress_pairs(n)
+    a[:8], b[:8], a[-8:], b[-8:] = sa, sb, sa, sb
+    check_add(bi, orc, a, b)
+    check_sub(bi, orc, a, b)
