@@ -74,7 +74,10 @@ __device__ __forceinline__ void st_stream2(uint64_t *p, ulonglong2 v) {
 // launched by chain_launch right behind this one) be scheduled as SM resources
 // allow, pdl_wait holds a kernel until the kernel before it has completed and
 // its writes are visible.  A kernel calls pdl_wait before it touches global
-// memory.  Both do nothing in kernels launched the ordinary way.
+// memory, and does not declare what it reads __restrict__: loads through such
+// pointers are taken to be of memory that nothing writes while the kernel runs,
+// which the kernel before it may do, and could move above the wait.  Both do
+// nothing in kernels launched the ordinary way.
 __device__ __forceinline__ void pdl_trigger() {
   asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
 }

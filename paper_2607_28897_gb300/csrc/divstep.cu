@@ -87,7 +87,7 @@ __device__ __forceinline__ bool regular(const uint64_t *, int, const uint64_t *v
 // tiny Newton steps in this kernel too, one CTA per instance, was measured
 // slower than their batched launches: 579 us for 4096 instances of 512
 // limbs, the long chains of block barriers of the one-CTA form again.)
-__global__ void k_ds_start(const uint64_t *__restrict__ U, const uint64_t *__restrict__ V, int nu,
+__global__ void k_ds_start(const uint64_t *U, const uint64_t *V, int nu,
                            int nv, int l, uint64_t *W, int64_t sw, int64_t count,
                            int32_t *irregular, int *nirr) {
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
@@ -127,7 +127,7 @@ struct SmallSteps {
 // the result (l + m + 2 limbs of the last step) to W0 or W1 as the batched
 // steps would leave it (W0 after an even number of steps).
 __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS)
-    k_ds_small(const uint64_t *__restrict__ V, int nv, uint64_t *W0, uint64_t *W1, int64_t sw,
+    k_ds_small(const uint64_t *V, int nv, uint64_t *W0, uint64_t *W1, int64_t sw,
                int64_t count, SmallSteps S) {
   extern __shared__ __align__(16) uint64_t ssm[];
   const int wi = threadIdx.x >> 5, lane = (int)lane_id();
@@ -156,49 +156,33 @@ __global__ void __launch_bounds__(32 * SMALL_STEP_WARPS)
 // One warp per instance: the sign of d from P = vt w mod B^nl and |d| (nl
 // limbs): P itself if its top bit is clear (d <= 0), else B^nl - P.
 __global__ void __launch_bounds__(WARP_CTA)
-    k_ds_mid(const uint64_t *__restrict__ P, int64_t sp, uint64_t *__restrict__ D, int64_t sd,
+    k_ds_mid(const uint64_t *P, int64_t sp, uint64_t *D, int64_t sd,
              int nl, int32_t *neg, int64_t count) {
   const int64_t i = (int64_t)blockIdx.x * (WARP_CTA / 32) + (threadIdx.x >> 5);
   pdl_trigger();
   pdl_wait();
   if (i >= count) return;
-  const uint64_t *p = P + i * sp;
-  uint64_t *d = D + i * sd;
-  const bool ng = (p[nl - 1] >> 63) == 0;
-  if (ng) {
-    for (int j = lane_id(); j < nl; j += 32) d[j] = p[j];
-  } else {
-    warp_addsub<true>(nl, 0u, [&](int j) { return make_ulonglong2(0ull, p[j]); },
-                      [&](int j, uint64_t x) { d[j] = x; });
-  }
+  const bool ng = ds_mid_warp(P + i * sp, D + i * sd, nl);
   if (lane_id() == 0) neg[i] = ng ? 1 : 0;
 }
 
 // One warp per instance: w' = w B^m + Y (d >= 0) or w B^m - Y - 1 (d < 0),
 // Y = floor(P2 / B^s) (ny limbs), into nout limbs of the next iterate record.
 __global__ void __launch_bounds__(WARP_CTA)
-    k_ds_update(const uint64_t *__restrict__ W, int64_t sw, int nw, const uint64_t *__restrict__ Z,
-                int64_t sz, int s, int ny, const int32_t *__restrict__ neg, int m,
-                uint64_t *__restrict__ Wn, int nout, int64_t count) {
+    k_ds_update(const uint64_t *W, int64_t sw, int nw, const uint64_t *Z,
+                int64_t sz, int s, int ny, const int32_t *neg, int m,
+                uint64_t *Wn, int nout, int64_t count) {
   const int64_t i = (int64_t)blockIdx.x * (WARP_CTA / 32) + (threadIdx.x >> 5);
   pdl_trigger();
   pdl_wait();
   if (i >= count) return;
-  const uint64_t *w = W + i * sw, *y = Z + i * sz + s;
-  uint64_t *wn = Wn + i * sw;
-  auto load = [&](int j) {
-    const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
-    return make_ulonglong2(x, j < ny ? y[j] : 0ull);
-  };
-  auto store = [&](int j, uint64_t x) { wn[j] = x; };
-  if (neg[i]) warp_addsub<true>(nout, 1u, load, store);
-  else warp_addsub<false>(nout, 0u, load, store);
+  ds_update_warp(W + i * sw, nw, Z + i * sz + s, ny, neg[i] != 0, m, Wn + i * sw, nout);
 }
 
 // The same two steps with one CTA per instance, for wide records (a warp
 // takes its limbs 32 at a time, one round after the other).
 __global__ void __launch_bounds__(LIN_THREADS_FEW)
-    k_ds_mid_cta(const uint64_t *__restrict__ P, int64_t sp, uint64_t *__restrict__ D, int64_t sd,
+    k_ds_mid_cta(const uint64_t *P, int64_t sp, uint64_t *D, int64_t sd,
                  int nl, int32_t *neg) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   pdl_trigger();
@@ -209,9 +193,9 @@ __global__ void __launch_bounds__(LIN_THREADS_FEW)
 }
 
 __global__ void __launch_bounds__(LIN_THREADS_FEW)
-    k_ds_update_cta(const uint64_t *__restrict__ W, int64_t sw, int nw,
-                    const uint64_t *__restrict__ Z, int64_t sz, int s, int ny,
-                    const int32_t *__restrict__ neg, int m, uint64_t *__restrict__ Wn, int nout) {
+    k_ds_update_cta(const uint64_t *W, int64_t sw, int nw,
+                    const uint64_t *Z, int64_t sz, int s, int ny,
+                    const int32_t *neg, int m, uint64_t *Wn, int nout) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];
   pdl_trigger();
   pdl_wait();
@@ -230,8 +214,8 @@ constexpr int64_t FEW = 128;
 // kernel.  A tensor-core product of this division that gave up at a wait
 // limit (*aborted) voids the results: BIGINT_ETIMEOUT.
 __global__ void __launch_bounds__(LIN_THREADS_FEW)
-    k_ds_finish(const uint64_t *__restrict__ U, int nu, const uint64_t *__restrict__ V, int nv,
-                const uint64_t *__restrict__ R, int64_t sp, uint64_t *Rh, int64_t sd, uint64_t *Qh,
+    k_ds_finish(const uint64_t *U, int nu, const uint64_t *V, int nv,
+                const uint64_t *R, int64_t sp, uint64_t *Rh, int64_t sd, uint64_t *Qh,
                 int64_t sq, int nqh, uint64_t *Qo, int nq, uint64_t *Ro, int32_t *status,
                 const int *aborted) {
   __shared__ uint32_t scr[BLK_SCRATCH_WORDS];

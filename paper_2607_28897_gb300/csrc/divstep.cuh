@@ -97,7 +97,8 @@ __device__ __forceinline__ void ds_small_step(const uint64_t *vt, Step S, const 
 
 // One CTA: the sign of d from P = vt w mod B^nl and |d| (nl limbs): P itself
 // if its top bit is clear (d <= 0; returns true), else B^nl - P.
-__device__ __forceinline__ bool ds_mid_cta(const uint64_t *p, uint64_t *d, int nl, uint32_t *scr) {
+__device__ __forceinline__ bool ds_mid_cta(const uint64_t *__restrict__ p,
+                                           uint64_t *__restrict__ d, int nl, uint32_t *scr) {
   const bool ng = (p[nl - 1] >> 63) == 0;
   if (ng) {
     for (int j = threadIdx.x; j < nl; j += blockDim.x) d[j] = p[j];
@@ -110,8 +111,9 @@ __device__ __forceinline__ bool ds_mid_cta(const uint64_t *p, uint64_t *d, int n
 
 // One CTA: w' = w B^m + Y (d >= 0) or w B^m - Y - 1 (d < 0), Y (ny limbs) =
 // floor(P2 / B^s), into nout limbs of the next iterate.
-__device__ __forceinline__ void ds_update_cta(const uint64_t *w, int nw, const uint64_t *y, int ny,
-                                              bool neg, int m, uint64_t *wn, int nout,
+__device__ __forceinline__ void ds_update_cta(const uint64_t *__restrict__ w, int nw,
+                                              const uint64_t *__restrict__ y, int ny, bool neg,
+                                              int m, uint64_t *__restrict__ wn, int nout,
                                               uint32_t *scr) {
   auto load = [&](int j) {
     const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
@@ -122,13 +124,38 @@ __device__ __forceinline__ void ds_update_cta(const uint64_t *w, int nw, const u
   else blk_addsub<false>(nout, 0u, load, store, scr);
 }
 
+// The same two by one warp.
+__device__ __forceinline__ bool ds_mid_warp(const uint64_t *__restrict__ p,
+                                            uint64_t *__restrict__ d, int nl) {
+  const bool ng = (p[nl - 1] >> 63) == 0;
+  if (ng) {
+    for (int j = lane_id(); j < nl; j += 32) d[j] = p[j];
+  } else {
+    warp_addsub<true>(nl, 0u, [&](int j) { return make_ulonglong2(0ull, p[j]); },
+                      [&](int j, uint64_t x) { d[j] = x; });
+  }
+  return ng;
+}
+__device__ __forceinline__ void ds_update_warp(const uint64_t *__restrict__ w, int nw,
+                                               const uint64_t *__restrict__ y, int ny, bool neg,
+                                               int m, uint64_t *__restrict__ wn, int nout) {
+  auto load = [&](int j) {
+    const uint64_t x = (j >= m && j - m < nw) ? w[j - m] : 0ull;
+    return make_ulonglong2(x, j < ny ? y[j] : 0ull);
+  };
+  auto store = [&](int j, uint64_t x) { wn[j] = x; };
+  if (neg) warp_addsub<true>(nout, 1u, load, store);
+  else warp_addsub<false>(nout, 0u, load, store);
+}
+
 // One CTA: r^ = (u - R) mod B^(nv+1) with R the low nv + 1 limbs of q^ v, the
 // exact correction of q^ (nqcap limbs, in place) and r^, and the results q
 // (nq limbs) and r (nv limbs).  Returns the status.
-__device__ __forceinline__ int ds_finish_cta(const uint64_t *u, int nu, const uint64_t *v, int nv,
-                                             const uint64_t *rr, uint64_t *rh, uint64_t *qh,
-                                             int nqcap, uint64_t *q, int nq, uint64_t *r,
-                                             uint32_t *scr) {
+__device__ __forceinline__ int ds_finish_cta(const uint64_t *__restrict__ u, int nu,
+                                             const uint64_t *__restrict__ v, int nv,
+                                             const uint64_t *__restrict__ rr, uint64_t *rh,
+                                             uint64_t *qh, int nqcap, uint64_t *q, int nq,
+                                             uint64_t *r, uint32_t *scr) {
   {
     auto load = [&](int j) { return make_ulonglong2(j < nu ? u[j] : 0ull, rr[j]); };
     auto store = [&](int j, uint64_t x) { rh[j] = x; };

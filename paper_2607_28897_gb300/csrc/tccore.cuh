@@ -375,7 +375,7 @@ __device__ __forceinline__ uint32_t unbias_h2(uint32_t m) {
 // i - 16 R, so a warp's loads are coalesced; a thread issues the loads of
 // four limbs before it recodes any, so their latencies overlap.
 template <bool XC, int KB = 128>
-__device__ __forceinline__ void fill_x(uint8_t *xs, const uint64_t *x, int nx, int ptot) {
+__device__ __forceinline__ void fill_x(uint8_t *xs, const uint64_t *__restrict__ x, int nx, int ptot) {
   constexpr int U = 4, R = KB / 8, LR = KB == 128 ? 4 : (KB == 64 ? 3 : 2);
   const int total = R * ptot, step = (int)blockDim.x;
   for (int i0 = threadIdx.x; i0 < total; i0 += U * step) {
@@ -404,7 +404,7 @@ __device__ __forceinline__ void fill_x(uint8_t *xs, const uint64_t *x, int nx, i
 
 // The same for the blocks p0 <= p < p1 of 128 digits only, with x's carry
 // digit.
-__device__ __forceinline__ void fill_x_window(uint8_t *xs, const uint64_t *x, int nx, int ptot,
+__device__ __forceinline__ void fill_x_window(uint8_t *xs, const uint64_t *__restrict__ x, int nx, int ptot,
                                               int p0, int p1) {
   constexpr int U = 8;
   const int total = 16 * (p1 - p0), step = (int)blockDim.x;
@@ -685,7 +685,7 @@ __device__ void tc_release(TcCtx &c) {
 //
 // Returns false (and sets c.aborted) if a wait hit its limit.
 template <int NT, int G, bool IW = false, bool XC = true, bool SPLIT = false, int KB = 128>
-__device__ __forceinline__ bool tc_product(TcCtx &c, const uint64_t *x, int nx, const uint64_t *y,
+__device__ __forceinline__ bool tc_product(TcCtx &c, const uint64_t *__restrict__ x, int nx, const uint64_t *__restrict__ y,
                                            int ny, uint64_t *out, int nout, int lo, int tile = 0,
                                            uint64_t *tile_carry = nullptr) {
   constexpr int DRAIN = 2 * NT;                // threads that drain and build

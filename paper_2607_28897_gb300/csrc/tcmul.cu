@@ -35,8 +35,8 @@ namespace tcm {
 // chaining products (the step-batched division) can report it per instance.
 template <int NT, int G, bool XC, int KB = 128>
 __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
-    k_mul_tc(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
-             uint64_t *__restrict__ Out, int nx, int ny, int nout, int64_t count, int64_t sx,
+    k_mul_tc(const uint64_t *X, const uint64_t *Y,
+             uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
              int64_t sy, int64_t so, int lo, int *abort_flag) {
   extern __shared__ __align__(1024) uint8_t sm[];
   __shared__ TcShared sh;
@@ -64,7 +64,7 @@ __global__ void __launch_bounds__(2 * NT + 32, 256 / NT)
 // and 32 W threads per CTA, 512 / (NT ACC) CTAs per SM.  add + i sadd: nout limbs added to product i (null: none).
 template <int NT, int W, bool ADD, int ACC>
 __global__ void __launch_bounds__(32 * W, 512 / (NT * ACC))
-    k_mul_one(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
+    k_mul_one(const uint64_t *X, const uint64_t *Y,
               uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
               int64_t sy, int64_t so, int lo, int *abort_flag, const uint64_t *add,
               int64_t sadd) {
@@ -91,7 +91,7 @@ __global__ void __launch_bounds__(32 * W, 512 / (NT * ACC))
 // The same by the pipeline of tcpipe.cuh: one CTA per SM.
 template <int KB, int NT>
 __global__ void __launch_bounds__(PIPE_THREADS, 1)
-    k_mul_pipe(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y,
+    k_mul_pipe(const uint64_t *X, const uint64_t *Y,
                uint64_t *Out, int nx, int ny, int nout, int64_t count, int64_t sx,
                int64_t sy, int64_t so, int lo, int *abort_flag, const uint64_t *add, int64_t sadd,
                PipeLayout L) {
@@ -155,7 +155,7 @@ struct SkPlan {
 
 template <int NT, int G>
 __global__ void __launch_bounds__(2 * NT + 32, 1)
-    k_mul_tc_sk(const uint64_t *__restrict__ X, const uint64_t *__restrict__ Y, int nx, int ny,
+    k_mul_tc_sk(const uint64_t *X, const uint64_t *Y, int nx, int ny,
                 int64_t sx, int64_t sy, int64_t count, SkPlan P, int *colsum, int64_t cs_stride,
                 int *abort_flag) {
   extern __shared__ __align__(1024) uint8_t sm[];

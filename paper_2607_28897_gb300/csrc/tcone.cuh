@@ -178,7 +178,7 @@ __device__ __forceinline__ void limb_of(const uint32_t (&w)[8], uint64_t add, bo
 // and the one below.
 // A thread issues the loads of two matrices before it recodes either.
 template <int THREADS>
-__device__ __forceinline__ void one_hankel(uint8_t *hk, const uint64_t *y, int ny, int eb, int nb) {
+__device__ __forceinline__ void one_hankel(uint8_t *hk, const uint64_t *__restrict__ y, int ny, int eb, int nb) {
   for (int j0 = threadIdx.x; j0 < nb; j0 += 2 * THREADS) {
     uint64_t v[2][3];
 #pragma unroll
@@ -334,8 +334,8 @@ __device__ void one_release(OneCtx &c) {
 // holds one_layout<W>(nx, ny, blocks of the widest tile).  Returns false
 // (and sets c.aborted) if a wait hit its limit.
 template <int NT, int W, bool ADD = false, int ACC = 1>
-__device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *x, int nx,
-                                            const uint64_t *y, int ny, uint64_t *out, int nout,
+__device__ __forceinline__ bool one_product(OneCtx &c, const uint64_t *__restrict__ x, int nx,
+                                            const uint64_t *__restrict__ y, int ny, uint64_t *out, int nout,
                                             int lo, const uint64_t *add = nullptr) {
   constexpr int THREADS = 32 * W, RUN = 8 * W, NRUN = NT / RUN, S = ONE_S, R = ONE_R;
   constexpr int BUFS = one_bufs<W>();

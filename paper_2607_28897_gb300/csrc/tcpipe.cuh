@@ -169,7 +169,7 @@ __device__ __forceinline__ bool pipe_wait_warp(PipeShared *sh, uint64_t *bar, ui
 // alone would leave the others of its warp at the next __syncwarp for ever.
 // x into the B layout (fill_x without the carry digit), by the builders.
 template <int KB>
-__device__ __forceinline__ void pipe_fill(uint8_t *xs, const uint64_t *x, int nx, int t) {
+__device__ __forceinline__ void pipe_fill(uint8_t *xs, const uint64_t *__restrict__ x, int nx, int t) {
   constexpr int U = 4, R = KB / 8, LR = KB == 128 ? 4 : (KB == 64 ? 3 : 2), STEP = 32 * PIPE_BUILD;
   const int ptot = pipe_ptot<KB>(nx), total = R * ptot;
   for (int i0 = t; i0 < total; i0 += U * STEP) {
