@@ -17,8 +17,9 @@
 // operands (top limb of v nonzero, "regular") the same precision k = nv - 1
 // and the exponent h = nu, so the Newton schedule (l, m, t per step) is
 // known on the host.  Instances whose divisor has a zero top limb
-// (including v = 0) take the one-CTA-per-division kernel in a last launch;
-// the step kernels run over them too (their values are never used, and
+// (including v = 0) are listed and divided in a last launch, a warp each
+// (k_ds_listed) or, longer ones, a CTA each (divmod.cu); the step kernels run
+// over them too (their values are never used, and
 // every size is fixed, so nothing reads out of bounds).
 //
 // Per step, with the iterate w ~ B^(k+l) / v kept to l + 2 limbs,
@@ -210,8 +211,8 @@ constexpr int64_t FEW = 128;
 
 // One CTA per regular instance: r^ = (u - R) mod B^(nv+1) with R the low
 // nv + 1 limbs of q^ v, the exact correction of q^ (in place: the top limbs
-// of the banded product) and r^ (divmod.cu), and the results.  Irregular instances are left to the one-CTA-per-division
-// kernel.  A tensor-core product of this division that gave up at a wait
+// of the banded product) and r^ (divmod.cu), and the results.  Irregular
+// instances are left to the last launch.  A tensor-core product of this division that gave up at a wait
 // limit (*aborted) voids the results: BIGINT_ETIMEOUT.
 __global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_finish(const uint64_t *U, int nu, const uint64_t *V, int nv,
@@ -231,6 +232,186 @@ __global__ void __launch_bounds__(LIN_THREADS_FEW)
                          scr);
   if (*(volatile const int *)aborted) st = BIGINT_ETIMEOUT;
   if (status != nullptr && threadIdx.x == 0) status[i] = st;
+}
+
+// ---------------------------------------------------------------------------
+// The listed instances of short shapes: long division by 64-bit digits (Knuth's
+// Algorithm D), one warp per instance, everything in shared memory.  Any divisor
+// and quotient: v = 0, a quotient beyond nq limbs, u < v.
+//
+// Why: the one-CTA-per-division kernel takes the Newton steps again, one CTA's
+// block barriers after the other, on top of the steps the batch has just been
+// through.  Batches of divisors that all have a zero top limb (padded arrays):
+// 300 of 144 by 96 limbs 149 -> 85 us, 20000 of 64 by 32 limbs 2736 -> 362 (99
+// and 2450 without the step form).  Bound by latency: a quotient limb takes 0.3 us
+// below 32 divisor limbs, 0.5 us at 127, so that the longest quotients taken
+// here are no faster than a CTA's (one of 508 by 127 limbs 292 us, of which the
+// steps 97; 341 with the CTA form in this place), and longer ones stay there.
+// ---------------------------------------------------------------------------
+constexpr int LIST_WARPS = 4, LIST_NV = 128, LIST_NU = 512;
+constexpr int64_t LIST_CTAS = 2048;  // more than are ever resident; they loop over the list
+__host__ __device__ inline bool list_warps_ok(int nu, int nv) {
+  return nv < LIST_NV && nu <= LIST_NU;
+}
+__host__ __device__ inline int list_warp_limbs(int nu, int nv) { return nu + 1 + nv; }
+
+// One warp: precision of x[0 .. n).
+__device__ __forceinline__ int warp_prec(const uint64_t *x, int n) {
+  for (int base = (n - 1) & ~31; base >= 0; base -= 32) {
+    const int j = base + (int)lane_id();
+    const uint32_t nz = __ballot_sync(FULL, j < n && x[j] != 0);
+    if (nz) return base + 32 - __clz((int)nz);
+  }
+  return 0;
+}
+
+// One warp: x (nx limbs) shifted up by s bits (s < 64) into out, n >= nx limbs.
+__device__ __forceinline__ void warp_shl(const uint64_t *x, int nx, int s, uint64_t *out, int n) {
+  for (int j = lane_id(); j < n; j += 32) {
+    const uint64_t a = j < nx ? x[j] : 0ull, b = j >= 1 && j - 1 < nx ? x[j - 1] : 0ull;
+    out[j] = s ? a << s | b >> (64 - s) : a;
+  }
+}
+
+// One warp: x[0 .. n] -= d y[0 .. n), n < 32 R, x in shared memory, lane i's R
+// limbs of y from limb R i on in its registers (zero from n on); the borrow out
+// of limb n (d one too large).  A lane subtracts the low R limbs of its product
+// and the high word of the lane's below, then what that one borrowed (at most
+// 2), and one scan settles the rest.
+template <int R>
+__device__ __forceinline__ bool warp_submul(uint64_t *x, const uint64_t (&y)[R], int n, uint64_t d) {
+  const int lane = (int)lane_id(), j0 = R * lane;
+  uint64_t t[R], hi = 0;
+  uint32_t c = 0;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint64_t lo = d * y[r] + hi;  // hi <= B - 2 before, so no overflow after
+    hi = __umul64hi(d, y[r]) + (lo < hi);
+    const uint64_t xv = j0 + r <= n ? x[j0 + r] : 0ull;
+    const uint64_t u = xv - lo;
+    t[r] = u - c;
+    c = (uint32_t)(xv < lo) + (uint32_t)(u < c);
+  }
+  uint64_t in = __shfl_up_sync(FULL, hi, 1);
+  if (lane == 0) in = 0;
+  uint64_t b = in;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint64_t u = t[r];
+    t[r] = u - b;
+    b = u < b;
+  }
+  c += (uint32_t)b;
+  uint32_t cb = __shfl_up_sync(FULL, c, 1);
+  if (lane == 0) cb = 0;
+  b = cb;
+  uint64_t any = 0;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint64_t u = t[r];
+    t[r] = u - b;
+    b = u < b;
+    any |= t[r];
+  }
+  const uint64_t bm = warp_carries(warp_gp((uint32_t)b, b == 0 && any == 0), 0);
+  b = (bm >> lane) & 1u;
+#pragma unroll
+  for (int r = 0; r < R; r++) {
+    const uint64_t u = t[r];
+    if (j0 + r <= n) x[j0 + r] = u - b;
+    b = u < b;
+  }
+  return __shfl_sync(FULL, c, 31) != 0 || (bm >> 32) != 0;
+}
+
+// One warp: the quotient digits of un / vn (normalised: vn of pv < 32 R limbs,
+// bit 63 of the last set), L of them, into q (nq limbs); un becomes the
+// remainder.  False if the quotient does not fit.
+template <int R>
+__device__ __forceinline__ bool warp_longdiv(uint64_t *un, const uint64_t *vn, int pv, int L,
+                                             uint64_t *q, int nq) {
+  typedef unsigned __int128 u128;
+  const int lane = (int)lane_id();
+  const uint64_t vt = vn[pv - 1], v2 = pv > 1 ? vn[pv - 2] : 0ull;
+  const uint64_t rec = (uint64_t)((((u128)~vt << 64) | ~0ull) / vt);  // floor((B^2 - 1) / vt) - B
+  uint64_t y[R];
+#pragma unroll
+  for (int r = 0; r < R; r++) y[r] = R * lane + r < pv ? vn[R * lane + r] : 0ull;
+  bool fits = true;
+  for (int j = L - 1; j >= 0; j--) {
+    // the digit from the top limbs (Moeller and Granlund, as divcore.cuh's
+    // small_div), at most one too large
+    const uint64_t n1 = un[j + pv], n0 = un[j + pv - 1], n2 = pv > 1 ? un[j + pv - 2] : 0ull;
+    uint64_t d = ~0ull;
+    u128 rh = (u128)n0 + vt;
+    if (n1 < vt) {
+      const u128 f = (u128)rec * n1 + (((u128)n1 << 64) | n0);
+      d = (uint64_t)(f >> 64) + 1;
+      uint64_t r0 = n0 - d * vt;
+      if (r0 > (uint64_t)f) {
+        d--;
+        r0 += vt;
+      }
+      if (r0 >= vt) {
+        d++;
+        r0 -= vt;
+      }
+      rh = r0;
+    }
+    for (int k = 0; k < 2 && (rh >> 64) == 0 && (u128)d * v2 > ((rh << 64) | n2); k++) {
+      d--;
+      rh += vt;
+    }
+    __syncwarp();
+    if (warp_submul<R>(un + j, y, pv, d)) {
+      d--;
+      __syncwarp();
+      warp_addsub<false>(pv, 0u, [&](int k) { return make_ulonglong2(un[j + k], vn[k]); },
+                         [&](int k, uint64_t x) { un[j + k] = x; });
+    }
+    __syncwarp();
+    if (j < nq) {
+      if (lane == 0) q[j] = d;
+    } else if (d != 0) {
+      fits = false;
+    }
+  }
+  return fits;
+}
+
+__global__ void __launch_bounds__(32 * LIST_WARPS)
+    k_ds_listed(const uint64_t *U, int nu, const uint64_t *V, int nv, uint64_t *Qo, int nq,
+                uint64_t *Ro, int32_t *status, const int32_t *list, const int *nlist) {
+  extern __shared__ __align__(16) uint64_t lsm[];
+  const int lane = (int)lane_id(), wi = (int)(threadIdx.x >> 5), n = *nlist;
+  uint64_t *un = lsm + (size_t)wi * list_warp_limbs(nu, nv), *vn = un + nu + 1;
+  for (int64_t e = (int64_t)blockIdx.x * LIST_WARPS + wi; e < n; e += (int64_t)gridDim.x * LIST_WARPS) {
+    const int64_t i = list[e];
+    const uint64_t *u = U + i * nu, *v = V + i * nv;
+    uint64_t *q = Qo + i * nq, *r = Ro + i * nv;
+    const int pv = warp_prec(v, nv), pu = warp_prec(u, nu);
+    int st = pv == 0 ? BIGINT_EDIVZERO : BIGINT_OK;
+    const int L = pv > 0 && pu >= pv ? pu - pv + 1 : 0;  // limbs the quotient may have
+    for (int j = L + lane; j < nq; j += 32) q[j] = 0;
+    if (L == 0) {  // v = 0: q = r = 0; u < v: r = u
+      for (int j = lane; j < nv; j += 32) r[j] = pv > 0 && j < pu ? u[j] : 0ull;
+    } else {
+      const int s = __clzll((long long)v[pv - 1]);
+      warp_shl(v, pv, s, vn, pv);
+      warp_shl(u, pu, s, un, pu + 1);
+      __syncwarp();
+      const bool fits = pv < 32 ? warp_longdiv<1>(un, vn, pv, L, q, nq)
+                                : (pv < 64 ? warp_longdiv<2>(un, vn, pv, L, q, nq)
+                                           : warp_longdiv<4>(un, vn, pv, L, q, nq));
+      if (!fits) st = BIGINT_ERANGE;
+      for (int j = lane; j < nv; j += 32) {
+        const uint64_t a = j < pv ? un[j] : 0ull, b = j + 1 < pv ? un[j + 1] : 0ull;
+        r[j] = s ? a >> s | b << (64 - s) : a;
+      }
+    }
+    if (status != nullptr && lane == 0) status[i] = st;
+    __syncwarp();
+  }
 }
 
 // The Newton schedule of a regular instance.
@@ -333,8 +514,7 @@ bool divmod_steps_default(int64_t count, int nu, int nv) {
 }
 
 // q = floor(u / v), r = u - q v for a uniform batch, step by step across the
-// batch (see the top of this file); irregular instances by the
-// one-CTA-per-division kernel at the end.
+// batch (see the top of this file); irregular instances at the end.
 // ws: ws_bytes for the step records (the one-CTA-per-division kernel's
 // per-instance regions, reused); list_and_counters: 4 count bytes rounded to
 // 256, then two ints, OUTSIDE those regions (that kernel reads the list
@@ -437,8 +617,15 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   rc = chain_launch(few, k_ds_finish, (unsigned)count, lin, 0, st, u, nu, v, nv, P, Y.sp, D, Y.sd,
                     Z + h, Y.sz, nqh, q, nq, r, status, ctr + 1);
   if (rc != BIGINT_OK) return rc;
-  // the irregular instances, one CTA per division (the workspace is free
-  // again: everything above is stream-ordered before this launch)
+  // the irregular instances: a warp each, or one CTA per division (the workspace
+  // is free again: everything above is stream-ordered before this launch)
+  if (list_warps_ok(nu, nv)) {
+    const int64_t ctas = (count + LIST_WARPS - 1) / LIST_WARPS;
+    k_ds_listed<<<(unsigned)(ctas < LIST_CTAS ? ctas : LIST_CTAS), 32 * LIST_WARPS,
+                  8 * LIST_WARPS * (size_t)list_warp_limbs(nu, nv), st>>>(u, nu, v, nv, q, nq, r,
+                                                                          status, list, ctr);
+    return bigint_launch_status();
+  }
   return launch_divmod_cta(u, v, q, r, status, count, nu, nv, ws, list, ctr, st);
 }
 

@@ -172,3 +172,43 @@ def test_long_quotients(bi, orc, nu, nv, mul):
     oq, orr, est = expect(bi, orc, u, v)
     assert np.array_equal(st, est)
     assert np.array_equal(q, oq) and np.array_equal(r, orr)
+
+
+@pytest.mark.parametrize("nu,nv", [(8, 8), (9, 8), (12, 8), (16, 8), (40, 12), (64, 33), (97, 96),
+                                   (130, 127), (200, 100), (140, 8), (256, 127), (300, 40),
+                                   (512, 127), (513, 127), (512, 8), (513, 8)])
+def test_zero_topped_divisors(bi, orc, nu, nv):
+    """Short divisors with every number of zero top limbs beside regular ones,
+    below dividends with as many, one fewer and none (a quotient that may not
+    fit), and a zero divisor: the step form lists them for one warp each, about
+    the longest dividends it takes and beyond for one CTA each."""
+    from paper_2607_28897_gb300 import inputs
+
+    count = 3 * nv + 2
+    u = inputs.limbs(nu * 19 + nv, count, nu, top_nonzero=True)
+    v = inputs.limbs(nu * 23 + nv, count, nv, top_nonzero=True)
+    v[1::2, :nv // 2] = np.uint64(2**64 - 1)
+    for s in range(nv + 1):
+        for k in range(3):
+            i = 3 * s + k
+            if i >= count:
+                break
+            v[i, nv - s:] = 0
+            if 0 < s < nv and s % 2:
+                v[i, nv - s - 1] = np.uint64(1)
+            zeros = s if k == 0 else (max(s - 1, 0) if k == 1 else 0)
+            u[i, nu - zeros:] = 0
+    oq, orr, est = expect(bi, orc, u, v)
+    for variant in (3, 1):
+        q, r, st = run(bi, u, v, variant)
+        assert np.array_equal(st, est), variant
+        assert np.array_equal(q, oq) and np.array_equal(r, orr), variant
+    # every divisor zero-topped, as a caller's padded array has them
+    u[:, nu - 1] = 0
+    v[:, nv - 1] = 0
+    v[:, nv - 2] |= np.uint64(1)
+    oq, orr, est = expect(bi, orc, u, v)
+    for n in (1, count):
+        q, r, st = run(bi, u[:n], v[:n], 3)
+        assert np.array_equal(st, est[:n])
+        assert np.array_equal(q, oq[:n]) and np.array_equal(r, orr[:n])
