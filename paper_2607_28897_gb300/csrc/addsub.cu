@@ -232,18 +232,6 @@ struct Shape {
 constexpr int MANY = 3;
 constexpr int64_t MANY_LIMBS = 3 << 20, HALF_LIMBS = 2048;
 
-static int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0, v = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess ||
-        cudaDeviceGetAttribute(&v, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
-      return 0;
-    sms = v;
-  }
-  return sms;
-}
-
 template <int MODE, int LPL>
 static Shape shape_of(int64_t count, int n) {
   constexpr int ROUND = 32 * LPL;  // limbs of a warp's round

@@ -164,7 +164,7 @@ bool op_tc(const bigint_op &o) {
   return false;
 }
 
-int op_tc_words(const bigint_op &o, int max_words) {
+int op_tc_words(const bigint_op &o) {
   int ns, nl;
   if (o.op == BIGINT_OP_MUL) {
     ns = std::min(o.na, o.nb);
@@ -175,9 +175,7 @@ int op_tc_words(const bigint_op &o, int max_words) {
   } else {
     return 0;
   }
-  const int w8 = (int)(tcm::layout<256, 8>(ns, nl).total / 4);
-  const int w4 = (int)(tcm::layout<256, 4>(ns, nl).total / 4);
-  return w8 <= max_words ? w8 : w4;
+  return (int)(tcm::layout<256, 8>(ns, nl).total / 4);
 }
 
 int op_units(const bigint_op &o) {
@@ -334,7 +332,7 @@ int batch_configure(bigint_batch *B) {
     units = std::max(units, op_units(o));
     if (B->use_tc && op_tc(o)) {
       tc = true;
-      tc_words = std::max(tc_words, op_tc_words(o, max_words_tc));
+      tc_words = std::max(tc_words, op_tc_words(o));
     }
   }
   Launch &P = B->persistent;
@@ -371,7 +369,7 @@ int batch_configure(bigint_batch *B) {
       u = std::max(u, op_units(o));
       if (B->use_tc && op_tc(o)) {
         ltc = true;
-        tw = std::max(tw, op_tc_words(o, max_words_tc));
+        tw = std::max(tw, op_tc_words(o));
       }
       j++;
     }

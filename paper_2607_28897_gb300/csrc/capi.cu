@@ -27,13 +27,11 @@ int launch_mul_kara(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t
 int mul_set_variant(int v);
 int mul_variant_for(int na, int nb, int nout);
 int tc_take_timeout();
-int programs_take_timeout();
 int div_take_timeout();
 int batch_take_timeout();
 int rag_take_timeout();
 int tc_set_wait_limit(long long cycles);
 int div_set_wait_limit(long long cycles);
-int programs_set_wait_limit(long long cycles);
 int batch_set_wait_limit(long long cycles);
 int rag_set_wait_limit(long long cycles);
 int launch_add_chain(const uint64_t *a, const uint64_t *b, uint64_t *out, uint8_t *carry,
@@ -303,8 +301,8 @@ int bigint_host_sync(void) { return host_sync(); }
 int bigint_check_timeout(void) {
   // every translation unit that launches tensor-core products keeps its own
   // record: ask them all (each read clears it)
-  const int rc[5] = {tc_take_timeout(), div_take_timeout(), programs_take_timeout(),
-                     batch_take_timeout(), rag_take_timeout()};
+  const int rc[4] = {tc_take_timeout(), div_take_timeout(), batch_take_timeout(),
+                     rag_take_timeout()};
   int out = BIGINT_OK;
   for (int x : rc) {
     if (x == BIGINT_ECUDA) return BIGINT_ECUDA;
@@ -318,9 +316,8 @@ unsigned long long bigint_kernel_launches(void) {
 }
 
 int bigint_set_wait_limit(long long cycles) {
-  const int rc[5] = {tc_set_wait_limit(cycles), div_set_wait_limit(cycles),
-                     programs_set_wait_limit(cycles), batch_set_wait_limit(cycles),
-                     rag_set_wait_limit(cycles)};
+  const int rc[4] = {tc_set_wait_limit(cycles), div_set_wait_limit(cycles),
+                     batch_set_wait_limit(cycles), rag_set_wait_limit(cycles)};
   for (int x : rc)
     if (x != BIGINT_OK) return x;
   return BIGINT_OK;

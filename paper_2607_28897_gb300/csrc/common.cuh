@@ -6,6 +6,7 @@
 // limb pointer as a digit pointer.
 #pragma once
 
+#include <atomic>
 #include <cstdint>
 #include <cuda_runtime.h>
 
@@ -104,6 +105,20 @@ static inline int bigint_cuda_error() {
 namespace bigint {
 // Counts the kernel launches the library enqueues (bigint_kernel_launches).
 void count_launch();
+
+// SMs of the current device (0: a CUDA error).
+inline int sm_count() {
+  static std::atomic<int> sms{0};
+  int n = sms.load(std::memory_order_relaxed);
+  if (n == 0) {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess)
+      return 0;
+    sms.store(n, std::memory_order_relaxed);
+  }
+  return n;
+}
 
 // Column sums of a chain of split-K products: two buffers of `bytes`, all
 // zero at the start; a product takes buf[cur], and its finish clears what the

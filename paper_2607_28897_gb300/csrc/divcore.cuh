@@ -179,10 +179,9 @@ __device__ Work carve(uint64_t *base, int nu, int nv, int h) {
 // 512 TMEM columns (tccore.cuh; the last warp issues the MMAs), as one
 // out-of-line copy.
 // ---------------------------------------------------------------------------
-template <int G>
 __device__ __noinline__ bool tc_call(tcm::TcCtx *c, const uint64_t *x, int nx, const uint64_t *y,
                                      int ny, uint64_t *out, int nout, int lo) {
-  return tcm::tc_product<256, G, true>(*c, x, nx, y, ny, out, nout, lo);
+  return tcm::tc_product<256, 8, true>(*c, x, nx, y, ny, out, nout, lo);
 }
 
 // out[0..nout) = x * y on the tensor cores when the shorter operand has
@@ -218,17 +217,13 @@ __device__ __forceinline__ bool tc_mul(tcm::TcCtx *tc, const uint64_t *x, int nx
   // MMAs (a low product whose longer operand has most of the columns: an
   // MMA narrower than ~136 columns costs its A operand's read, so fewer,
   // wider MMAs win) and the longer one fits shared memory as x
-  if (ns != nl && tcm::layout<256, 4>(nl, ns).total <= bytes &&
+  if (ns != nl && tcm::layout<256, 8>(nl, ns).total <= bytes &&
       tc_blocks256(nl, ns, no, lo) < tc_blocks256(ns, nl, no, lo)) {
     const uint64_t *t = xs; xs = ys; ys = t;
     const int tn = ns; ns = nl; nl = tn;
   }
-  if (tcm::layout<256, 8>(ns, nl).total <= bytes)
-    tc_call<8>(tc, xs, ns, ys, nl, out, no, lo);
-  else if (tcm::layout<256, 4>(ns, nl).total <= bytes)
-    tc_call<4>(tc, xs, ns, ys, nl, out, no, lo);
-  else
-    return false;
+  if (tcm::layout<256, 8>(ns, nl).total > bytes) return false;
+  tc_call(tc, xs, ns, ys, nl, out, no, lo);
   for (int j = no + (int)threadIdx.x; j < nout; j += blockDim.x) out[j] = 0;
   __syncthreads();
   return true;

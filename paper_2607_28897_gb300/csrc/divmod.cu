@@ -242,10 +242,7 @@ static int launch_div_variant(const uint64_t *u, const uint64_t *v, uint64_t *q,
   int need = blk_mul_smem_words<RB, Q>(H, H);
   if (TC) {  // tensor-core products: shorter operand up to max(H - nv, nv) + a few limbs
     const int ns = (H - nv > nv ? H - nv : nv) + 8;
-    const tcm::Layout L8 = tcm::layout<256, 8>(ns, H + 8);
-    const tcm::Layout L4 = tcm::layout<256, 4>(ns, H + 8);
-    const int w8 = (int)(L8.total / 4), w4 = (int)(L4.total / 4);
-    const int tcw = w8 <= smem_words ? w8 : w4;
+    const int tcw = (int)(tcm::layout<256, 8>(ns, H + 8).total / 4);
     if (tcw > need) need = tcw;
   }
   if (need < smem_words) smem_words = need;
@@ -265,12 +262,8 @@ static int launch_div_variant(const uint64_t *u, const uint64_t *v, uint64_t *q,
   const int64_t stride = ws_limbs(nu, nv, hcap);
   int64_t grid = count;
   if (x.list != nullptr) {  // a listed subset: as many CTAs as fit loop over it
-    static int sms = 0;
-    if (sms == 0) {
-      int dev = 0;
-      BIGINT_CUDA_TRY(cudaGetDevice(&dev));
-      BIGINT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
-    }
+    const int sms = sm_count();
+    if (sms == 0) return BIGINT_ECUDA;
     int per = 1;
     if (!TC && grid > sms)
       BIGINT_CUDA_TRY(cudaOccupancyMaxActiveBlocksPerMultiprocessor(

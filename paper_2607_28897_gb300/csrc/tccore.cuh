@@ -53,9 +53,8 @@
 //
 // Schedule: a persistent CTA of 2 NT drain threads and one issuer warp loops
 // over instances; per instance over tiles of NT output columns; per tile
-// over groups of G Toeplitz blocks (8; 7 for NT = 64; 4 when the longer
-// Hankel buffers do not fit).  Fewer, larger groups matter: every drain
-// reads the whole accumulator out of tensor memory.  The issuer warp's lane
+// over groups of G Toeplitz blocks (8; 7 for NT = 64).  Fewer, larger groups
+// matter: every drain reads the whole accumulator out of tensor memory.  The issuer warp's lane
 // 0 issues a group's MMAs into one of two NT-column fp32 accumulators in
 // tensor memory and commits them to an mbarrier (it blocks on the tensor
 // core's shallow instruction queue for most of a group, hence a warp of its

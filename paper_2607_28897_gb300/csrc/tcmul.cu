@@ -374,8 +374,7 @@ static size_t tc_smem(int nx, int ny) {
   return d > 0 && L.total <= (uint32_t)d ? L.total : 0;
 }
 
-// Shared memory of a shape for x of nx and y of ny limbs, 0 if it does not
-// fit (the 256-column tile falls back to groups of 4 blocks).
+// Shared memory of a shape for x of nx and y of ny limbs, 0 if it does not fit.
 static size_t shape_smem(TcShape sh, int nx, int ny) {
   switch (sh) {
     case TC_64_XC: return tc_smem<64, 7, true, 128>(nx, ny);
@@ -386,10 +385,7 @@ static size_t shape_smem(TcShape sh, int nx, int ny) {
     case TC_N64_NOXC: return tc_smem<128, 15, false, 64>(nx, ny);
     case TC_N32_XC: return tc_smem<128, 12, true, 32>(nx, ny);
     case TC_N32_NOXC: return tc_smem<128, 12, false, 32>(nx, ny);
-    default: {
-      const size_t s8 = tc_smem<256, 8, true, 128>(nx, ny);
-      return s8 ? s8 : tc_smem<256, 4, true, 128>(nx, ny);
-    }
+    default: return tc_smem<256, 8, true, 128>(nx, ny);
   }
 }
 
@@ -437,16 +433,6 @@ static int tc_per_sm(size_t smem) {
   return per_sm < 1 ? 1 : per_sm;
 }
 
-static int sm_count() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  }
-  return sms;
-}
-
 template <int NT, int G, bool XC, int KB>
 static int launch_tc(const TcArgs &A, int64_t count, int nx, int ny, int nout, cudaStream_t st) {
   const size_t smem = tc_smem<NT, G, XC, KB>(nx, ny);
@@ -471,10 +457,7 @@ static int launch_shape(TcShape sh, const TcArgs &A, int64_t count, int nx, int 
     case TC_N64_NOXC: return launch_tc<128, 15, false, 64>(A, count, nx, ny, nout, st);
     case TC_N32_XC: return launch_tc<128, 12, true, 32>(A, count, nx, ny, nout, st);
     case TC_N32_NOXC: return launch_tc<128, 12, false, 32>(A, count, nx, ny, nout, st);
-    default:
-      return tc_smem<256, 8, true, 128>(nx, ny)
-                 ? launch_tc<256, 8, true, 128>(A, count, nx, ny, nout, st)
-                 : launch_tc<256, 4, true, 128>(A, count, nx, ny, nout, st);
+    default: return launch_tc<256, 8, true, 128>(A, count, nx, ny, nout, st);
   }
 }
 
@@ -794,11 +777,7 @@ static int launch_form(int form, TcArgs A, bool sw, int64_t count, int nx, int n
 }
 
 // out = low n limbs of a b + c for a batch of n-limb operands (instance i at
-// a + i sa, ...; c may be null or out), by a form that takes an addend.
-bool mul_add_ok(int n) {
-  bool sw = false;
-  return n >= 64 && best_form(n, n, n, 0, -1, &sw) >= 0;
-}
+// a + i sa, ...; c may be null or out), n >= 64, by a form that takes an addend.
 int launch_mul_add(const uint64_t *a, const uint64_t *b, const uint64_t *c, uint64_t *out,
                    int64_t count, int n, cudaStream_t st) {
   bool sw = false;
@@ -899,7 +878,8 @@ int launch_mul_tc(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t c
 // ---- split-K products (host) --------------------------------------------------
 namespace {
 
-template <int G>
+constexpr int SK_G = 8;  // Toeplitz blocks per group
+
 int sk_dyn_max() {
   static int dyn = -1;
   if (dyn < 0) {
@@ -909,9 +889,9 @@ int sk_dyn_max() {
         cudaSuccess)
       return 0;
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, tcm::k_mul_tc_sk<256, G>) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, tcm::k_mul_tc_sk<256, SK_G>) != cudaSuccess) return 0;
     const int d = optin - (int)fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(tcm::k_mul_tc_sk<256, G>,
+    if (cudaFuncSetAttribute(tcm::k_mul_tc_sk<256, SK_G>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, d) != cudaSuccess)
       return 0;
     dyn = d;
@@ -919,20 +899,10 @@ int sk_dyn_max() {
   return dyn;
 }
 
-int sm_count_cached() {
-  static int sms = 0;
-  if (sms == 0) {
-    int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess) return 0;
-    if (cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) return 0;
-  }
-  return sms;
-}
-
 // Tiles of 256 columns of the low nout limbs of x * y (x with its carry
 // digit) from the column of limb lo on, as tc_product computes them; groups
-// of G blocks per tile.  Returns false if there are more than SK_MAX_TILES.
-bool sk_tiles(int nx, int ny, int nout, int lo, int G, tcm::SkPlan &P, int *groups) {
+// of SK_G blocks per tile.  Returns false if there are more than SK_MAX_TILES.
+bool sk_tiles(int nx, int ny, int nout, int lo, tcm::SkPlan &P, int *groups) {
   const int mx = (8 * nx + 1 + 127) / 128, ey = (8 * ny + 127) / 128, ctot = mx + ey;
   P.cfirst = lo > 0 ? lo / 16 : 0;
   P.T = 0;
@@ -946,7 +916,7 @@ bool sk_tiles(int nx, int ny, int nout, int lo, int G, tcm::SkPlan &P, int *grou
     const int e_lo = c0 - mx + 1 > 0 ? c0 - mx + 1 : 0, e_hi = c0 + W - 1 < ey ? c0 + W - 1 : ey;
     P.c0[P.T] = c0;
     P.W[P.T] = W;
-    groups[P.T] = e_hi >= e_lo ? (e_hi - e_lo + G) / G : 0;
+    groups[P.T] = e_hi >= e_lo ? (e_hi - e_lo + SK_G) / SK_G : 0;
     P.T++;
   }
   return P.T > 0;
@@ -966,8 +936,8 @@ size_t mul_sk_bytes_per_product(int na, int nb, int nout, int lo) {
   int groups[tcm::SK_MAX_TILES];
   if (nx < 1 || nx > 16383 || ny > 32768 || nout < 1 || nout > na + nb || lo < 0 || lo >= nout)
     return 0;
-  if (tcm::layout<256, 4, true>(nx, ny).total > SK_SMEM_CAP) return 0;
-  if (!sk_tiles(nx, ny, nout, lo, 8, P, groups)) return 0;
+  if (tcm::layout<256, SK_G>(nx, ny).total > SK_SMEM_CAP) return 0;
+  if (!sk_tiles(nx, ny, nout, lo, P, groups)) return 0;
   return (size_t)P.T * 256 * 128 * sizeof(int);
 }
 
@@ -980,8 +950,8 @@ bool mul_sk_worth(int64_t count, int na, int nb, int nout, int lo) {
   if (nx <= tcm::ONE_MAX || mul_sk_bytes_per_product(na, nb, nout, lo) == 0) return false;
   tcm::SkPlan P;
   int groups[tcm::SK_MAX_TILES];
-  if (!sk_tiles(nx, ny, nout, lo, 8, P, groups)) return false;
-  const int sms = sm_count_cached();
+  if (!sk_tiles(nx, ny, nout, lo, P, groups)) return false;
+  const int sms = sm_count();
   return sms > 0 && count * P.T * 2 <= sms;
 }
 
@@ -1003,18 +973,13 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
     return BIGINT_EINVAL;
   const size_t per = mul_sk_bytes_per_product(na, nb, nout, lo);
   if (per == 0 || colsum == nullptr || colsum_bytes < per * (size_t)count) return BIGINT_EINVAL;
-  const int sms = sm_count_cached();
+  const int sms = sm_count();
   if (sms == 0) return BIGINT_ECUDA;
-  int G = 8;
-  size_t smem = tcm::layout<256, 8, true>(nx, ny).total;
-  if (sk_dyn_max<8>() <= 0 || smem > (size_t)sk_dyn_max<8>()) {
-    G = 4;
-    smem = tcm::layout<256, 4, true>(nx, ny).total;
-    if (sk_dyn_max<4>() <= 0 || smem > (size_t)sk_dyn_max<4>()) return BIGINT_EINVAL;
-  }
+  const size_t smem = tcm::layout<256, SK_G>(nx, ny).total;
+  if (sk_dyn_max() <= 0 || smem > (size_t)sk_dyn_max()) return BIGINT_EINVAL;
   tcm::SkPlan P;
   int groups[tcm::SK_MAX_TILES];
-  if (!sk_tiles(nx, ny, nout, lo, G, P, groups)) return BIGINT_EINVAL;
+  if (!sk_tiles(nx, ny, nout, lo, P, groups)) return BIGINT_EINVAL;
   // groups per unit: about one unit per SM over the whole launch (each unit
   // first stages x and its first Hankel buffer, so units are not cut finer)
   int64_t total = 0;
@@ -1038,8 +1003,7 @@ int launch_mul_tc_sk(const uint64_t *a, int64_t sa, const uint64_t *b, int64_t s
   }
   const int64_t stride = (int64_t)(per / sizeof(int));
   const unsigned grid = (unsigned)(units < sms ? units : sms);
-  int rc = chain_launch(true, G == 8 ? tcm::k_mul_tc_sk<256, 8> : tcm::k_mul_tc_sk<256, 4>, grid,
-                        2 * 256 + 32, smem, st, x, y, nx, ny, sx, sy, count, P,
+  int rc = chain_launch(true, tcm::k_mul_tc_sk<256, SK_G>, grid, 2 * 256 + 32, smem, st, x, y, nx, ny, sx, sy, count, P,
                         static_cast<int *>(colsum), stride, abort_flag);
   if (rc != BIGINT_OK) return rc;
   const int L0 = 16 * P.cfirst;
@@ -1059,9 +1023,8 @@ int launch_mul(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t coun
 
 namespace {
 
-constexpr int SPLIT_NT = 256, SPLIT_TILE_LIMBS = 16 * SPLIT_NT;
+constexpr int SPLIT_NT = 256, SPLIT_G = 8, SPLIT_TILE_LIMBS = 16 * SPLIT_NT;
 
-template <int G>
 int split_dyn_max() {
   static int dyn = -1;
   if (dyn < 0) {
@@ -1071,9 +1034,9 @@ int split_dyn_max() {
         cudaSuccess)
       return 0;
     cudaFuncAttributes fa;
-    if (cudaFuncGetAttributes(&fa, tcm::k_mul_tc_split<SPLIT_NT, G>) != cudaSuccess) return 0;
+    if (cudaFuncGetAttributes(&fa, tcm::k_mul_tc_split<SPLIT_NT, SPLIT_G>) != cudaSuccess) return 0;
     const int d = optin - (int)fa.sharedSizeBytes;
-    if (cudaFuncSetAttribute(tcm::k_mul_tc_split<SPLIT_NT, G>,
+    if (cudaFuncSetAttribute(tcm::k_mul_tc_split<SPLIT_NT, SPLIT_G>,
                              cudaFuncAttributeMaxDynamicSharedMemorySize, d) != cudaSuccess)
       return 0;
     dyn = d;
@@ -1081,18 +1044,17 @@ int split_dyn_max() {
   return dyn;
 }
 
-template <int G>
 int launch_split(const uint64_t *x, const uint64_t *y, uint64_t *out, int64_t count, int nx, int ny,
                  int T, uint64_t *tile_carry, cudaStream_t st) {
-  const size_t smem = tcm::layout<SPLIT_NT, G>(nx, ny).total;
-  const int dyn = split_dyn_max<G>();
+  const size_t smem = tcm::layout<SPLIT_NT, SPLIT_G>(nx, ny).total;
+  const int dyn = split_dyn_max();
   if (dyn <= 0 || smem > (size_t)dyn) return BIGINT_EINVAL;
   int dev = 0, sms = 0;
   BIGINT_CUDA_TRY(cudaGetDevice(&dev));
   BIGINT_CUDA_TRY(cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
   const int64_t units = count * T, grid = units < sms ? units : sms;
   const int nout = nx + ny;
-  tcm::k_mul_tc_split<SPLIT_NT, G><<<(unsigned)grid, 2 * SPLIT_NT + 32, smem, st>>>(
+  tcm::k_mul_tc_split<SPLIT_NT, SPLIT_G><<<(unsigned)grid, 2 * SPLIT_NT + 32, smem, st>>>(
       x, y, out, nx, ny, nout, count, T, tile_carry);
   int rc = bigint_launch_status();
   if (rc != BIGINT_OK) return rc;
@@ -1110,7 +1072,7 @@ constexpr size_t SPLIT_SMEM_CAP = 232448 - 2048;
 // or a single tile).
 int split_tiles(int nx, int ny) {
   if (nx < 1 || ny > 16383 || (8 * nx + 127) / 128 + (8 * ny + 127) / 128 <= 128) return 0;
-  if (tcm::layout<SPLIT_NT, 4>(nx, ny).total > SPLIT_SMEM_CAP) return 0;
+  if (tcm::layout<SPLIT_NT, SPLIT_G>(nx, ny).total > SPLIT_SMEM_CAP) return 0;
   const int T = (nx + ny + SPLIT_TILE_LIMBS - 1) / SPLIT_TILE_LIMBS;
   return T >= 2 ? T : 0;
 }
@@ -1149,13 +1111,7 @@ int launch_mul_split(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_
   const int T = split_tiles(nx, ny);
   if (T == 0) return launch_mul(a, b, out, count, na, nb, na + nb, st);
   uint64_t *tcarry = static_cast<uint64_t *>(ws);
-  const size_t s8 = tcm::layout<SPLIT_NT, 8>(nx, ny).total;
-  const size_t s4 = tcm::layout<SPLIT_NT, 4>(nx, ny).total;
-  if (split_dyn_max<8>() > 0 && s8 <= (size_t)split_dyn_max<8>())
-    return launch_split<8>(x, y, out, count, nx, ny, T, tcarry, st);
-  if (split_dyn_max<4>() > 0 && s4 <= (size_t)split_dyn_max<4>())
-    return launch_split<4>(x, y, out, count, nx, ny, T, tcarry, st);
-  return launch_mul(a, b, out, count, na, nb, na + nb, st);
+  return launch_split(x, y, out, count, nx, ny, T, tcarry, st);
 }
 
 // BIGINT_ETIMEOUT if a tensor-core product hit a wait limit since the last
