@@ -100,8 +100,8 @@ int bigint_mul_lo(const uint64_t *a, const uint64_t *b, uint64_t *out,
 
 /* The products of bigint_mul with each product spread over several CTAs,
  * for few, large products (serving), where one CTA per product would leave
- * most SMs idle.  Up to 16 products with a shorter operand of 256 limbs or
- * more: each product's output tiles (4096 limbs each) are cut further into
+ * most SMs idle.  Up to 16 products with a shorter operand of more than 512
+ * limbs: each product's output tiles (4096 limbs each) are cut further into
  * units of consecutive groups of Toeplitz blocks, about one unit per SM;
  * every unit adds its tile's partial column sums into a buffer in the
  * workspace with integer atomic adds (exact, in any order), and a cluster of
@@ -124,7 +124,7 @@ int bigint_mul_split(const uint64_t *a, const uint64_t *b, uint64_t *out,
  * disjoint from a and b), by `levels` levels of Karatsuba's method in its
  * subtractive form -- x y = z2 B^2k + (z0 + z2 + (x0 - x1)(y1 - y0)) B^k +
  * z0 with n = 2k -- every step batched across the instances, the leaf
- * products those of bigint_mul (tensor cores from 256 limbs).  The paper
+ * products batched the same way (tensor cores from 256 limbs).  The paper
  * names sub-quadratic multiplication as its next step; this is its exact
  * integer form.  levels: 0..3, or -1 for the measured choice on GB300 (two
  * from 8192 limbs, one from 4096, none below); a level that would not halve
@@ -157,9 +157,11 @@ int bigint_mul_kara(const uint64_t *a, const uint64_t *b, uint64_t *out, int64_t
  * step runs for all instances at once -- the leading ones in one launch, then
  * each product one batched launch of the multiply kernels, each linear step
  * one small launch -- and only instances whose divisor has a zero top limb
- * are divided one CTA each at the end.  Smaller divisions, and small batches
- * with quotients of at most four limbs, run one CTA per division (the
- * paper's intragroup form).  Results are the same either way.             */
+ * are divided at the end, a warp each (up to 512 by 127 limbs) or one CTA
+ * each.  Smaller divisions, small batches with quotients of at most four
+ * limbs, and quotients too long for every form of such a product (some
+ * 11,200 limbs) run one CTA per division (the paper's intragroup form).
+ * Results are the same either way.                                         */
 int bigint_divmod(const uint64_t *u, const uint64_t *v, uint64_t *q,
                   uint64_t *r, int32_t *status, int64_t count, int32_t nu,
                   int32_t nv, void *workspace, size_t workspace_bytes,
@@ -467,7 +469,7 @@ int bigint_host_sync(void);
  *   schoolbook product (Sec. V-B) as fp16 matrix products (tcgen05.mma)
  *   over signed base-256 digits with exact fp32 accumulation -- with its
  *   tile chosen by a cost model of its MMAs; bit-identical results.  Needs the shorter operand to fit shared memory
- *   (about 10700 limbs; otherwise variant 8).
+ *   (11215 limbs; otherwise variant 8).
  *   variants 13, 14, 15: variant 12 with 128-digit x blocks and tiles of
  *   64, 128, 256 output columns (three, two, one CTAs per SM)
  *   variants 16, 17: variant 12 with x blocks of 64 or 32 digits (128-column
