@@ -215,8 +215,8 @@ __global__ void __launch_bounds__(1024)
 //    2.9 us, 3.2 with 16), of four rounds above 4096 limbs (6000 limbs 3.6 us, 3.7
 //    with two), and one of two 24 if that makes one super-round.
 // Against 8 warps of four rounds (32 up to two instances per SM) at every size:
-// 64 additions of 512 limbs 1.97 -> 1.68 us, 400 of 1024 limbs 2.79 -> 2.63, 600
-// of 1536 limbs 3.70 -> 3.31, 304 of 8192 limbs 8.54 -> 7.29, 400 of 8193 limbs
+// 64 additions of 512 limbs 1.78 -> 1.45 us, 400 of 1024 limbs 2.77 -> 2.51, 600
+// of 1536 limbs 3.70 -> 3.29, 304 of 8192 limbs 8.54 -> 7.09, 400 of 8193 limbs
 // 15.4 -> 12.0, 2^26 limbs of 300 242 -> 224.
 //
 // The chain keeps 4 warps of four rounds (32 up to two instances per SM): its

@@ -212,8 +212,8 @@ constexpr int64_t FEW = 128;
 // One CTA per regular instance: r^ = (u - R) mod B^(nv+1) with R the low
 // nv + 1 limbs of q^ v, the exact correction of q^ (in place: the top limbs
 // of the banded product) and r^ (divmod.cu), and the results.  Irregular
-// instances are left to the last launch.  A tensor-core product of this division that gave up at a wait
-// limit (*aborted) voids the results: BIGINT_ETIMEOUT.
+// instances are left to the last launch.  A tensor-core product of this division
+// that gave up at a wait limit (*aborted) voids the results: BIGINT_ETIMEOUT.
 __global__ void __launch_bounds__(LIN_THREADS_FEW)
     k_ds_finish(const uint64_t *U, int nu, const uint64_t *V, int nv,
                 const uint64_t *R, int64_t sp, uint64_t *Rh, int64_t sd, uint64_t *Qh,
@@ -385,7 +385,8 @@ __global__ void __launch_bounds__(32 * LIST_WARPS)
   extern __shared__ __align__(16) uint64_t lsm[];
   const int lane = (int)lane_id(), wi = (int)(threadIdx.x >> 5), n = *nlist;
   uint64_t *un = lsm + (size_t)wi * list_warp_limbs(nu, nv), *vn = un + nu + 1;
-  for (int64_t e = (int64_t)blockIdx.x * LIST_WARPS + wi; e < n; e += (int64_t)gridDim.x * LIST_WARPS) {
+  for (int64_t e = (int64_t)blockIdx.x * LIST_WARPS + wi; e < n;
+       e += (int64_t)gridDim.x * LIST_WARPS) {
     const int64_t i = list[e];
     const uint64_t *u = U + i * nu, *v = V + i * nv;
     uint64_t *q = Qo + i * nq, *r = Ro + i * nv;
@@ -609,10 +610,12 @@ int launch_divmod_steps(const uint64_t *u, const uint64_t *v, uint64_t *q, uint6
   }
   // q^ = floor(u w / B^h), w of L + 2 limbs
   const int nw = L + 2, nz = nu + nw, nqh = nz - h;
-  rc = launch_mul_ex(u, nu, W[cur], Y.sw, Z, Y.sz, count, nu, nw, nz, h - 2, ctr + 1, st, STEP_TC_MIN, skp);
+  rc = launch_mul_ex(u, nu, W[cur], Y.sw, Z, Y.sz, count, nu, nw, nz, h - 2, ctr + 1, st,
+                     STEP_TC_MIN, skp);
   if (rc != BIGINT_OK) return rc;
   // R = q^ v mod B^(nv+1)
-  rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st, STEP_TC_MIN, skp);
+  rc = launch_mul_ex(Z + h, Y.sz, v, nv, P, Y.sp, count, nqh, nv, nv + 1, 0, ctr + 1, st,
+                     STEP_TC_MIN, skp);
   if (rc != BIGINT_OK) return rc;
   rc = chain_launch(few, k_ds_finish, (unsigned)count, lin, 0, st, u, nu, v, nv, P, Y.sp, D, Y.sd,
                     Z + h, Y.sz, nqh, q, nq, r, status, ctr + 1);

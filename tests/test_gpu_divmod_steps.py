@@ -152,7 +152,8 @@ def test_single_division_2_20_bits(bi, orc):
 
 @pytest.mark.parametrize("nu,nv,mul", [(12000, 8, 0), (16384, 8, 0), (12000, 64, 0),
                                        (16384, 64, 0), (12000, 127, 0), (16384, 127, 0),
-                                       (12000, 1000, 0), (16384, 1000, 0), (16384, 4096, 0), (16384, 5500, 0),
+                                       (12000, 1000, 0), (16384, 1000, 0), (16384, 4096, 0),
+                                       (16384, 5500, 0),
                                        (11224, 12, 0), (11225, 12, 0), (11700, 12, 0),
                                        (16384, 8192, 8)])
 def test_long_quotients(bi, orc, nu, nv, mul):
